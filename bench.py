@@ -735,11 +735,13 @@ def stage_work(rz, needed, V, pixels, blended):
     bits = max(1, int(np.ceil(np.log2(max(tiles, 2)))))
     passes = max(1, (bits + 7) // 8)
     vb = max(1, int(R - 1).bit_length())  # record-id bits
+    # the measure of the tile sort's work: the bytes a radix sort of all (record,
+    # tile) entries moves, so that its fraction stays comparable (the lists are
+    # built through coarser bins and move fewer bytes than this)
     if passes == 2 and (bits - 8) + vb <= 32:
-        # packed two-pass tile sort: duplication writes a 16-bit tile id and a
-        # record id, pass 0 reads them and writes one word, pass 1 reads it
-        # twice (histogram, scatter) and writes the record id; the duplication
-        # reads each record's id, descriptor and entry offset
+        # packed two passes: a 16-bit tile id and a record id generated, read
+        # and written as one word, which is read twice (histogram, scatter) and
+        # leaves the record id; each record's id, descriptor and offset
         tile_sort_bytes = 28.0 * K + 20.0 * R
     else:
         tile_sort_bytes = 8.0 * K + passes * 16.0 * K - 4.0 * K + 20.0 * R

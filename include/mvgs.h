@@ -30,7 +30,7 @@
  *     needs into a caller-owned `state` buffer.  Sizes come from
  *     mvgs_render_layout() / mvgs_dssim_workspace_size().
  *   - Every call is asynchronous on the given CUDA stream, except that
- *     mvgs_render_views synchronises the stream twice to read the number of
+ *     mvgs_render_views synchronises the stream once to read the number of
  *     visible (Gaussian, view) records and of duplicated keys back to the
  *     host (they size the sorts) -- unless MVGS_FLAG_CAPTURABLE is set.
  *   - Every call returns an mvgs_status; no exception crosses the ABI.
@@ -132,8 +132,9 @@ typedef struct mvgs_config {
  * captured in a CUDA graph (with the backward, the losses and the ADC call).
  * `needed` gets -1s.  Results are valid only if the counts block of the state
  * (layout.off_counts) shows needed counts within the capacity afterwards:
- * otherwise the records and keys past it were dropped, and the caller grows
- * the buffers and runs again. */
+ * otherwise the records past it were dropped -- and with too few keys every
+ * tile's list is empty, so the images show the background -- and the caller
+ * grows the buffers and runs again. */
 #define MVGS_FLAG_CAPTURABLE 4u
 /* cfg->flags bit for the forward calls: also write the per-pixel statistics
  * (layout.off_pixel_stats: where the pixel stopped and how many Gaussians it
@@ -200,7 +201,7 @@ mvgs_status mvgs_count_views(const mvgs_scene* scene, const mvgs_camera* cams, i
  *   needed     out (host): the record and key counts this batch needs.
  * If a count exceeds `cap`, returns MVGS_ENOSPACE after reporting `needed`;
  * the caller re-sizes with mvgs_render_layout and calls again.
- * Synchronises `stream` twice (record and key count read-back). */
+ * Synchronises `stream` once (record and key count read-back). */
 mvgs_status mvgs_render_views(const mvgs_scene* scene, const mvgs_camera* cams, int32_t V, const mvgs_config* cfg,
                               const mvgs_capacity* cap, float* images, void* state, size_t state_bytes,
                               void* workspace, size_t workspace_bytes, mvgs_capacity* needed, mvgs_stream stream);
@@ -440,10 +441,10 @@ typedef enum mvgs_stage {
     MVGS_STAGE_SCAN_RECORDS,      /* record offsets                            */
     MVGS_STAGE_PREPROCESS,        /* projection, colour, radius, rect          */
     MVGS_STAGE_DEPTH_SORT,        /* records by depth                          */
-    MVGS_STAGE_SCAN_TILES,        /* key offsets                               */
-    MVGS_STAGE_TILE_SORT,         /* one entry per (record, tile), generated
-                                     in the first pass, sorted by (view, tile) */
-    MVGS_STAGE_RANGES,            /* per-tile list ranges from the rectangles  */
+    MVGS_STAGE_SCAN_TILES,        /* offsets of the (record, bin) entries      */
+    MVGS_STAGE_TILE_SORT,         /* (record, bin) entries sorted by bin, then
+                                     expanded into the tiles' lists            */
+    MVGS_STAGE_RANGES,            /* per-tile list ranges and processing order */
     MVGS_STAGE_BLEND_FORWARD,
     MVGS_STAGE_ZERO_GRADS,
     MVGS_STAGE_BLEND_BACKWARD,

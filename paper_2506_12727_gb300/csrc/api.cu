@@ -118,12 +118,12 @@ struct Plan {
     int V = 0;
     long long n = 0;
     std::vector<DevCam> cams;
-    long long tiles = 0, pixels = 0;
+    long long tiles = 0, pixels = 0, bins = 0;
     mvgs_layout L{};
     // workspace offsets (forward)
     size_t w_cams = 0, w_counts = 0, w_vis = 0, w_scan = 0, w_dkeys_a = 0, w_dkeys_b = 0, w_ids_a = 0, w_ids_b = 0,
-           w_order = 0, w_tiles = 0, w_desc = 0, w_tile_off = 0, w_keys_a = 0, w_keys_b = 0, w_vals_a = 0, w_vals_b = 0,
-           w_radix = 0, w_tcount = 0, w_torder = 0, w_counter = 0, w_dcount = 0;
+           w_order = 0, w_bins = 0, w_desc = 0, w_bin_off = 0, w_keys_a = 0, w_keys_b = 0, w_vals_a = 0, w_vals_b = 0,
+           w_radix = 0, w_lists = 0, w_torder = 0, w_counter = 0, w_dcount = 0;
     // workspace offsets of the sampled blend (forward and backward each carve their own)
     size_t w_chunk_off = 0, w_chunk_map = 0, w_chunk_tmp = 0, w_mask = 0;
     size_t b_chunk_off = 0, b_chunk_map = 0, b_chunk_tmp = 0, b_mask = 0;
@@ -166,13 +166,13 @@ mvgs_status make_plan(long long n, const mvgs_camera* cams, int V, const mvgs_co
     P.V = V;
     P.n = n;
     P.cams.resize(V);
-    long long tiles = 0, pixels = 0, cells = 0;
+    long long tiles = 0, pixels = 0, bins = 0;
     for (int v = 0; v < V; v++) {
         const mvgs_camera& c = cams[v];
         if (c.width < 1 || c.height < 1) return fail(MVGS_EINVAL, "view %d: empty image", v);
         if (!(c.fx > 0.f) || !(c.fy > 0.f)) return fail(MVGS_EINVAL, "view %d: focal lengths must be > 0", v);
         const int txs = (c.width + tw - 1) / tw, tys = (c.height + th - 1) / th;
-        // tile coordinates travel in 12-bit fields of the duplication's record descriptors
+        // tile coordinates travel in 12-bit fields of the records' tile descriptors
         if (txs > 4095 || tys > 4095) return fail(MVGS_EOVERFLOW, "view %d: more than 4095 tiles per axis", v);
         DevCam& d = P.cams[v];
         for (int i = 0; i < 3; i++) {
@@ -188,14 +188,15 @@ mvgs_status make_plan(long long n, const mvgs_camera* cams, int V, const mvgs_co
         d.tiles_x = txs; d.tiles_y = tys;
         d.tile_base = tiles;
         d.pix_base = pixels;
-        d.diff_base = cells;
-        cells += (long long)(txs + 1) * (tys + 1);
+        d.bin_base = bins;
+        bins += (long long)bins_across(txs) * bins_across(tys);
         tiles += (long long)txs * tys;
         pixels += (long long)c.width * c.height;
     }
     if (tiles >= (1LL << 32)) return fail(MVGS_EOVERFLOW, "more than 2^32 tiles over all views");
     P.tiles = tiles;
     P.pixels = pixels;
+    P.bins = bins;
 
     const size_t R = (size_t)cap->records, K = (size_t)cap->keys;
     mvgs_layout& L = P.L;
@@ -233,19 +234,19 @@ mvgs_status make_plan(long long n, const mvgs_camera* cams, int V, const mvgs_co
     P.w_ids_a = w.take(R * sizeof(uint32_t));
     P.w_ids_b = w.take(R * sizeof(uint32_t));
     P.w_order = w.take(R * sizeof(uint32_t));
-    P.w_tiles = w.take(R * sizeof(uint32_t));
+    P.w_bins = w.take(R * sizeof(uint32_t));
     P.w_desc = w.take(R * sizeof(unsigned long long));
-    P.w_tile_off = w.take((R + 1) * sizeof(unsigned long long));
+    P.w_bin_off = w.take((R + 1) * sizeof(unsigned long long));
     P.w_keys_a = w.take(K * sizeof(uint32_t));
     P.w_keys_b = w.take(K * sizeof(uint32_t));
     P.w_vals_a = w.take(K * sizeof(uint32_t));
     P.w_vals_b = w.take(K * sizeof(uint32_t));
-    P.w_radix = w.take(radix_temp_bytes(big) > tile_sort_temp_bytes(K) ? radix_temp_bytes(big)
-                                                                          : tile_sort_temp_bytes(K));
-    P.w_tcount = w.take(tile_count_temp_bytes(P.cams.data(), V, tiles));
+    P.w_radix = w.take(radix_temp_bytes(big));
+    // every (record, bin) entry holds at least one tile: at most K of them
+    P.w_lists = w.take(tile_lists_temp_bytes(K, bins, tiles));
     P.w_torder = w.take(tile_order_temp_bytes(tiles));
     P.w_counter = w.take(sizeof(int));
-    P.w_dcount = w.take(4 * sizeof(unsigned long long));
+    P.w_dcount = w.take((8 + 2 * kSumSlots) * sizeof(unsigned long long));
     // runs of at least 32 samples: at most one partial run per tile
     P.chunk_cap = tiles + pixels / 32 + 1;
     P.w_chunk_off = w.take((size_t)(tiles + 1) * sizeof(long long));
@@ -323,15 +324,28 @@ __global__ void set_counts_kernel(long long* c, long long R, long long K, long l
     c[5] = K;
 }
 
-// capturable mode: the counts stay on the device
-__global__ void clamp_records_kernel(const long long* rec_total, long long cap, unsigned long long* dcnt) {
-    const long long R = *rec_total;
-    dcnt[0] = (unsigned long long)(R < cap ? R : cap);
-}
-
-__global__ void clamp_keys_kernel(long long cap, unsigned long long* dcnt) {
-    const unsigned long long K = dcnt[1];
-    dcnt[2] = K < (unsigned long long)cap ? K : (unsigned long long)cap;
+// The batch's counts, from the record scan and the preprocessing's sums:
+// dcnt = records held, keys needed, keys held, (record, bin) entries held,
+// records needed ("held": within the capacity).
+__global__ void total_counts_kernel(const long long* rec_total, const unsigned long long* sums, long long rec_cap,
+                                    long long key_cap, unsigned long long* dcnt) {
+    unsigned long long k = 0, b = 0;
+    for (int i = threadIdx.x; i < kSumSlots; i += 32) {
+        k += sums[2 * i];
+        b += sums[2 * i + 1];
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        k += __shfl_xor_sync(0xffffffffu, k, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    if (threadIdx.x == 0) {
+        const unsigned long long r = (unsigned long long)*rec_total, kc = (unsigned long long)key_cap;
+        dcnt[0] = r < (unsigned long long)rec_cap ? r : (unsigned long long)rec_cap;
+        dcnt[1] = k;
+        dcnt[2] = k < kc ? k : kc;
+        dcnt[3] = b < kc ? b : kc;
+        dcnt[4] = r;
+    }
 }
 
 __global__ void set_counts_dev_kernel(long long* c, const long long* rec_total, const unsigned long long* dcnt,
@@ -342,12 +356,6 @@ __global__ void set_counts_dev_kernel(long long* c, const long long* rec_total, 
     c[3] = P;
     c[4] = *rec_total;
     c[5] = (long long)dcnt[1];
-}
-
-int bits_for(long long tiles) {
-    int b = 0;
-    while (b < 63 && (1LL << b) < tiles) b++;
-    return b;
 }
 
 // Points the blend at a sample set: sampled runs (Alg. 3) or, with the
@@ -458,7 +466,9 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
     const long long n = scene->n;
     const int tw = cfg->tile_w, th = cfg->tile_h;
     DevCam* dcams = at<DevCam>(workspace, P.w_cams);
-    upload_cams(P.cams.data(), V, dcams, s);
+    unsigned long long* dcnt = at<unsigned long long>(workspace, P.w_dcount);
+    unsigned long long* sums = dcnt + 8;
+    upload_cams(P.cams.data(), V, dcams, s, sums, 2 * kSumSlots);
     const SceneArgs sc = scene_args(scene);
     RecordArgs rec = record_args(state, L);
     long long* counts_dev = at<long long>(state, L.off_counts);
@@ -473,18 +483,30 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
         StageTimer t(MVGS_STAGE_SCAN_RECORDS, s);
         scan_i32_to_i64(counts, rec.rec_off, (uint64_t)n, at<void>(workspace, P.w_scan), s);
     }
-    // Without MVGS_FLAG_CAPTURABLE the record and key counts are read back to
-    // size the sorts exactly; with it they stay on the device and every
-    // launch is sized by the capacity (the kernels stop at the device count),
-    // so the call can be captured in a CUDA graph.
+    // projection, colour, radius and tile rectangle of every record, its bin
+    // count and its tile descriptor (rectangle and view in 8 bytes), and the
+    // batch's totals; records past the capacity are not written
+    rec.cap = cap->records;
+    uint32_t* bins = at<uint32_t>(workspace, P.w_bins);
+    unsigned long long* desc = at<unsigned long long>(workspace, P.w_desc);
+    {
+        StageTimer t(MVGS_STAGE_PREPROCESS, s);
+        launch_preprocess(sc, dcams, V, tw, th, at<uint8_t>(workspace, P.w_vis), rec, bins, desc, sums, s);
+        total_counts_kernel<<<1, 32, 0, s>>>(rec.rec_off + n, sums, cap->records, cap->keys, dcnt);
+        note_launches(1);
+    }
+    // Without MVGS_FLAG_CAPTURABLE the counts are read back to size the sorts
+    // exactly; with it they stay on the device and every launch is sized by
+    // the capacity (the kernels stop at the device count), so the call can be
+    // captured in a CUDA graph.
     const bool capt = (cfg->flags & MVGS_FLAG_CAPTURABLE) != 0;
-    unsigned long long* dcnt = at<unsigned long long>(workspace, P.w_dcount);
-    long long R = 0;
+    unsigned long long c[5] = {0, 0, 0, 0, 0};
     if (!capt) {
-        if (cudaMemcpyAsync(&R, rec.rec_off + n, sizeof(long long), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        if (cudaMemcpyAsync(c, dcnt, sizeof(c), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess)
-            return cuda_check("record count read-back");
-        if ((st = cuda_check("participation")) != MVGS_OK) return st;
+            return cuda_check("count read-back");
+        if ((st = cuda_check("participation and preprocess")) != MVGS_OK) return st;
+        const long long R = (long long)c[4];
         if (needed) {
             needed->records = R;
             needed->keys = 0;
@@ -492,80 +514,49 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
         if (R > cap->records)
             return fail(MVGS_ENOSPACE, "%lld visible records exceed the capacity of %lld", R,
                         (long long)cap->records);
-        rec.cap = R;
-    } else {
-        clamp_records_kernel<<<1, 1, 0, s>>>(rec.rec_off + n, cap->records, dcnt);
-        note_launches(1);
-        rec.cap = cap->records;
-        if (needed) {
-            needed->records = -1;  // on the device: counts block of the state
-            needed->keys = -1;
-        }
+        if (needed) needed->keys = (long long)c[1];
+        if (c[1] >= (1ULL << 32)) return fail(MVGS_EOVERFLOW, "%llu keys do not fit 32-bit positions", c[1]);
+        if ((long long)c[1] > cap->keys)
+            return fail(MVGS_ENOSPACE, "%llu keys exceed the capacity of %lld", c[1], (long long)cap->keys);
+    } else if (needed) {
+        needed->records = -1;  // on the device: counts block of the state
+        needed->keys = -1;
     }
-    const Count Rc = capt ? Count((unsigned long long)cap->records, dcnt) : Count((unsigned long long)R);
-
-    // projection, colour, radius and tile rectangle of every record, its tile
-    // count and its tile descriptor (rectangle and view in 8 bytes)
-    uint32_t* tiles = at<uint32_t>(workspace, P.w_tiles);
-    unsigned long long* desc = at<unsigned long long>(workspace, P.w_desc);
-    {
-        StageTimer t(MVGS_STAGE_PREPROCESS, s);
-        launch_preprocess(sc, dcams, V, tw, th, at<uint8_t>(workspace, P.w_vis), rec, tiles, desc, s);
-    }
+    const Count Rc = capt ? Count((unsigned long long)cap->records, dcnt) : Count(c[0]);
+    const Count Kc = capt ? Count((unsigned long long)cap->keys, dcnt + 2) : Count(c[1]);
+    const Count Sc = capt ? Count((unsigned long long)cap->keys, dcnt + 3) : Count(c[3]);
 
     // records by depth (the keys are the records' float32 depths, positive, so
     // their bits sort as unsigned integers; the values the record indices),
-    // with each record's tile count carried into depth order by the last pass;
-    // then keys per covered tile in that order
+    // with each record's bin count carried into depth order by the last pass;
+    // then the tiles' lists in that order
     uint32_t* order = at<uint32_t>(workspace, P.w_order);
-    uint32_t* tiles_by_depth = at<uint32_t>(workspace, P.w_ids_a);
+    uint32_t* bins_by_depth = at<uint32_t>(workspace, P.w_ids_a);
     {
         StageTimer t(MVGS_STAGE_DEPTH_SORT, s);
         radix_sort_pairs(reinterpret_cast<const uint32_t*>(rec.depth), nullptr, at<uint32_t>(workspace, P.w_dkeys_a),
-                         tiles_by_depth, at<uint32_t>(workspace, P.w_dkeys_b), at<uint32_t>(workspace, P.w_ids_b),
-                         order, Rc, 32, at<void>(workspace, P.w_radix), s, tiles, tiles_by_depth);
+                         bins_by_depth, at<uint32_t>(workspace, P.w_dkeys_b), at<uint32_t>(workspace, P.w_ids_b),
+                         order, Rc, 32, at<void>(workspace, P.w_radix), s, bins, bins_by_depth);
     }
-    unsigned long long* tile_off = at<unsigned long long>(workspace, P.w_tile_off);
+    unsigned long long* bin_off = at<unsigned long long>(workspace, P.w_bin_off);
     {
         StageTimer t(MVGS_STAGE_SCAN_TILES, s);
-        scan_u32_to_u64_count(tiles_by_depth, tile_off, Rc, capt ? dcnt + 1 : nullptr, at<void>(workspace, P.w_scan),
-                              s);
+        scan_u32_to_u64_count(bins_by_depth, bin_off, Rc, nullptr, at<void>(workspace, P.w_scan), s);
     }
-    unsigned long long K = 0;
-    if (!capt) {
-        if (cudaMemcpyAsync(&K, tile_off + R, sizeof(K), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess)
-            return cuda_check("key count read-back");
-        if ((st = cuda_check("preprocess")) != MVGS_OK) return st;
-        if (needed) needed->keys = (long long)K;
-        if (K >= (1ULL << 32)) return fail(MVGS_EOVERFLOW, "%llu keys do not fit 32-bit positions", K);
-        if ((long long)K > cap->keys)
-            return fail(MVGS_ENOSPACE, "%llu keys exceed the capacity of %lld", K, (long long)cap->keys);
-    } else {
-        clamp_keys_kernel<<<1, 1, 0, s>>>(cap->keys, dcnt);
-        note_launches(1);
-    }
-    const Count Kc = capt ? Count((unsigned long long)cap->keys, dcnt + 2) : Count(K);
-
     uint32_t* sorted = at<uint32_t>(state, L.off_sorted_records);
-    {
-        StageTimer t(MVGS_STAGE_TILE_SORT, s);
-        tile_sort(order, tile_off, Rc, Kc, desc, dcams, P.tiles, bits_for(P.tiles),
-                  at<uint32_t>(workspace, P.w_keys_a), at<uint32_t>(workspace, P.w_vals_a),
-                  at<uint32_t>(workspace, P.w_keys_b), at<uint32_t>(workspace, P.w_vals_b), sorted,
-                  at<void>(workspace, P.w_radix), s);
-    }
     long long* ranges = at<long long>(state, L.off_tile_ranges);
+    tile_lists(order, bin_off, Rc, Sc, Kc, desc, dcams, V, P.bins, P.tiles, at<uint32_t>(workspace, P.w_keys_a),
+               at<uint32_t>(workspace, P.w_vals_a), at<uint32_t>(workspace, P.w_keys_b),
+               at<uint32_t>(workspace, P.w_vals_b), sorted, ranges, (uint64_t)cap->keys,
+               at<void>(workspace, P.w_lists), at<void>(workspace, P.w_radix), s);
     {
         StageTimer t(MVGS_STAGE_RANGES, s);
-        tile_ranges_from_rects(rec.rect, rec.rec_v, Rc, Kc, dcams, P.cams.data(), V, P.tiles, ranges,
-                               at<void>(workspace, P.w_tcount), s);
         tile_order(ranges, P.tiles, at<uint32_t>(state, L.off_tile_order), at<void>(workspace, P.w_torder), s);
     }
     if (capt)
         set_counts_dev_kernel<<<1, 1, 0, s>>>(counts_dev, rec.rec_off + n, dcnt, P.tiles, P.pixels);
     else
-        set_counts_kernel<<<1, 1, 0, s>>>(counts_dev, R, (long long)K, P.tiles, P.pixels);
+        set_counts_kernel<<<1, 1, 0, s>>>(counts_dev, (long long)c[0], (long long)c[1], P.tiles, P.pixels);
     note_launches(1);
 
     BlendArgs ba;

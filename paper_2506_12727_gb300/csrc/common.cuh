@@ -31,7 +31,7 @@ struct __align__(16) DevCam {
     int W, H, tiles_x, tiles_y;
     long long tile_base;  // first global tile id of the view
     long long pix_base;   // first pixel of the view in the packed layout
-    long long diff_base;  // first cell of the view's (tiles_y + 1) x (tiles_x + 1) count grid
+    long long bin_base;   // first bin of the view (8 x 8 tiles each, row-major)
 };
 static_assert(sizeof(DevCam) == 128, "camera table entry is 128 bytes");
 
@@ -148,6 +148,14 @@ __device__ __forceinline__ short4 tile_desc_rect(unsigned long long d) {
                        (short)(d >> 36 & 0xfffu));
 }
 __device__ __forceinline__ int tile_desc_view(unsigned long long d) { return (int)(d >> 48); }
+
+// Bins of 8 x 8 tiles (sort.cu): bins along an axis of `tiles` tiles, and the
+// bins a tile rectangle reaches.
+__host__ __device__ __forceinline__ int bins_across(int tiles) { return (tiles + 7) >> 3; }
+__device__ __forceinline__ uint32_t bins_touched(short4 rc) {
+    if (rc.z <= rc.x || rc.w <= rc.y) return 0u;
+    return (uint32_t)((((rc.z - 1) >> 3) - (rc.x >> 3) + 1) * (((rc.w - 1) >> 3) - (rc.y >> 3) + 1));
+}
 
 struct ColTerms {
     float xx, x;  // qa dx^2 and qb dx

@@ -31,7 +31,9 @@ class StageTimer {
 };
 
 // ---- preprocess.cu -------------------------------------------------------
-void upload_cams(const DevCam* host, int V, DevCam* dst, cudaStream_t s);
+// Uploads the camera table; also zeroes `zero_count` words at `zero` when given.
+void upload_cams(const DevCam* host, int V, DevCam* dst, cudaStream_t s, unsigned long long* zero = nullptr,
+                 int zero_count = 0);
 
 struct SceneArgs {
     long long n;
@@ -63,11 +65,13 @@ void launch_count_keys(const SceneArgs& sc, const DevCam* cams, int V, int tw, i
 // vis: [n * V] bytes, 1 where (g, v) is visible; counts: visible views per Gaussian.
 void launch_count_visible(const SceneArgs& sc, const DevCam* cams, int V, int tw, int th, int* counts, uint8_t* vis,
                           cudaStream_t s);
-// Writes all records of the visible pairs, the number of tiles each record
-// touches and its tile descriptor (pack_tile_desc).
+// Writes all records of the visible pairs, the number of bins each record
+// touches and its tile descriptor (pack_tile_desc), and adds the records' tile
+// and bin totals into kSumSlots pairs of sums (zeroed by the caller).
+constexpr int kSumSlots = 128;
 void launch_preprocess(const SceneArgs& sc, const DevCam* cams, int V, int tw, int th, const uint8_t* vis,
-                       const RecordArgs& rec, uint32_t* tiles_touched, unsigned long long* tile_desc,
-                       cudaStream_t s);
+                       const RecordArgs& rec, uint32_t* bins, unsigned long long* tile_desc,
+                       unsigned long long* sums, cudaStream_t s);
 void launch_zero_f32(float* p, size_t count, cudaStream_t s);
 // rec_grad: [records, kGradStride] float (mean2d x, y, opacity, rgb, e1 at
 // 0, 1, 2, 3..5, 6); rec_conic: [records, 3] double (conic A, B, C).
@@ -86,15 +90,11 @@ void scan_i32_to_i64(const int* in, long long* out, uint64_t n, void* tmp, cudaS
 // scans in[i] & mask
 void scan_masked_i32_to_i64(const int* in, int mask, long long* out, uint64_t n, void* tmp, cudaStream_t s);
 void scan_u32_to_u64(const uint32_t* in, unsigned long long* out, uint64_t n, void* tmp, cudaStream_t s);
-// gathered variant: scans in[idx[i]]
 // (also the total into *total when given; n may be a device count)
 void scan_u32_to_u64_count(const uint32_t* in, unsigned long long* out, Count n, unsigned long long* total,
                            void* tmp, cudaStream_t s);
-void scan_gather_u32_to_u64(const uint32_t* in, const uint32_t* idx, unsigned long long* out, Count n,
-                            unsigned long long* total, void* tmp, cudaStream_t s);
 
 size_t radix_temp_bytes(uint64_t n);
-size_t tile_sort_temp_bytes(uint64_t K);
 // Stable LSD sort of (key, value) pairs on key bits [0, bits).  Input in
 // (keys0, vals0), read only; vals0 == nullptr sorts the identity permutation
 // (values generated, not read).  keys_a/b and vals_a/b are scratch; the sorted
@@ -104,27 +104,22 @@ void radix_sort_pairs(const uint32_t* keys0, const uint32_t* vals0, uint32_t* ke
                       uint32_t* keys_b, uint32_t* vals_b, uint32_t* vals_out, Count n, int bits, void* tmp,
                       cudaStream_t s, const uint32_t* gather_src = nullptr, uint32_t* gather_out = nullptr);
 
-// Stable sort, by global (view, tile) id, of one entry per (record, covered
-// tile) taken in the order of `order` (records sorted by depth); tile_off is
-// the exclusive scan of the records' tile counts in that order; desc holds the
-// records' tile descriptors (pack_tile_desc, record order).  The entries
-// are generated by the first pass's histogram kernel (the duplication) and
-// written to keys_a / vals_a (16-bit tile ids when the sort runs packed).
-// Sorted record ids end in vals_out; keys_a/b and vals_a/b are scratch of K
-// entries.
-void tile_sort(const uint32_t* order, const unsigned long long* tile_off, Count R, Count K,
-               const unsigned long long* desc, const DevCam* cams, long long tiles, int bits, uint32_t* keys_a,
-               uint32_t* vals_a, uint32_t* keys_b, uint32_t* vals_b, uint32_t* vals_out, void* tmp, cudaStream_t s);
+// The per-tile lists: record ids by (view, tile, depth), of one entry per
+// (record, covered tile), and every tile's [start, end).  `order`: records
+// sorted by depth; bin_off: exclusive scan of their bin counts in that order;
+// S: (record, bin) entries; K: room in `sorted` (nothing is placed, and every
+// range is empty, when the lists hold more); desc: tile descriptors
+// (pack_tile_desc, record order).  keys_a/b and vals_a/b are scratch of S_cap
+// entries each.
+size_t tile_lists_temp_bytes(uint64_t S, long long bins, long long tiles);
+void tile_lists(const uint32_t* order, const unsigned long long* bin_off, Count R, Count S, Count K,
+                const unsigned long long* desc, const DevCam* cams, int V, long long bins, long long tiles,
+                uint32_t* keys_a, uint32_t* vals_a, uint32_t* keys_b, uint32_t* vals_b, uint32_t* sorted,
+                long long* ranges, uint64_t S_cap, void* tmp, void* radix_tmp, cudaStream_t s);
 
 // Tiles ordered by decreasing list length (the blend's processing order).
 size_t tile_order_temp_bytes(long long tiles);
 void tile_order(const long long* ranges, long long tiles, uint32_t* order, void* tmp, cudaStream_t s);
-
-// Per-tile [start, end) of the sorted list, from the records' rectangles.
-size_t tile_count_temp_bytes(const DevCam* host_cams, int V, long long tiles);
-void tile_ranges_from_rects(const short4* rect, const int* rec_v, Count R, Count K, const DevCam* cams,
-                            const DevCam* host_cams, int V, long long tiles, long long* ranges, void* tmp,
-                            cudaStream_t s);
 
 // ---- blend.cu --------------------------------------------------------------
 struct BlendArgs {

@@ -233,8 +233,9 @@ __device__ __forceinline__ bool project(const Gauss& G, const DevCam& cam, int t
 }
 
 // ---- kernels ---------------------------------------------------------------
-__global__ void upload_cams_kernel(CamChunk chunk, int count, DevCam* dst) {
+__global__ void upload_cams_kernel(CamChunk chunk, int count, DevCam* dst, unsigned long long* zero, int zero_count) {
     if ((int)threadIdx.x < count) dst[threadIdx.x] = chunk.c[threadIdx.x];
+    for (int i = threadIdx.x; i < zero_count; i += blockDim.x) zero[i] = 0ull;
 }
 
 // Visibility of every (Gaussian, view) pair: one byte per pair (view-minor)
@@ -331,8 +332,9 @@ constexpr int PRE_THREADS = 128;
 template <int DEG>
 __global__ void __launch_bounds__(PRE_THREADS, 8) preprocess_kernel(SceneArgs sc, const DevCam* __restrict__ cams, int V,
                                                                  int tw, int th, const uint8_t* __restrict__ vis,
-                                                                 RecordArgs rec, uint32_t* __restrict__ tiles_touched,
-                                                                 unsigned long long* __restrict__ tile_desc) {
+                                                                 RecordArgs rec, uint32_t* __restrict__ bins,
+                                                                 unsigned long long* __restrict__ tile_desc,
+                                                                 unsigned long long* __restrict__ sums) {
     constexpr int NK = (DEG + 1) * (DEG + 1);
     const int lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
@@ -362,37 +364,50 @@ __global__ void __launch_bounds__(PRE_THREADS, 8) preprocess_kernel(SceneArgs sc
         const uint32_t bal = __ballot_sync(0xffffffffu, on);
         const long long r = rbase + __popc(bal & lt);
         rbase += __popc(bal);
-        // capturable mode past its record capacity: not written (reported through the counts)
-        if (!on || r >= rec.cap) continue;
-        const DevCam& cam = cams[v];
-        Proj P;
-        const bool ok = project(G, cam, tw, th, P);
-        if (!ok) P.rect = make_short4(0, 0, 0, 0);  // same decision as the count pass, kept safe regardless
-        const float inv = 1.f / P.det;
-        rec.rec_g[r] = (int)g;
-        rec.rec_v[r] = v;
-        rec.xy[r] = P.xy;
-        rec.conic_o[r] = make_float4(P.c * inv, -P.b * inv, P.a * inv, G.o);
-        // colour from the direction camera -> mean
-        float dx = G.mu[0] - cam.campos[0], dy = G.mu[1] - cam.campos[1], dz = G.mu[2] - cam.campos[2];
-        const float il = rsqrtf(dx * dx + dy * dy + dz * dz);
-        dx *= il; dy *= il; dz *= il;
-        float Y[NK];
-        sh_basis<DEG>(dx, dy, dz, Y);
-        float rgb[3] = {0.5f, 0.5f, 0.5f};
-        int clamp = 0;
+        // past the record capacity nothing is written (the counts tell)
+        uint32_t nt = 0, nb = 0;  // the record's tiles and bins
+        if (on && r < rec.cap) {
+            const DevCam& cam = cams[v];
+            Proj P;
+            const bool ok = project(G, cam, tw, th, P);
+            if (!ok) P.rect = make_short4(0, 0, 0, 0);  // same decision as the count pass, kept safe regardless
+            const float inv = 1.f / P.det;
+            rec.rec_g[r] = (int)g;
+            rec.rec_v[r] = v;
+            rec.xy[r] = P.xy;
+            rec.conic_o[r] = make_float4(P.c * inv, -P.b * inv, P.a * inv, G.o);
+            // colour from the direction camera -> mean
+            float dx = G.mu[0] - cam.campos[0], dy = G.mu[1] - cam.campos[1], dz = G.mu[2] - cam.campos[2];
+            const float il = rsqrtf(dx * dx + dy * dy + dz * dz);
+            dx *= il; dy *= il; dz *= il;
+            float Y[NK];
+            sh_basis<DEG>(dx, dy, dz, Y);
+            float rgb[3] = {0.5f, 0.5f, 0.5f};
+            int clamp = 0;
 #pragma unroll
-        for (int e = 0; e < E; e++) rgb[e % 3] += Y[e / 3] * shc[e];
+            for (int e = 0; e < E; e++) rgb[e % 3] += Y[e / 3] * shc[e];
 #pragma unroll
-        for (int ch = 0; ch < 3; ch++) {
-            if (rgb[ch] < 0.f) { clamp |= 1 << ch; rgb[ch] = 0.f; }
+            for (int ch = 0; ch < 3; ch++) {
+                if (rgb[ch] < 0.f) { clamp |= 1 << ch; rgb[ch] = 0.f; }
+            }
+            rec.rgb_r[r] = make_float4(rgb[0], rgb[1], rgb[2], (float)P.radius);
+            rec.clamp[r] = clamp;
+            rec.depth[r] = P.depth;
+            rec.rect[r] = P.rect;
+            const uint32_t touched = bins_touched(P.rect);
+            bins[r] = touched;
+            tile_desc[r] = pack_tile_desc(P.rect, v);
+            nt = (uint32_t)((P.rect.z - P.rect.x) * (P.rect.w - P.rect.y));
+            nb = touched;
         }
-        rec.rgb_r[r] = make_float4(rgb[0], rgb[1], rgb[2], (float)P.radius);
-        rec.clamp[r] = clamp;
-        rec.depth[r] = P.depth;
-        rec.rect[r] = P.rect;
-        tiles_touched[r] = (uint32_t)((P.rect.z - P.rect.x) * (P.rect.w - P.rect.y));
-        tile_desc[r] = pack_tile_desc(P.rect, v);
+        // the warp's totals, spread over kSumSlots pairs of counters
+        nt = __reduce_add_sync(0xffffffffu, nt);
+        nb = __reduce_add_sync(0xffffffffu, nb);
+        if (lane == 0 && nb > 0) {
+            unsigned long long* slot = sums + 2 * (blockIdx.x % kSumSlots);
+            atomicAdd(slot, (unsigned long long)nt);
+            atomicAdd(slot + 1, (unsigned long long)nb);
+        }
     }
 }
 
@@ -597,12 +612,12 @@ unsigned blocks_for(long long n, int threads) { return (unsigned)((n + threads -
 
 }  // namespace
 
-void upload_cams(const DevCam* host, int V, DevCam* dst, cudaStream_t s) {
+void upload_cams(const DevCam* host, int V, DevCam* dst, cudaStream_t s, unsigned long long* zero, int zero_count) {
     for (int start = 0; start < V; start += kCamChunk) {
         CamChunk chunk;
         const int cnt = V - start < kCamChunk ? V - start : kCamChunk;
         for (int i = 0; i < cnt; i++) chunk.c[i] = host[start + i];
-        upload_cams_kernel<<<1, kCamChunk, 0, s>>>(chunk, cnt, dst + start);
+        upload_cams_kernel<<<1, kCamChunk, 0, s>>>(chunk, cnt, dst + start, zero, start == 0 ? zero_count : 0);
         note_launches(1);
     }
 }
@@ -622,14 +637,14 @@ void launch_count_visible(const SceneArgs& sc, const DevCam* cams, int V, int tw
 }
 
 void launch_preprocess(const SceneArgs& sc, const DevCam* cams, int V, int tw, int th, const uint8_t* vis,
-                       const RecordArgs& rec, uint32_t* tiles_touched, unsigned long long* tile_desc,
-                       cudaStream_t s) {
+                       const RecordArgs& rec, uint32_t* bins, unsigned long long* tile_desc,
+                       unsigned long long* sums, cudaStream_t s) {
     if (sc.n == 0) return;
     const long long gpw = V < 32 ? 32 / V : 1;  // Gaussians per warp
     const long long warps = (sc.n + gpw - 1) / gpw;
     const unsigned nb = (unsigned)((warps + PRE_THREADS / 32 - 1) / (PRE_THREADS / 32));
 #define MVGS_PP(D) \
-    preprocess_kernel<D><<<nb, PRE_THREADS, 0, s>>>(sc, cams, V, tw, th, vis, rec, tiles_touched, tile_desc)
+    preprocess_kernel<D><<<nb, PRE_THREADS, 0, s>>>(sc, cams, V, tw, th, vis, rec, bins, tile_desc, sums)
     switch (sc.sh_degree) {
         case 0: MVGS_PP(0); break;
         case 1: MVGS_PP(1); break;

@@ -1,16 +1,24 @@
-// Key duplication, exclusive scans, stable LSD radix sort and tile ranges.
+// Exclusive scans, stable LSD radix sort and the per-tile lists.
 //
 // The supplement ("Rasterization in multi-view training") sorts duplicated
 // (tile, viewpoint, depth) keys so each (tile, view) list is depth ordered.
-// Here the same order is reached in two cheaper sorts: the visible records
-// are first sorted by depth (32-bit keys, one entry per record), then
-// duplicated per covered tile in that order, and the duplicated entries are
-// sorted stably on the global (view, tile) id alone -- ceil(log2(tiles)) bits
-// instead of 32 + that.  Stability keeps depth order, and equal depths keep
-// the record order, which is Gaussian-major, so ties inside a tile list are
-// broken by Gaussian index.
+// Here the same lists are built without sorting the duplicated keys at all:
+//   1. the visible records are sorted by depth (32-bit keys, one entry per
+//      record);
+//   2. in that order, one entry per (record, bin) is generated -- a bin is
+//      8 x 8 tiles of one view, so a record has few of them -- and the entries
+//      are sorted stably by bin (usually one 8-bit pass);
+//   3. every chunk of a bin's entries is expanded to the bin's 64 tiles at
+//      once: entry i covers tile t when bit t of its 64-bit coverage mask is
+//      set, so transposing the masks of 32 entries gives each tile its part of
+//      the list in depth order.  A first kernel counts per (chunk, tile), a
+//      scan over the chunks gives every chunk its place in every tile's list,
+//      and a second kernel writes the record ids there, in runs.
+// Stability keeps depth order, and equal depths keep the record order, which
+// is Gaussian-major, so ties inside a tile list are broken by Gaussian index.
 #include <cstddef>
 
+#include "../../include/mvgs.h"
 #include "kernels.h"
 
 namespace mvgs {
@@ -68,13 +76,6 @@ struct LoadMasked {
     const int* in;
     int mask;
     __device__ __forceinline__ long long operator()(uint64_t i) const { return (long long)(in[i] & mask); }
-};
-
-template <class Tout>
-struct LoadGather {
-    const uint32_t* in;
-    const uint32_t* idx;
-    __device__ __forceinline__ Tout operator()(uint64_t i) const { return (Tout)in[idx[i]]; }
 };
 
 template <class Load, class T>
@@ -181,27 +182,18 @@ struct RankSmem {
     uint32_t svals[RS_TILE];         // values in block-local sorted order
 };
 
-// How a pass stores its output.  A two-pass sort of keys of at most 16 bits
-// whose values fit beside the high key bits in one word packs the first pass's
-// output: word = (key >> 8) << vb | value (vb value bits); the second pass
-// sorts these words on bits [vb, 32) and writes word & (2^vb - 1).  The first
-// pass of such a sort reads its keys as 16-bit words.
-enum PassMode { kPlain = 0, kPackOut = 1, kPackIn = 2 };
-
 // Stable rank of the block's keys (held in registers, warp w owning the
 // contiguous segment [w*SEG, (w+1)*SEG) in rounds of 32 lanes) and scatter:
 // first into shared memory in block-local digit order, then to global memory
 // in runs of consecutive positions per digit.  Equal digits inside a round are
 // found with one ballot per digit bit.  Values are fetched after the ranking
 // (get_val(block-local index)), so they do not occupy registers during it.
-// MODE kPackOut writes packed words to kout (shift 0); kPackIn takes the
-// values from the packed words and writes them to vout (shift vb).
-template <bool WRITE_KEYS, int NB, int MODE, class GetVal>
+template <bool WRITE_KEYS, int NB, class GetVal>
 __device__ __forceinline__ void rank_and_scatter(RankSmem& sm, const uint32_t (&k)[RS_ITEMS], uint64_t n, int shift,
                                                  const uint32_t* __restrict__ offsets, uint32_t nblocks,
                                                  uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
                                                  GetVal get_val, const uint32_t* __restrict__ gsrc,
-                                                 uint32_t* __restrict__ gout, int vb) {
+                                                 uint32_t* __restrict__ gout) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     const uint64_t block0 = (uint64_t)blockIdx.x * RS_TILE;
@@ -233,10 +225,8 @@ __device__ __forceinline__ void rank_and_scatter(RankSmem& sm, const uint32_t (&
     // values are read before the barrier that precedes the scatter, so a
     // source may keep them in the staging the scatter overwrites
     uint32_t vv[RS_ITEMS];
-    if (MODE != kPackIn) {
 #pragma unroll
-        for (int j = 0; j < RS_ITEMS; j++) vv[j] = base + (uint64_t)j * 32 < n ? get_val(local0 + j * 32) : 0u;
-    }
+    for (int j = 0; j < RS_ITEMS; j++) vv[j] = base + (uint64_t)j * 32 < n ? get_val(local0 + j * 32) : 0u;
     __syncthreads();
     uint32_t run = 0;
 #pragma unroll
@@ -254,7 +244,7 @@ __device__ __forceinline__ void rank_and_scatter(RankSmem& sm, const uint32_t (&
             const uint32_t d = (k[j] >> shift) & 0xffu;
             const uint32_t lp = sm.dstart[d] + wh[d] + lr[j];
             sm.skeys[lp] = k[j];
-            if (MODE != kPackIn) sm.svals[lp] = vv[j];
+            sm.svals[lp] = vv[j];
         }
     }
     __syncthreads();
@@ -263,15 +253,9 @@ __device__ __forceinline__ void rank_and_scatter(RankSmem& sm, const uint32_t (&
         const uint32_t key = sm.skeys[i];
         const uint32_t d = (key >> shift) & 0xffu;
         const uint32_t pos = sm.boff[d] + (uint32_t)i - sm.dstart[d];
-        if (MODE == kPackOut) {
-            kout[pos] = (key >> 8) << vb | sm.svals[i];
-        } else if (MODE == kPackIn) {
-            vout[pos] = key & ((1u << vb) - 1u);
-        } else {
-            vout[pos] = sm.svals[i];
-            if (WRITE_KEYS) kout[pos] = key;
-            if (gout) gout[pos] = gsrc[sm.svals[i]];
-        }
+        vout[pos] = sm.svals[i];
+        if (WRITE_KEYS) kout[pos] = key;
+        if (gout) gout[pos] = gsrc[sm.svals[i]];
     }
 }
 
@@ -297,11 +281,8 @@ __global__ void __launch_bounds__(RS_THREADS) rs_upsweep(const uint32_t* __restr
     counts[(uint64_t)threadIdx.x * nblocks + blockIdx.x] = sum;
 }
 
-// vin == nullptr: the values are the keys' positions (an identity
-// permutation, generated instead of read).  gout != nullptr: also writes
-// gout[pos] = gsrc[value] (a per-element array carried into sorted order).
-// The same table for a pass whose digits take at most 32 values (the tile
-// sort's last pass over the tile ids' high bits): each lane counts into its
+// The same table for a pass whose digits take at most 32 values (few bins, or
+// the bin ids' high bits): each lane counts into its
 // own column of a per-warp table (digit-major, lane-minor: a lane's updates
 // hit its own bank, and are plain read-modify-writes, not atomics, since no
 // other lane touches the column), then a skewed sweep sums the columns.
@@ -338,16 +319,18 @@ __global__ void __launch_bounds__(RS_THREADS) rs_upsweep_narrow(const uint32_t* 
 }
 
 // NB: significant bits of this pass's digit (8, or fewer in a last pass over
-// the high bits of keys narrower than a whole number of digits); MODE and vb:
-// see PassMode.
-template <bool WRITE_KEYS, int NB = 8, int MODE = kPlain>
+// the high bits of keys narrower than a whole number of digits).  vin ==
+// nullptr: the values are the keys' positions (an identity permutation,
+// generated instead of read).  gout != nullptr: also writes gout[pos] =
+// gsrc[value] (a per-element array carried into sorted order).
+template <bool WRITE_KEYS, int NB = 8>
 __global__ void __launch_bounds__(RS_THREADS, 3) rs_downsweep(const uint32_t* __restrict__ kin,
                                                              const uint32_t* __restrict__ vin,
                                                              uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
                                                              Count cn, int shift,
                                                              const uint32_t* __restrict__ offsets, uint32_t nblocks,
                                                              const uint32_t* __restrict__ gsrc = nullptr,
-                                                             uint32_t* __restrict__ gout = nullptr, int vb = 0) {
+                                                             uint32_t* __restrict__ gout = nullptr) {
     __shared__ RankSmem sm;
     const uint64_t n = cn.get();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -358,333 +341,356 @@ __global__ void __launch_bounds__(RS_THREADS, 3) rs_downsweep(const uint32_t* __
 #pragma unroll
     for (int j = 0; j < RS_ITEMS; j++) {
         const uint64_t idx = base + (uint64_t)j * 32;
-        // kPackOut reads the 16-bit keys of a two-pass sort
-        k[j] = idx >= n ? 0u : MODE == kPackOut ? (uint32_t)reinterpret_cast<const uint16_t*>(kin)[idx] : kin[idx];
+        k[j] = idx < n ? kin[idx] : 0u;
     }
-    rank_and_scatter<WRITE_KEYS, NB, MODE>(
+    rank_and_scatter<WRITE_KEYS, NB>(
         sm, k, n, shift, offsets, nblocks, kout, vout,
-        [&](int local) { return vin ? vin[block0 + local] : (uint32_t)(block0 + local); }, gsrc, gout, vb);
+        [&](int local) { return vin ? vin[block0 + local] : (uint32_t)(block0 + local); }, gsrc, gout);
 }
 
 // ---------------------------------------------------------------------------
-// duplication: one (tile, record) entry per tile a record's rectangle covers,
-// in the order of the depth-sorted records (rectangle tiles row-major).  Key
-// index k belongs to the record r with off[r] <= k < off[r+1].  Each block
-// emits one radix tile of entries and the histogram of their first digit, so
-// the first radix pass needs no separate histogram sweep.
+// per-tile lists through bins of 8 x 8 tiles
 // ---------------------------------------------------------------------------
-struct DupSrc {
-    const uint32_t* order;             // records by depth
-    const unsigned long long* off;     // [R + 1] exclusive scan of tiles in that order
-    Count R;
-    const unsigned long long* desc;    // tile descriptors (pack_tile_desc), record order
-    const DevCam* cams;
-    uint32_t tiles;
-};
+// Sorting one entry per (record, tile) moved 28 bytes per entry (generation,
+// histogram, two radix passes).  Here only the (record, bin) entries are
+// sorted -- about 1.7 per record at 32 x 64 tiles and 4 at 16 x 16, against 14
+// and 58 tiles -- and the record id of a (record, tile) pair is written once,
+// straight into its tile's list.  Bound by the random descriptor fetches of
+// the entries and the 4 bytes written per (record, tile) pair.  Tile sort with
+// ranges, radix sort of all pairs -> bins: 3M Gaussians x 8 views at 32 x 64
+// tiles (340M pairs, 41M entries) 4.83 -> 1.64 ms; 1M x 16 views at 16 x 64
+// (236M pairs) 3.83 -> 1.21 ms; 500k x 4 views at 16 x 16 (116M pairs, 8M
+// entries) 1.81 -> 0.44 ms; 500k x 1 view at 16 x 16 0.49 -> 0.17 ms; 20k x 3
+// small views 0.115 -> 0.097 ms.  Bins of 64 tiles because a coverage mask then
+// is two words and a warp transposes 32 of them in ten shuffles.
+//
+// Sort key of an entry: the bin id above 12 bits holding the part of the
+// record's rectangle inside the bin (x0, y0, x1, y1 inclusive, 3 bits each),
+// so the expansion needs no record fetch.  With more than 2^20 bins (LOCAL
+// false) the key is the bin id alone and the expansion clips the record's
+// rectangle again.
+constexpr int BIN_LOCAL_BITS = 12;
+constexpr long long BIN_LOCAL_MAX = 1LL << (32 - BIN_LOCAL_BITS);
+constexpr int BC_THREADS = 256;
+constexpr int BC_WARPS = BC_THREADS / 32;
+constexpr int BC_CHUNK = 1024;            // entries of one bin expanded together
+constexpr int BC_GROUPS = BC_CHUNK / 32;  // groups of 32 entries, one lane per group when a list is placed
+static_assert(BC_GROUPS == 32, "one lane per group");
 
-// Index of the record holding entry k: a binary search over the offsets of
-// the records that cover the block (staged in shared memory, relative to k0),
-// or over all offsets when they did not fit.
-__device__ __forceinline__ uint64_t dup_record(const DupSrc& src, const int* s_off, uint64_t rlo, int nr, uint64_t k0,
-                                               uint64_t k) {
-    if (nr > 0) {
-        const int kk = (int)(k - k0);
-        int lo = 0, hi = nr - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (s_off[mid] <= kk) lo = mid; else hi = mid - 1;
-        }
-        return rlo + lo;
-    }
-    uint64_t lo = 0, hi = src.R.get() - 1;
+// The part of rectangle rc inside bin (bx, by), packed as in the sort key.
+__device__ __forceinline__ uint32_t clip_to_bin(short4 rc, int bx, int by) {
+    const int x0 = max(rc.x - 8 * bx, 0), x1 = min(rc.z - 1 - 8 * bx, 7);
+    const int y0 = max(rc.y - 8 * by, 0), y1 = min(rc.w - 1 - 8 * by, 7);
+    return (uint32_t)(x0 | y0 << 3 | x1 << 6 | y1 << 9);
+}
+
+// Coverage mask over the bin's tiles (bit 8 y + x) of a packed local rectangle.
+__device__ __forceinline__ uint2 bin_mask(uint32_t l) {
+    const int x0 = l & 7, y0 = (l >> 3) & 7, x1 = (l >> 6) & 7, y1 = (l >> 9) & 7;
+    const uint32_t rep = ((0xffu >> (7 - x1)) & (0xffu << x0)) * 0x01010101u;
+    const unsigned long long rows = (~0ull >> (8 * (7 - y1))) & (~0ull << (8 * y0));
+    return make_uint2(rep & (uint32_t)rows, rep & (uint32_t)(rows >> 32));
+}
+
+__device__ __forceinline__ int find_bin_view(const DevCam* cams, int V, long long bin) {
+    int lo = 0, hi = V - 1;
     while (lo < hi) {
-        const uint64_t mid = (lo + hi + 1) >> 1;
-        if (src.off[mid] <= k) lo = mid; else hi = mid - 1;
+        const int mid = (lo + hi + 1) >> 1;
+        if (cams[mid].bin_base <= bin) lo = mid; else hi = mid - 1;
     }
     return lo;
 }
 
-constexpr int DUP_ITEMS = RS_ITEMS;  // consecutive entries per thread
-constexpr int DUP_MAXR = 1024;       // records a block stages in shared memory
-
-// first[b] = the record holding entry b * TILE, for every radix block b:
-// each record fills the blocks whose first entry it holds, so no block has to
-// search for its records; the block after the last entry gets R - 1.
-__global__ void block_starts_kernel(const unsigned long long* __restrict__ off, Count Rc, uint32_t nblocks,
-                                    uint32_t* __restrict__ first) {
-    const uint64_t R = Rc.get();
-    const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r == 0) {
-        const uint64_t end = (off[R] + RS_TILE - 1) / RS_TILE;
-        first[end < nblocks ? end : nblocks] = (uint32_t)(R - 1);
+// One entry per (record, bin), in depth order; off is the exclusive scan of
+// the records' bin counts in that order.  A warp takes 32 records and walks
+// their entries 32 at a time (each lane finds its entry's record by a search
+// over the warp's offsets), so the stores are coalesced however uneven the
+// records' counts are.
+template <bool LOCAL>
+__global__ void __launch_bounds__(256) bin_entries_kernel(const uint32_t* __restrict__ order,
+                                                          const unsigned long long* __restrict__ off, Count Rc,
+                                                          Count Sc, const unsigned long long* __restrict__ desc,
+                                                          const DevCam* __restrict__ cams,
+                                                          uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+    const uint64_t R = Rc.get(), S = Sc.get();
+    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    const uint64_t w0 = i - lane;
+    if (w0 >= R) return;  // the whole warp
+    const uint64_t r = i < R ? i : R;
+    const unsigned long long o = off[r];
+    const unsigned long long first = __shfl_sync(kFull, o, 0);
+    const uint32_t total = (uint32_t)(off[w0 + 32 < R ? w0 + 32 : R] - first);
+    uint32_t rec = 0, b0 = 0;
+    int bxs = 1;
+    unsigned long long d = 0;
+    if (i < R) {
+        rec = order[i];
+        d = desc[rec];
+        const short4 rc = tile_desc_rect(d);
+        const DevCam& c = cams[tile_desc_view(d)];
+        bxs = bins_across(c.tiles_x);
+        b0 = (uint32_t)(c.bin_base + (long long)(rc.y >> 3) * bxs + (rc.x >> 3));
     }
-    if (r >= R) return;
-    const uint64_t b0 = (off[r] + RS_TILE - 1) / RS_TILE;
-    const uint64_t b1 = (off[r + 1] + RS_TILE - 1) / RS_TILE;  // exclusive
-    for (uint64_t b = b0; b < b1 && b < nblocks; b++) first[b] = (uint32_t)r;
+    const uint32_t rel = (uint32_t)(o - first);
+    for (uint32_t j0 = 0; j0 < total; j0 += 32) {
+        const uint32_t j = j0 + lane;
+        // the last record starting at or before entry j (records without
+        // bins share the next one's offset)
+        int src = 0;
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1) {
+            const uint32_t v = __shfl_sync(kFull, rel, src + step);
+            if (v <= j) src += step;
+        }
+        const uint32_t k = j - __shfl_sync(kFull, rel, src);
+        const unsigned long long ds = __shfl_sync(kFull, d, src);
+        const uint32_t recs = __shfl_sync(kFull, rec, src), b0s = __shfl_sync(kFull, b0, src);
+        const int bxss = __shfl_sync(kFull, bxs, src);
+        const short4 rc = tile_desc_rect(ds);
+        const int bx0 = rc.x >> 3, by0 = rc.y >> 3;
+        const int w = max(((rc.z - 1) >> 3) - bx0 + 1, 1);
+        const int ty = (int)(k / (uint32_t)w), tx = (int)(k % (uint32_t)w);
+        const uint32_t bin = b0s + (uint32_t)ty * (uint32_t)bxss + (uint32_t)tx;
+        if (j < total && first + j < S) {
+            keys[first + j] = LOCAL ? bin << BIN_LOCAL_BITS | clip_to_bin(rc, bx0 + tx, by0 + ty) : bin;
+            vals[first + j] = recs;
+        }
+    }
 }
 
-// K16: keys stored as 16-bit words (tile ids below 2^16; see PassMode).
-template <bool K16>
-__global__ void __launch_bounds__(RS_THREADS, 4) dup_hist_kernel(DupSrc src, const uint32_t* __restrict__ first_rec,
-                                                             Count Kc, uint32_t* __restrict__ keys,
-                                                             uint32_t* __restrict__ vals,
-                                                             uint32_t* __restrict__ counts, uint32_t nblocks) {
-    __shared__ uint32_t hist[RS_WARPS * 256];
-    // the block's record offsets and records (ids and tile descriptors,
-    // gathered once by all threads together: the loads are independent, so
-    // they are all in flight at once); after the generation the same bytes
-    // stage the block's entries for coalesced stores
-    constexpr int OFF_BYTES = (RS_TILE + 4) * 4;
-    constexpr int RAW_BYTES = OFF_BYTES + DUP_MAXR * 20;
-    static_assert(RAW_BYTES >= RS_TILE * 8, "entry staging");
-    __shared__ __align__(16) unsigned char s_raw[RAW_BYTES];
-    int* s_off = reinterpret_cast<int*>(s_raw);
-    short4* s_rect = reinterpret_cast<short4*>(s_raw + OFF_BYTES);
-    uint32_t* s_rec = reinterpret_cast<uint32_t*>(s_raw + OFF_BYTES + DUP_MAXR * 8);
-    uint32_t* s_base = s_rec + DUP_MAXR;
-    int* s_tx = reinterpret_cast<int*>(s_base + DUP_MAXR);
-    const uint64_t K = Kc.get();
-    const uint64_t k0 = (uint64_t)blockIdx.x * RS_TILE;
-    if (k0 >= K) {  // a block past the entries (capturable mode): empty histogram
-        counts[(uint64_t)threadIdx.x * nblocks + blockIdx.x] = 0u;
+// First and one past the last position of every bin's entries (zeroed before:
+// a bin without entries keeps an empty range).
+__global__ void __launch_bounds__(256) bin_bounds_kernel(const uint32_t* __restrict__ keys, Count Sc, int shift,
+                                                         uint32_t* __restrict__ begin, uint32_t* __restrict__ end) {
+    const uint64_t S = Sc.get();
+    const uint64_t i0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
+    if (i0 >= S) return;
+    uint32_t b[6];
+    b[0] = i0 > 0 ? keys[i0 - 1] >> shift : 0xffffffffu;
+#pragma unroll
+    for (int q = 1; q < 6; q++) b[q] = i0 + q - 1 < S ? keys[i0 + q - 1] >> shift : 0xffffffffu;
+#pragma unroll
+    for (int q = 1; q < 5; q++) {
+        const uint64_t i = i0 + q - 1;
+        if (i >= S) break;
+        if (i == 0 || b[q] != b[q - 1]) begin[b[q]] = (uint32_t)i;
+        if (i + 1 == S || b[q] != b[q + 1]) end[b[q]] = (uint32_t)i + 1;
+    }
+}
+
+// First chunk of every bin (one block; bins that no entry touches have none).
+// A single bin holds all S entries.
+__global__ void __launch_bounds__(SPINE_THREADS) bin_chunks_kernel(uint32_t* __restrict__ begin,
+                                                                   uint32_t* __restrict__ end, Count Sc, long long bins,
+                                                                   uint32_t* __restrict__ chunk_off) {
+    __shared__ uint32_t buf[33];
+    if (bins == 1) {
+        if (threadIdx.x == 0) {
+            const uint32_t S = (uint32_t)Sc.get();
+            begin[0] = 0;
+            end[0] = S;
+            chunk_off[0] = 0;
+            chunk_off[1] = S / BC_CHUNK + (S % BC_CHUNK != 0);
+        }
         return;
     }
-    for (int i = threadIdx.x; i < RS_WARPS * 256; i += RS_THREADS) hist[i] = 0;
-    // records [rlo, rlo + nr) hold this block's entries (the next block's
-    // first record may start inside it); a record without tiles shares its
-    // offset with the next, so they can outnumber the entries: then search
-    // all offsets instead
-    const uint64_t rlo = first_rec[blockIdx.x];
-    const uint64_t rhi = first_rec[blockIdx.x + 1];
-    const int nr = rhi - rlo + 1 <= (uint64_t)RS_TILE ? (int)(rhi - rlo + 1) : -1;
-    for (int i = threadIdx.x; i <= nr; i += RS_THREADS) s_off[i] = (int)((long long)src.off[rlo + i] - (long long)k0);
-    const bool staged = nr > 0 && nr <= DUP_MAXR;
-    if (staged) {
-        for (int i = threadIdx.x; i < nr; i += RS_THREADS) {
-            const uint32_t rec = src.order[rlo + i];
-            const unsigned long long d = src.desc[rec];
-            const DevCam& c = src.cams[tile_desc_view(d)];
-            s_rec[i] = rec;
-            s_rect[i] = tile_desc_rect(d);
-            s_base[i] = (uint32_t)c.tile_base;
-            s_tx[i] = c.tiles_x;
-        }
+    uint32_t carry = 0;
+    for (long long base = 0; base < bins; base += SPINE_THREADS) {
+        const long long b = base + threadIdx.x;
+        const uint32_t len = b < bins ? end[b] - begin[b] : 0u;
+        uint32_t total;
+        const uint32_t ex = block_exclusive_scan<uint32_t>(len / BC_CHUNK + (len % BC_CHUNK != 0), buf, total);
+        if (b < bins) chunk_off[b] = carry + ex;
+        carry += total;
     }
+    if (threadIdx.x == 0) chunk_off[bins] = carry;
+}
+
+// The bin of chunk c: the last one whose first chunk is c or earlier (a warp
+// narrows the range 32-fold per step).
+__device__ __forceinline__ uint32_t bin_of_chunk(const uint32_t* chunk_off, uint32_t bins, uint32_t c, int lane) {
+    uint32_t lo = 0, hi = bins;
+    while (hi - lo > 1) {
+        const uint32_t step = (hi - lo + 31) / 32, at = lo + (uint32_t)lane * step;
+        const uint32_t n = __popc(__ballot_sync(kFull, at < hi && chunk_off[at] <= c));
+        lo += (n - 1) * step;
+        hi = lo + step < hi ? lo + step : hi;
+    }
+    return lo;
+}
+
+// 32 x 32 bit transpose over the warp: bit r of lane t's result is bit t of
+// lane r's word.
+__device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane) {
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) {
+        const uint32_t m = j == 16 ? 0x0000ffffu : j == 8 ? 0x00ff00ffu : j == 4 ? 0x0f0f0f0fu
+                                               : j == 2 ? 0x33333333u : 0x55555555u;
+        const uint32_t y = __shfl_xor_sync(kFull, x, j);
+        x = lane & j ? (x & ~m) | ((y & ~m) >> j) : (x & m) | ((y & m) << j);
+    }
+    return x;
+}
+
+struct BinLists {
+    const uint32_t* keys;              // entries sorted by bin
+    const uint32_t* vals;              // their record ids
+    const unsigned long long* desc;    // tile descriptors (LOCAL false only)
+    const uint32_t* begin;             // [bins] the bin's entries: [begin, end)
+    const uint32_t* end;
+    const uint32_t* chunk_off;         // [bins + 1] first chunk of every bin
+    uint32_t* chunk_bin;               // [chunks]
+    uint32_t* counts;                  // [chunks, 64] entries per tile, then the entries of the chunks before
+    uint32_t bins;
+};
+
+// Coverage mask of entry p (clipped to bin (bx, by) when the key does not hold it).
+template <bool LOCAL>
+__device__ __forceinline__ uint2 entry_mask(const BinLists& L, uint64_t p, int bx, int by) {
+    if (LOCAL) return bin_mask(L.keys[p]);
+    return bin_mask(clip_to_bin(tile_desc_rect(L.desc[L.vals[p]]), bx, by));
+}
+
+// Entries per tile of every chunk.
+template <bool LOCAL>
+__global__ void __launch_bounds__(BC_THREADS) bin_count_kernel(BinLists L, const DevCam* __restrict__ cams, int V) {
+    __shared__ uint32_t part[BC_WARPS][64];
+    const uint32_t c = blockIdx.x;
+    if (c >= L.chunk_off[L.bins]) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t b = bin_of_chunk(L.chunk_off, L.bins, c, lane);
+    const uint32_t p0 = L.begin[b] + (c - L.chunk_off[b]) * BC_CHUNK;
+    const uint32_t cnt = min(L.end[b] - p0, (uint32_t)BC_CHUNK);
+    int bx = 0, by = 0;
+    if (!LOCAL) {
+        const DevCam& cam = cams[find_bin_view(cams, V, b)];
+        const long long lb = (long long)b - cam.bin_base;
+        bx = (int)(lb % bins_across(cam.tiles_x));
+        by = (int)(lb / bins_across(cam.tiles_x));
+    }
+    uint32_t lo = 0, hi = 0;
+#pragma unroll
+    for (int q = 0; q < BC_GROUPS / BC_WARPS; q++) {
+        const uint32_t e = (warp * (BC_GROUPS / BC_WARPS) + q) * 32 + lane;
+        const uint2 m = e < cnt ? entry_mask<LOCAL>(L, (uint64_t)p0 + e, bx, by) : make_uint2(0u, 0u);
+        lo += __popc(warp_transpose(m.x, lane));
+        hi += __popc(warp_transpose(m.y, lane));
+    }
+    part[warp][lane] = lo;
+    part[warp][32 + lane] = hi;
+    if (threadIdx.x == 0) L.chunk_bin[c] = b;
     __syncthreads();
-    // record rr: id, rectangle, view tile base, tiles per row, end of its
-    // entries relative to the block's first entry (32-bit arithmetic in the
-    // walk: tile ids and entry positions are below 2^32)
-    auto load = [&](uint64_t rr, uint32_t& rec, short4& rc, uint32_t& base, int& txs, uint32_t& rend) {
-        if (staged) {
-            const int li = (int)(rr - rlo);
-            rec = s_rec[li];
-            rc = s_rect[li];
-            base = s_base[li];
-            txs = s_tx[li];
-            rend = (uint32_t)s_off[li + 1];
-        } else {
-            rec = src.order[rr];
-            const unsigned long long d = src.desc[rec];
-            rc = tile_desc_rect(d);
-            const DevCam& c = src.cams[tile_desc_view(d)];
-            base = (uint32_t)c.tile_base;
-            txs = c.tiles_x;
-            rend = (uint32_t)(src.off[rr + 1] - k0);
-        }
-    };
-    uint32_t* wh = hist + (threadIdx.x >> 5) * 256;
-    const uint32_t cnt_l = (uint32_t)(K - k0 < (uint64_t)RS_TILE ? K - k0 : (uint64_t)RS_TILE);
-    const uint32_t first_l = (uint32_t)threadIdx.x * DUP_ITEMS;
-    const uint32_t tmax = src.tiles - 1u;
-    uint32_t kk[DUP_ITEMS], vv[DUP_ITEMS];
+    if (threadIdx.x < 64) {
+        uint32_t sum = 0;
 #pragma unroll
-    for (int i = 0; i < DUP_ITEMS; i++) kk[i] = vv[i] = 0u;
-    if (first_l < cnt_l) {
-        const uint64_t first = k0 + first_l;
-        uint64_t r = dup_record(src, s_off, rlo, nr, k0, first);
-        uint32_t rend, rec, base;
-        short4 rc;
-        int txs;
-        load(r, rec, rc, base, txs, rend);
-        int w = max(rc.z - rc.x, 1);
-        const uint64_t rstart = staged ? k0 + (uint64_t)(long long)s_off[r - rlo] : src.off[r];
-        const uint32_t j = (uint32_t)(first - rstart);
-        int tx = rc.x + (int)(j % (uint32_t)w), ty = rc.y + (int)(j / (uint32_t)w);
-#pragma unroll
-        for (int i = 0; i < DUP_ITEMS; i++) {
-            const uint32_t l = first_l + i;
-            if (l < cnt_l) {
-                while (l >= rend) {  // next record (skipping any without tiles)
-                    r++;
-                    load(r, rec, rc, base, txs, rend);
-                    w = max(rc.z - rc.x, 1);
-                    tx = rc.x;
-                    ty = rc.y;
-                }
-                const uint32_t t = base + (uint32_t)ty * (uint32_t)txs + (uint32_t)tx;
-                const uint32_t key = t < tmax ? t : tmax;
-                kk[i] = key;
-                vv[i] = rec;
-                atomicAdd(&wh[key & 0xffu], 1u);
-                if (++tx == rc.x + w) {
-                    tx = rc.x;
-                    ty++;
-                }
-            }
-        }
+        for (int w = 0; w < BC_WARPS; w++) sum += part[w][threadIdx.x];
+        L.counts[(uint64_t)c * 64 + threadIdx.x] = sum;
     }
-    // stage the entries, then store them coalesced.  Thread t's quads of
-    // 32-bit words go to slots 4t + ((q + t/2) & 3), its pairs of 8 16-bit
-    // keys to 2t + ((q + t/4) & 1): the eight threads of a 128-byte phase hit
-    // distinct banks.
-    __syncthreads();
-    uint4* sv = reinterpret_cast<uint4*>(s_raw);
-    uint4* sk = sv + RS_TILE / 4;
-    const int t = threadIdx.x;
-#pragma unroll
-    for (int q = 0; q < DUP_ITEMS / 4; q++)
-        sv[4 * t + ((q + (t >> 1)) & 3)] = make_uint4(vv[4 * q], vv[4 * q + 1], vv[4 * q + 2], vv[4 * q + 3]);
-    if (K16) {
-#pragma unroll
-        for (int q = 0; q < DUP_ITEMS / 8; q++) {
-            const uint32_t* h = kk + 8 * q;
-            sk[2 * t + ((q + (t >> 2)) & 1)] = make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16, h[4] | h[5] << 16,
-                                                          h[6] | h[7] << 16);
-        }
-    } else {
-#pragma unroll
-        for (int q = 0; q < DUP_ITEMS / 4; q++)
-            sk[4 * t + ((q + (t >> 1)) & 3)] = make_uint4(kk[4 * q], kk[4 * q + 1], kk[4 * q + 2], kk[4 * q + 3]);
-    }
-    __syncthreads();
-    const uint64_t cnt = K - k0 < (uint64_t)RS_TILE ? K - k0 : (uint64_t)RS_TILE;
-    for (int L = t; L < RS_TILE / 4; L += RS_THREADS) {  // values, 4 per quad
-        const int owner = L >> 2;
-        const uint4 a = sv[4 * owner + (((L & 3) + (owner >> 1)) & 3)];
-        const uint64_t e = (uint64_t)L * 4;
-        if (e + 4 <= cnt) {
-            reinterpret_cast<uint4*>(vals + k0)[L] = a;
-        } else {
-            const uint32_t va[4] = {a.x, a.y, a.z, a.w};
-            for (int i = 0; i < 4 && e + i < cnt; i++) vals[k0 + e + i] = va[i];
-        }
-    }
-    constexpr int KPER = K16 ? 8 : 4;  // keys per quad
-    for (int L = t; L < RS_TILE / KPER; L += RS_THREADS) {
-        const int owner = K16 ? L >> 1 : L >> 2;
-        const uint4 a = K16 ? sk[2 * owner + (((L & 1) + (owner >> 2)) & 1)]
-                            : sk[4 * owner + (((L & 3) + (owner >> 1)) & 3)];
-        const uint64_t e = (uint64_t)L * KPER;
-        if (e + KPER <= cnt) {
-            if (K16) reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(keys) + k0)[L] = a;
-            else reinterpret_cast<uint4*>(keys + k0)[L] = a;
-        } else {
-            const uint32_t ka[4] = {a.x, a.y, a.z, a.w};
-            for (int i = 0; i < KPER && e + i < cnt; i++) {
-                if (K16) reinterpret_cast<uint16_t*>(keys)[k0 + e + i] = (uint16_t)(ka[i >> 1] >> (16 * (i & 1)));
-                else keys[k0 + e + i] = ka[i];
-            }
-        }
-    }
+}
+
+// One block per bin: every chunk's counts become the number of entries in the
+// chunks before it, tile by tile, and the totals the tiles' list lengths.
+constexpr int BS_PARTS = 8;  // stretches of chunks scanned side by side
+__global__ void __launch_bounds__(64 * BS_PARTS) bin_scan_kernel(BinLists L, const DevCam* __restrict__ cams, int V,
+                                                                 uint32_t* __restrict__ tile_counts) {
+    __shared__ uint32_t sums[BS_PARTS][64];
+    const uint32_t b = blockIdx.x;
+    const int t = threadIdx.x & 63, part = threadIdx.x >> 6;
+    const uint32_t c0 = L.chunk_off[b], n = L.chunk_off[b + 1] - c0;
+    const uint32_t per = (n + BS_PARTS - 1) / BS_PARTS;
+    const uint32_t r0 = min(part * per, n), r1 = min(r0 + per, n);
+    uint32_t* row = L.counts + (uint64_t)c0 * 64 + t;
     uint32_t sum = 0;
+#pragma unroll 8
+    for (uint32_t r = r0; r < r1; r++) sum += row[(uint64_t)r * 64];
+    sums[part][t] = sum;
+    __syncthreads();
+    uint32_t run = 0;
+    for (int q = 0; q < part; q++) run += sums[q][t];
+#pragma unroll 8
+    for (uint32_t r = r0; r < r1; r++) {
+        const uint32_t v = row[(uint64_t)r * 64];
+        row[(uint64_t)r * 64] = run;
+        run += v;
+    }
+    if (part == BS_PARTS - 1) {
+        const DevCam& cam = cams[find_bin_view(cams, V, b)];
+        const int lb = (int)((long long)b - cam.bin_base), across = bins_across(cam.tiles_x);
+        const int tx = (lb % across) * 8 + (t & 7), ty = (lb / across) * 8 + (t >> 3);
+        if (tx < cam.tiles_x && ty < cam.tiles_y)
+            tile_counts[cam.tile_base + (long long)ty * cam.tiles_x + tx] = run;
+    }
+}
+
+// Writes every chunk's record ids into the tiles' lists.  A warp takes one
+// tile at a time: lane g holds the tile's coverage word of the chunk's group g
+// (32 entries), a warp scan of the popcounts gives each lane its part of the
+// run, the set bits are compacted in shared memory and the run is stored by
+// consecutive lanes.
+template <bool LOCAL>
+__global__ void __launch_bounds__(BC_THREADS) bin_place_kernel(BinLists L, const DevCam* __restrict__ cams, int V,
+                                                               const long long* __restrict__ ranges,
+                                                               const unsigned long long* __restrict__ total, Count Kc,
+                                                               uint32_t* __restrict__ sorted) {
+    __shared__ uint32_t words[64][BC_GROUPS + 1];
+    __shared__ uint32_t recs[BC_CHUNK];
+    __shared__ uint32_t first[64];
+    __shared__ uint16_t stage[BC_WARPS][BC_CHUNK];
+    const uint32_t c = blockIdx.x;
+    // nothing is placed when the lists do not fit (capturable mode)
+    if (c >= L.chunk_off[L.bins] || *total > Kc.max) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t b = L.chunk_bin[c];
+    const uint32_t p0 = L.begin[b] + (c - L.chunk_off[b]) * BC_CHUNK;
+    const uint32_t cnt = min(L.end[b] - p0, (uint32_t)BC_CHUNK);
+    const DevCam& cam = cams[find_bin_view(cams, V, b)];
+    const int lb = (int)((long long)b - cam.bin_base), across = bins_across(cam.tiles_x);
+    const int bx = lb % across, by = lb / across;
+    if (threadIdx.x < 64) {
+        const int tx = bx * 8 + (threadIdx.x & 7), ty = by * 8 + (threadIdx.x >> 3);
+        first[threadIdx.x] = tx < cam.tiles_x && ty < cam.tiles_y
+                                 ? (uint32_t)ranges[2 * (cam.tile_base + (long long)ty * cam.tiles_x + tx)] +
+                                       L.counts[(uint64_t)c * 64 + threadIdx.x]
+                                 : 0u;
+    }
 #pragma unroll
-    for (int w2 = 0; w2 < RS_WARPS; w2++) sum += hist[w2 * 256 + threadIdx.x];
-    counts[(uint64_t)threadIdx.x * nblocks + blockIdx.x] = sum;
-}
-
-// ---------------------------------------------------------------------------
-// per-tile list lengths from the records' rectangles (2D difference counts),
-// so the tile ranges need no pass over the sorted keys
-// ---------------------------------------------------------------------------
-__global__ void rect_diff_kernel(const short4* __restrict__ rect, const int* __restrict__ rec_v, Count Rc,
-                                 const DevCam* __restrict__ cams, int* __restrict__ diff) {
-    const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= Rc.get()) return;
-    const short4 rc = rect[r];
-    if (rc.z <= rc.x || rc.w <= rc.y) return;
-    const DevCam& cam = cams[rec_v[r]];
-    const long long W1 = cam.tiles_x + 1;
-    int* d = diff + cam.diff_base;
-    atomicAdd(d + rc.y * W1 + rc.x, 1);
-    atomicAdd(d + rc.y * W1 + rc.z, -1);
-    atomicAdd(d + rc.w * W1 + rc.x, -1);
-    atomicAdd(d + rc.w * W1 + rc.z, 1);
-}
-
-// The same difference grid accumulated in shared memory: each block adds the
-// corners of a contiguous chunk of records into its own copy of the grid of
-// all views (no contention between blocks), then writes it out as one partial
-// grid; sum_parts_kernel adds the partial grids.  Same-address atomics in L2
-// serialise when many small rectangles share corners; shared-memory atomics
-// spread over 32 banks per SM do not.
-constexpr int RD_PARTS = 304;      // partial grids (2 per SM on 152 SMs)
-constexpr int RD_THREADS = 512;
-constexpr long long RD_MAX_CELLS = 54 * 1024;  // 216 KB of int counters
-
-__global__ void __launch_bounds__(RD_THREADS)
-rect_diff_smem_kernel(const short4* __restrict__ rect, const int* __restrict__ rec_v, Count Rc,
-                      const DevCam* __restrict__ cams, int cells, int* __restrict__ parts) {
-    extern __shared__ int grid[];
-    const uint64_t R = Rc.get();
-    for (int c = threadIdx.x; c < cells; c += blockDim.x) grid[c] = 0;
-    __syncthreads();
-    const uint64_t chunk = (R + gridDim.x - 1) / gridDim.x;
-    const uint64_t r0 = (uint64_t)blockIdx.x * chunk;
-    const uint64_t r1 = r0 + chunk < R ? r0 + chunk : R;
-    for (uint64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-        const short4 rc = rect[r];
-        if (rc.z <= rc.x || rc.w <= rc.y) continue;
-        const DevCam& cam = cams[rec_v[r]];
-        const int W1 = cam.tiles_x + 1;
-        int* d = grid + cam.diff_base;
-        atomicAdd(d + rc.y * W1 + rc.x, 1);
-        atomicAdd(d + rc.y * W1 + rc.z, -1);
-        atomicAdd(d + rc.w * W1 + rc.x, -1);
-        atomicAdd(d + rc.w * W1 + rc.z, 1);
-    }
-    __syncthreads();
-    int* out = parts + (size_t)blockIdx.x * cells;
-    for (int c = threadIdx.x; c < cells; c += blockDim.x) out[c] = grid[c];
-}
-
-__global__ void sum_parts_kernel(const int* __restrict__ parts, int cells, int nparts, int* __restrict__ diff) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cells) return;
-    int acc = 0;
-    for (int p = 0; p < nparts; p++) acc += parts[(size_t)p * cells + c];
-    diff[c] = acc;
-}
-
-// One block per view: prefix sums along rows, then along columns, give the
-// number of records covering each tile.
-__global__ void diff_to_counts_kernel(const DevCam* __restrict__ cams, int* __restrict__ diff,
-                                      uint32_t* __restrict__ counts) {
-    const DevCam& cam = cams[blockIdx.x];
-    const int W1 = cam.tiles_x + 1, H1 = cam.tiles_y + 1;
-    int* d = diff + cam.diff_base;
-    for (int y = threadIdx.x; y < H1; y += blockDim.x) {
-        int run = 0;
-        for (int x = 0; x < W1; x++) {
-            run += d[y * W1 + x];
-            d[y * W1 + x] = run;
+    for (int q = 0; q < BC_GROUPS / BC_WARPS; q++) {
+        const int g = warp * (BC_GROUPS / BC_WARPS) + q;
+        const uint32_t e = g * 32 + lane;
+        uint2 m = make_uint2(0u, 0u);
+        if (e < cnt) {
+            m = entry_mask<LOCAL>(L, (uint64_t)p0 + e, bx, by);
+            recs[e] = L.vals[(uint64_t)p0 + e];
         }
+        words[lane][g] = warp_transpose(m.x, lane);
+        words[32 + lane][g] = warp_transpose(m.y, lane);
     }
     __syncthreads();
-    for (int x = threadIdx.x; x < W1; x += blockDim.x) {
-        int run = 0;
-        for (int y = 0; y < H1; y++) {
-            run += d[y * W1 + x];
-            d[y * W1 + x] = run;
+    uint16_t* st = stage[warp];
+    for (int t = warp; t < 64; t += BC_WARPS) {
+        uint32_t word = words[t][lane];
+        const uint32_t n = __popc(word);
+        uint32_t inc = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += y;
         }
+        const uint32_t all = __shfl_sync(kFull, inc, 31);
+        if (all == 0) continue;
+        uint32_t at = inc - n;
+        while (word) {
+            st[at++] = (uint16_t)(lane * 32 + __ffs(word) - 1);
+            word &= word - 1;
+        }
+        __syncwarp();
+        uint32_t* out = sorted + first[t];
+        for (uint32_t j = lane; j < all; j += 32) out[j] = recs[st[j]];
+        __syncwarp();
     }
-    __syncthreads();
-    const int n = cam.tiles_x * cam.tiles_y;
-    for (int i = threadIdx.x; i < n; i += blockDim.x)
-        counts[cam.tile_base + i] = (uint32_t)d[(i / cam.tiles_x) * W1 + (i % cam.tiles_x)];
 }
 
-// Sort key of a tile for the blend's processing order: longest lists first.
 // Blend processing order: tiles by decreasing list length, in 256 length
 // classes (8 per octave: the exponent and three mantissa bits of length + 1),
 // tile id order inside a class; the persistent blend kernels take the longest
@@ -748,15 +754,16 @@ __global__ void __launch_bounds__(TO_THREADS) tile_order_kernel(const long long*
     }
 }
 
-// Ranges are clamped to the entries that were generated (all of them unless
-// a capturable call ran out of key capacity).
+// [start, end) of every tile's list.  All lists are empty when they hold more
+// entries than there is room for (a capturable call that ran out of key
+// capacity: nothing is placed then, so no range may point at the array).
 __global__ void ranges_kernel(const unsigned long long* __restrict__ starts, long long tiles, Count Kc,
                               long long* __restrict__ ranges) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= tiles) return;
-    const unsigned long long K = Kc.get();
-    ranges[2 * t] = (long long)(starts[t] < K ? starts[t] : K);
-    ranges[2 * t + 1] = (long long)(starts[t + 1] < K ? starts[t + 1] : K);
+    const bool fits = starts[tiles] <= Kc.max;
+    ranges[2 * t] = fits ? (long long)starts[t] : 0;
+    ranges[2 * t + 1] = fits ? (long long)starts[t + 1] : 0;
 }
 
 }  // namespace
@@ -783,21 +790,12 @@ void scan_u32_to_u64_count(const uint32_t* in, unsigned long long* out, Count n,
     scan_impl(LoadDirect<uint32_t, unsigned long long>{in}, out, n, true, total, tmp, s);
 }
 
-void scan_gather_u32_to_u64(const uint32_t* in, const uint32_t* idx, unsigned long long* out, Count n,
-                            unsigned long long* total, void* tmp, cudaStream_t s) {
-    scan_impl(LoadGather<unsigned long long>{in, idx}, out, n, true, total, tmp, s);
-}
-
 static uint64_t radix_blocks(uint64_t n) { return ceil_div_u64(n, RS_TILE); }
 
 size_t radix_temp_bytes(uint64_t n) {
     const uint64_t nb = radix_blocks(n > 0 ? n : 1);
     const size_t counts = ((256 * nb * sizeof(uint32_t)) + 255) / 256 * 256;
     return counts + (scan_temp_bytes(256 * nb) + 255) / 256 * 256;
-}
-
-size_t tile_sort_temp_bytes(uint64_t K) {
-    return radix_temp_bytes(K) + ((radix_blocks(K > 0 ? K : 1) + 1) * sizeof(uint32_t) + 255) / 256 * 256;
 }
 
 namespace {
@@ -843,63 +841,108 @@ void radix_sort_pairs(const uint32_t* keys0, const uint32_t* vals0, uint32_t* ke
     }
 }
 
-void tile_sort(const uint32_t* order, const unsigned long long* tile_off, Count R, Count K,
-               const unsigned long long* desc, const DevCam* cams, long long tiles, int bits, uint32_t* keys_a,
-               uint32_t* vals_a, uint32_t* keys_b, uint32_t* vals_b, uint32_t* vals_out, void* tmp, cudaStream_t s) {
-    if (K.max == 0 || R.max == 0) return;
-    // the radix pass uses the front of tmp; the block starts go behind it
-    uint32_t* first_rec = reinterpret_cast<uint32_t*>(static_cast<char*>(tmp) + radix_temp_bytes(K.max));
-    const DupSrc src{order, tile_off, R, desc, cams, (uint32_t)tiles};
-    const int passes = bits > 8 ? (bits + 7) / 8 : 1;
-    // record ids take vb bits; two passes whose second digit fits beside them
-    // in one word run packed (PassMode)
-    int vb = 1;
-    while (vb < 32 && (R.max - 1) >> vb) vb++;
-    const bool packed = passes == 2 && (bits - 8) + vb <= 32;
-    uint32_t *kin = keys_a, *vin = vals_a, *kout = keys_b, *vout = vals_b;
-    for (int p = 0; p < passes; p++) {
-        const bool last = p == passes - 1;
-        if (last) vout = vals_out;
-        const int shift = packed && last ? vb : 8 * p;
-        const int hi = bits - 8 * p;  // significant bits of this pass's digit
-        radix_pass(
-            K.max, tmp, s,
-            [&](unsigned nb, uint32_t* counts) {
-                // pass 0 writes the entries and the histogram of their first digit
-                if (p == 0) {
-                    block_starts_kernel<<<(unsigned)ceil_div_u64(R.max, 256), 256, 0, s>>>(tile_off, R, nb, first_rec);
-                    if (packed)
-                        dup_hist_kernel<true><<<nb, RS_THREADS, 0, s>>>(src, first_rec, K, keys_a, vals_a, counts, nb);
+namespace {
+uint64_t bin_chunks(uint64_t S, long long bins) { return S / BC_CHUNK + (uint64_t)bins; }
+size_t round256(size_t x) { return (x + 255) / 256 * 256; }
+
+// The scratch of the tile lists inside one buffer.
+struct BinTemp {
+    size_t begin, end, chunk_off, chunk_bin, counts, tile_counts, starts, scan, bytes;
+    BinTemp(uint64_t S, long long bins, long long tiles) {
+        size_t o = 0;
+        auto take = [&](size_t n) { const size_t at = o; o += round256(n); return at; };
+        const uint64_t chunks = bin_chunks(S, bins);
+        begin = take((size_t)bins * sizeof(uint32_t));
+        end = take((size_t)bins * sizeof(uint32_t));
+        chunk_off = take((size_t)(bins + 1) * sizeof(uint32_t));
+        chunk_bin = take(chunks * sizeof(uint32_t));
+        counts = take(chunks * 64 * sizeof(uint32_t));
+        tile_counts = take((size_t)tiles * sizeof(uint32_t));
+        starts = take((size_t)(tiles + 1) * sizeof(unsigned long long));
+        scan = take(scan_temp_bytes((uint64_t)tiles));
+        bytes = o;
+    }
+};
+
+template <class T>
+T* part(void* tmp, size_t off) { return reinterpret_cast<T*>(static_cast<char*>(tmp) + off); }
+}  // namespace
+
+size_t tile_lists_temp_bytes(uint64_t S, long long bins, long long tiles) { return BinTemp(S, bins, tiles).bytes; }
+
+void tile_lists(const uint32_t* order, const unsigned long long* bin_off, Count R, Count S, Count K,
+                const unsigned long long* desc, const DevCam* cams, int V, long long bins, long long tiles,
+                uint32_t* keys_a, uint32_t* vals_a, uint32_t* keys_b, uint32_t* vals_b, uint32_t* sorted,
+                long long* ranges, uint64_t S_cap, void* tmp, void* radix_tmp, cudaStream_t s) {
+    const BinTemp T(S_cap, bins, tiles);
+    uint32_t* tile_counts = part<uint32_t>(tmp, T.tile_counts);
+    unsigned long long* starts = part<unsigned long long>(tmp, T.starts);
+    const bool any = S.max > 0 && R.max > 0;
+    const bool local = bins <= BIN_LOCAL_MAX;
+    BinLists L{};
+    const unsigned chunks = (unsigned)bin_chunks(S.max, bins);
+    if (!any) {
+        cudaMemsetAsync(tile_counts, 0, (size_t)tiles * sizeof(uint32_t), s);
+    } else {
+        StageTimer timer(MVGS_STAGE_TILE_SORT, s);
+        uint32_t *kin = keys_a, *vin = vals_a, *kout = keys_b, *vout = vals_b;
+        const unsigned rblocks = (unsigned)ceil_div_u64(R.max, 256);
+        if (local) bin_entries_kernel<true><<<rblocks, 256, 0, s>>>(order, bin_off, R, S, desc, cams, kin, vin);
+        else bin_entries_kernel<false><<<rblocks, 256, 0, s>>>(order, bin_off, R, S, desc, cams, kin, vin);
+        const int low = local ? BIN_LOCAL_BITS : 0;
+        int bits = 0;
+        while ((1LL << bits) < bins) bits++;
+        for (int p = 0; 8 * p < bits; p++) {
+            const int shift = low + 8 * p, hi = bits - 8 * p;  // hi: significant bits from this digit up
+            radix_pass(
+                S.max, radix_tmp, s,
+                [&](unsigned nb, uint32_t* counts) {
+                    if (hi <= 5)
+                        rs_upsweep_narrow<<<nb, RS_THREADS, 0, s>>>(kin, S, shift, (1u << hi) - 1u, counts, nb);
                     else
-                        dup_hist_kernel<false><<<nb, RS_THREADS, 0, s>>>(src, first_rec, K, keys_a, vals_a, counts, nb);
-                    note_launches(1);
-                } else if (hi <= 5) {
-                    rs_upsweep_narrow<<<nb, RS_THREADS, 0, s>>>(kin, K, shift, (1u << hi) - 1u, counts, nb);
-                } else {
-                    rs_upsweep<<<nb, RS_THREADS, 0, s>>>(kin, K, shift, counts, nb);
-                }
-            },
-            [&](unsigned nb, uint32_t* counts) {
-                if (packed && !last)
-                    rs_downsweep<true, 8, kPackOut><<<nb, RS_THREADS, 0, s>>>(kin, vin, kout, nullptr, K, shift, counts,
-                                                                               nb, nullptr, nullptr, vb);
-                else if (packed && hi <= 5)
-                    rs_downsweep<false, 5, kPackIn><<<nb, RS_THREADS, 0, s>>>(kin, nullptr, nullptr, vout, K, shift,
-                                                                               counts, nb, nullptr, nullptr, vb);
-                else if (packed)
-                    rs_downsweep<false, 8, kPackIn><<<nb, RS_THREADS, 0, s>>>(kin, nullptr, nullptr, vout, K, shift,
-                                                                               counts, nb, nullptr, nullptr, vb);
-                else if (last && hi <= 5)
-                    rs_downsweep<false, 5><<<nb, RS_THREADS, 0, s>>>(kin, vin, kout, vout, K, shift, counts, nb);
-                else if (last) rs_downsweep<false><<<nb, RS_THREADS, 0, s>>>(kin, vin, kout, vout, K, shift, counts, nb);
-                else rs_downsweep<true><<<nb, RS_THREADS, 0, s>>>(kin, vin, kout, vout, K, shift, counts, nb);
-            });
-        uint32_t* nk = kin;
-        uint32_t* nv = vin;
-        kin = kout;
-        vin = vout;
-        kout = nk;
-        vout = nv;
+                        rs_upsweep<<<nb, RS_THREADS, 0, s>>>(kin, S, shift, counts, nb);
+                },
+                [&](unsigned nb, uint32_t* counts) {
+                    if (hi <= 5)
+                        rs_downsweep<true, 5><<<nb, RS_THREADS, 0, s>>>(kin, vin, kout, vout, S, shift, counts, nb);
+                    else
+                        rs_downsweep<true><<<nb, RS_THREADS, 0, s>>>(kin, vin, kout, vout, S, shift, counts, nb);
+                });
+            uint32_t *nk = kin, *nv = vin;
+            kin = kout;
+            vin = vout;
+            kout = nk;
+            vout = nv;
+        }
+        uint32_t* begin = part<uint32_t>(tmp, T.begin);
+        uint32_t* end = part<uint32_t>(tmp, T.end);
+        uint32_t* chunk_off = part<uint32_t>(tmp, T.chunk_off);
+        L = BinLists{kin, vin, desc, begin, end, chunk_off, part<uint32_t>(tmp, T.chunk_bin),
+                     part<uint32_t>(tmp, T.counts), (uint32_t)bins};
+        if (bins > 1) {
+            cudaMemsetAsync(begin, 0, T.chunk_off - T.begin, s);  // begin and end
+            bin_bounds_kernel<<<(unsigned)ceil_div_u64(S.max, 1024), 256, 0, s>>>(kin, S, low, begin, end);
+            note_launches(1);
+        }
+        bin_chunks_kernel<<<1, SPINE_THREADS, 0, s>>>(begin, end, S, bins, chunk_off);
+        if (local) bin_count_kernel<true><<<chunks, BC_THREADS, 0, s>>>(L, cams, V);
+        else bin_count_kernel<false><<<chunks, BC_THREADS, 0, s>>>(L, cams, V);
+        bin_scan_kernel<<<(unsigned)bins, 64 * BS_PARTS, 0, s>>>(L, cams, V, tile_counts);
+        note_launches(4);
+    }
+    {
+        StageTimer timer(MVGS_STAGE_RANGES, s);
+        scan_u32_to_u64(tile_counts, starts, (uint64_t)tiles, part<void>(tmp, T.scan), s);
+        ranges_kernel<<<(unsigned)ceil_div_u64((uint64_t)tiles, 256), 256, 0, s>>>(starts, tiles, K, ranges);
+        note_launches(1);
+    }
+    if (any) {
+        StageTimer timer(MVGS_STAGE_TILE_SORT, s);
+        if (local)
+            bin_place_kernel<true><<<chunks, BC_THREADS, 0, s>>>(L, cams, V, ranges, starts + tiles, K, sorted);
+        else
+            bin_place_kernel<false><<<chunks, BC_THREADS, 0, s>>>(L, cams, V, ranges, starts + tiles, K, sorted);
+        note_launches(1);
     }
 }
 
@@ -909,64 +952,6 @@ void tile_order(const long long* ranges, long long tiles, uint32_t* order, void*
     if (tiles <= 0) return;
     tile_order_kernel<<<1, TO_THREADS, 0, s>>>(ranges, tiles, order);
     note_launches(1);
-}
-
-static long long diff_cells(const DevCam* host_cams, int V) {
-    long long cells = 0;
-    for (int v = 0; v < V; v++) cells += (long long)(host_cams[v].tiles_x + 1) * (host_cams[v].tiles_y + 1);
-    return cells;
-}
-
-size_t tile_count_temp_bytes(const DevCam* host_cams, int V, long long tiles) {
-    const long long cells = diff_cells(host_cams, V);
-    const size_t a = ((size_t)cells * sizeof(int) + 255) / 256 * 256;
-    const size_t b = ((size_t)tiles * sizeof(uint32_t) + 255) / 256 * 256;
-    const size_t c = ((size_t)(tiles + 1) * sizeof(unsigned long long) + 255) / 256 * 256;
-    const size_t d = cells <= RD_MAX_CELLS ? (size_t)RD_PARTS * a : 0;
-    return a + b + c + d + scan_temp_bytes((uint64_t)tiles);
-}
-
-void tile_ranges_from_rects(const short4* rect, const int* rec_v, Count R, Count K, const DevCam* cams,
-                            const DevCam* host_cams, int V, long long tiles, long long* ranges, void* tmp,
-                            cudaStream_t s) {
-    const long long cells = diff_cells(host_cams, V);
-    const size_t a = ((size_t)cells * sizeof(int) + 255) / 256 * 256;
-    char* base = static_cast<char*>(tmp);
-    int* diff = reinterpret_cast<int*>(base);
-    base += a;
-    uint32_t* counts = reinterpret_cast<uint32_t*>(base);
-    base += ((size_t)tiles * sizeof(uint32_t) + 255) / 256 * 256;
-    unsigned long long* starts = reinterpret_cast<unsigned long long*>(base);
-    base += ((size_t)(tiles + 1) * sizeof(unsigned long long) + 255) / 256 * 256;
-    if (cells <= RD_MAX_CELLS) {
-        int* parts = reinterpret_cast<int*>(base);
-        base += (size_t)RD_PARTS * a;
-        const size_t smem = (size_t)cells * sizeof(int);
-        // raise the kernel's shared-memory limit once per device, to the
-        // largest size used (not at every call: the call may be captured)
-        static thread_local int raised[64] = {0};
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (dev < 64 && raised[dev] < (int)(RD_MAX_CELLS * sizeof(int))) {
-            cudaFuncSetAttribute(rect_diff_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(RD_MAX_CELLS * sizeof(int)));
-            raised[dev] = (int)(RD_MAX_CELLS * sizeof(int));
-        }
-        rect_diff_smem_kernel<<<RD_PARTS, RD_THREADS, smem, s>>>(rect, rec_v, R, cams, (int)cells, parts);
-        sum_parts_kernel<<<(unsigned)ceil_div_u64((uint64_t)cells, 256), 256, 0, s>>>(parts, (int)cells, RD_PARTS,
-                                                                                       diff);
-        note_launches(2);
-    } else {
-        cudaMemsetAsync(diff, 0, (size_t)cells * sizeof(int), s);
-        if (R.max > 0) {
-            rect_diff_kernel<<<(unsigned)ceil_div_u64(R.max, 256), 256, 0, s>>>(rect, rec_v, R, cams, diff);
-            note_launches(1);
-        }
-    }
-    diff_to_counts_kernel<<<V, 256, 0, s>>>(cams, diff, counts);
-    scan_u32_to_u64(counts, starts, (uint64_t)tiles, base, s);
-    ranges_kernel<<<(unsigned)ceil_div_u64((uint64_t)tiles, 256), 256, 0, s>>>(starts, tiles, K, ranges);
-    note_launches(2);
 }
 
 }  // namespace mvgs
