@@ -120,6 +120,7 @@ struct Plan {
     std::vector<DevCam> cams;
     long long tiles = 0, pixels = 0, bins = 0;
     mvgs_layout L{};
+    size_t s_geom = 0;  // state: the records' Geom array (not part of the public layout)
     // workspace offsets (forward)
     size_t w_cams = 0, w_counts = 0, w_vis = 0, w_scan = 0, w_dkeys_a = 0, w_dkeys_b = 0, w_ids_a = 0, w_ids_b = 0,
            w_order = 0, w_bins = 0, w_desc = 0, w_bin_off = 0, w_keys_a = 0, w_keys_b = 0, w_vals_a = 0, w_vals_b = 0,
@@ -219,6 +220,7 @@ mvgs_status make_plan(long long n, const mvgs_camera* cams, int V, const mvgs_co
     L.off_n_contrib = s.take((size_t)pixels * sizeof(uint32_t));
     L.off_pixel_stats = s.take((size_t)pixels * 2 * sizeof(uint32_t));
     L.off_pixel_depth = s.take((size_t)pixels * sizeof(float));
+    P.s_geom = s.take(R * sizeof(Geom));
     L.state_bytes = s.off;
     L.tiles = tiles;
     L.pixels = pixels;
@@ -285,7 +287,8 @@ const T* at(const void* base, size_t off) {
     return reinterpret_cast<const T*>(static_cast<const char*>(base) + off);
 }
 
-RecordArgs record_args(void* state, const mvgs_layout& L) {
+RecordArgs record_args(void* state, const Plan& P) {
+    const mvgs_layout& L = P.L;
     RecordArgs r;
     r.rec_off = at<long long>(state, L.off_rec_offsets);
     r.rec_g = at<int>(state, L.off_rec_gauss);
@@ -296,6 +299,7 @@ RecordArgs record_args(void* state, const mvgs_layout& L) {
     r.clamp = at<int>(state, L.off_rec_clamp);
     r.depth = at<float>(state, L.off_rec_depth);
     r.rect = at<short4>(state, L.off_rec_rect);
+    r.geom = at<Geom>(state, P.s_geom);
     r.cap = 0;
     return r;
 }
@@ -470,7 +474,7 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
     unsigned long long* sums = dcnt + 8;
     upload_cams(P.cams.data(), V, dcams, s, sums, 2 * kSumSlots);
     const SceneArgs sc = scene_args(scene);
-    RecordArgs rec = record_args(state, L);
+    RecordArgs rec = record_args(state, P);
     long long* counts_dev = at<long long>(state, L.off_counts);
 
     // participation: which (Gaussian, view) pairs are visible, Gaussian-major
@@ -573,8 +577,7 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
     ba.ranges = ranges;
     ba.order = at<uint32_t>(state, L.off_tile_order);
     ba.sorted = sorted;
-    ba.xy = rec.xy;
-    ba.conic_o = rec.conic_o;
+    ba.geom = rec.geom;
     ba.rgb_r = rec.rgb_r;
     for (int i = 0; i < 3; i++) ba.bg[i] = cfg->bg[i];
     ba.rec_depth = rec.depth;
@@ -613,7 +616,7 @@ static mvgs_status backward_impl(const mvgs_scene* scene, const mvgs_camera* cam
     DevCam* dcams = at<DevCam>(workspace, P.b_cams);
     upload_cams(P.cams.data(), V, dcams, s);
     void* st_mut = const_cast<void*>(state);  // read only below; RecordArgs carries non-const pointers
-    RecordArgs rec = record_args(st_mut, L);
+    RecordArgs rec = record_args(st_mut, P);
     rec.cap = cap->records;
     float* rec_grad = at<float>(workspace, P.b_grad);
     double* rec_conic = reinterpret_cast<double*>(rec_grad + (size_t)cap->records * kGradStride);
@@ -636,8 +639,7 @@ static mvgs_status backward_impl(const mvgs_scene* scene, const mvgs_camera* cam
     ba.ranges = at<long long>(state, L.off_tile_ranges);
     ba.order = at<uint32_t>(state, L.off_tile_order);
     ba.sorted = at<uint32_t>(state, L.off_sorted_records);
-    ba.xy = rec.xy;
-    ba.conic_o = rec.conic_o;
+    ba.geom = rec.geom;
     ba.rgb_r = rec.rgb_r;
     for (int i = 0; i < 3; i++) ba.bg[i] = cfg->bg[i];
     ba.rec_depth = rec.depth;

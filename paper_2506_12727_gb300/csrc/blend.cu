@@ -30,8 +30,8 @@
 // lane's one column), then over the
 // warp by a reduce-scatter (12 shuffles for 10 values), and one lane per
 // value adds it with one atomic.
+#include <map>
 #include <mutex>
-#include <unordered_map>
 
 #include "kernels.h"
 
@@ -163,114 +163,300 @@ __device__ __forceinline__ bool next_work(const BlendArgs& a, int* counter, int 
     else return next_strip<PPT>(a, counter, lane, w);
 }
 
-// Resident blocks per SM the forward is compiled for: six (at most 80
-// registers) for 4 pixels per lane without the depth and statistics outputs
-// (strips and sample runs), where the extra warps hide more latency than the
-// registers given up cost (3-4% faster); no bound elsewhere (more state
-// there, and a bound spills it).
-constexpr int fwd_min_blocks(int ppt, bool extra) { return ppt == 4 && !extra ? 6 : 1; }
+// A Gaussian staged by the forward: the values of the per-pixel arithmetic
+// twice each, as operands of the packed instructions.
+struct alignas(16) FwdEntry {
+    float4 m;     // -mx, -mx, -my, -my
+    float4 qab;   // qa, qa, qb, qb
+    float4 qco;   // qc, qc, -o, -o
+    float4 rg;    // -r, -r, -g, -g
+    float4 brp;   // -b, -b, radius, list position (bit 31: every test of pair_eval is needed)
+};
+static_assert(sizeof(FwdEntry) == 80, "five 16-byte reads");
+constexpr uint32_t kTestAll = 0x80000000u;  // a list has fewer than 2^31 entries, one per record at most
+
+// The forward looks at FWD_SCAN list entries at a time until more than FWD_FLUSH
+// of them reach the work item (or the list ends), then blends those: where few
+// do, the scan goes on at the pace of its own loads.  The staging takes 30 KB
+// per block; with 40 KB the L1 cache that is left thrashes under the fetches.
+constexpr int FWD_SCAN = 64, FWD_FLUSH = 32, FWD_STAGE = FWD_SCAN + FWD_FLUSH;
+
+// Resident blocks per SM the forward is compiled for: four (at most 128
+// registers) for 4 pixels per lane without the depth and statistics outputs.
+// More warps fetch more records at once than the L1 cache holds (five blocks:
+// 3M Gaussians x 8 views 3.13 -> 3.44 ms, 500k x 4 0.62 -> 0.73), fewer leave
+// latency open (three: 3.6 ms).  No bound elsewhere: more state there.
+constexpr int fwd_min_blocks(int ppt, bool extra) { return ppt == 4 && !extra ? 4 : 1; }
 
 // DEPTH: also the expected depth per pixel; STATS: also the per-pixel
 // statistics (list position where the pixel stopped, Gaussians blended).
-template <int PPT, bool SAMPLED, int WBATCH, bool DEPTH, bool STATS>
+//
+// Bound by instruction issue where most staged Gaussians are blended, by the L2
+// sectors of the scanned list entries where few are.  So a lane's pixels are
+// taken two at a time with packed float32 arithmetic and without branches: a
+// pixel that the Gaussian does not reach blends it with alpha 0, which leaves T
+// and C as they are, bit for bit; a stopped pixel's threshold is raised out of
+// reach; the rare stop is found with one vote per Gaussian.  Gaussians for which
+// that could differ (plain_gaussian) take the pixels one by one with every
+// test.  Warp instructions per staged Gaussian (128 pixels) 109 -> 75, per 32
+// list entries scanned 193 -> 110, L2 sectors per entry 3.1 -> 1.4 (Geom).
+// 3M Gaussians x 8 views at 32 x 64 tiles (2.1e9 blended pairs) 5.46 -> 3.13 ms,
+// 1M x 16 views at 16 x 64 3.59 -> 2.60, 500k x 4 views 0.94 -> 0.62, 2M x 5
+// views 2.34 -> 1.28, 500k x 1 view at 16 x 16 0.33 -> 0.21.
+template <int PPT, bool SAMPLED, bool DEPTH, bool STATS>
 __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, fwd_min_blocks(PPT, DEPTH || STATS))
-    blend_forward_kernel(BlendArgs a, int* __restrict__ counter,
-                                                                             float* __restrict__ img,
-                                                                             float* __restrict__ final_T,
-                                                                             uint32_t* __restrict__ n_contrib,
-                                                                             uint2* __restrict__ pixel_stats) {
-    __shared__ float2 s_xy[WARPS_PER_BLOCK][WBATCH];
-    __shared__ float4 s_co[WARPS_PER_BLOCK][WBATCH];
-    __shared__ float4 s_rgb[WARPS_PER_BLOCK][WBATCH];
-    __shared__ uint32_t s_pos[WARPS_PER_BLOCK][WBATCH];
-    __shared__ float s_dep[WARPS_PER_BLOCK][DEPTH ? WBATCH : 1];
+    blend_forward_kernel(BlendArgs a, int* __restrict__ counter, float* __restrict__ img,
+                         float* __restrict__ final_T, uint32_t* __restrict__ n_contrib,
+                         uint2* __restrict__ pixel_stats) {
+    __shared__ FwdEntry s_ent[WARPS_PER_BLOCK][FWD_STAGE];
+    __shared__ uint32_t s_rid[WARPS_PER_BLOCK][FWD_STAGE];
+    __shared__ float s_dep[WARPS_PER_BLOCK][DEPTH ? FWD_STAGE : 1];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t lt = (1u << lane) - 1u;
-    float2* wxy = s_xy[w];
-    float4* wco = s_co[w];
-    float4* wrgb = s_rgb[w];
-    uint32_t* wpos = s_pos[w];
+    FwdEntry* ent = s_ent[w];
+    uint32_t* wrid = s_rid[w];
     float* wdep = s_dep[w];
-    constexpr uint32_t ALL = (1u << PPT) - 1u;
+    constexpr float kStopped = 2.f;  // no alpha reaches it
+    constexpr int NP = (PPT + 1) / 2, NK = 2 * NP;  // pairs, pixel slots (one idle slot with 1 pixel per lane)
+    float one1, one2;  // kept in registers (a constant would be moved there at every use)
+    asm volatile("mov.f32 %0, %1;" : "=f"(one1) : "f"(1.f));
+    asm volatile("mov.f32 %0, %1;" : "=f"(one2) : "f"(1.f));
+    const f32x2 one = pack2(one1, one2);
     const long long total = SAMPLED ? min(a.chunk_off[a.tiles], a.chunk_cap) : 0;
     Work<PPT> st;
     while (next_work<PPT, SAMPLED>(a, counter, lane, total, st)) {
         const DevCam& cam = *st.cam;
         const long long start = a.ranges[2 * st.gt], end = a.ranges[2 * st.gt + 1];
-        float T[PPT], C0[PPT], C1[PPT], C2[PPT], D[PPT];
-        uint32_t last[PPT], stop[PPT], nblend[PPT];
-        uint32_t done = 0;
+        f32x2 T[NP], C0[NP], C1[NP], C2[NP], D[NP], FX[SAMPLED ? NP : 1], FY[NP];
+        float nmin[NK];  // minus the least alpha that blends; -kStopped once the pixel has stopped
+        uint32_t last[NK], stop[NK], nblend[NK];
 #pragma unroll
-        for (int k = 0; k < PPT; k++) {
-            T[k] = 1.f;
-            C0[k] = C1[k] = C2[k] = D[k] = 0.f;
+        for (int p = 0; p < NP; p++) {
+            const int k = 2 * p, l = k + 1 < PPT ? k + 1 : k;
+            T[p] = pack2(1.f, 1.f);
+            C0[p] = C1[p] = C2[p] = D[p] = pack2(0.f, 0.f);
+            if (SAMPLED || p == 0) FX[SAMPLED ? p : 0] = pack2(st.fx[k], st.fx[l]);
+            FY[p] = pack2(st.fy[k], st.fy[l]);
+        }
+#pragma unroll
+        for (int k = 0; k < NK; k++) {
             last[k] = 0;
             stop[k] = (uint32_t)(end - start);  // list position where the pixel stopped
             nblend[k] = 0;
-            if (st.pix[k] < 0) done |= 1u << k;
+            nmin[k] = k >= PPT || st.pix[k < PPT ? k : 0] < 0 ? -kStopped : -kAlphaMin;
         }
-        for (long long b = start; b < end; b += WBATCH) {
-            if (__all_sync(kFull, done == ALL)) break;
-            // stage the Gaussians of this batch that can reach a pixel of the work item
+        auto all_stopped = [&]() {
+            bool d = true;
+#pragma unroll
+            for (int k = 0; k < NK; k++) d = d && nmin[k] == -kStopped;
+            return d;
+        };
+        const uint32_t len = (uint32_t)(end - start);  // one entry per record at most: below 2^31
+        const uint32_t* list = a.sorted + start;
+        // one Gaussian that plain_gaussian lets through, on all pixels; true
+        // when the warp's last pixel has stopped (votes keep the warp together)
+        auto plain_step = [&](const FwdEntry& e, float dep) {
+            const float4 em = e.m, eq = e.qab, eo = e.qco, ec = e.rg, eb = e.brp;
+            const uint32_t pos1 = __float_as_uint(eb.w) + 1;
+            const float radius = eb.z;
+            const f32x2 nmx = pack2(em.x, em.y), nmy = pack2(em.z, em.w), qa = pack2(eq.x, eq.y),
+                        qb = pack2(eq.z, eq.w), qc = pack2(eo.x, eo.y), no = pack2(eo.z, eo.w);
+            f32x2 xx{}, x{}, na[NP], om[NP];  // na: minus alpha, om: 1 - alpha
+            bool in0 = true, in1 = true, ok[NK];
+            float tmin;
+#pragma unroll
+            for (int p = 0; p < NP; p++) {
+                const int k = 2 * p, l = 2 * p + 1;
+                if (SAMPLED || p == 0) {
+                    const f32x2 dx = add2(FX[SAMPLED ? p : 0], nmx);
+                    xx = mul2(mul2(qa, dx), dx);
+                    x = mul2(qb, dx);
+                    float dx0, dx1;
+                    unpack2(dx, dx0, dx1);
+                    in0 = fabsf(dx0) <= radius;
+                    in1 = SAMPLED ? fabsf(dx1) <= radius : in0;
+                }
+                const f32x2 dy = add2(FY[p], nmy);
+                float dy0, dy1, e0, e1, v0, v1, t0, t1;
+                unpack2(dy, dy0, dy1);
+                unpack2(fma2(dy, fma2(qc, dy, x), xx), e0, e1);
+                unpack2(mul2(no, pack2(ex2_approx(e0), ex2_approx(e1))), v0, v1);
+                ok[k] = in0 & (fabsf(dy0) <= radius) & (v0 <= nmin[k]);
+                ok[l] = in1 & (fabsf(dy1) <= radius) & (v1 <= nmin[l]);
+                na[p] = pack2(ok[k] ? v0 : 0.f, ok[l] ? v1 : 0.f);
+                om[p] = add2(na[p], one);
+                unpack2(mul2(T[p], om[p]), t0, t1);
+                tmin = p == 0 ? fminf(t0, t1) : fminf(tmin, fminf(t0, t1));
+            }
+            const f32x2 r2 = pack2(ec.x, ec.y), g2 = pack2(ec.z, ec.w), b2 = pack2(eb.x, eb.y);
+            auto add_colour = [&](int p, f32x2 nal) {
+                const f32x2 nw = mul2(nal, T[p]);  // minus the weight, times minus the colour
+                C0[p] = fma2(r2, nw, C0[p]);
+                C1[p] = fma2(g2, nw, C1[p]);
+                C2[p] = fma2(b2, nw, C2[p]);
+                if (DEPTH) D[p] = fma2(pack2(-dep, -dep), nw, D[p]);
+            };
+            if (!__any_sync(kFull, tmin < kTMin)) {
+#pragma unroll
+                for (int p = 0; p < NP; p++) {
+                    add_colour(p, na[p]);
+                    T[p] = mul2_fresh(T[p], om[p]);
+                }
+#pragma unroll
+                for (int k = 0; k < NK; k++) {
+                    last[k] = ok[k] ? pos1 : last[k];
+                    if (STATS) nblend[k] += ok[k];
+                }
+                return false;
+            }
+            // some pixel of the warp stops here: its alpha becomes 0
+#pragma unroll
+            for (int p = 0; p < NP; p++) {
+                float t[2], al[2];
+                unpack2(mul2(T[p], om[p]), t[0], t[1]);
+                unpack2(na[p], al[0], al[1]);
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const int k = 2 * p + h;
+                    if (t[h] < kTMin) {
+                        al[h] = 0.f;
+                        nmin[k] = -kStopped;
+                        if (STATS) stop[k] = pos1;
+                    }
+                    if (al[h] < 0.f) {
+                        last[k] = pos1;
+                        if (STATS) nblend[k]++;
+                    }
+                }
+                const f32x2 nal = pack2(al[0], al[1]);
+                add_colour(p, nal);
+                T[p] = mul2(T[p], add2(nal, one));
+            }
+            return (bool)__all_sync(kFull, all_stopped());
+        };
+        // any Gaussian, pixel by pixel with every test
+        auto general_step = [&](const FwdEntry& e, float dep) {
+            const float4 em = e.m, eq = e.qab, eo = e.qco, ec = e.rg, eb = e.brp;
+            const float radius = eb.z;
+            const float4 q = make_float4(eq.x, eq.z, eo.x, -eo.z);
+            const uint32_t pos1 = (__float_as_uint(eb.w) & ~kTestAll) + 1;
+            auto blend_one = [&](int k, float fx, float fy, float& Tk, float& c0, float& c1, float& c2, float& d) {
+                if (nmin[k] == -kStopped) return;
+                const float dx = fx + em.x;
+                float alpha, G;
+                if (!pair_eval(dx, fy + em.z, col_terms(dx, q), q, radius, alpha, G)) return;
+                const float Tn = __fmul_rn(Tk, __fsub_rn(1.f, alpha));
+                if (Tn < kTMin) {
+                    nmin[k] = -kStopped;
+                    if (STATS) stop[k] = pos1;
+                    return;
+                }
+                const float wgt = __fmul_rn(alpha, Tk);
+                c0 = __fmaf_rn(-ec.x, wgt, c0);
+                c1 = __fmaf_rn(-ec.z, wgt, c1);
+                c2 = __fmaf_rn(-eb.x, wgt, c2);
+                if (DEPTH) d = __fmaf_rn(dep, wgt, d);
+                Tk = Tn;
+                last[k] = pos1;
+                if (STATS) nblend[k]++;
+            };
+#pragma unroll
+            for (int p = 0; p < NP; p++) {
+                float u[5][2], f0, f1, y0, y1;
+                unpack2(T[p], u[0][0], u[0][1]);
+                unpack2(C0[p], u[1][0], u[1][1]);
+                unpack2(C1[p], u[2][0], u[2][1]);
+                unpack2(C2[p], u[3][0], u[3][1]);
+                unpack2(D[p], u[4][0], u[4][1]);
+                unpack2(FX[SAMPLED ? p : 0], f0, f1);
+                unpack2(FY[p], y0, y1);
+                blend_one(2 * p, f0, y0, u[0][0], u[1][0], u[2][0], u[3][0], u[4][0]);
+                blend_one(2 * p + 1, f1, y1, u[0][1], u[1][1], u[2][1], u[3][1], u[4][1]);
+                T[p] = pack2(u[0][0], u[0][1]);
+                C0[p] = pack2(u[1][0], u[1][1]);
+                C1[p] = pack2(u[2][0], u[2][1]);
+                C2[p] = pack2(u[3][0], u[3][1]);
+                if (DEPTH) D[p] = pack2(u[4][0], u[4][1]);
+            }
+            return (bool)__all_sync(kFull, all_stopped());
+        };
+        // the next batch's geometry (and the ids of the one after it) is fetched
+        // while the present one is blended
+        uint32_t rec[2], nid[2];
+        Geom g[2];
+        auto fetch_ids = [&](uint32_t b) {
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const uint32_t i = b + 32 * h + lane;
+                nid[h] = i < len ? list[i] : 0u;
+            }
+        };
+        auto fetch_geometry = [&](uint32_t b) {
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                rec[h] = nid[h];
+                if (b + 32 * h + lane < len) g[h] = load_geom(a.geom + rec[h]);
+            }
+        };
+        fetch_ids(0);
+        fetch_geometry(0);
+        fetch_ids(FWD_SCAN);
+        for (uint32_t b = 0; b < len;) {
+            if (__all_sync(kFull, all_stopped())) break;
+            // stage the Gaussians that can reach a pixel of the work item
             __syncwarp();
             int n = 0;
-            for (int i0 = 0; i0 < WBATCH; i0 += 32) {
-                const long long idx = b + i0 + lane;
-                bool hit = false;
-                float2 m;
-                float4 co, cr;
-                uint32_t r = 0;
-                if (idx < end) {
-                    r = a.sorted[idx];
-                    m = a.xy[r];
-                    co = a.conic_o[r];
-                    cr = a.rgb_r[r];
-                    hit = rect_reaches(st.sx0 - m.x, st.sx1 - m.x, st.sy0 - m.y, st.sy1 - m.y, co, cr.w);
+            bool odd = false;
+            do {
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const bool hit = b + 32 * h + lane < len && rect_reaches(st.sx0, st.sx1, st.sy0, st.sy1, g[h]);
+                    const uint32_t bal = __ballot_sync(kFull, hit);
+                    if (hit) {
+                        const int slot = n + __popc(bal & lt);
+                        const bool plain = g[h].radius >= 0.f;
+                        odd |= !plain;
+                        ent[slot].m = make_float4(-g[h].mx, -g[h].mx, -g[h].my, -g[h].my);
+                        ent[slot].qab = make_float4(g[h].qa, g[h].qa, g[h].qb, g[h].qb);
+                        ent[slot].qco = make_float4(g[h].qc, g[h].qc, -g[h].o, -g[h].o);
+                        ent[slot].brp.w = __uint_as_float((b + 32 * h + lane) | (plain ? 0u : kTestAll));
+                        wrid[slot] = rec[h];
+                    }
+                    n += __popc(bal);
                 }
-                const uint32_t bal = __ballot_sync(kFull, hit);
-                if (hit) {
-                    const int slot = n + __popc(bal & lt);
-                    wxy[slot] = m;
-                    wco[slot] = exp2_coeffs(co);
-                    wrgb[slot] = cr;
-                    wpos[slot] = (uint32_t)(idx - start);
-                    if (DEPTH) wdep[slot] = a.rec_depth[r];
+                b += FWD_SCAN;
+                if (b < len) {
+                    fetch_geometry(b);
+                    fetch_ids(b + FWD_SCAN);
                 }
-                n += __popc(bal);
+            } while (n <= FWD_FLUSH && b < len);
+            __syncwarp();
+            // their colours, each lane's entries (at most three) in flight together
+            float4 cr[(FWD_STAGE + 31) / 32];
+#pragma unroll
+            for (int i = 0; i < (FWD_STAGE + 31) / 32; i++)
+                if (32 * i + lane < n) cr[i] = a.rgb_r[wrid[32 * i + lane]];
+#pragma unroll
+            for (int i = 0; i < (FWD_STAGE + 31) / 32; i++) {
+                const int e = 32 * i + lane;
+                if (e < n) {
+                    ent[e].rg = make_float4(-cr[i].x, -cr[i].x, -cr[i].y, -cr[i].y);
+                    *reinterpret_cast<float2*>(&ent[e].brp) = make_float2(-cr[i].z, -cr[i].z);
+                    ent[e].brp.z = cr[i].w;
+                    if (DEPTH) wdep[e] = a.rec_depth[wrid[e]];
+                }
             }
             __syncwarp();
-            for (int j = 0; j < n; j++) {
-                const float2 m = wxy[j];
-                const float4 cr = wrgb[j];
-                const float dx0 = st.fx[0] - m.x;
-                if (!SAMPLED && fabsf(dx0) > cr.w) continue;  // outside the support for the whole column
-                const float4 q = wco[j];
-                const uint32_t pos = wpos[j];
-                const float dep = DEPTH ? wdep[j] : 0.f;
-                const ColTerms ct0 = col_terms(dx0, q);
-#pragma unroll
-                for (int k = 0; k < PPT; k++) {
-                    if ((done >> k) & 1u) continue;
-                    const float dx = SAMPLED ? st.fx[k] - m.x : dx0;
-                    const ColTerms ct = SAMPLED ? col_terms(dx, q) : ct0;
-                    float alpha, G;
-                    if (!pair_eval(dx, st.fy[k] - m.y, ct, q, cr.w, alpha, G)) continue;
-                    const float Tn = __fmul_rn(T[k], __fsub_rn(1.f, alpha));
-                    if (Tn < kTMin) {
-                        done |= 1u << k;
-                        if (STATS) stop[k] = pos + 1;
-                        continue;
-                    }
-                    const float wgt = __fmul_rn(alpha, T[k]);
-                    C0[k] = __fmaf_rn(cr.x, wgt, C0[k]);
-                    C1[k] = __fmaf_rn(cr.y, wgt, C1[k]);
-                    C2[k] = __fmaf_rn(cr.z, wgt, C2[k]);
-                    if (DEPTH) D[k] = __fmaf_rn(dep, wgt, D[k]);
-                    T[k] = Tn;
-                    last[k] = pos + 1;
-                    if (STATS) nblend[k]++;
+            if (!__any_sync(kFull, odd)) {
+                for (int j = 0; j < n; j++)
+                    if (plain_step(ent[j], DEPTH ? wdep[j] : 0.f)) break;
+            } else {
+                for (int j = 0; j < n; j++) {
+                    const float dep = DEPTH ? wdep[j] : 0.f;
+                    if (__any_sync(kFull, __float_as_uint(ent[j].brp.w) >= kTestAll) ? general_step(ent[j], dep)
+                                                                                     : plain_step(ent[j], dep))
+                        break;
                 }
-                if (done == ALL) break;
             }
         }
         const long long HW = (long long)cam.W * cam.H;
@@ -279,13 +465,19 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, fwd_min_blocks(PPT, DEPT
         for (int k = 0; k < PPT; k++) {
             const long long p = st.pix[k];
             if (p >= 0) {
-                out[p] = __fmaf_rn(T[k], a.bg[0], C0[k]);
-                out[HW + p] = __fmaf_rn(T[k], a.bg[1], C1[k]);
-                out[2 * HW + p] = __fmaf_rn(T[k], a.bg[2], C2[k]);
-                final_T[cam.pix_base + p] = T[k];
+                auto half = [k](f32x2 v) {
+                    float lo, hi;
+                    unpack2(v, lo, hi);
+                    return k & 1 ? hi : lo;
+                };
+                const float t = half(T[k / 2]);
+                out[p] = __fmaf_rn(t, a.bg[0], half(C0[k / 2]));
+                out[HW + p] = __fmaf_rn(t, a.bg[1], half(C1[k / 2]));
+                out[2 * HW + p] = __fmaf_rn(t, a.bg[2], half(C2[k / 2]));
+                final_T[cam.pix_base + p] = t;
                 n_contrib[cam.pix_base + p] = last[k];
                 if (STATS) pixel_stats[cam.pix_base + p] = make_uint2(stop[k], nblend[k]);
-                if (DEPTH) a.depth_out[cam.pix_base + p] = D[k];
+                if (DEPTH) a.depth_out[cam.pix_base + p] = half(D[k / 2]);
             }
         }
     }
@@ -392,22 +584,19 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK) blend_backward_kernel(Bl
                 const long long pos = (long long)maxlast - 1 - b - i0 - lane;
                 bool hit = false;
                 uint32_t r = 0;
-                float2 m;
-                float4 co, cr;
+                Geom g;
                 if (pos >= 0) {
                     r = a.sorted[start + pos];
-                    m = a.xy[r];
-                    co = a.conic_o[r];
-                    cr = a.rgb_r[r];
-                    hit = rect_reaches(st.sx0 - m.x, st.sx1 - m.x, st.sy0 - m.y, st.sy1 - m.y, co, cr.w);
+                    g = load_geom(a.geom + r);
+                    hit = rect_reaches(st.sx0, st.sx1, st.sy0, st.sy1, g);
                 }
                 const uint32_t bal = __ballot_sync(kFull, hit);
                 if (hit) {
                     const int slot = n + __popc(bal & lt);
                     wrid[slot] = r;
-                    wxy[slot] = m;
-                    wco[slot] = exp2_coeffs(co);
-                    wrgb[slot] = cr;
+                    wxy[slot] = make_float2(g.mx, g.my);
+                    wco[slot] = make_float4(g.qa, g.qb, g.qc, g.o);
+                    wrgb[slot] = a.rgb_r[r];
                     wpos[slot] = (uint32_t)pos;
                 }
                 n += __popc(bal);
@@ -497,19 +686,20 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK) blend_backward_kernel(Bl
     }
 }
 
-// Resident blocks over the whole GPU for a kernel (cached per kernel).
+// Resident blocks over the whole GPU for a kernel (cached per kernel and device).
 int persistent_blocks(const void* kernel) {
     static std::mutex mu;
-    static std::unordered_map<const void*, int> cache;
-    std::lock_guard<std::mutex> lk(mu);
-    auto it = cache.find(kernel);
-    if (it != cache.end()) return it->second;
+    static std::map<std::pair<const void*, int>, int> cache;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(mu);
+    const auto key = std::make_pair(kernel, dev);
+    auto it = cache.find(key);
+    if (it != cache.end()) return it->second;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * WARPS_PER_BLOCK, 0);
     const int n = (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
-    cache[kernel] = n;
+    cache[key] = n;
     return n;
 }
 
@@ -545,37 +735,33 @@ void launch_blend_forward(const BlendArgs& a, int* counter, float* img, float* f
     // full persistent grid
     const bool depth = a.depth_out != nullptr, stats = pixel_stats != nullptr;
     const long long items = sampled ? (1LL << 40) : a.tiles * a.strips;
-#define MVGS_BF1(P, S, B, D, ST)                                                                  \
-    blend_forward_kernel<P, S, B, D, ST><<<grid_for(blend_forward_kernel<P, S, B, D, ST>, items),          \
-                                           32 * WARPS_PER_BLOCK, 0, s>>>(a, counter, img, final_T, n_contrib, \
-                                                                         pixel_stats)
-#define MVGS_BF(P, S, B)                        \
-    do {                                        \
-        if (depth && stats)                     \
-            MVGS_BF1(P, S, B, true, true);      \
-        else if (depth)                         \
-            MVGS_BF1(P, S, B, true, false);     \
-        else if (stats)                         \
-            MVGS_BF1(P, S, B, false, true);     \
-        else                                    \
-            MVGS_BF1(P, S, B, false, false);    \
+#define MVGS_BF1(P, S, D, ST)                                                                             \
+    blend_forward_kernel<P, S, D, ST><<<grid_for(blend_forward_kernel<P, S, D, ST>, items),               \
+                                        32 * WARPS_PER_BLOCK, 0, s>>>(a, counter, img, final_T, n_contrib, \
+                                                                      pixel_stats)
+#define MVGS_BF(P, S)                        \
+    do {                                     \
+        if (depth && stats)                  \
+            MVGS_BF1(P, S, true, true);      \
+        else if (depth)                      \
+            MVGS_BF1(P, S, true, false);     \
+        else if (stats)                      \
+            MVGS_BF1(P, S, false, true);     \
+        else                                 \
+            MVGS_BF1(P, S, false, false);    \
     } while (0)
-#define MVGS_BF2(P, B)              \
-    do {                            \
-        if (sampled)                \
-            MVGS_BF(P, true, B);    \
-        else                        \
-            MVGS_BF(P, false, B);   \
+#define MVGS_BF2(P)              \
+    do {                         \
+        if (sampled)             \
+            MVGS_BF(P, true);    \
+        else                     \
+            MVGS_BF(P, false);   \
     } while (0)
     switch (a.ppt) {
-        case 1: MVGS_BF2(1, WBATCH_DEFAULT); break;
-        case 2: MVGS_BF2(2, WBATCH_DEFAULT); break;
-        case 8: MVGS_BF2(8, WBATCH_DEFAULT); break;
-        default:
-            if (a.wbatch == 64) MVGS_BF2(4, 64);
-            else if (a.wbatch == 192) MVGS_BF2(4, 192);
-            else MVGS_BF2(4, WBATCH_DEFAULT);
-            break;
+        case 1: MVGS_BF2(1); break;
+        case 2: MVGS_BF2(2); break;
+        case 8: MVGS_BF2(8); break;
+        default: MVGS_BF2(4); break;
     }
 #undef MVGS_BF2
 #undef MVGS_BF

@@ -157,6 +157,27 @@ __device__ __forceinline__ uint32_t bins_touched(short4 rc) {
     return (uint32_t)((((rc.z - 1) >> 3) - (rc.x >> 3) + 1) * (((rc.w - 1) >> 3) - (rc.y >> 3) + 1));
 }
 
+// Packed float32 arithmetic of sm_100 and later on a pair of registers: one
+// instruction, two IEEE round-to-nearest results (the bits of the scalar
+// operations).  It takes the FMA pipe as long as two scalar instructions but
+// one issue slot.
+typedef float2 f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) { a = v.x; b = v.y; }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) { return __ffma2_rn(a, b, c); }
+
+// A product the compiler may not merge with an equal one before it: where the
+// first is only looked at and the second replaces its factor, merging them
+// would cost a register copy per value.
+__device__ __forceinline__ f32x2 mul2_fresh(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm volatile("{.reg .b64 a, b, r; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %5}; mul.rn.f32x2 r, a, b; mov.b64 {%0, %1}, r;}"
+                 : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+
 struct ColTerms {
     float xx, x;  // qa dx^2 and qb dx
 };
@@ -184,37 +205,68 @@ __device__ __forceinline__ bool pair_eval(float dx, float dy, ColTerms ct, float
     return fabsf(dx) <= radius && fabsf(dy) <= radius && e <= 0.f && alpha >= kAlphaMin;
 }
 
-// Whether a Gaussian can pass the support rule and alpha >= 1/255 at any
-// pixel centre of the rectangle [x0, x1] x [y0, y1] (centre coordinates,
-// relative to the projected mean).  The exponent is largest where the
-// quadratic form q = A dx^2 + 2 B dx dy + C dy^2 is smallest; over a
-// rectangle that is 0 if it holds the mean, else on an edge, where q is a
-// 1D quadratic minimised in closed form.  alpha >= 1/255 needs
-// q <= 2 ln(255 o); the margin keeps the test a superset of what any pixel's
-// float32 evaluation lets through.  The edge minimisers use approximate
-// reciprocals: a point off the minimiser by a relative 1e-7 raises q by a
-// second-order amount, far inside the margin.
-__device__ __forceinline__ bool rect_reaches(float x0, float x1, float y0, float y1, float4 co, float radius) {
-    if (x0 > radius || x1 < -radius || y0 > radius || y1 < -radius) return false;
-    const float lvl = 2.f * __logf(255.f * co.w);
-    if (!(lvl > 0.f)) return false;
-    if (x0 <= 0.f && x1 >= 0.f && y0 <= 0.f && y1 >= 0.f) return true;
+// What the blend kernels read of a record to decide whether it reaches a
+// strip, in one 32-byte sector (a list entry is looked at by every strip of its
+// tile; the separate arrays of the state took three sectors).  The colour is
+// fetched for the entries that do.
+struct alignas(32) Geom {
+    float mx, my;        // projected mean
+    float qa, qb, qc;    // base-2 exponent coefficients (exp2_coeffs)
+    float o;             // opacity
+    float radius;        // in pixels; negative: not plain (plain_gaussian)
+    float reach;         // alpha >= 1/255 needs an exponent of at least -reach (base 2), with a margin
+};
+static_assert(sizeof(Geom) == 32, "one sector");
+
+__device__ __forceinline__ Geom load_geom(const Geom* g) {
+    const float4 a = reinterpret_cast<const float4*>(g)[0], b = reinterpret_cast<const float4*>(g)[1];
+    return Geom{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+}
+
+// Whether two tests of pair_eval cannot matter for a Gaussian, so that the
+// forward blend may leave them out, and blending it with alpha 0 changes
+// nothing:
+//   - e <= 0: with B^2 <= 0.99 AC the quadratic form is at least 1/400 of the
+//     sum of its terms' magnitudes, which rounding (a few 2^-24 of that sum)
+//     cannot turn negative.  The bounds on A and C keep the terms of a pixel
+//     distance (0, or at least 2^-25) clear of underflow and overflow.
+//   - the clamp at 0.99: o G stays below it when o does (G <= 1 up to the
+//     error of ex2.approx).
+//   - colour and depth are finite (their sum is only then).
+// NaN fails every comparison.
+__device__ __forceinline__ bool plain_gaussian(float4 co, float3 rgb, float depth) {
     const float A = co.x, B = co.y, C = co.z;
-    auto q = [&](float x, float y) { return A * x * x + 2.f * B * x * y + C * y * y; };
-    // edges x = x0, x = x1: minimise over y in [y0, y1]
-    const float iC = rcp_approx(C), iA = rcp_approx(A);
-    float best = 3.4e38f;
-    {
-        const float ya = fminf(fmaxf(-B * x0 * iC, y0), y1);
-        const float yb = fminf(fmaxf(-B * x1 * iC, y0), y1);
-        best = fminf(best, fminf(q(x0, ya), q(x1, yb)));
-    }
-    {
-        const float xa = fminf(fmaxf(-B * y0 * iA, x0), x1);
-        const float xb = fminf(fmaxf(-B * y1 * iA, x0), x1);
-        best = fminf(best, fminf(q(xa, y0), q(xb, y1)));
-    }
-    return best <= lvl * 1.001f + 1e-3f;
+    return (A >= 1e-15f) & (A <= 1e10f) & (C >= 1e-15f) & (C <= 1e10f) & (B * B <= 0.99f * (A * C)) &
+           (co.w <= 0.989f) & (fabsf(rgb.x) + fabsf(rgb.y) + fabsf(rgb.z) + fabsf(depth) <= 3e38f);
+}
+
+__device__ __forceinline__ Geom make_geom(float2 m, float4 co, float radius, bool plain) {
+    const float4 q = exp2_coeffs(co);
+    const float l2 = __log2f(255.f * co.w);  // o G >= 1/255 where the exponent is -l2 or more
+    return Geom{m.x, m.y, q.x, q.y, q.z, co.w, plain ? radius : -radius, l2 > 0.f ? l2 * 1.001f + 1e-3f : -1.f};
+}
+
+// Whether a Gaussian can pass the support rule and alpha >= 1/255 at any
+// pixel centre of the rectangle [x0, x1] x [y0, y1].  From the point of the
+// rectangle (relative to the mean) where the exponent is largest, the way to
+// the mean, along which it grows, must leave the rectangle, so that point lies
+// on an edge facing the mean: at most one in x and one in y, and on an edge the
+// exponent is a 1D quadratic with its maximum in closed form.  (On an axis on
+// which the rectangle holds the mean there is no such edge; its candidate below
+// is then some point of the rectangle, and the mean itself when that is
+// inside.)  The margin in `reach` keeps the test a superset of what any pixel's
+// float32 evaluation lets through; a maximiser off by a relative 1e-7 (the
+// approximate reciprocals) lowers the exponent by a second-order amount, far
+// inside it.  NaN fails the first comparisons or the last.
+__device__ __forceinline__ bool rect_reaches(float sx0, float sx1, float sy0, float sy1, const Geom& g) {
+    const float x0 = sx0 - g.mx, x1 = sx1 - g.mx, y0 = sy0 - g.my, y1 = sy1 - g.my, r = fabsf(g.radius);
+    const float xe = fminf(fmaxf(0.f, x0), x1), ye = fminf(fmaxf(0.f, y0), y1);
+    const float hb = -0.5f * g.qb;
+    const float ys = fminf(fmaxf(hb * xe * rcp_approx(g.qc), y0), y1);
+    const float xs = fminf(fmaxf(hb * ye * rcp_approx(g.qa), x0), x1);
+    const float e1 = fmaf(xe, fmaf(g.qb, ys, g.qa * xe), g.qc * ys * ys);
+    const float e2 = fmaf(xs, fmaf(g.qb, ye, g.qa * xs), g.qc * ye * ye);
+    return (x0 <= r) & (x1 >= -r) & (y0 <= r) & (y1 >= -r) & (fmaxf(e1, e2) >= -g.reach) & (g.reach > 0.f);
 }
 
 }  // namespace mvgs

@@ -56,6 +56,7 @@ struct RecordArgs {
     int* clamp;
     float* depth;
     short4* rect;
+    Geom* geom;          // what the blend tests and evaluates of a record
     long long cap;       // records the arrays hold: no record index reaches it
 };
 
@@ -127,7 +128,7 @@ struct BlendArgs {
     int V;
     int tw, th;
     int ppt;                 // pixels per lane (resolved, 1..8)
-    int wbatch;              // Gaussians per warp batch in shared memory (64, 128 or 192; 128 unless ppt 4)
+    int wbatch;              // Gaussians per warp batch of the backward (64, 128 or 192; 128 unless ppt 4)
     int sw;                  // columns of a warp's strip (blend_strip_width)
     int strip_h;             // rows of a warp's strip: (32 / sw) * ppt
     int strips;              // strips per tile: (tw / sw) * (th / strip_h)
@@ -135,9 +136,8 @@ struct BlendArgs {
     const long long* ranges;
     const uint32_t* order;   // tiles in processing order (longest lists first)
     const uint32_t* sorted;
-    const float2* xy;
-    const float4* conic_o;
-    const float4* rgb_r;
+    const Geom* geom;        // [records]
+    const float4* rgb_r;     // [records] rgb, radius
     float bg[3];
     // sampled mode (thread-efficient partial rendering, Alg. 3); s_off null
     // for the full render

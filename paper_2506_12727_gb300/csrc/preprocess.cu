@@ -375,7 +375,8 @@ __global__ void __launch_bounds__(PRE_THREADS, 8) preprocess_kernel(SceneArgs sc
             rec.rec_g[r] = (int)g;
             rec.rec_v[r] = v;
             rec.xy[r] = P.xy;
-            rec.conic_o[r] = make_float4(P.c * inv, -P.b * inv, P.a * inv, G.o);
+            const float4 co = make_float4(P.c * inv, -P.b * inv, P.a * inv, G.o);
+            rec.conic_o[r] = co;
             // colour from the direction camera -> mean
             float dx = G.mu[0] - cam.campos[0], dy = G.mu[1] - cam.campos[1], dz = G.mu[2] - cam.campos[2];
             const float il = rsqrtf(dx * dx + dy * dy + dz * dz);
@@ -391,6 +392,11 @@ __global__ void __launch_bounds__(PRE_THREADS, 8) preprocess_kernel(SceneArgs sc
                 if (rgb[ch] < 0.f) { clamp |= 1 << ch; rgb[ch] = 0.f; }
             }
             rec.rgb_r[r] = make_float4(rgb[0], rgb[1], rgb[2], (float)P.radius);
+            const bool plain = plain_gaussian(co, make_float3(rgb[0], rgb[1], rgb[2]), P.depth);
+            const Geom ge = make_geom(P.xy, co, (float)P.radius, plain);
+            float4* gout = reinterpret_cast<float4*>(rec.geom + r);
+            gout[0] = make_float4(ge.mx, ge.my, ge.qa, ge.qb);
+            gout[1] = make_float4(ge.qc, ge.o, ge.radius, ge.reach);
             rec.clamp[r] = clamp;
             rec.depth[r] = P.depth;
             rec.rect[r] = P.rect;

@@ -1,0 +1,75 @@
+"""The forward blend's two paths -- packed pixel pairs for plain Gaussians, pixel
+by pixel with every test for the others -- and its pixel counts per lane: images
+against the oracle with Gaussians of both kinds (opacities on either side of the
+0.99 clamp, needles whose conic is nearly degenerate, supports that cut the
+alpha >= 1/255 ellipse), bit for bit the same for 1, 2, 4 and 8 pixels per lane,
+and a colour that is not finite changes only the pixels that blend it."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+from gpu_helpers import assert_close_frac, gpu_forward, scene_to_device
+
+pytestmark = pytest.mark.gpu
+
+
+def _mixed_scene(n, seed):
+    rng = np.random.default_rng(seed)
+    sc = synth.make_scene(n, 1, seed=seed)
+    kind = rng.integers(0, 4, n)
+    sc.opacity_logits[kind == 0] = rng.uniform(3.0, 9.0, int((kind == 0).sum())).astype(np.float32)  # o 0.953 .. 0.9999
+    needle = kind == 1
+    sc.log_scales[needle] = np.float32(-8.0)
+    sc.log_scales[needle, 0] = rng.uniform(-2.0, -0.5, int(needle.sum())).astype(np.float32)
+    return sc
+
+
+@pytest.mark.parametrize("n,sizes", [(40, [(120, 90)]), (700, [(97, 61), (64, 128)])])
+def test_plain_and_other_gaussians_match_the_oracle(cuda_lib, n, sizes):
+    scene, cams = _mixed_scene(n, 100 + n), synth.make_cameras(sizes, radius=3.0, seed=5)
+    ref = oracle.forward(scene, cams, (16, 16), bg=(0.1, 0.2, 0.3))
+    rz, _, _, img = gpu_forward(cuda_lib, scene, cams, (16, 16), (0.1, 0.2, 0.3))
+    amb = ref["amb"] != 0
+    _, _, _, base = oracle.layout(cams, (16, 16))
+    amb3 = np.concatenate([np.tile(amb[base[v]:base[v + 1]], 3) for v in range(cams.V)])
+    assert amb.mean() < 0.1
+    assert_close_frac(img.cpu().numpy()[~amb3], ref["img"][~amb3], 0, 1e-4, "image")
+    assert_close_frac(rz.records()["final_T"].cpu().numpy()[~amb], ref["T"][~amb], 0, 1e-4, "final T")
+
+
+@pytest.mark.parametrize("seed", [1, 2])
+def test_pixels_per_lane_do_not_change_a_bit(cuda_lib, seed):
+    scene, cams = _mixed_scene(3000, seed), synth.make_cameras([(203, 157), (90, 301)], radius=3.0, seed=seed)
+    params = scene_to_device(scene)
+    sc = cuda_lib.make_scene(params, scene.sh_degree)
+    runs = []
+    for ppt in (0, 1, 2, 4, 8):
+        rz = cuda_lib.Rasterizer(cams, tile=(32, 64), pixels_per_thread=ppt)
+        img = rz.forward(sc, depth=True, stats=True)
+        rec = rz.records()
+        runs.append([img] + [rec[k].clone() for k in ("final_T", "n_contrib", "depth_acc", "pixel_stats")])
+        img2 = rz.forward(sc)
+        assert torch.equal(img, img2)
+    for r in runs[1:]:
+        for a, b in zip(r, runs[0]):
+            assert torch.equal(a, b)
+
+
+def test_a_colour_that_is_not_finite_stays_where_it_blends(cuda_lib):
+    scene, cams = synth.make_scene(400, 0, seed=9), synth.make_cameras([(150, 110)], radius=3.0, seed=9)
+    params = scene_to_device(scene)
+    g = int(torch.argmin((params["means"] ** 2).sum(1)))
+    imgs, T = [], []
+    for value in (0.5, 1.5, float("inf"), float("nan")):
+        params["sh"][g] = value
+        rz = cuda_lib.Rasterizer(cams, tile=(16, 16))
+        imgs.append(rz.forward(cuda_lib.make_scene(params, 0)))
+        T.append(rz.records()["final_T"].clone())
+    apart = imgs[0] == imgs[1]  # pixels whose colour does not hold Gaussian g
+    assert 0 < int((~apart).sum()) and int(apart.sum()) > 0
+    for img, t in zip(imgs[2:], T[2:]):
+        assert torch.equal(img[apart], imgs[0][apart])
+        assert torch.equal(t, T[0])
+        assert not torch.isfinite(img[~apart]).any()
