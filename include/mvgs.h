@@ -109,11 +109,10 @@ typedef struct mvgs_config {
                                    across wider tiles): 0 = automatic, else
                                    1, 2, 4 or 8 with the strip height dividing
                                    tile_h.  Results do not depend on it. */
-    int32_t smem_batch;         /* Gaussians a warp of the backward stages in shared
-                                   memory per batch: 0 = automatic (128), else 64,
-                                   128 or 192 (used with 4 pixels per lane; other
-                                   pixel counts use 128).  Results do not depend
-                                   on it. */
+    int32_t smem_batch;         /* 0, 64, 128 or 192.  Once the Gaussians a warp staged
+                                   in shared memory per batch; the blend kernels
+                                   now size their staging themselves, and nothing
+                                   depends on it. */
 } mvgs_config;
 
 /* cfg->flags bit for the sampled calls: blend whole strips and leave the

@@ -569,7 +569,6 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
     ba.tw = tw;
     ba.th = th;
     ba.ppt = blend_pixels_per_thread(tw, th, cfg->pixels_per_thread);
-    ba.wbatch = cfg->smem_batch ? cfg->smem_batch : 128;
     ba.sw = blend_strip_width(tw);
     ba.strip_h = (32 / ba.sw) * ba.ppt;
     ba.strips = (tw / ba.sw) * (th / ba.strip_h);
@@ -631,7 +630,6 @@ static mvgs_status backward_impl(const mvgs_scene* scene, const mvgs_camera* cam
     ba.tw = cfg->tile_w;
     ba.th = cfg->tile_h;
     ba.ppt = blend_pixels_per_thread(ba.tw, ba.th, cfg->pixels_per_thread);
-    ba.wbatch = cfg->smem_batch ? cfg->smem_batch : 128;
     ba.sw = blend_strip_width(ba.tw);
     ba.strip_h = (32 / ba.sw) * ba.ppt;
     ba.strips = (ba.tw / ba.sw) * (ba.th / ba.strip_h);

@@ -27,9 +27,9 @@
 // dC/dalpha_i = c_i T_i - S_i / (1 - alpha_i), S_i the colour blended behind
 // i plus T_final bg.  The gradients of one Gaussian are summed over the
 // lane's pixels (in a strip, as sums of dL/dpower times 1, dy, dy^2 for the
-// lane's one column), then over the
-// warp by a reduce-scatter (12 shuffles for 10 values), and one lane per
-// value adds it with one atomic.
+// lane's one column), then over the warp: the lanes' values of three Gaussians
+// go through shared memory, where one lane per value adds up the 32 of them
+// and adds the sum to the record with one atomic.
 #include <map>
 #include <mutex>
 
@@ -40,7 +40,6 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-constexpr int WBATCH_DEFAULT = 128;  // Gaussians per warp batch in shared memory (64 and 192 with 4 px/lane)
 constexpr int WARPS_PER_BLOCK = 4;
 
 // One warp's work item: PPT pixels per lane of one (view, tile) pair -- a
@@ -483,204 +482,370 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, fwd_min_blocks(PPT, DEPT
     }
 }
 
-// Sum over the warp of 10 values per lane, scattered: 12 shuffles in five
-// halving steps (5 + 3 + 2 + 1 + 1), after which every lane holds the full sum
-// of one value, value_of_lane(lane).
-__device__ __forceinline__ int value_of_lane(int lane) {
-    const int b4 = (lane >> 4) & 1, b3 = (lane >> 3) & 1, b2 = (lane >> 2) & 1, b1 = (lane >> 1) & 1;
-    return 5 * b4 + (b3 ? 3 + b2 : (b2 ? 2 : b1));
-}
+// The backward's staging: list entries looked at together, staged entries that
+// end a scan, and Gaussians whose lane sums are added up together (three: ten
+// values each take 30 lanes).
+constexpr int BWD_GROUP = 3;
+constexpr int BWD_SCAN = 64, BWD_FLUSH = 16, BWD_STAGE = (BWD_SCAN + BWD_FLUSH + BWD_GROUP - 1) / BWD_GROUP * BWD_GROUP;
 
-__device__ __forceinline__ float warp_reduce_scatter10(const float (&g)[10], int lane) {
-    const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0, b2 = (lane & 4) != 0, b1 = (lane & 2) != 0;
-    // step 1 (lanes l, l^16): values 0-4 stay in the lower, 5-9 in the upper half
-    float a[5];
-#pragma unroll
-    for (int i = 0; i < 5; i++) {
-        const float send = b4 ? g[i] : g[i + 5];
-        const float keep = b4 ? g[i + 5] : g[i];
-        a[i] = keep + __shfl_xor_sync(kFull, send, 16);
-    }
-    // step 2 (l^8): a0-a2 stay in the lower, a3-a4 in the upper half
-    float b[3];
-#pragma unroll
-    for (int i = 0; i < 2; i++) {
-        const float send = b3 ? a[i] : a[3 + i];
-        const float keep = b3 ? a[3 + i] : a[i];
-        b[i] = keep + __shfl_xor_sync(kFull, send, 8);
-    }
-    b[2] = a[2] + __shfl_xor_sync(kFull, a[2], 8);
-    // step 3 (l^4): three values split 2 + 1, two values 1 + 1
-    const float send0 = b2 ? b[0] : (b3 ? b[1] : b[2]);
-    const float keep0 = b2 ? (b3 ? b[1] : b[2]) : b[0];
-    const float c0 = keep0 + __shfl_xor_sync(kFull, send0, 4);
-    const float c1 = b[1] + __shfl_xor_sync(kFull, b[1], 4);
-    // step 4 (l^2): the two-value lanes split 1 + 1, the others add
-    const bool two = !b3 && !b2;
-    const float send = (two && !b1) ? c1 : c0;
-    const float keep = (two && b1) ? c1 : c0;
-    const float d = keep + __shfl_xor_sync(kFull, send, 2);
-    return d + __shfl_xor_sync(kFull, d, 1);
-}
+// A Gaussian staged by the backward (operands of the packed instructions twice).
+struct alignas(16) BwdEntry {
+    float4 m;     // -mx, -mx, -my, -my
+    float4 qab;   // qa, qa, qb, qb
+    float4 qco;   // qc, qc, -o, -o
+    float4 rg;    // r, r, g, g
+    float4 brp;   // b, b, radius, list position (bit 31: every test of pair_eval is needed)
+};
 
-template <int PPT, bool SAMPLED, int WBATCH>
-__global__ void __launch_bounds__(32 * WARPS_PER_BLOCK) blend_backward_kernel(BlendArgs a, int* __restrict__ counter,
-                                                                              const float* __restrict__ dimg,
-                                                                              const float* __restrict__ final_T,
-                                                                              const uint32_t* __restrict__ n_contrib,
-                                                                              float* __restrict__ rec_grad,
-                                                                              double* __restrict__ rec_conic) {
-    __shared__ float2 s_xy[WARPS_PER_BLOCK][WBATCH];
-    __shared__ float4 s_co[WARPS_PER_BLOCK][WBATCH];
-    __shared__ float4 s_rgb[WARPS_PER_BLOCK][WBATCH];
-    __shared__ uint32_t s_rid[WARPS_PER_BLOCK][WBATCH];
-    __shared__ uint32_t s_pos[WARPS_PER_BLOCK][WBATCH];
+// The lane sums of a group of Gaussians: ten rows of 32 lanes each, added up by
+// one lane per row.  Rows are 136 bytes apart, so that the 16 lanes of an
+// 8-byte read hit different banks.
+struct BwdSums {
+    static constexpr int ROW = 34;  // floats
+    float v[32 * ROW];
+};
+
+// Resident blocks per SM the backward is compiled for: four (at most 128
+// registers; three: 3M Gaussians x 8 views 6.39 -> 6.88 ms, five spill: 6.86).
+constexpr int bwd_min_blocks(int ppt) { return ppt == 4 ? 4 : 1; }
+
+// Bound by instruction issue and the FMA pipe (two thirds of the issue slots,
+// half of the pipe's cycles, 16 warps per SM).  As in the forward, pixels are
+// taken two at a time with packed arithmetic and without branches: a pixel that
+// the Gaussian does not reach takes part with alpha 0, which leaves T and the
+// sums as they are.  That needs finite factors: strips with an image gradient
+// that is not of ordinary size, and Gaussians that are not plain, take every
+// pixel with every test.  The steps of a group of three Gaussians follow each
+// other without a branch, so one's latency hides behind the next.  A warp's
+// sums go through shared memory (ten stores a lane, 16 reads by one lane
+// per value: half the instructions of a shuffle reduction with its selects).  Every sum is
+// taken in a fixed order -- a lane's pixels one after the other, then lanes 16,
+// 8, 4, 2, 1 apart: the conic gradients of long thin Gaussians cancel to a small
+// rest, and their error is the order's.
+// Warp instructions per staged Gaussian (128 pixels) 240 -> 180.  3M Gaussians x
+// 8 views at 32 x 64 tiles 8.44 -> 6.49 ms, 1M x 16 views at 16 x 64 7.70 ->
+// 5.47, 500k x 4 views 1.74 -> 1.34, the sampled pixels of 500k x 4 at 16 x 16
+// 1.21 -> 1.02, 10k at 128 x 128 0.224 -> 0.125.
+
+template <int PPT, bool SAMPLED>
+__global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
+    blend_backward_kernel(BlendArgs a, int* __restrict__ counter, const float* __restrict__ dimg,
+                          const float* __restrict__ final_T, const uint32_t* __restrict__ n_contrib,
+                          float* __restrict__ rec_grad, double* __restrict__ rec_conic) {
+    __shared__ BwdEntry s_ent[WARPS_PER_BLOCK][BWD_STAGE];
+    __shared__ uint32_t s_rid[WARPS_PER_BLOCK][BWD_STAGE];
+    __shared__ __align__(16) BwdSums s_sum[WARPS_PER_BLOCK];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t lt = (1u << lane) - 1u;
-    float2* wxy = s_xy[w];
-    float4* wco = s_co[w];
-    float4* wrgb = s_rgb[w];
+    BwdEntry* ent = s_ent[w];
     uint32_t* wrid = s_rid[w];
-    uint32_t* wpos = s_pos[w];
-    // the value this lane holds after the reduce-scatter
-    const int my_val = value_of_lane(lane);
-    // one lane per value: value_of_lane is the same for lanes l, l^1 and, where
-    // it ignores bit 1, for l^2
-    const bool adder = (lane & 1) == 0 && ((lane & 12) == 0 || (lane & 2) == 0);
+    BwdSums& sums = s_sum[w];
+    constexpr int NP = (PPT + 1) / 2, NK = 2 * NP;  // pairs, pixel slots (one idle slot with 1 pixel per lane)
+    constexpr float LN2 = 0.6931471805599453f;
+    float one1, one2;  // kept in registers (a constant would be moved there at every use)
+    asm volatile("mov.f32 %0, %1;" : "=f"(one1) : "f"(1.f));
+    asm volatile("mov.f32 %0, %1;" : "=f"(one2) : "f"(1.f));
+    const f32x2 one = pack2(one1, one2);
+    // the row this lane adds up: Gaussian of the group, value, and what the sum
+    // is multiplied with
+    const int my_group = lane / 10, my_val = lane % 10;
+    const float my_factor = my_val < 6 ? -1.f : my_val == 6 ? LN2 : my_val == 8 ? 1.f : 0.5f;
+
+    // adds the sums of the k Gaussians from entry j on to their records (lanes
+    // l and l + 16 first, then 8, 4, 2 and 1 apart)
+    auto add_sums = [&](int j, int k) {
+        __syncwarp();
+        const float2* row = reinterpret_cast<const float2*>(sums.v + lane * BwdSums::ROW);
+        f32x2 t[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) t[i] = add2(row[i], row[i + 8]);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+            for (int i = 0; i < o; i++) t[i] = add2(t[i], t[i + o]);
+        const float sum = t[0].x + t[0].y;
+        const float other = __shfl_xor_sync(kFull, sum, 1);
+        float out = my_factor * sum;
+        if (my_group < k) {
+            const BwdEntry& e = ent[j + my_group];
+            const uint32_t r = wrid[j + my_group];
+            // dL/d mean = sum dL/dpower (A dx + B dy, B dx + C dy), in base-2 coefficients
+            if (my_val < 2)
+                out = LN2 * fmaf(2.f * (my_val == 0 ? e.qab.x : e.qco.x), sum, e.qab.z * other);
+            // the conic gradients sum terms weighted by dx^2 ~ 1e4 px^2 of both
+            // signs: they are added across warps in double precision
+            if (my_val < 7) atomicAdd(rec_grad + (size_t)kGradStride * r + my_val, out);
+            else atomicAdd(rec_conic + (size_t)3 * r + (my_val - 7), (double)out);
+        }
+        __syncwarp();
+    };
+
     const long long total = SAMPLED ? min(a.chunk_off[a.tiles], a.chunk_cap) : 0;
     Work<PPT> st;
     while (next_work<PPT, SAMPLED>(a, counter, lane, total, st)) {
         const DevCam& cam = *st.cam;
         const long long HW = (long long)cam.W * cam.H;
         const float* din = dimg + 3 * cam.pix_base;
-        // per pixel: T in front of the current Gaussian, dL/dC, and
-        // U = dL/dC . (colour blended behind the current Gaussian + T_final bg)
-        float T[PPT], d0[PPT], d1[PPT], d2[PPT], U[PPT];
-        uint32_t last[PPT];
+        // per pixel: T in front of the current Gaussian, dL/dC, and V = minus
+        // dL/dC . (colour blended behind the current Gaussian + T_final bg)
+        f32x2 T[NP], d0[NP], d1[NP], d2[NP], V[NP], FX[SAMPLED ? NP : 1], FY[NP];
+        uint32_t last[NK];
         uint32_t mylast = 0;
+        bool odd_pixels = false;
+        {
+            float t[NK], e0[NK], e1[NK], e2[NK], u[NK];
 #pragma unroll
-        for (int k = 0; k < PPT; k++) {
-            T[k] = 1.f;
-            d0[k] = d1[k] = d2[k] = 0.f;
-            last[k] = 0;
-            const long long p = st.pix[k];
-            if (p >= 0) {
-                d0[k] = din[p];
-                d1[k] = din[HW + p];
-                d2[k] = din[2 * HW + p];
-                T[k] = final_T[cam.pix_base + p];
-                last[k] = n_contrib[cam.pix_base + p];
+            for (int k = 0; k < NK; k++) {
+                t[k] = 1.f;
+                e0[k] = e1[k] = e2[k] = 0.f;
+                last[k] = 0;
+                const long long p = k < PPT ? st.pix[k < PPT ? k : 0] : -1;
+                if (p >= 0) {
+                    e0[k] = din[p];
+                    e1[k] = din[HW + p];
+                    e2[k] = din[2 * HW + p];
+                    t[k] = final_T[cam.pix_base + p];
+                    last[k] = n_contrib[cam.pix_base + p];
+                }
+                u[k] = -t[k] * (e0[k] * a.bg[0] + e1[k] * a.bg[1] + e2[k] * a.bg[2]);
+                mylast = last[k] > mylast ? last[k] : mylast;
+                // gradients a Gaussian of weight 0 may be multiplied with
+                odd_pixels |= !(fabsf(e0[k]) + fabsf(e1[k]) + fabsf(e2[k]) <= 1e25f && fabsf(u[k]) <= 1e35f);
             }
-            U[k] = T[k] * (d0[k] * a.bg[0] + d1[k] * a.bg[1] + d2[k] * a.bg[2]);
-            mylast = last[k] > mylast ? last[k] : mylast;
+#pragma unroll
+            for (int p = 0; p < NP; p++) {
+                const int k = 2 * p, l = 2 * p + 1;
+                T[p] = pack2(t[k], t[l]);
+                d0[p] = pack2(e0[k], e0[l]);
+                d1[p] = pack2(e1[k], e1[l]);
+                d2[p] = pack2(e2[k], e2[l]);
+                V[p] = pack2(u[k], u[l]);
+                if (SAMPLED || p == 0) FX[SAMPLED ? p : 0] = pack2(st.fx[k], st.fx[l < PPT ? l : k]);
+                FY[p] = pack2(st.fy[k], st.fy[l < PPT ? l : k]);
+            }
         }
-        const uint32_t maxlast = __reduce_max_sync(kFull, mylast);
-        const long long start = a.ranges[2 * st.gt];
-        for (uint32_t b = 0; b < maxlast; b += WBATCH) {
-            // stage, back to front, the Gaussians that can reach the work item
+        odd_pixels = __any_sync(kFull, odd_pixels);
+        const uint32_t len = __reduce_max_sync(kFull, mylast);
+        const uint32_t* list = a.sorted + a.ranges[2 * st.gt];
+        // back to front: entry i of the walk is list position len - 1 - i
+        uint32_t rec[2], nid[2];
+        Geom g[2];
+        auto fetch_ids = [&](uint32_t b) {
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const uint32_t i = b + 32 * h + lane;
+                nid[h] = i < len ? list[len - 1 - i] : 0u;
+            }
+        };
+        auto fetch_geometry = [&](uint32_t b) {
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                rec[h] = nid[h];
+                if (b + 32 * h + lane < len) g[h] = load_geom(a.geom + rec[h]);
+            }
+        };
+        auto hand_over = [&](int u, float v0, float v1, float v2, float v3, float v4, float v5, float v6, float v7,
+                             float v8, float v9) {
+            const float v[10] = {v0, v1, v2, v3, v4, v5, v6, v7, v8, v9};
+#pragma unroll
+            for (int i = 0; i < 10; i++) sums.v[(10 * u + i) * BwdSums::ROW + lane] = v[i];
+        };
+        // One Gaussian on all pixels: the lane's sums over its pixels -- minus
+        // dL/dpower times 1, dy, dy^2, dx, dx^2 and dx dy, minus the colour
+        // gradients, the E_1 term -- into place u of the group.
+        auto plain_step = [&](const BwdEntry& e, int u) {
+            const float4 em = e.m, eq = e.qab, eo = e.qco, ec = e.rg, eb = e.brp;
+            const uint32_t tag = __float_as_uint(eb.w);
+            const float radius = eb.z;
+            const f32x2 nmx = pack2(em.x, em.y), nmy = pack2(em.z, em.w), qa = pack2(eq.x, eq.y),
+                        qb = pack2(eq.z, eq.w), qc = pack2(eo.x, eo.y), no = pack2(eo.z, eo.w),
+                        r2 = pack2(ec.x, ec.y), g2 = pack2(ec.z, ec.w), b2 = pack2(eb.x, eb.y);
+            const f32x2 qc2 = add2(qc, qc);
+            f32x2 dx{}, t2{}, xx{}, x{}, sr{}, sg{}, sb{};
+            float P0 = 0.f, P1 = 0.f, P2 = 0.f, Sx = 0.f, Sxx = 0.f, Sxy = 0.f;
+            bool in0 = true, in1 = true;
+            float E = 0.f;
+#pragma unroll
+            for (int p = 0; p < NP; p++) {
+                const int k = 2 * p, l = 2 * p + 1;
+                if (SAMPLED || p == 0) {
+                    dx = add2(FX[SAMPLED ? p : 0], nmx);
+                    const f32x2 t = mul2(qa, dx);
+                    t2 = add2(t, t);
+                    xx = mul2(t, dx);
+                    x = mul2(qb, dx);
+                    float dx0, dx1;
+                    unpack2(dx, dx0, dx1);
+                    in0 = fabsf(dx0) <= radius;
+                    in1 = SAMPLED ? fabsf(dx1) <= radius : in0;
+                }
+                const f32x2 dy = add2(FY[p], nmy);
+                float dy0, dy1, e0, e1, v0, v1, o0, o1;
+                unpack2(dy, dy0, dy1);
+                unpack2(fma2(dy, fma2(qc, dy, x), xx), e0, e1);
+                unpack2(mul2(no, pack2(ex2_approx(e0), ex2_approx(e1))), v0, v1);
+                const bool ok0 = in0 & (fabsf(dy0) <= radius) & (v0 <= -kAlphaMin) & (tag < last[k]);
+                const bool ok1 = in1 & (fabsf(dy1) <= radius) & (v1 <= -kAlphaMin) & (tag < last[l]);
+                const f32x2 na = pack2(ok0 ? v0 : 0.f, ok1 ? v1 : 0.f);  // minus alpha
+                unpack2(add2(na, one), o0, o1);
+                const f32x2 inv = pack2(rcp_approx(o0), rcp_approx(o1));
+                T[p] = mul2(T[p], inv);  // transmittance in front of this Gaussian
+                const f32x2 nw = mul2(na, T[p]);
+                const f32x2 dc = fma2(d2[p], b2, fma2(d0[p], r2, mul2(d1[p], g2)));
+                const f32x2 da = fma2(T[p], dc, mul2(V[p], inv));  // dL/dalpha
+                V[p] = fma2(dc, nw, V[p]);
+                const f32x2 nd = mul2(da, na);  // minus dL/dpower
+                const f32x2 ed = mul2(nd, dy);
+                const f32x2 ax = fma2(qb, dy, t2), ay = fma2(qc2, dy, x);
+                float n0, n1, h0, h1, w0, w1;
+                unpack2(fma2(ay, ay, mul2(ax, ax)), n0, n1);
+                unpack2(nd, h0, h1);
+                unpack2(ed, w0, w1);
+                E = fmaf(fabsf(h0), sqrt_approx(n0), E);
+                E = fmaf(fabsf(h1), sqrt_approx(n1), E);
+                // pixel by pixel: where these cancel, a result is as good as their order
+                P0 = p == 0 ? h0 + h1 : P0 + h0 + h1;
+                P1 = p == 0 ? w0 + w1 : P1 + w0 + w1;
+                P2 = fmaf(w1, dy1, p == 0 ? w0 * dy0 : fmaf(w0, dy0, P2));
+                if (SAMPLED) {
+                    float dx0, dx1;
+                    unpack2(dx, dx0, dx1);
+                    const float x0 = h0 * dx0, x1 = h1 * dx1;
+                    Sx += x0 + x1;
+                    Sxx = fmaf(x1, dx1, fmaf(x0, dx0, Sxx));
+                    Sxy = fmaf(x1, dy1, fmaf(x0, dy0, Sxy));
+                }
+                sr = p == 0 ? mul2(d0[p], nw) : fma2(d0[p], nw, sr);
+                sg = p == 0 ? mul2(d1[p], nw) : fma2(d1[p], nw, sg);
+                sb = p == 0 ? mul2(d2[p], nw) : fma2(d2[p], nw, sb);
+            }
+            auto sum = [](f32x2 v) {
+                float lo, hi;
+                unpack2(v, lo, hi);
+                return lo + hi;
+            };
+            if (!SAMPLED) {
+                float dx0, dx1;
+                unpack2(dx, dx0, dx1);
+                Sx = dx0 * P0;
+                Sxx = dx0 * dx0 * P0;
+                Sxy = dx0 * P1;
+            }
+            hand_over(u, Sx, P1, P0, sum(sr), sum(sg), sum(sb), E, Sxx, Sxy, P2);
+        };
+        // the same for any Gaussian and gradient, pixel by pixel with every test
+        auto general_step = [&](const BwdEntry& e, int u) {
+            const float4 em = e.m, eq = e.qab, eo = e.qco, ec = e.rg, eb = e.brp;
+            const uint32_t tag = __float_as_uint(eb.w);
+            const float radius = eb.z;
+            const float4 q = make_float4(eq.x, eq.z, eo.x, -eo.z);
+            const uint32_t pos = tag & ~kTestAll;
+            float P0 = 0.f, P1 = 0.f, P2 = 0.f, Sx = 0.f, Sxx = 0.f, Sxy = 0.f, R = 0.f, Gn = 0.f, B = 0.f, E = 0.f;
+            auto one_pixel = [&](int k, float fx, float fy, float e0, float e1, float e2, float& Tk, float& Vk) {
+                if (pos >= last[k]) return;
+                const float dx = fx + em.x, dy = fy + em.z;
+                float alpha, G;
+                if (!pair_eval(dx, dy, col_terms(dx, q), q, radius, alpha, G)) return;
+                const float inv = rcp_approx(1.f - alpha);
+                Tk *= inv;
+                const float nw = -alpha * Tk;
+                R += e0 * nw;
+                Gn += e1 * nw;
+                B += e2 * nw;
+                const float dc = e0 * ec.x + e1 * ec.z + e2 * eb.x;
+                const float da = fmaf(Tk, dc, Vk * inv);
+                Vk += dc * nw;
+                if (alpha < kAlphaMax) {  // below the clamp alpha = o G
+                    const float nd = -da * alpha, nx = nd * dx, ny = nd * dy;
+                    const float ax = fmaf(q.y, dy, 2.f * q.x * dx), ay = fmaf(2.f * q.z, dy, q.y * dx);
+                    P0 += nd;
+                    P1 += ny;
+                    P2 = fmaf(ny, dy, P2);
+                    Sx += nx;
+                    Sxx = fmaf(nx, dx, Sxx);
+                    Sxy = fmaf(nx, dy, Sxy);
+                    E = fmaf(fabsf(nd), sqrt_approx(ax * ax + ay * ay), E);
+                }
+            };
+#pragma unroll
+            for (int p = 0; p < NP; p++) {
+                float t[2], u[2], f[2], y[2], a0[2], a1[2], a2[2];
+                unpack2(T[p], t[0], t[1]);
+                unpack2(V[p], u[0], u[1]);
+                unpack2(FX[SAMPLED ? p : 0], f[0], f[1]);
+                unpack2(FY[p], y[0], y[1]);
+                unpack2(d0[p], a0[0], a0[1]);
+                unpack2(d1[p], a1[0], a1[1]);
+                unpack2(d2[p], a2[0], a2[1]);
+#pragma unroll
+                for (int h = 0; h < 2; h++) one_pixel(2 * p + h, f[h], y[h], a0[h], a1[h], a2[h], t[h], u[h]);
+                T[p] = pack2(t[0], t[1]);
+                V[p] = pack2(u[0], u[1]);
+            }
+            hand_over(u, Sx, P1, P0, R, Gn, B, E, Sxx, Sxy, P2);
+        };
+        fetch_ids(0);
+        fetch_geometry(0);
+        fetch_ids(BWD_SCAN);
+        for (uint32_t b = 0; b < len;) {
+            // stage the Gaussians that can reach a pixel of the work item
             __syncwarp();
             int n = 0;
-            for (int i0 = 0; i0 < WBATCH; i0 += 32) {
-                const long long pos = (long long)maxlast - 1 - b - i0 - lane;
-                bool hit = false;
-                uint32_t r = 0;
-                Geom g;
-                if (pos >= 0) {
-                    r = a.sorted[start + pos];
-                    g = load_geom(a.geom + r);
-                    hit = rect_reaches(st.sx0, st.sx1, st.sy0, st.sy1, g);
+            do {
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const uint32_t i = b + 32 * h + lane;
+                    const bool hit = i < len && rect_reaches(st.sx0, st.sx1, st.sy0, st.sy1, g[h]);
+                    const uint32_t bal = __ballot_sync(kFull, hit);
+                    if (hit) {
+                        const int slot = n + __popc(bal & lt);
+                        ent[slot].m = make_float4(-g[h].mx, -g[h].mx, -g[h].my, -g[h].my);
+                        ent[slot].qab = make_float4(g[h].qa, g[h].qa, g[h].qb, g[h].qb);
+                        ent[slot].qco = make_float4(g[h].qc, g[h].qc, -g[h].o, -g[h].o);
+                        ent[slot].brp.w = __uint_as_float((len - 1 - i) | (g[h].radius >= 0.f && !odd_pixels ? 0u : kTestAll));
+                        wrid[slot] = rec[h];
+                    }
+                    n += __popc(bal);
                 }
-                const uint32_t bal = __ballot_sync(kFull, hit);
-                if (hit) {
-                    const int slot = n + __popc(bal & lt);
-                    wrid[slot] = r;
-                    wxy[slot] = make_float2(g.mx, g.my);
-                    wco[slot] = make_float4(g.qa, g.qb, g.qc, g.o);
-                    wrgb[slot] = a.rgb_r[r];
-                    wpos[slot] = (uint32_t)pos;
+                b += BWD_SCAN;
+                if (b < len) {
+                    fetch_geometry(b);
+                    fetch_ids(b + BWD_SCAN);
                 }
-                n += __popc(bal);
+            } while (n <= BWD_FLUSH && b < len);
+            __syncwarp();
+            float4 cr[(BWD_STAGE + 31) / 32];
+#pragma unroll
+            for (int i = 0; i < (BWD_STAGE + 31) / 32; i++)
+                if (32 * i + lane < n) cr[i] = a.rgb_r[wrid[32 * i + lane]];
+#pragma unroll
+            for (int i = 0; i < (BWD_STAGE + 31) / 32; i++) {
+                const int e = 32 * i + lane;
+                if (e < n) {
+                    ent[e].rg = make_float4(cr[i].x, cr[i].x, cr[i].y, cr[i].y);
+                    *reinterpret_cast<float2*>(&ent[e].brp) = make_float2(cr[i].z, cr[i].z);
+                    ent[e].brp.z = cr[i].w;
+                }
+            }
+            // fill the last group with Gaussians that reach no pixel
+            if (lane < BWD_GROUP - 1 && (n + lane) % BWD_GROUP != 0 && (n + lane) / BWD_GROUP == (n - 1) / BWD_GROUP) {
+                const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+                ent[n + lane].m = ent[n + lane].qab = ent[n + lane].qco = ent[n + lane].rg = ent[n + lane].brp = zero;
             }
             __syncwarp();
-            // two Gaussians per loop trip: one's reduce-scatter overlaps the next one's pixels
-#pragma unroll 2
-            for (int j = 0; j < n; j++) {
-                const uint32_t pos = wpos[j];
-                float g[10];
+            // in groups, straight through: the steps of a group overlap
+            for (int j = 0; j < n; j += BWD_GROUP) {
+                uint32_t tags = 0;
 #pragma unroll
-                for (int i = 0; i < 10; i++) g[i] = 0.f;
-                bool any = false;
-                const float2 m = wxy[j];
-                const float4 cr = wrgb[j];
-                const float dx0 = st.fx[0] - m.x;
-                if (pos < mylast && (SAMPLED || fabsf(dx0) <= cr.w)) {
-                    const float4 q = wco[j];
-                    const float3 cn = conic_of(q);  // (A, B, C)
-                    const ColTerms ct0 = col_terms(dx0, q);
-                    const float adx0 = cn.x * dx0, bdx0 = cn.y * dx0;
-                    // strips (one column per lane): sums over the lane's pixels of
-                    // dL/dpower times 1, dy and dy^2, turned into the mean and conic
-                    // gradients once per Gaussian below
-                    float P0 = 0.f, P1 = 0.f, P2 = 0.f;
+                for (int u = 0; u < BWD_GROUP; u++) tags |= __float_as_uint(ent[j + u].brp.w);
+                if (!__any_sync(kFull, tags >= kTestAll)) {
 #pragma unroll
-                    for (int k = 0; k < PPT; k++) {
-                        if (pos >= last[k]) continue;
-                        const float dx = SAMPLED ? st.fx[k] - m.x : dx0;
-                        const float dy = st.fy[k] - m.y;
-                        const ColTerms ct = SAMPLED ? col_terms(dx, q) : ct0;
-                        float alpha, G;
-                        if (!pair_eval(dx, dy, ct, q, cr.w, alpha, G)) continue;
-                        any = true;
-                        const float inv = rcp_approx(1.f - alpha);
-                        T[k] *= inv;  // transmittance in front of this Gaussian
-                        const float wgt = alpha * T[k];
-                        g[6] += d0[k] * wgt;
-                        g[7] += d1[k] * wgt;
-                        g[8] += d2[k] * wgt;
-                        const float dc = d0[k] * cr.x + d1[k] * cr.y + d2[k] * cr.z;
-                        const float dLda = T[k] * dc - U[k] * inv;
-                        U[k] += dc * wgt;
-                        if (alpha < kAlphaMax) {  // below the clamp alpha = o G
-                            const float dLdp = dLda * alpha;  // dL/d power = dL/dalpha o G
-                            // d power / d mean2d = (ax, ay) = (A dx + B dy, B dx + C dy)
-                            const float ax = fmaf(cn.y, dy, SAMPLED ? cn.x * dx : adx0);
-                            const float ay = fmaf(cn.z, dy, SAMPLED ? cn.y * dx : bdx0);
-                            if (SAMPLED) {
-                                const float h = -0.5f * dLdp;
-                                g[0] += dLdp * ax;
-                                g[1] += dLdp * ay;
-                                g[2] += h * dx * dx;
-                                g[3] += 2.f * h * dx * dy;
-                                g[4] += h * dy * dy;
-                            } else {
-                                const float e = dLdp * dy;
-                                P0 += dLdp;
-                                P1 += e;
-                                P2 = fmaf(e, dy, P2);
-                            }
-                            g[5] += dLda * G;
-                            g[9] += fabsf(dLdp) * sqrt_approx(ax * ax + ay * ay);
-                        }
-                    }
-                    if (!SAMPLED) {
-                        // sum_k dL/dpower_k (ax_k, ay_k) and -1/2 sum_k dL/dpower_k (dx^2, 2 dx dy_k, dy_k^2)
-                        g[0] = fmaf(adx0, P0, cn.y * P1);
-                        g[1] = fmaf(bdx0, P0, cn.z * P1);
-                        g[2] = -0.5f * dx0 * dx0 * P0;
-                        g[3] = -dx0 * P1;
-                        g[4] = -0.5f * P2;
-                    }
+                    for (int u = 0; u < BWD_GROUP; u++) plain_step(ent[j + u], u);
+                } else {
+#pragma unroll 1
+                    for (int u = 0; u < BWD_GROUP; u++) general_step(ent[j + u], u);
                 }
-                if (__ballot_sync(kFull, any) == 0u) continue;
-                const float sum = warp_reduce_scatter10(g, lane);
-                if (adder) {
-                    // the conic gradients sum terms weighted by dx^2 ~ 1e4 px^2 of both
-                    // signs: they are added across warps in double precision
-                    if (my_val >= 2 && my_val <= 4)
-                        atomicAdd(rec_conic + (size_t)3 * wrid[j] + (my_val - 2), (double)sum);
-                    else
-                        atomicAdd(rec_grad + (size_t)kGradStride * wrid[j] + grad_slot(my_val), sum);
-                }
+                add_sums(j, min(n - j, BWD_GROUP));
             }
         }
     }
@@ -775,19 +940,15 @@ void launch_blend_backward(const BlendArgs& a, int* counter, const float* dimg, 
     cudaMemsetAsync(counter, 0, sizeof(int), s);
     const bool sampled = a.s_off != nullptr;
     const long long items = sampled ? (1LL << 40) : a.tiles * a.strips;
-#define MVGS_BB(P, S, B)                                                                                         \
-    blend_backward_kernel<P, S, B><<<grid_for(blend_backward_kernel<P, S, B>, items), 32 * WARPS_PER_BLOCK, 0,   \
-                                     s>>>(a, counter, dimg, final_T, n_contrib, rec_grad, rec_conic)
-#define MVGS_BB2(P, B) if (sampled) MVGS_BB(P, true, B); else MVGS_BB(P, false, B)
+#define MVGS_BB(P, S)                                                                                      \
+    blend_backward_kernel<P, S><<<grid_for(blend_backward_kernel<P, S>, items), 32 * WARPS_PER_BLOCK, 0, s>>>( \
+        a, counter, dimg, final_T, n_contrib, rec_grad, rec_conic)
+#define MVGS_BB2(P) if (sampled) MVGS_BB(P, true); else MVGS_BB(P, false)
     switch (a.ppt) {
-        case 1: MVGS_BB2(1, WBATCH_DEFAULT); break;
-        case 2: MVGS_BB2(2, WBATCH_DEFAULT); break;
-        case 8: MVGS_BB2(8, WBATCH_DEFAULT); break;
-        default:
-            if (a.wbatch == 64) MVGS_BB2(4, 64);
-            else if (a.wbatch == 192) MVGS_BB2(4, 192);
-            else MVGS_BB2(4, WBATCH_DEFAULT);
-            break;
+        case 1: MVGS_BB2(1); break;
+        case 2: MVGS_BB2(2); break;
+        case 8: MVGS_BB2(8); break;
+        default: MVGS_BB2(4); break;
     }
 #undef MVGS_BB2
 #undef MVGS_BB

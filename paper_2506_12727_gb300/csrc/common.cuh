@@ -55,14 +55,10 @@ struct CamChunk {
 };
 
 // Per-record float gradient slots written by the blend backward and read by
-// the preprocessing backward: mean2d x, y, opacity, r, g, b, E_1 term,
-// padding (the conic's three go to a separate double array).  The blend
-// backward's reduced value v (0, 1 mean2d; 2..4 conic; 5 opacity; 6..8 rgb;
-// 9 E_1) goes to float slot grad_slot(v).
+// the preprocessing backward: mean2d x, y, opacity (times the opacity), r, g, b,
+// E_1 term, padding (the conic's three go to a separate double array).
 constexpr int kGradStride = 8;
-__host__ __device__ constexpr int grad_slot(int v) { return v < 2 ? v : v - 3; }
 
-// Global tile ids index the view-major list of (view, tile) pairs.
 // Single-instruction approximations (PTX rcp.approx / sqrt.approx, about
 // 1 ulp; flush-to-zero) for per-pair arithmetic, where the correctly rounded
 // forms (__frcp_rn, IEEE sqrtf and division) are instruction sequences with a
@@ -232,12 +228,13 @@ __device__ __forceinline__ Geom load_geom(const Geom* g) {
 //     distance (0, or at least 2^-25) clear of underflow and overflow.
 //   - the clamp at 0.99: o G stays below it when o does (G <= 1 up to the
 //     error of ex2.approx).
-//   - colour and depth are finite (their sum is only then).
+//   - colour and depth are finite (and the colour small enough for its product
+//     with any image gradient the backward takes this way, see there).
 // NaN fails every comparison.
 __device__ __forceinline__ bool plain_gaussian(float4 co, float3 rgb, float depth) {
     const float A = co.x, B = co.y, C = co.z;
     return (A >= 1e-15f) & (A <= 1e10f) & (C >= 1e-15f) & (C <= 1e10f) & (B * B <= 0.99f * (A * C)) &
-           (co.w <= 0.989f) & (fabsf(rgb.x) + fabsf(rgb.y) + fabsf(rgb.z) + fabsf(depth) <= 3e38f);
+           (co.w <= 0.989f) & (fabsf(rgb.x) + fabsf(rgb.y) + fabsf(rgb.z) <= 1e10f) & (fabsf(depth) <= 3e38f);
 }
 
 __device__ __forceinline__ Geom make_geom(float2 m, float4 co, float radius, bool plain) {

@@ -74,8 +74,8 @@ void launch_preprocess(const SceneArgs& sc, const DevCam* cams, int V, int tw, i
                        const RecordArgs& rec, uint32_t* bins, unsigned long long* tile_desc,
                        unsigned long long* sums, cudaStream_t s);
 void launch_zero_f32(float* p, size_t count, cudaStream_t s);
-// rec_grad: [records, kGradStride] float (mean2d x, y, opacity, rgb, e1 at
-// 0, 1, 2, 3..5, 6); rec_conic: [records, 3] double (conic A, B, C).
+// rec_grad: [records, kGradStride] float (mean2d x, y, opacity times dL/dopacity,
+// rgb, e1 at 0, 1, 2, 3..5, 6); rec_conic: [records, 3] double (conic A, B, C).
 void launch_preprocess_backward(const SceneArgs& sc, const DevCam* cams, int V, const RecordArgs& rec,
                                 const float* rec_grad, const double* rec_conic, float* g_means,
                                 float* g_log_scales, float* g_quats, float* g_logits, float* g_sh,
@@ -128,7 +128,6 @@ struct BlendArgs {
     int V;
     int tw, th;
     int ppt;                 // pixels per lane (resolved, 1..8)
-    int wbatch;              // Gaussians per warp batch of the backward (64, 128 or 192; 128 unless ppt 4)
     int sw;                  // columns of a warp's strip (blend_strip_width)
     int strip_h;             // rows of a warp's strip: (32 / sw) * ppt
     int strips;              // strips per tile: (tw / sw) * (th / strip_h)

@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(128, 3) preprocess_backward_kernel(SceneArgs s
     }
 #pragma unroll
     for (int j = 0; j < 3; j++) g_means[3 * g + j] = gmu[j];
-    g_logits[g] = go * G.o * (1.f - G.o);
+    g_logits[g] = go * (1.f - G.o);  // go: sum of o dL/do
     float* gshg = g_sh + (size_t)g * NK * 3;
     if constexpr ((NK * 3) % 4 == 0) {
         if ((reinterpret_cast<uintptr_t>(g_sh) & 15) == 0) {

@@ -10,17 +10,17 @@ import torch
 
 import oracle
 import synth
-from gpu_helpers import assert_close_frac, gpu_forward, scene_to_device
+from gpu_helpers import PARAMS, assert_close_frac, assert_close_rows, gpu_forward, grads_like, scene_to_device
 
 pytestmark = pytest.mark.gpu
 
 
-def _mixed_scene(n, seed):
+def _mixed_scene(n, seed, needles=True):
     rng = np.random.default_rng(seed)
     sc = synth.make_scene(n, 1, seed=seed)
     kind = rng.integers(0, 4, n)
     sc.opacity_logits[kind == 0] = rng.uniform(3.0, 9.0, int((kind == 0).sum())).astype(np.float32)  # o 0.953 .. 0.9999
-    needle = kind == 1
+    needle = (kind == 1) & needles
     sc.log_scales[needle] = np.float32(-8.0)
     sc.log_scales[needle, 0] = rng.uniform(-2.0, -0.5, int(needle.sum())).astype(np.float32)
     return sc
@@ -73,3 +73,54 @@ def test_a_colour_that_is_not_finite_stays_where_it_blends(cuda_lib):
         assert torch.equal(img[apart], imgs[0][apart])
         assert torch.equal(t, T[0])
         assert not torch.isfinite(img[~apart]).any()
+
+
+@pytest.mark.parametrize("n,sizes,ppt", [(40, [(120, 90)], 0), (700, [(97, 61), (64, 128)], 0), (700, [(97, 61), (64, 128)], 1),
+                                         (700, [(97, 61), (64, 128)], 2), (700, [(97, 61), (64, 128)], 8)])
+def test_gradients_with_opacities_around_the_clamp_match_the_oracle(cuda_lib, n, sizes, ppt):
+    # (no needles: the gradient of a nearly degenerate covariance is a float32
+    # cancellation that no order of summation brings within the tolerance)
+    scene, cams = _mixed_scene(n, 100 + n, needles=False), synth.make_cameras(sizes, radius=3.0, seed=5)
+    tile, bg = (32, 64), (0.1, 0.2, 0.3)
+    ref = oracle.forward(scene, cams, tile, bg=bg)
+    amb = ref["amb"] != 0
+    _, _, _, base = oracle.layout(cams, tile)
+    dimg = np.random.default_rng(3).normal(size=ref["img"].shape).astype(np.float32)
+    dimg[np.concatenate([np.tile(amb[base[v]:base[v + 1]], 3) for v in range(cams.V)])] = 0.0
+    grads, _, _ = oracle.backward(scene, cams, ref, dimg.astype(np.float64), tile, bg)
+    params = scene_to_device(scene)
+    sc = cuda_lib.make_scene(params, scene.sh_degree)
+    rz = cuda_lib.Rasterizer(cams, tile=tile, bg=bg, pixels_per_thread=ppt)
+    rz.forward(sc)
+    got = grads_like(params)
+    rz.backward(sc, torch.tensor(dimg, device="cuda"), got)
+    bad = np.zeros(scene.n, bool)
+    bad[np.nonzero(ref["P"]["amb"])[0] % scene.n] = True
+    for k in PARAMS:
+        ref_k = grads[k][~bad]
+        assert_close_rows(got[k].cpu().numpy()[~bad], ref_k, 1e-3, 1e-5 * np.abs(ref_k).max(), k)
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), 1e30])
+def test_a_pixel_gradient_reaches_only_the_gaussians_it_blends(cuda_lib, value):
+    scene, cams = synth.make_scene(400, 0, seed=9), synth.make_cameras([(150, 110)], radius=3.0, seed=9)
+    params = scene_to_device(scene)
+    sc = cuda_lib.make_scene(params, 0)
+    rz = cuda_lib.Rasterizer(cams, tile=(16, 16))
+    img = rz.forward(sc)
+    pixel = 55 * 150 + 75
+    one = torch.zeros_like(img)
+    one[pixel] = 1.0
+    base = torch.randn(img.shape, device="cuda", generator=torch.Generator("cuda").manual_seed(2))
+    base[pixel] = 0.0
+    runs = []
+    for dimg in (one, base, torch.where(one > 0, torch.full_like(base, value), base)):
+        g = grads_like(params)
+        rz.backward(sc, dimg, g)
+        runs.append(g)
+    apart = (runs[0]["sh"].reshape(scene.n, -1) == 0).all(1)  # not blended at the pixel
+    assert 0 < int((~apart).sum()) < scene.n
+    for k in PARAMS:
+        a, b = runs[1][k][apart], runs[2][k][apart]
+        assert torch.isfinite(b).all(), k
+        torch.testing.assert_close(b, a, rtol=1e-4, atol=1e-6 * float(a.abs().max()))
