@@ -929,7 +929,7 @@ mvgs_status mvgs_densify(const mvgs_scene* scene, const float* accum_e1, const f
         return fail(MVGS_ENOSPACE, "%lld output Gaussians exceed the capacity of %lld", total, (long long)capacity);
     DensifyOut o{out_means, out_log_scales, out_quats, out_opacity_logits, out_sh,
                  reinterpret_cast<long long*>(out_src), out_kind};
-    launch_densify_write(a, o, workspace, s);
+    launch_densify_write(a, o, total, workspace, s);
     return cuda_check("densify");
 }
 

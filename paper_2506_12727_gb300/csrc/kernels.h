@@ -216,7 +216,7 @@ struct DensifyOut {
 constexpr float kLogSplitDiv = 0.47000362924573558f;  // ln 1.6
 size_t densify_temp_bytes(long long n);
 const long long* launch_densify_plan(const DensifyArgs& a, void* tmp, cudaStream_t s);
-void launch_densify_write(const DensifyArgs& a, const DensifyOut& o, void* tmp, cudaStream_t s);
+void launch_densify_write(const DensifyArgs& a, const DensifyOut& o, long long n_out, void* tmp, cudaStream_t s);
 void launch_carry(long long n_out, const long long* src, const int* kind, int width, const float* in, float* out,
                   cudaStream_t s);
 void launch_adam(long long count, float* p, const float* g, float* m, float* v, float lr, float b1, float b2,
