@@ -19,9 +19,8 @@ constexpr float kGuard = 1.3f;
 constexpr float kSigmas = 3.0f;
 constexpr float kEigFloor = 0.1f;
 
-// Per-view camera table entry, built on the host from mvgs_camera and
-// uploaded once per call; every kernel reads it from global memory.
-struct __align__(16) DevCam {
+// What the projection reads of a view.
+struct ProjCam {
     float R[9];      // world -> camera rotation, row-major
     float t[3];
     float fx, fy, cx, cy;
@@ -29,6 +28,11 @@ struct __align__(16) DevCam {
     float near_z;
     float limx, limy;  // guard band on x/z and y/z
     int W, H, tiles_x, tiles_y;
+};
+
+// Per-view camera table entry, built on the host from mvgs_camera and
+// uploaded once per call; every kernel reads it from global memory.
+struct __align__(16) DevCam : ProjCam {
     long long tile_base;  // first global tile id of the view
     long long pix_base;   // first pixel of the view in the packed layout
     long long bin_base;   // first bin of the view (8 x 8 tiles each, row-major)
@@ -48,6 +52,21 @@ struct Count {
         return v < max ? v : max;
     }
 };
+
+// Asynchronous copies from global to shared memory: no register holds the data,
+// so a warp goes on until it waits for them.  N: 4, 8 or 16 bytes, both sides
+// aligned to it.
+template <int N>
+__device__ __forceinline__ void cp_async(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "n"(N)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int PENDING>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+}
 
 constexpr int kCamChunk = 32;
 struct CamChunk {
