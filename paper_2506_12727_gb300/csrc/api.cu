@@ -123,7 +123,7 @@ struct Plan {
     size_t s_geom = 0;  // state: the records' Geom array (not part of the public layout)
     // workspace offsets (forward)
     size_t w_cams = 0, w_counts = 0, w_vis = 0, w_scan = 0, w_dkeys_a = 0, w_dkeys_b = 0, w_ids_a = 0, w_ids_b = 0,
-           w_order = 0, w_bins = 0, w_desc = 0, w_bin_off = 0, w_keys_a = 0, w_keys_b = 0, w_vals_a = 0, w_vals_b = 0,
+           w_order = 0, w_bins = 0, w_desc = 0, w_bins_by_depth = 0, w_bin_off = 0, w_keys_a = 0, w_keys_b = 0, w_vals_a = 0, w_vals_b = 0,
            w_radix = 0, w_lists = 0, w_torder = 0, w_counter = 0, w_dcount = 0;
     // workspace offsets of the sampled blend (forward and backward each carve their own)
     size_t w_chunk_off = 0, w_chunk_map = 0, w_chunk_tmp = 0, w_mask = 0;
@@ -238,6 +238,7 @@ mvgs_status make_plan(long long n, const mvgs_camera* cams, int V, const mvgs_co
     P.w_order = w.take(R * sizeof(uint32_t));
     P.w_bins = w.take(R * sizeof(uint32_t));
     P.w_desc = w.take(R * sizeof(unsigned long long));
+    P.w_bins_by_depth = w.take(R * sizeof(uint32_t));
     P.w_bin_off = w.take((R + 1) * sizeof(unsigned long long));
     P.w_keys_a = w.take(K * sizeof(uint32_t));
     P.w_keys_b = w.take(K * sizeof(uint32_t));
@@ -248,7 +249,7 @@ mvgs_status make_plan(long long n, const mvgs_camera* cams, int V, const mvgs_co
     P.w_lists = w.take(tile_lists_temp_bytes(K, bins, tiles));
     P.w_torder = w.take(tile_order_temp_bytes(tiles));
     P.w_counter = w.take(sizeof(int));
-    P.w_dcount = w.take((8 + 2 * kSumSlots) * sizeof(unsigned long long));
+    P.w_dcount = w.take((8 + kSumWords) * sizeof(unsigned long long));
     // runs of at least 32 samples: at most one partial run per tile
     P.chunk_cap = tiles + pixels / 32 + 1;
     P.w_chunk_off = w.take((size_t)(tiles + 1) * sizeof(long long));
@@ -330,14 +331,21 @@ __global__ void set_counts_kernel(long long* c, long long R, long long K, long l
 
 // The batch's counts, from the record scan and the preprocessing's sums:
 // dcnt = records held, keys needed, keys held, (record, bin) entries held,
-// records needed ("held": within the capacity).
+// records needed ("held": within the capacity), the least of the depths' bits
+// and how far the largest is above it.
 __global__ void total_counts_kernel(const long long* rec_total, const unsigned long long* sums, long long rec_cap,
                                     long long key_cap, unsigned long long* dcnt) {
     unsigned long long k = 0, b = 0;
+    uint32_t lo = 0, hi = 0;
     for (int i = threadIdx.x; i < kSumSlots; i += 32) {
         k += sums[2 * i];
         b += sums[2 * i + 1];
+        const uint2 e = reinterpret_cast<const uint2*>(sums + 2 * kSumSlots)[i];
+        lo = max(lo, e.x);
+        hi = max(hi, e.y);
     }
+    lo = ~__reduce_max_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
     for (int o = 16; o > 0; o >>= 1) {
         k += __shfl_xor_sync(0xffffffffu, k, o);
         b += __shfl_xor_sync(0xffffffffu, b, o);
@@ -349,6 +357,8 @@ __global__ void total_counts_kernel(const long long* rec_total, const unsigned l
         dcnt[2] = k < kc ? k : kc;
         dcnt[3] = b < kc ? b : kc;
         dcnt[4] = r;
+        dcnt[5] = lo;
+        dcnt[6] = hi > lo ? hi - lo : 0u;
     }
 }
 
@@ -472,7 +482,7 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
     DevCam* dcams = at<DevCam>(workspace, P.w_cams);
     unsigned long long* dcnt = at<unsigned long long>(workspace, P.w_dcount);
     unsigned long long* sums = dcnt + 8;
-    upload_cams(P.cams.data(), V, dcams, s, sums, 2 * kSumSlots);
+    upload_cams(P.cams.data(), V, dcams, s, sums, kSumWords);
     const SceneArgs sc = scene_args(scene);
     RecordArgs rec = record_args(state, P);
     long long* counts_dev = at<long long>(state, L.off_counts);
@@ -504,7 +514,7 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
     // the capacity (the kernels stop at the device count), so the call can be
     // captured in a CUDA graph.
     const bool capt = (cfg->flags & MVGS_FLAG_CAPTURABLE) != 0;
-    unsigned long long c[5] = {0, 0, 0, 0, 0};
+    unsigned long long c[7] = {0, 0, 0, 0, 0, 0, 0};
     if (!capt) {
         if (cudaMemcpyAsync(c, dcnt, sizeof(c), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess)
@@ -531,21 +541,26 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
     const Count Sc = capt ? Count((unsigned long long)cap->keys, dcnt + 3) : Count(c[3]);
 
     // records by depth (the keys are the records' float32 depths, positive, so
-    // their bits sort as unsigned integers; the values the record indices),
-    // with each record's bin count carried into depth order by the last pass;
-    // then the tiles' lists in that order
+    // their bits sort as unsigned integers, less the least of them; only the
+    // bits that the largest difference has are sorted, all 32 when it is not
+    // known here), with each record's bin count carried into depth order by the
+    // last pass; then the tiles' lists in that order
     uint32_t* order = at<uint32_t>(workspace, P.w_order);
-    uint32_t* bins_by_depth = at<uint32_t>(workspace, P.w_ids_a);
+    uint32_t* bins_by_depth = at<uint32_t>(workspace, P.w_bins_by_depth);
+    int depth_bits = 32;
+    if (!capt)
+        while (depth_bits > 1 && (c[6] >> (depth_bits - 1)) == 0) depth_bits--;
     {
         StageTimer t(MVGS_STAGE_DEPTH_SORT, s);
-        radix_sort_pairs(reinterpret_cast<const uint32_t*>(rec.depth), nullptr, at<uint32_t>(workspace, P.w_dkeys_a),
-                         bins_by_depth, at<uint32_t>(workspace, P.w_dkeys_b), at<uint32_t>(workspace, P.w_ids_b),
-                         order, Rc, 32, at<void>(workspace, P.w_radix), s, bins, bins_by_depth);
+        radix_sort_ids(reinterpret_cast<const uint32_t*>(rec.depth), dcnt + 5, at<uint32_t>(workspace, P.w_dkeys_a),
+                       at<uint32_t>(workspace, P.w_ids_a), at<uint32_t>(workspace, P.w_dkeys_b),
+                       at<uint32_t>(workspace, P.w_ids_b), order, Rc, depth_bits, at<void>(workspace, P.w_radix), s,
+                       bins, bins_by_depth);
     }
     unsigned long long* bin_off = at<unsigned long long>(workspace, P.w_bin_off);
     {
         StageTimer t(MVGS_STAGE_SCAN_TILES, s);
-        scan_u32_to_u64_count(bins_by_depth, bin_off, Rc, nullptr, at<void>(workspace, P.w_scan), s);
+        scan_u32_to_u64_count(bins_by_depth, bin_off, Rc, at<void>(workspace, P.w_scan), s);
     }
     uint32_t* sorted = at<uint32_t>(state, L.off_sorted_records);
     long long* ranges = at<long long>(state, L.off_tile_ranges);

@@ -67,9 +67,11 @@ void launch_count_keys(const SceneArgs& sc, const DevCam* cams, int V, int tw, i
 void launch_count_visible(const SceneArgs& sc, const DevCam* cams, int V, int tw, int th, int* counts, uint8_t* vis,
                           cudaStream_t s);
 // Writes all records of the visible pairs, the number of bins each record
-// touches and its tile descriptor (pack_tile_desc), and adds the records' tile
-// and bin totals into kSumSlots pairs of sums (zeroed by the caller).
-constexpr int kSumSlots = 128;
+// touches and its tile descriptor (pack_tile_desc), adds the records' tile and
+// bin totals into kSumSlots pairs of sums (zeroed by the caller), and behind
+// those leaves kSumSlots pairs of 32-bit words: the largest complement and the
+// largest of the depths' bits.
+constexpr int kSumSlots = 128, kSumWords = 3 * kSumSlots;
 void launch_preprocess(const SceneArgs& sc, const DevCam* cams, int V, int tw, int th, const uint8_t* vis,
                        const RecordArgs& rec, uint32_t* bins, unsigned long long* tile_desc,
                        unsigned long long* sums, cudaStream_t s);
@@ -91,19 +93,18 @@ void scan_i32_to_i64(const int* in, long long* out, uint64_t n, void* tmp, cudaS
 // scans in[i] & mask
 void scan_masked_i32_to_i64(const int* in, int mask, long long* out, uint64_t n, void* tmp, cudaStream_t s);
 void scan_u32_to_u64(const uint32_t* in, unsigned long long* out, uint64_t n, void* tmp, cudaStream_t s);
-// (also the total into *total when given; n may be a device count)
-void scan_u32_to_u64_count(const uint32_t* in, unsigned long long* out, Count n, unsigned long long* total,
-                           void* tmp, cudaStream_t s);
+// (n may be a device count)
+void scan_u32_to_u64_count(const uint32_t* in, unsigned long long* out, Count n, void* tmp, cudaStream_t s);
 
 size_t radix_temp_bytes(uint64_t n);
-// Stable LSD sort of (key, value) pairs on key bits [0, bits).  Input in
-// (keys0, vals0), read only; vals0 == nullptr sorts the identity permutation
-// (values generated, not read).  keys_a/b and vals_a/b are scratch; the sorted
-// values end in vals_out.  With gather_src, the last pass also writes
-// gather_out[i] = gather_src[vals_out[i]] (gather_out may be vals_a).
-void radix_sort_pairs(const uint32_t* keys0, const uint32_t* vals0, uint32_t* keys_a, uint32_t* vals_a,
-                      uint32_t* keys_b, uint32_t* vals_b, uint32_t* vals_out, Count n, int bits, void* tmp,
-                      cudaStream_t s, const uint32_t* gather_src = nullptr, uint32_t* gather_out = nullptr);
+// Stable LSD sort of the ids 0 .. n by key bits [0, bits); sub (optional): a
+// device word subtracted from every key, the bits being those of the
+// differences.  keys_a/b and vals_a/b are scratch; the sorted ids end in
+// vals_out.  With gather_src, the last pass also writes
+// gather_out[i] = gather_src[vals_out[i]].
+void radix_sort_ids(const uint32_t* keys, const unsigned long long* sub, uint32_t* keys_a, uint32_t* vals_a,
+                    uint32_t* keys_b, uint32_t* vals_b, uint32_t* vals_out, Count n, int bits, void* tmp,
+                    cudaStream_t s, const uint32_t* gather_src, uint32_t* gather_out);
 
 // The per-tile lists: record ids by (view, tile, depth), of one entry per
 // (record, covered tile), and every tile's [start, end).  `order`: records

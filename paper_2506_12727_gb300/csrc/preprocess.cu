@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(PRE_THREADS, SHARED_CAMS ? 10 : 8) preprocess_
         }
         cp_async_wait<0>();
         __syncwarp();
-        uint32_t nt = 0, nb = 0;  // the record's tiles and bins
+        uint32_t nt = 0, nb = 0, depth = 0;  // the record's tiles, bins and depth
         if (write) {
             const float inv = 1.f / P.det;
             rec.rec_g[r] = (int)g;
@@ -435,19 +435,24 @@ __global__ void __launch_bounds__(PRE_THREADS, SHARED_CAMS ? 10 : 8) preprocess_
             rec.clamp[r] = clamp;
             rec.depth[r] = P.depth;
             rec.rect[r] = P.rect;
-            const uint32_t touched = bins_touched(P.rect);
-            bins[r] = touched;
+            bins[r] = nb = bins_touched(P.rect);
             tile_desc[r] = pack_tile_desc(P.rect, v);
             nt = (uint32_t)((P.rect.z - P.rect.x) * (P.rect.w - P.rect.y));
-            nb = touched;
+            depth = __float_as_uint(P.depth);
         }
         // the warp's totals, spread over kSumSlots pairs of counters
         nt = __reduce_add_sync(0xffffffffu, nt);
         nb = __reduce_add_sync(0xffffffffu, nb);
+        const uint32_t lo = __reduce_max_sync(0xffffffffu, write ? ~depth : 0u);
+        const uint32_t hi = __reduce_max_sync(0xffffffffu, depth);
         if (lane == 0 && nb > 0) {
             unsigned long long* slot = sums + 2 * (blockIdx.x % kSumSlots);
             atomicAdd(slot, (unsigned long long)nt);
             atomicAdd(slot + 1, (unsigned long long)nb);
+            uint32_t* ext = reinterpret_cast<uint32_t*>(sums + 2 * kSumSlots) + 2 * (blockIdx.x % kSumSlots);
+            const uint2 now = __ldcg(reinterpret_cast<const uint2*>(ext));  // seldom exceeded once warps have passed
+            if (lo > now.x) atomicMax(ext, lo);
+            if (hi > now.y) atomicMax(ext + 1, hi);
         }
     }
 }

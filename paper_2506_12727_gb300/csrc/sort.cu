@@ -27,7 +27,7 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 
 // ---------------------------------------------------------------------------
-// exclusive scan (reduce, spine, downsweep)
+// exclusive scan (reduce, spine, downsweep; fewer launches for fewer blocks)
 // ---------------------------------------------------------------------------
 constexpr int SC_THREADS = 256;
 constexpr int SC_ITEMS = 16;
@@ -113,8 +113,13 @@ __global__ void __launch_bounds__(SPINE_THREADS) scan_spine_kernel(T* partials, 
 
 __device__ __forceinline__ int pad_index(int i) { return i + (i >> 5); }
 
+// What the blocks before sum to: the scanned partials (SPINE), the sum of the
+// raw ones (PARTIALS), or of their input read again (INPUT; not in place).
+enum ScanBase { SPINE, PARTIALS, INPUT };
+
 template <class Load, class T>
-__global__ void __launch_bounds__(SC_THREADS) scan_down_kernel(Load ld, Count cn, const T* partials, T* out) {
+__global__ void __launch_bounds__(SC_THREADS) scan_down_kernel(Load ld, Count cn, ScanBase mode, const T* partials, T* out,
+                                                               T* total_out, T* end_out) {
     __shared__ T tile[SC_TILE + SC_TILE / 32];
     __shared__ T buf[33];
     const uint64_t n = cn.get();
@@ -131,8 +136,26 @@ __global__ void __launch_bounds__(SC_THREADS) scan_down_kernel(Load ld, Count cn
         local[k] = tile[pad_index(threadIdx.x * SC_ITEMS + k)];
         sum += local[k];
     }
+    T first = 0;
+    if (mode == SPINE) {
+        first = partials[blockIdx.x];
+    } else {
+        T before = 0;
+        if (mode == PARTIALS) {
+            for (unsigned i = threadIdx.x; i < blockIdx.x; i += SC_THREADS) before += partials[i];
+        } else {
+            const uint64_t end = base < n ? base : n;
+#pragma unroll 8
+            for (uint64_t i = threadIdx.x; i < end; i += SC_THREADS) before += ld(i);
+        }
+        block_exclusive_scan<T>(before, buf, first);
+    }
     T total;
-    T run = block_exclusive_scan<T>(sum, buf, total) + partials[blockIdx.x];
+    T run = block_exclusive_scan<T>(sum, buf, total) + first;
+    if (mode != SPINE && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+        if (total_out) *total_out = first + total;
+        if (end_out) end_out[n] = first + total;
+    }
 #pragma unroll
     for (int k = 0; k < SC_ITEMS; k++) {
         tile[pad_index(threadIdx.x * SC_ITEMS + k)] = run;
@@ -158,127 +181,99 @@ void scan_impl(Load ld, T* out, Count n, bool write_end, T* total_out, void* tmp
     }
     const uint64_t nb = ceil_div_u64(n.max, SC_TILE);
     T* partials = static_cast<T*>(tmp);
-    scan_reduce_kernel<Load, T><<<(unsigned)nb, SC_THREADS, 0, s>>>(ld, n, partials);
-    scan_spine_kernel<T><<<1, SPINE_THREADS, 0, s>>>(partials, nb, total_out, write_end ? out : nullptr, n);
-    scan_down_kernel<Load, T><<<(unsigned)nb, SC_THREADS, 0, s>>>(ld, n, partials, out);
-    note_launches(3);
+    T* end = write_end ? out : nullptr;
+    // A launch costs a dependent kernel some 3 us: up to 5 blocks sum what
+    // lies before them from the input, up to 1024 from the blocks' sums.
+    const ScanBase mode = nb <= 5 ? INPUT : nb <= 1024 ? PARTIALS : SPINE;
+    if (mode != INPUT) {
+        scan_reduce_kernel<Load, T><<<(unsigned)nb, SC_THREADS, 0, s>>>(ld, n, partials);
+        note_launches(1);
+    }
+    if (mode == SPINE) {
+        scan_spine_kernel<T><<<1, SPINE_THREADS, 0, s>>>(partials, nb, total_out, end, n);
+        note_launches(1);
+    }
+    scan_down_kernel<Load, T><<<(unsigned)nb, SC_THREADS, 0, s>>>(ld, n, mode, partials, out, total_out, end);
+    note_launches(1);
 }
 
 // ---------------------------------------------------------------------------
 // stable LSD radix sort of (uint32 key, uint32 value), 8-bit digits
 // ---------------------------------------------------------------------------
+// A pass is a histogram per block, a scan per digit over the blocks and the
+// scatter: three launches instead of five (the scan over the digits is the
+// scatter's own), two when there are few blocks.  Bound by the scatter: 16
+// ballot rounds per key in the ranking, then runs of about 16 keys.  Sort of the
+// depths: 22M (3M Gaussians x 8 views) 0.93 -> 0.61 ms, 500k 138 -> 57 us, 10k
+// 118 -> 42 us, with three passes for four where their range allows it (below
+// 2^24 apart: the farthest up to about four times as far as the nearest).
+// Digits of 9 bits, three passes for 27 bits, took 0.77 ms at 22M keys against
+// 0.74 with four passes, and as long at 2M.
 constexpr int RS_THREADS = 256;  // == number of digit values
 constexpr int RS_ITEMS = 16;
 constexpr int RS_WARPS = RS_THREADS / 32;
 constexpr int RS_SEG = RS_ITEMS * 32;  // contiguous keys per warp
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
+// Blocks up to which the scatter sums the histograms itself: at 64 blocks its
+// loads take 1 us more than reading a scanned table, the scan 2 us and a launch.
+constexpr uint64_t RS_DIRECT = 64;
+
+// The histograms of a pass: per digit over the blocks (direct false: scanned
+// in place, totals beside) or per block over the digits (direct true).
+struct RadixTable {
+    uint32_t* counts;
+    uint32_t* totals;
+    uint32_t nblocks;
+    bool direct;
+};
 
 struct RankSmem {
     uint32_t whist[RS_WARPS * 256];  // per-warp digit counts, then per-warp prefixes
     uint32_t boff[256];              // first output position of each digit of the block
     uint32_t dstart[256];            // first block-local position of each digit
-    uint32_t scan_buf[33];
+    unsigned long long scan_buf[33];
     uint32_t skeys[RS_TILE];         // keys in block-local sorted order
     uint32_t svals[RS_TILE];         // values in block-local sorted order
 };
 
-// Stable rank of the block's keys (held in registers, warp w owning the
-// contiguous segment [w*SEG, (w+1)*SEG) in rounds of 32 lanes) and scatter:
-// first into shared memory in block-local digit order, then to global memory
-// in runs of consecutive positions per digit.  Equal digits inside a round are
-// found with one ballot per digit bit.  Values are fetched after the ranking
-// (get_val(block-local index)), so they do not occupy registers during it.
-template <bool WRITE_KEYS, int NB, class GetVal>
-__device__ __forceinline__ void rank_and_scatter(RankSmem& sm, const uint32_t (&k)[RS_ITEMS], uint64_t n, int shift,
-                                                 const uint32_t* __restrict__ offsets, uint32_t nblocks,
-                                                 uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
-                                                 GetVal get_val, const uint32_t* __restrict__ gsrc,
-                                                 uint32_t* __restrict__ gout) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t lt = (1u << lane) - 1u;
-    const uint64_t block0 = (uint64_t)blockIdx.x * RS_TILE;
-    const int local0 = warp * RS_SEG + lane;
-    const uint64_t base = block0 + local0;
-    for (int i = threadIdx.x; i < RS_WARPS * 256; i += RS_THREADS) sm.whist[i] = 0;
-    sm.boff[threadIdx.x] = offsets[(uint64_t)threadIdx.x * nblocks + blockIdx.x];
-    __syncthreads();
-    uint32_t* wh = sm.whist + warp * 256;
-    uint32_t lr[RS_ITEMS];
-#pragma unroll
-    for (int j = 0; j < RS_ITEMS; j++) {
-        const bool ok = base + (uint64_t)j * 32 < n;
-        const uint32_t d = (k[j] >> shift) & 0xffu;
-        uint32_t peers = __ballot_sync(kFull, ok);
-#pragma unroll
-        for (int b = 0; b < NB; b++) {  // digit bits above NB are zero in this pass
-            const uint32_t bit = (d >> b) & 1u;
-            const uint32_t bb = __ballot_sync(kFull, bit);
-            peers &= bit ? bb : ~bb;
+// Keys of the thread's digit in all blocks and in the blocks before.
+__device__ __forceinline__ void digit_counts(const RadixTable& tab, uint32_t& tot, uint32_t& pre) {
+    if (tab.direct) {
+        tot = pre = 0;
+#pragma unroll 8
+        for (uint32_t b = 0; b < tab.nblocks; b++) {
+            const uint32_t c = tab.counts[b * 256 + threadIdx.x];
+            if (b < blockIdx.x) pre += c;
+            tot += c;
         }
-        const uint32_t rank = __popc(peers & lt);
-        const uint32_t before = wh[d];
-        __syncwarp();
-        if (ok && rank == 0) wh[d] = before + __popc(peers);
-        __syncwarp();
-        lr[j] = before + rank;
-    }
-    // values are read before the barrier that precedes the scatter, so a
-    // source may keep them in the staging the scatter overwrites
-    uint32_t vv[RS_ITEMS];
-#pragma unroll
-    for (int j = 0; j < RS_ITEMS; j++) vv[j] = base + (uint64_t)j * 32 < n ? get_val(local0 + j * 32) : 0u;
-    __syncthreads();
-    uint32_t run = 0;
-#pragma unroll
-    for (int w = 0; w < RS_WARPS; w++) {
-        const uint32_t c = sm.whist[w * 256 + threadIdx.x];
-        sm.whist[w * 256 + threadIdx.x] = run;
-        run += c;
-    }
-    uint32_t total;
-    sm.dstart[threadIdx.x] = block_exclusive_scan<uint32_t>(run, sm.scan_buf, total);
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < RS_ITEMS; j++) {
-        if (base + (uint64_t)j * 32 < n) {
-            const uint32_t d = (k[j] >> shift) & 0xffu;
-            const uint32_t lp = sm.dstart[d] + wh[d] + lr[j];
-            sm.skeys[lp] = k[j];
-            sm.svals[lp] = vv[j];
-        }
-    }
-    __syncthreads();
-    const int cnt = (int)(n - block0 < (uint64_t)RS_TILE ? n - block0 : (uint64_t)RS_TILE);
-    for (int i = threadIdx.x; i < cnt; i += RS_THREADS) {
-        const uint32_t key = sm.skeys[i];
-        const uint32_t d = (key >> shift) & 0xffu;
-        const uint32_t pos = sm.boff[d] + (uint32_t)i - sm.dstart[d];
-        vout[pos] = sm.svals[i];
-        if (WRITE_KEYS) kout[pos] = key;
-        if (gout) gout[pos] = gsrc[sm.svals[i]];
+    } else {
+        pre = tab.counts[(uint64_t)threadIdx.x * tab.nblocks + blockIdx.x];
+        tot = tab.totals[threadIdx.x];
     }
 }
 
-// Per-block digit histogram, stored digit-major so that one exclusive scan of
-// the whole table gives every block's first output position per digit.
+// Per-block digit histogram.  sub (optional): subtracted from every key.
 __global__ void __launch_bounds__(RS_THREADS) rs_upsweep(const uint32_t* __restrict__ keys, Count cn, int shift,
-                                                        uint32_t* __restrict__ counts, uint32_t nblocks) {
+                                                        const unsigned long long* __restrict__ sub, RadixTable tab) {
     __shared__ uint32_t hist[RS_WARPS * 256];
     const uint64_t n = cn.get();
-    for (int i = threadIdx.x; i < RS_WARPS * 256; i += RS_THREADS) hist[i] = 0;
-    __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t base = (uint64_t)blockIdx.x * RS_TILE + warp * RS_SEG + lane;
+    uint32_t k[RS_ITEMS];
 #pragma unroll
-    for (int j = 0; j < RS_ITEMS; j++) {
-        const uint64_t idx = base + (uint64_t)j * 32;
-        if (idx < n) atomicAdd(&hist[warp * 256 + ((keys[idx] >> shift) & 0xffu)], 1u);
-    }
+    for (int j = 0; j < RS_ITEMS; j++) k[j] = base + (uint64_t)j * 32 < n ? keys[base + (uint64_t)j * 32] : 0u;
+    const uint32_t k0 = sub ? (uint32_t)*sub : 0u;
+    for (int i = threadIdx.x; i < RS_WARPS * 256; i += RS_THREADS) hist[i] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < RS_ITEMS; j++)
+        if (base + (uint64_t)j * 32 < n) atomicAdd(&hist[warp * 256 + (((k[j] - k0) >> shift) & 0xffu)], 1u);
     __syncthreads();
     uint32_t sum = 0;
 #pragma unroll
     for (int w = 0; w < RS_WARPS; w++) sum += hist[w * 256 + threadIdx.x];
-    counts[(uint64_t)threadIdx.x * nblocks + blockIdx.x] = sum;
+    if (tab.direct) tab.counts[(uint64_t)blockIdx.x * 256 + threadIdx.x] = sum;
+    else tab.counts[(uint64_t)threadIdx.x * tab.nblocks + blockIdx.x] = sum;
 }
 
 // The same table for a pass whose digits take at most 32 values (few bins, or
@@ -288,8 +283,7 @@ __global__ void __launch_bounds__(RS_THREADS) rs_upsweep(const uint32_t* __restr
 // other lane touches the column), then a skewed sweep sums the columns.
 // Shared-memory atomics from 32 lanes on a handful of digits serialise.
 __global__ void __launch_bounds__(RS_THREADS) rs_upsweep_narrow(const uint32_t* __restrict__ keys, Count cn, int shift,
-                                                               uint32_t mask, uint32_t* __restrict__ counts,
-                                                               uint32_t nblocks) {
+                                                               uint32_t mask, RadixTable tab) {
     __shared__ uint32_t cnt[RS_WARPS][32 * 32];
     __shared__ uint32_t wsum[RS_WARPS][32];
     const uint64_t n = cn.get();
@@ -315,37 +309,133 @@ __global__ void __launch_bounds__(RS_THREADS) rs_upsweep_narrow(const uint32_t* 
 #pragma unroll
         for (int w = 0; w < RS_WARPS; w++) total += wsum[w][threadIdx.x];
     }
-    counts[(uint64_t)threadIdx.x * nblocks + blockIdx.x] = threadIdx.x < 32 ? total : 0u;
+    if (tab.direct) tab.counts[(uint64_t)blockIdx.x * 256 + threadIdx.x] = total;
+    else tab.counts[(uint64_t)threadIdx.x * tab.nblocks + blockIdx.x] = total;
 }
 
-// NB: significant bits of this pass's digit (8, or fewer in a last pass over
-// the high bits of keys narrower than a whole number of digits).  vin ==
-// nullptr: the values are the keys' positions (an identity permutation,
-// generated instead of read).  gout != nullptr: also writes gout[pos] =
-// gsrc[value] (a per-element array carried into sorted order).
-template <bool WRITE_KEYS, int NB = 8>
+// One block per digit: its counts become the number of its keys in the blocks
+// before, and their sum its total.  A warp takes a stretch of the blocks.
+__global__ void __launch_bounds__(RS_THREADS) rs_scan_kernel(RadixTable tab) {
+    __shared__ uint32_t buf[33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t* row = tab.counts + (uint64_t)blockIdx.x * tab.nblocks;
+    const uint32_t per = (tab.nblocks + RS_THREADS - 1) / RS_THREADS * 32;
+    const uint32_t r0 = min(warp * per, tab.nblocks), r1 = min(r0 + per, tab.nblocks);
+    uint32_t sum = 0;
+#pragma unroll 4
+    for (uint32_t r = r0 + lane; r < r1; r += 32) sum += row[r];
+    uint32_t total;
+    const uint32_t ex = block_exclusive_scan<uint32_t>(sum, buf, total);
+    uint32_t run = __shfl_sync(kFull, ex, 0);
+#pragma unroll 4
+    for (uint32_t r = r0; r < r1; r += 32) {
+        const uint32_t v = r + lane < r1 ? row[r + lane] : 0u;
+        uint32_t inc = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (r + lane < r1) row[r + lane] = run + inc - v;
+        run += __shfl_sync(kFull, inc, 31);
+    }
+    if (threadIdx.x == 0) tab.totals[blockIdx.x] = total;
+}
+
+// Stable rank of the block's keys (held in registers, warp w owning the
+// contiguous segment [w*SEG, (w+1)*SEG) in rounds of 32 lanes) and scatter:
+// first into shared memory in block-local digit order, then to global memory
+// in runs of consecutive positions per digit.  Equal digits inside a round are
+// found with one ballot per digit bit.  Values are fetched after the ranking,
+// so they do not occupy registers during it.
+// NB: significant bits of this pass's digit.  vin == nullptr: the values are
+// the keys' positions (an identity permutation, generated instead of read).
+// sub: subtracted from every key (the keys written are the differences).
+// gout != nullptr: also writes gout[pos] = gsrc[value] (a per-element array
+// carried into sorted order).
+template <bool WRITE_KEYS, int NB>
 __global__ void __launch_bounds__(RS_THREADS, 3) rs_downsweep(const uint32_t* __restrict__ kin,
                                                              const uint32_t* __restrict__ vin,
                                                              uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
                                                              Count cn, int shift,
-                                                             const uint32_t* __restrict__ offsets, uint32_t nblocks,
+                                                             const unsigned long long* __restrict__ sub, RadixTable tab,
                                                              const uint32_t* __restrict__ gsrc = nullptr,
                                                              uint32_t* __restrict__ gout = nullptr) {
     __shared__ RankSmem sm;
     const uint64_t n = cn.get();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
     const uint64_t block0 = (uint64_t)blockIdx.x * RS_TILE;
     if (block0 >= n) return;  // a block past the keys (capturable mode)
-    const uint64_t base = block0 + warp * RS_SEG + lane;
+    const int here = (int)(n - block0 < (uint64_t)RS_TILE ? n - block0 : (uint64_t)RS_TILE);
+    const int local0 = warp * RS_SEG + lane;
+    for (int i = threadIdx.x; i < RS_WARPS * 256; i += RS_THREADS) sm.whist[i] = 0;
+    kin += block0;
     uint32_t k[RS_ITEMS];
+    const uint32_t k0 = sub ? (uint32_t)*sub : 0u;
+#pragma unroll
+    for (int j = 0; j < RS_ITEMS; j++) k[j] = (local0 + j * 32 < here ? kin[local0 + j * 32] : 0u) - k0;
+    uint32_t tot, pre;
+    digit_counts(tab, tot, pre);
+    __syncthreads();
+    uint32_t* wh = sm.whist + warp * 256;
+    uint32_t lr[RS_ITEMS];
 #pragma unroll
     for (int j = 0; j < RS_ITEMS; j++) {
-        const uint64_t idx = base + (uint64_t)j * 32;
-        k[j] = idx < n ? kin[idx] : 0u;
+        const bool ok = local0 + j * 32 < here;
+        const uint32_t d = (k[j] >> shift) & 0xffu;
+        uint32_t peers = __ballot_sync(kFull, ok);
+#pragma unroll
+        for (int b = 0; b < NB; b++) {  // digit bits above NB are zero in this pass
+            const uint32_t bit = (d >> b) & 1u;
+            const uint32_t bb = __ballot_sync(kFull, bit);
+            peers &= bit ? bb : ~bb;
+        }
+        const uint32_t rank = __popc(peers & lt);
+        const uint32_t before = wh[d];
+        __syncwarp();
+        if (ok && rank == 0) wh[d] = before + __popc(peers);
+        __syncwarp();
+        lr[j] = before + rank;
     }
-    rank_and_scatter<WRITE_KEYS, NB>(
-        sm, k, n, shift, offsets, nblocks, kout, vout,
-        [&](int local) { return vin ? vin[block0 + local] : (uint32_t)(block0 + local); }, gsrc, gout);
+    uint32_t vv[RS_ITEMS];
+#pragma unroll
+    for (int j = 0; j < RS_ITEMS; j++)
+        vv[j] = !vin ? (uint32_t)block0 + local0 + j * 32 : local0 + j * 32 < here ? vin[block0 + local0 + j * 32] : 0u;
+    __syncthreads();
+    uint32_t run = 0;
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; w++) {
+        const uint32_t c = sm.whist[w * 256 + threadIdx.x];
+        sm.whist[w * 256 + threadIdx.x] = run;
+        run += c;
+    }
+    // both prefixes over the digits in one scan: of the totals (high words) and
+    // of the block's counts
+    unsigned long long all;
+    const unsigned long long at =
+        block_exclusive_scan<unsigned long long>((unsigned long long)tot << 32 | run, sm.scan_buf, all);
+    sm.dstart[threadIdx.x] = (uint32_t)at;
+    sm.boff[threadIdx.x] = (uint32_t)(at >> 32) + pre;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < RS_ITEMS; j++) {
+        if (local0 + j * 32 < here) {
+            const uint32_t d = (k[j] >> shift) & 0xffu;
+            const uint32_t lp = sm.dstart[d] + wh[d] + lr[j];
+            sm.skeys[lp] = k[j];
+            sm.svals[lp] = vv[j];
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < here; i += RS_THREADS) {
+        const uint32_t key = sm.skeys[i];
+        const uint32_t d = (key >> shift) & 0xffu;
+        const uint32_t pos = sm.boff[d] + (uint32_t)i - sm.dstart[d];
+        vout[pos] = sm.svals[i];
+        if (WRITE_KEYS) kout[pos] = key;
+        if (gout) gout[pos] = gsrc[sm.svals[i]];
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -785,57 +875,53 @@ void scan_u32_to_u64(const uint32_t* in, unsigned long long* out, uint64_t n, vo
     scan_impl(LoadDirect<uint32_t, unsigned long long>{in}, out, n, true, (unsigned long long*)nullptr, tmp, s);
 }
 
-void scan_u32_to_u64_count(const uint32_t* in, unsigned long long* out, Count n, unsigned long long* total,
-                           void* tmp, cudaStream_t s) {
-    scan_impl(LoadDirect<uint32_t, unsigned long long>{in}, out, n, true, total, tmp, s);
+void scan_u32_to_u64_count(const uint32_t* in, unsigned long long* out, Count n, void* tmp, cudaStream_t s) {
+    scan_impl(LoadDirect<uint32_t, unsigned long long>{in}, out, n, true, (unsigned long long*)nullptr, tmp, s);
 }
 
 static uint64_t radix_blocks(uint64_t n) { return ceil_div_u64(n, RS_TILE); }
 
-size_t radix_temp_bytes(uint64_t n) {
-    const uint64_t nb = radix_blocks(n > 0 ? n : 1);
-    const size_t counts = ((256 * nb * sizeof(uint32_t)) + 255) / 256 * 256;
-    return counts + (scan_temp_bytes(256 * nb) + 255) / 256 * 256;
-}
+size_t radix_temp_bytes(uint64_t n) { return (radix_blocks(n > 0 ? n : 1) + 1) * 256 * sizeof(uint32_t); }
 
 namespace {
-// One radix pass: histogram, scan, scatter.
-template <class Up, class Down>
-void radix_pass(uint64_t n, void* tmp, cudaStream_t s, Up up, Down down) {
-    const uint64_t nb = radix_blocks(n);
-    uint32_t* counts = static_cast<uint32_t*>(tmp);
-    void* scan_tmp = static_cast<char*>(tmp) + ((256 * nb * sizeof(uint32_t)) + 255) / 256 * 256;
-    up((unsigned)nb, counts);
-    scan_impl(LoadDirect<uint32_t, uint32_t>{counts}, counts, Count(256 * nb), false, (uint32_t*)nullptr, scan_tmp, s);
-    down((unsigned)nb, counts);
+// One radix pass over the 8 bits from `shift` up; the keys' bits from
+// shift + bits up are zero.
+void radix_pass(const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout, Count n, int shift, int bits,
+                bool write_keys, const unsigned long long* sub, void* tmp, cudaStream_t s,
+                const uint32_t* gsrc = nullptr, uint32_t* gout = nullptr) {
+    const uint64_t nb64 = radix_blocks(n.max);
+    const unsigned nb = (unsigned)nb64;
+    uint32_t* totals = static_cast<uint32_t*>(tmp);
+    const RadixTable tab{totals + 256, totals, nb, nb64 <= RS_DIRECT};
+    if (bits <= 5 && !sub) rs_upsweep_narrow<<<nb, RS_THREADS, 0, s>>>(kin, n, shift, (1u << bits) - 1u, tab);
+    else rs_upsweep<<<nb, RS_THREADS, 0, s>>>(kin, n, shift, sub, tab);
+    if (!tab.direct) {
+        rs_scan_kernel<<<256, RS_THREADS, 0, s>>>(tab);
+        note_launches(1);
+    }
+#define MVGS_DOWN(W, B) \
+    rs_downsweep<W, B><<<nb, RS_THREADS, 0, s>>>(kin, vin, kout, vout, n, shift, sub, tab, gsrc, gout)
+    if (bits <= 5 && !sub && write_keys) MVGS_DOWN(true, 5);
+    else if (write_keys) MVGS_DOWN(true, 8);
+    else MVGS_DOWN(false, 8);
+#undef MVGS_DOWN
     note_launches(2);
 }
 }  // namespace
 
-void radix_sort_pairs(const uint32_t* keys0, const uint32_t* vals0, uint32_t* keys_a, uint32_t* vals_a,
-                      uint32_t* keys_b, uint32_t* vals_b, uint32_t* vals_out, Count n, int bits, void* tmp,
-                      cudaStream_t s, const uint32_t* gather_src, uint32_t* gather_out) {
+void radix_sort_ids(const uint32_t* keys, const unsigned long long* sub, uint32_t* keys_a, uint32_t* vals_a,
+                    uint32_t* keys_b, uint32_t* vals_b, uint32_t* vals_out, Count n, int bits, void* tmp,
+                    cudaStream_t s, const uint32_t* gather_src, uint32_t* gather_out) {
     if (n.max == 0) return;
     const int passes = (bits + 7) / 8 > 0 ? (bits + 7) / 8 : 1;
-    // pass 0 reads (keys0, vals0); later passes ping-pong b -> a -> b ...
-    const uint32_t* kin = keys0;
-    const uint32_t* vin = vals0;
+    const uint32_t* kin = keys;
+    const uint32_t* vin = nullptr;
     for (int p = 0; p < passes; p++) {
         const bool last = p == passes - 1;
         uint32_t* kout = (p & 1) ? keys_a : keys_b;
         uint32_t* vout = last ? vals_out : ((p & 1) ? vals_a : vals_b);
-        const int shift = 8 * p;
-        const uint32_t* gs = last ? gather_src : nullptr;
-        uint32_t* go = last ? gather_out : nullptr;
-        radix_pass(
-            n.max, tmp, s,
-            [&](unsigned nb, uint32_t* counts) { rs_upsweep<<<nb, RS_THREADS, 0, s>>>(kin, n, shift, counts, nb); },
-            [&](unsigned nb, uint32_t* counts) {
-                if (last)
-                    rs_downsweep<false><<<nb, RS_THREADS, 0, s>>>(kin, vin, kout, vout, n, shift, counts, nb, gs, go);
-                else
-                    rs_downsweep<true><<<nb, RS_THREADS, 0, s>>>(kin, vin, kout, vout, n, shift, counts, nb);
-            });
+        radix_pass(kin, vin, kout, vout, n, 8 * p, bits - 8 * p, !last, p == 0 ? sub : nullptr, tmp, s,
+                   last ? gather_src : nullptr, last ? gather_out : nullptr);
         kin = kout;
         vin = vout;
     }
@@ -893,21 +979,7 @@ void tile_lists(const uint32_t* order, const unsigned long long* bin_off, Count 
         int bits = 0;
         while ((1LL << bits) < bins) bits++;
         for (int p = 0; 8 * p < bits; p++) {
-            const int shift = low + 8 * p, hi = bits - 8 * p;  // hi: significant bits from this digit up
-            radix_pass(
-                S.max, radix_tmp, s,
-                [&](unsigned nb, uint32_t* counts) {
-                    if (hi <= 5)
-                        rs_upsweep_narrow<<<nb, RS_THREADS, 0, s>>>(kin, S, shift, (1u << hi) - 1u, counts, nb);
-                    else
-                        rs_upsweep<<<nb, RS_THREADS, 0, s>>>(kin, S, shift, counts, nb);
-                },
-                [&](unsigned nb, uint32_t* counts) {
-                    if (hi <= 5)
-                        rs_downsweep<true, 5><<<nb, RS_THREADS, 0, s>>>(kin, vin, kout, vout, S, shift, counts, nb);
-                    else
-                        rs_downsweep<true><<<nb, RS_THREADS, 0, s>>>(kin, vin, kout, vout, S, shift, counts, nb);
-                });
+            radix_pass(kin, vin, kout, vout, S, low + 8 * p, bits - 8 * p, true, nullptr, radix_tmp, s);
             uint32_t *nk = kin, *nv = vin;
             kin = kout;
             vin = vout;
