@@ -583,7 +583,8 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
     ba.V = V;
     ba.tw = tw;
     ba.th = th;
-    ba.ppt = blend_pixels_per_thread(tw, th, cfg->pixels_per_thread);
+    ba.ppt = smp ? blend_pixels_per_thread(tw, th, cfg->pixels_per_thread)
+                 : blend_forward_pixels_per_thread(tw, th, cfg->pixels_per_thread, P.tiles);
     ba.sw = blend_strip_width(tw);
     ba.strip_h = (32 / ba.sw) * ba.ppt;
     ba.strips = (tw / ba.sw) * (th / ba.strip_h);

@@ -891,6 +891,25 @@ int blend_pixels_per_thread(int tw, int th, int req) {
     return 1;
 }
 
+// The forward's images do not depend on the pixels per lane (each pixel's
+// arithmetic is its own), so a small render may use fewer and fill the chip with
+// more, shorter strips; the backward sums a lane's pixels together and keeps its
+// count.  2432 warps are resident.  Up to 2048 strips of 4 pixels per lane all
+// warps have at most one strip and 1 pixel is fastest: 10k Gaussians at 128 x 128
+// (128 strips) 69 -> 38 us, 20k in three small views (1077) 256 -> 144, 300k at
+// 480 x 400 (1500) 179 -> 110, with 2 pixels 45, 179, 122.  Above, a strip's
+// staging is repeated too often, and 2 are fastest while the queue is short:
+// 100k at 800 x 600 (3750 strips) 83 us with 4, 73 with 2, 101 with 1; two views
+// of unlike sizes (7394) 267, 170, 202; from about three strips of 4 per warp on
+// it is even (7734 strips: 157 and 148, 55 and 59; 8216: 101 and 107).
+int blend_forward_pixels_per_thread(int tw, int th, int req, long long tiles) {
+    const int most = blend_pixels_per_thread(tw, th, req);
+    if (req > 0) return most;
+    const long long strips = tiles * tw * th / 128;
+    const int want = strips <= 2048 ? 1 : strips <= 7500 ? 2 : 4;
+    return want < most ? want : most;
+}
+
 void launch_blend_forward(const BlendArgs& a, int* counter, float* img, float* final_T, uint32_t* n_contrib,
                           uint2* pixel_stats, cudaStream_t s) {
     if (a.tiles == 0) return;

@@ -157,6 +157,8 @@ struct BlendArgs {
 int blend_strip_width(int tw);
 // Pixels per lane for a tile size (req > 0: the caller's choice, checked).
 int blend_pixels_per_thread(int tw, int th, int req);
+// of a forward over all pixels
+int blend_forward_pixels_per_thread(int tw, int th, int req, long long tiles);
 // Persistent launches; `counter` is one device int of scratch (reset here).
 void launch_blend_forward(const BlendArgs& a, int* counter, float* img, float* final_T, uint32_t* n_contrib,
                           uint2* pixel_stats, cudaStream_t s);

@@ -124,3 +124,26 @@ def test_a_pixel_gradient_reaches_only_the_gaussians_it_blends(cuda_lib, value):
         a, b = runs[1][k][apart], runs[2][k][apart]
         assert torch.isfinite(b).all(), k
         torch.testing.assert_close(b, a, rtol=1e-4, atol=1e-6 * float(a.abs().max()))
+
+
+@pytest.mark.parametrize("tile,size", [((16, 16), (512, 512)), ((16, 16), (528, 512)), ((32, 64), (960, 960)),
+                                       ((32, 64), (960, 1024)), ((8, 8), (512, 512))])
+def test_small_renders_choose_pixels_per_lane_freely(cuda_lib, tile, size):
+    scene, cams = _mixed_scene(2000, 9), synth.make_cameras([size], radius=3.0, seed=2)
+    params = scene_to_device(scene)
+    sc = cuda_lib.make_scene(params, scene.sh_degree)
+    # strips of 8 columns and 4 rows per pixel of a lane
+    most = min(4, tile[1] // 4)
+    runs = []
+    for ppt in (0, most):
+        rz = cuda_lib.Rasterizer(cams, tile=tile, pixels_per_thread=ppt)
+        img = rz.forward(sc, depth=True, stats=True)
+        rec = rz.records()
+        grads = grads_like(params)
+        rz.backward(sc, torch.ones_like(img), grads)
+        runs.append(([img] + [rec[k].clone() for k in ("final_T", "n_contrib", "depth_acc", "pixel_stats")], grads))
+    for a, b in zip(runs[0][0], runs[1][0]):
+        assert torch.equal(a, b)
+    for k in PARAMS:  # the same kernel on the same state: only the order of its atomics may differ
+        a, b = runs[0][1][k].double(), runs[1][1][k].double()
+        assert float((a - b).norm()) <= 1e-5 * float(b.norm()) + 1e-12
