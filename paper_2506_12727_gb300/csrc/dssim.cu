@@ -36,37 +36,101 @@ struct Views {
     int count;
     int H[kMaxViews], W[kMaxViews];
     int tiles_x[kMaxViews];
+    int run[kMaxViews];           // tiles below one another that a block takes
     long long pix[kMaxViews];     // first pixel of the view in the packed layout
-    long long blk[kMaxViews + 1]; // first block of the view (3 channel planes)
+    long long blk[kMaxViews + 1]; // first tile of the view (3 channel planes)
+    long long cta[kMaxViews + 1]; // first block of the view
     int first_view;               // global index of views[0]
     float w[TAPS];
 };
 
 __device__ __forceinline__ int block_view(const Views& vw, long long b) {
     int v = 0;
-    while (v + 1 < vw.count && vw.blk[v + 1] <= b) v++;
+    while (v + 1 < vw.count && vw.cta[v + 1] <= b) v++;
     return v;
 }
 
 struct BlockPos {
-    int v, ch, x0, y0, H, W;
-    long long plane;  // offset of the channel plane in the packed image
+    int x0, H, W;
+    int ty0, ty1;        // tile rows
+    int tiles_x;
+    long long plane;     // offset of the channel plane in the packed image
+    long long tile;      // index of tile (ty = 0, the block's column) of the plane
 };
 
 __device__ __forceinline__ BlockPos block_pos(const Views& vw) {
     BlockPos p;
     const long long b = blockIdx.x;
-    p.v = block_view(vw, b);
-    const long long lb = b - vw.blk[p.v];
-    p.H = vw.H[p.v];
-    p.W = vw.W[p.v];
-    const int tiles = vw.tiles_x[p.v] * ((p.H + TSY - 1) / TSY);
-    p.ch = (int)(lb / tiles);
-    const int t = (int)(lb % tiles);
-    p.x0 = (t % vw.tiles_x[p.v]) * TSX;
-    p.y0 = (t / vw.tiles_x[p.v]) * TSY;
-    p.plane = 3 * vw.pix[p.v] + (long long)p.ch * p.H * p.W;
+    const int v = block_view(vw, b);
+    const long long lb = b - vw.cta[v];
+    p.H = vw.H[v];
+    p.W = vw.W[v];
+    p.tiles_x = vw.tiles_x[v];
+    const int tiles_y = (p.H + TSY - 1) / TSY, runs = p.tiles_x * ((tiles_y + vw.run[v] - 1) / vw.run[v]);
+    const int ch = (int)(lb / runs);
+    const int t = (int)(lb % runs);
+    const int tx = t % p.tiles_x;
+    p.x0 = tx * TSX;
+    p.ty0 = t / p.tiles_x * vw.run[v];
+    p.ty1 = min(p.ty0 + vw.run[v], tiles_y);
+    p.plane = 3 * vw.pix[v] + (long long)ch * p.H * p.W;
+    p.tile = vw.blk[v] + (long long)ch * p.tiles_x * tiles_y + tx;
     return p;
+}
+
+// A block takes a run of tiles below one another: after the first, the row
+// pass's last HALO rows are the next tile's first, so that it stages and blurs
+// TSY rows per tile (one item per thread) instead of HSY (336 items for 256
+// threads: a second round a third full).  The row-blurred rows lie in a ring of
+// HSY; the next tile's rows arrive during the column pass.  Bound by the issue
+// slots in the forward (79%) and by loads and address arithmetic in the
+// backward.  Eight 1264 x 832 views: 439 + 351 -> 348 + 282 us.  The sums' order
+// is the tile's own, so results do not depend on the runs; packed arithmetic (I1
+// and I2 side by side) saves a fifth of the instructions but its 64-bit column
+// reads conflict, 357 us.
+constexpr int HALO = 2 * RADIUS;
+__device__ __forceinline__ int ring(int row) { return row < HSY ? row : row - HSY; }
+static_assert(TSY * (TSX / 4) == 256, "one item per thread");
+
+// The rows that the tile below y0 adds, fetched asynchronously (the caller waits
+// and synchronises).
+template <int NP>
+__device__ __forceinline__ void fetch_rows(const float* const (&src)[NP], const BlockPos& p, int y0,
+                                           float (&s)[NP][HSY][HSX + 2]) {
+    int r = threadIdx.x / HSX, c = threadIdx.x % HSX;
+    long long o = p.plane + (long long)(y0 + TSY + RADIUS + r) * p.W + (p.x0 + c - RADIUS);
+    const long long step = (long long)(256 / HSX) * p.W + 256 % HSX;
+    while (r < TSY) {
+        const int y = y0 + TSY + RADIUS + r, x = p.x0 + c - RADIUS;
+        const bool in = x >= 0 && x < p.W && y < p.H;
+#pragma unroll
+        for (int m = 0; m < NP; m++) {
+            if (in) cp_async<4>(&s[m][r][c], src[m] + o);
+            else s[m][r][c] = 0.f;
+        }
+        r += 256 / HSX;
+        c += 256 % HSX;
+        o += step;
+        if (c >= HSX) {
+            c -= HSX;
+            r++;
+            o += p.W - HSX;
+        }
+    }
+    cp_async_commit();
+}
+// All staged rows of a run's first tile.
+template <int NP>
+__device__ __forceinline__ void stage_rows(const float* const (&src)[NP], const BlockPos& p, int y0,
+                                           float (&s)[NP][HSY][HSX + 2]) {
+    for (int i = threadIdx.x; i < HSY * HSX; i += 256) {
+        const int r = i / HSX, c = i % HSX;
+        const int y = y0 + r - RADIUS, x = p.x0 + c - RADIUS;
+        const bool in = x >= 0 && y >= 0 && x < p.W && y < p.H;
+        const long long o = p.plane + (long long)y * p.W + x;
+#pragma unroll
+        for (int m = 0; m < NP; m++) s[m][r][c] = in ? src[m][o] : 0.f;
+    }
 }
 
 __global__ void __launch_bounds__(256) dssim_forward_kernel(Views vw, const float* __restrict__ img,
@@ -75,113 +139,116 @@ __global__ void __launch_bounds__(256) dssim_forward_kernel(Views vw, const floa
                                                            float* __restrict__ dm12, float2* __restrict__ bsum,
                                                            long long blk_offset) {
     // rows of 44 floats: 16-byte aligned, for the vector reads of the row pass
-    __shared__ __align__(16) float s1[HSY][HSX + 2], s2[HSY][HSX + 2];
+    __shared__ __align__(16) float s[2][HSY][HSX + 2];
     __shared__ float h[5][HSY][TSX + 1];
     __shared__ float red[2][8];
     const BlockPos p = block_pos(vw);
-    for (int i = threadIdx.x; i < HSY * HSX; i += blockDim.x) {
-        const int r = i / HSX, c = i % HSX;
-        const int y = p.y0 + r - RADIUS, x = p.x0 + c - RADIUS;
-        const bool in = x >= 0 && y >= 0 && x < p.W && y < p.H;
-        const long long o = p.plane + (long long)y * p.W + x;
-        s1[r][c] = in ? img[o] : 0.f;
-        s2[r][c] = in ? tgt[o] : 0.f;
-    }
-    __syncthreads();
-    // row pass, four adjacent outputs per item: their 14 inputs come in four
-    // 16-byte reads instead of 44 scalar ones
-    for (int i = threadIdx.x; i < HSY * (TSX / 4); i += blockDim.x) {
-        const int r = i / (TSX / 4), c0 = 4 * (i % (TSX / 4));
-        float x1[16], x2[16];
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const float4 u = reinterpret_cast<const float4*>(&s1[r][c0])[q];
-            const float4 v = reinterpret_cast<const float4*>(&s2[r][c0])[q];
-            x1[4 * q] = u.x; x1[4 * q + 1] = u.y; x1[4 * q + 2] = u.z; x1[4 * q + 3] = u.w;
-            x2[4 * q] = v.x; x2[4 * q + 1] = v.y; x2[4 * q + 2] = v.z; x2[4 * q + 3] = v.w;
-        }
-#pragma unroll
-        for (int o = 0; o < 4; o++) {
-            float a = 0.f, b = 0.f, aa = 0.f, bb = 0.f, ab = 0.f;
-#pragma unroll
-            for (int k = 0; k < TAPS; k++) {
-                const float u = x1[o + k], v = x2[o + k], w = vw.w[k];
-                a += w * u;
-                b += w * v;
-                aa += w * u * u;
-                bb += w * v * v;
-                ab += w * u * v;
-            }
-            const int c = c0 + o;
-            h[0][r][c] = a; h[1][r][c] = b; h[2][r][c] = aa; h[3][r][c] = bb; h[4][r][c] = ab;
-        }
-    }
-    __syncthreads();
-    float ssim = 0.f, l1 = 0.f;
-    const int c = threadIdx.x % TSX;
-    // a thread's ROWS consecutive output rows share ROWS + TAPS - 1 staged rows:
-    // each staged value is read once and used for every output it reaches
-    const int r0 = (threadIdx.x / TSX) * ROWS;
-    float mv[ROWS][5];
-#pragma unroll
-    for (int q = 0; q < ROWS; q++)
-#pragma unroll
-        for (int i = 0; i < 5; i++) mv[q][i] = 0.f;
-#pragma unroll
-    for (int k = 0; k < ROWS + TAPS - 1; k++) {
-        float hv[5];
-#pragma unroll
-        for (int i = 0; i < 5; i++) hv[i] = h[i][r0 + k][c];
-#pragma unroll
-        for (int q = 0; q < ROWS; q++) {
-            const int t = k - q;
-            if (t >= 0 && t < TAPS) {
-                const float w = vw.w[t];
-#pragma unroll
-                for (int i = 0; i < 5; i++) mv[q][i] += w * hv[i];
-            }
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < ROWS; q++) {
-        const int r = r0 + q;
-        const float m1 = mv[q][0], m2 = mv[q][1], m11 = mv[q][2], m22 = mv[q][3], m12 = mv[q][4];
-        const int x = p.x0 + c, y = p.y0 + r;
-        if (x < p.W && y < p.H) {
-            const float t11 = m11 - m1 * m1, t22 = m22 - m2 * m2, t12 = m12 - m1 * m2;
-            const float a1 = 2.f * m1 * m2 + kC1, a2 = 2.f * t12 + kC2;
-            const float b1 = m1 * m1 + m2 * m2 + kC1, b2 = t11 + t22 + kC2;
-            // only the denominators b1, b2 (>= C1, C2 > 0) are inverted: S / a_k
-            // is written as a product, so a vanishing a2 = 2 cov + C2 is harmless
-            const float ib1 = rcp_approx(b1), ib2 = rcp_approx(b2), q = ib1 * ib2;
-            const float sv = a1 * a2 * q;
-            ssim += sv;
-            const long long o = p.plane + (long long)y * p.W + x;
-            dm1[o] = 2.f * (m2 * (a2 - a1) * q + m1 * sv * (ib2 - ib1));
-            dm11[o] = -sv * ib2;
-            dm12[o] = 2.f * a1 * q;
-            l1 += fabsf(s1[r + RADIUS][c + RADIUS] - s2[r + RADIUS][c + RADIUS]);
-        }
-    }
-    // block sums of SSIM and |I1 - I2|
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        ssim += __shfl_xor_sync(0xffffffffu, ssim, o);
-        l1 += __shfl_xor_sync(0xffffffffu, l1, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        red[0][threadIdx.x >> 5] = ssim;
-        red[1][threadIdx.x >> 5] = l1;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    const float* const src[2] = {img, tgt};
+    auto put_sums = [&](int ty) {
         float a = 0.f, b = 0.f;
         for (int i = 0; i < 8; i++) {
             a += red[0][i];
             b += red[1][i];
         }
-        bsum[blk_offset + blockIdx.x] = make_float2(a, b);
+        bsum[blk_offset + p.tile + (long long)ty * p.tiles_x] = make_float2(a, b);
+    };
+    stage_rows(src, p, p.ty0 * TSY, s);
+    int base = 0;  // ring position of the tile's first staged row
+    for (int ty = p.ty0; ty < p.ty1; ty++) {
+        const int y0 = ty * TSY, skip = ty == p.ty0 ? 0 : HALO;
+        cp_async_wait<0>();
+        __syncthreads();
+        if (ty > p.ty0 && threadIdx.x == 0) put_sums(ty - 1);
+        // row pass, four adjacent outputs per item: their 14 inputs come in four
+        // 16-byte reads instead of 44 scalar ones
+        for (int i = threadIdx.x; i < (HSY - skip) * (TSX / 4); i += 256) {
+            const int r = i / (TSX / 4), c0 = 4 * (i % (TSX / 4)), hr = ring(base + skip + r);
+            float x1[16], x2[16];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const float4 u = reinterpret_cast<const float4*>(&s[0][r][c0])[q];
+                const float4 v = reinterpret_cast<const float4*>(&s[1][r][c0])[q];
+                x1[4 * q] = u.x; x1[4 * q + 1] = u.y; x1[4 * q + 2] = u.z; x1[4 * q + 3] = u.w;
+                x2[4 * q] = v.x; x2[4 * q + 1] = v.y; x2[4 * q + 2] = v.z; x2[4 * q + 3] = v.w;
+            }
+#pragma unroll
+            for (int o = 0; o < 4; o++) {
+                float a = 0.f, b = 0.f, aa = 0.f, bb = 0.f, ab = 0.f;
+#pragma unroll
+                for (int k = 0; k < TAPS; k++) {
+                    const float u = x1[o + k], v = x2[o + k], w = vw.w[k];
+                    a += w * u;
+                    b += w * v;
+                    aa += w * u * u;
+                    bb += w * v * v;
+                    ab += w * u * v;
+                }
+                const int c = c0 + o;
+                h[0][hr][c] = a; h[1][hr][c] = b; h[2][hr][c] = aa; h[3][hr][c] = bb; h[4][hr][c] = ab;
+            }
+        }
+        __syncthreads();
+        if (ty + 1 < p.ty1) fetch_rows(src, p, y0, s);  // the row pass is done with them
+        float ssim = 0.f, l1 = 0.f;
+        const int c = threadIdx.x % TSX;
+        // a thread's ROWS consecutive output rows share ROWS + TAPS - 1 staged rows:
+        // each staged value is read once and used for every output it reaches
+        const int r0 = (threadIdx.x / TSX) * ROWS;
+        float mv[ROWS][5];
+#pragma unroll
+        for (int q = 0; q < ROWS; q++)
+#pragma unroll
+            for (int i = 0; i < 5; i++) mv[q][i] = 0.f;
+#pragma unroll
+        for (int k = 0; k < ROWS + TAPS - 1; k++) {
+            float hv[5];
+#pragma unroll
+            for (int i = 0; i < 5; i++) hv[i] = h[i][ring(base + r0 + k)][c];
+#pragma unroll
+            for (int q = 0; q < ROWS; q++) {
+                const int t = k - q;
+                if (t >= 0 && t < TAPS) {
+                    const float w = vw.w[t];
+#pragma unroll
+                    for (int i = 0; i < 5; i++) mv[q][i] += w * hv[i];
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < ROWS; q++) {
+            const int r = r0 + q;
+            const float m1 = mv[q][0], m2 = mv[q][1], m11 = mv[q][2], m22 = mv[q][3], m12 = mv[q][4];
+            const int x = p.x0 + c, y = y0 + r;
+            if (x < p.W && y < p.H) {
+                const float t11 = m11 - m1 * m1, t22 = m22 - m2 * m2, t12 = m12 - m1 * m2;
+                const float a1 = 2.f * m1 * m2 + kC1, a2 = 2.f * t12 + kC2;
+                const float b1 = m1 * m1 + m2 * m2 + kC1, b2 = t11 + t22 + kC2;
+                // only the denominators b1, b2 (>= C1, C2 > 0) are inverted: S / a_k
+                // is written as a product, so a vanishing a2 = 2 cov + C2 is harmless
+                const float ib1 = rcp_approx(b1), ib2 = rcp_approx(b2), q = ib1 * ib2;
+                const float sv = a1 * a2 * q;
+                ssim += sv;
+                const long long o = p.plane + (long long)y * p.W + x;
+                dm1[o] = 2.f * (m2 * (a2 - a1) * q + m1 * sv * (ib2 - ib1));
+                dm11[o] = -sv * ib2;
+                dm12[o] = 2.f * a1 * q;
+                l1 += fabsf(img[o] - tgt[o]);
+            }
+        }
+        // block sums of SSIM and |I1 - I2|
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            ssim += __shfl_xor_sync(0xffffffffu, ssim, o);
+            l1 += __shfl_xor_sync(0xffffffffu, l1, o);
+        }
+        if ((threadIdx.x & 31) == 0) {
+            red[0][threadIdx.x >> 5] = ssim;
+            red[1][threadIdx.x >> 5] = l1;
+        }
+        base = ring(base + TSY);
     }
+    __syncthreads();
+    if (threadIdx.x == 0) put_sums(p.ty1 - 1);
 }
 
 __global__ void __launch_bounds__(256) dssim_backward_kernel(Views vw, const float* __restrict__ img,
@@ -193,73 +260,74 @@ __global__ void __launch_bounds__(256) dssim_backward_kernel(Views vw, const flo
     __shared__ __align__(16) float s[3][HSY][HSX + 2];
     __shared__ float h[3][HSY][TSX + 1];
     const BlockPos p = block_pos(vw);
-    for (int i = threadIdx.x; i < HSY * HSX; i += blockDim.x) {
-        const int r = i / HSX, c = i % HSX;
-        const int y = p.y0 + r - RADIUS, x = p.x0 + c - RADIUS;
-        const bool in = x >= 0 && y >= 0 && x < p.W && y < p.H;
-        const long long o = p.plane + (long long)y * p.W + x;
-        s[0][r][c] = in ? dm1[o] : 0.f;
-        s[1][r][c] = in ? dm11[o] : 0.f;
-        s[2][r][c] = in ? dm12[o] : 0.f;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < HSY * (TSX / 4); i += blockDim.x) {
-        const int r = i / (TSX / 4), c0 = 4 * (i % (TSX / 4));
-        float x[3][16];
+    const float* const src[3] = {dm1, dm11, dm12};
+    stage_rows(src, p, p.ty0 * TSY, s);
+    int base = 0;
+    for (int ty = p.ty0; ty < p.ty1; ty++) {
+        const int y0 = ty * TSY, skip = ty == p.ty0 ? 0 : HALO;
+        cp_async_wait<0>();
+        __syncthreads();
+        for (int i = threadIdx.x; i < (HSY - skip) * (TSX / 4); i += 256) {
+            const int r = i / (TSX / 4), c0 = 4 * (i % (TSX / 4)), hr = ring(base + skip + r);
+            float x[3][16];
 #pragma unroll
-        for (int m = 0; m < 3; m++)
+            for (int m = 0; m < 3; m++)
 #pragma unroll
-            for (int q = 0; q < 4; q++) {
-                const float4 u = reinterpret_cast<const float4*>(&s[m][r][c0])[q];
-                x[m][4 * q] = u.x; x[m][4 * q + 1] = u.y; x[m][4 * q + 2] = u.z; x[m][4 * q + 3] = u.w;
+                for (int q = 0; q < 4; q++) {
+                    const float4 u = reinterpret_cast<const float4*>(&s[m][r][c0])[q];
+                    x[m][4 * q] = u.x; x[m][4 * q + 1] = u.y; x[m][4 * q + 2] = u.z; x[m][4 * q + 3] = u.w;
+                }
+#pragma unroll
+            for (int o = 0; o < 4; o++) {
+                float a = 0.f, b = 0.f, d = 0.f;
+#pragma unroll
+                for (int k = 0; k < TAPS; k++) {
+                    const float w = vw.w[k];
+                    a += w * x[0][o + k];
+                    b += w * x[1][o + k];
+                    d += w * x[2][o + k];
+                }
+                const int c = c0 + o;
+                h[0][hr][c] = a; h[1][hr][c] = b; h[2][hr][c] = d;
             }
-#pragma unroll
-        for (int o = 0; o < 4; o++) {
-            float a = 0.f, b = 0.f, d = 0.f;
-#pragma unroll
-            for (int k = 0; k < TAPS; k++) {
-                const float w = vw.w[k];
-                a += w * x[0][o + k];
-                b += w * x[1][o + k];
-                d += w * x[2][o + k];
-            }
-            const int c = c0 + o;
-            h[0][r][c] = a; h[1][r][c] = b; h[2][r][c] = d;
         }
-    }
-    __syncthreads();
-    const int c = threadIdx.x % TSX;
-    const float inv_n = 1.f / (3.f * (float)p.H * (float)p.W);
-    const int r0 = (threadIdx.x / TSX) * ROWS;
-    float bv[ROWS][3];
+        __syncthreads();
+        if (ty + 1 < p.ty1) fetch_rows(src, p, y0, s);
+        const int c = threadIdx.x % TSX;
+        const float inv_n = 1.f / (3.f * (float)p.H * (float)p.W);
+        const int r0 = (threadIdx.x / TSX) * ROWS;
+        float bv[ROWS][3];
 #pragma unroll
-    for (int q = 0; q < ROWS; q++) bv[q][0] = bv[q][1] = bv[q][2] = 0.f;
+        for (int q = 0; q < ROWS; q++) bv[q][0] = bv[q][1] = bv[q][2] = 0.f;
 #pragma unroll
-    for (int k = 0; k < ROWS + TAPS - 1; k++) {
-        const float h0 = h[0][r0 + k][c], h1 = h[1][r0 + k][c], h2 = h[2][r0 + k][c];
+        for (int k = 0; k < ROWS + TAPS - 1; k++) {
+            const int hr = ring(base + r0 + k);
+            const float h0 = h[0][hr][c], h1 = h[1][hr][c], h2 = h[2][hr][c];
+#pragma unroll
+            for (int q = 0; q < ROWS; q++) {
+                const int t = k - q;
+                if (t >= 0 && t < TAPS) {
+                    const float w = vw.w[t];
+                    bv[q][0] += w * h0;
+                    bv[q][1] += w * h1;
+                    bv[q][2] += w * h2;
+                }
+            }
+        }
 #pragma unroll
         for (int q = 0; q < ROWS; q++) {
-            const int t = k - q;
-            if (t >= 0 && t < TAPS) {
-                const float w = vw.w[t];
-                bv[q][0] += w * h0;
-                bv[q][1] += w * h1;
-                bv[q][2] += w * h2;
-            }
+            const int r = r0 + q;
+            const int x = p.x0 + c, y = y0 + r;
+            if (x >= p.W || y >= p.H) continue;
+            const float B1 = bv[q][0], B11 = bv[q][1], B12 = bv[q][2];
+            const long long o = p.plane + (long long)y * p.W + x;
+            const float i1 = img[o], i2 = tgt[o];
+            const float diff = i1 - i2;
+            const float sgn = diff > 0.f ? 1.f : (diff < 0.f ? -1.f : 0.f);
+            const float dssim = B1 + 2.f * i1 * B11 + i2 * B12;
+            dimg[o] = inv_views * inv_n * ((1.f - lambda) * sgn - lambda * dssim);
         }
-    }
-#pragma unroll
-    for (int q = 0; q < ROWS; q++) {
-        const int r = r0 + q;
-        const int x = p.x0 + c, y = p.y0 + r;
-        if (x >= p.W || y >= p.H) continue;
-        const float B1 = bv[q][0], B11 = bv[q][1], B12 = bv[q][2];
-        const long long o = p.plane + (long long)y * p.W + x;
-        const float i1 = img[o], i2 = tgt[o];
-        const float diff = i1 - i2;
-        const float sgn = diff > 0.f ? 1.f : (diff < 0.f ? -1.f : 0.f);
-        const float dssim = B1 + 2.f * i1 * B11 + i2 * B12;
-        dimg[o] = inv_views * inv_n * ((1.f - lambda) * sgn - lambda * dssim);
+        base = ring(base + TSY);
     }
 }
 
@@ -307,6 +375,20 @@ Views make_views(const int* hw, int first, int count) {
         blk += 3LL * vw.tiles_x[i] * ((H + TSY - 1) / TSY);
     }
     vw.blk[count] = blk;
+    // Tiles per block: as many as leave three blocks for each of the 608 that are
+    // resident, up to 8, in runs of even length (eight 1264 x 832 views, 13 tiles
+    // by that count: 643 us with up to 8 or 13, 684 with up to 4; one such view
+    // has runs of one tile).
+    const long long most = blk / (3 * 608);
+    const int run = most < 1 ? 1 : most > 8 ? 8 : (int)most;
+    long long cta = 0;
+    for (int i = 0; i < count; i++) {
+        const int tiles_y = (vw.H[i] + TSY - 1) / TSY, runs = (tiles_y + run - 1) / run;
+        vw.run[i] = (tiles_y + runs - 1) / runs;
+        vw.cta[i] = cta;
+        cta += 3LL * vw.tiles_x[i] * ((tiles_y + vw.run[i] - 1) / vw.run[i]);
+    }
+    vw.cta[count] = cta;
     // 1D Gaussian taps, normalised to sum 1 (double on the host)
     double tap[TAPS], sum = 0.0;
     for (int k = 0; k < TAPS; k++) {
@@ -351,12 +433,12 @@ void launch_dssim(const float* img, const float* target, const int* hw, int V, f
     for (int first = 0; first < V; first += kMaxViews) {
         const int count = V - first < kMaxViews ? V - first : kMaxViews;
         const Views vw = make_views(hw, first, count);
-        const long long nb = vw.blk[count];
+        const long long nb = vw.blk[count], ctas = vw.cta[count];
         if (nb > 0) {
-            dssim_forward_kernel<<<(unsigned)nb, 256, 0, s>>>(vw, img, target, dm1, dm11, dm12, bsum, blk_offset);
+            dssim_forward_kernel<<<(unsigned)ctas, 256, 0, s>>>(vw, img, target, dm1, dm11, dm12, bsum, blk_offset);
             note_launches(1);
             if (dimg)
-                dssim_backward_kernel<<<(unsigned)nb, 256, 0, s>>>(vw, img, target, dm1, dm11, dm12, lambda,
+                dssim_backward_kernel<<<(unsigned)ctas, 256, 0, s>>>(vw, img, target, dm1, dm11, dm12, lambda,
                                                                    1.f / (float)V, dimg);
             if (dimg) note_launches(1);
         }
