@@ -761,9 +761,11 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
                     P0 += nd;
                     P1 += ny;
                     P2 = fmaf(ny, dy, P2);
-                    Sx += nx;
-                    Sxx = fmaf(nx, dx, Sxx);
-                    Sxy = fmaf(nx, dy, Sxy);
+                    if (SAMPLED) {
+                        Sx += nx;
+                        Sxx = fmaf(nx, dx, Sxx);
+                        Sxy = fmaf(nx, dy, Sxy);
+                    }
                     E = fmaf(fabsf(nd), sqrt_approx(ax * ax + ay * ay), E);
                 }
             };
@@ -781,6 +783,16 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
                 for (int h = 0; h < 2; h++) one_pixel(2 * p + h, f[h], y[h], a0[h], a1[h], a2[h], t[h], u[h]);
                 T[p] = pack2(t[0], t[1]);
                 V[p] = pack2(u[0], u[1]);
+            }
+            if (!SAMPLED) {  // one column per lane: the products of the sums, as in plain_step
+                float f0, f1;
+                unpack2(FX[0], f0, f1);
+                const float dx0 = f0 + em.x;
+                if (fabsf(dx0) <= radius) {
+                    Sx = dx0 * P0;
+                    Sxx = dx0 * dx0 * P0;
+                    Sxy = dx0 * P1;
+                }
             }
             hand_over(u, Sx, P1, P0, R, Gn, B, E, Sxx, Sxy, P2);
         };

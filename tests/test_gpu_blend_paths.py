@@ -147,3 +147,28 @@ def test_small_renders_choose_pixels_per_lane_freely(cuda_lib, tile, size):
     for k in PARAMS:  # the same kernel on the same state: only the order of its atomics may differ
         a, b = runs[0][1][k].double(), runs[1][1][k].double()
         assert float((a - b).norm()) <= 1e-5 * float(b.norm()) + 1e-12
+
+
+@pytest.mark.parametrize("tile,size", [((16, 16), (70, 53)), ((32, 64), (96, 128)), ((8, 8), (64, 64))])
+def test_both_backward_paths_round_alike(cuda_lib, tile, size):
+    """An enormous gradient on pixels that no Gaussian reaches sends their strips to
+    the general path: the conic gradients (summed in double precision) keep every bit."""
+    scene = synth.make_scene(150, 1, seed=3)
+    scene.log_scales[:] -= np.float32(0.5)
+    cams = synth.make_cameras([size], radius=5.0, seed=4)
+    params = scene_to_device(scene)
+    sc = cuda_lib.make_scene(params, scene.sh_degree)
+    rz = cuda_lib.Rasterizer(cams, tile=tile)
+    img = rz.forward(sc)
+    idle = rz.records()["n_contrib"].flatten() == 0
+    assert 0 < int(idle.sum()) < idle.numel()
+    dimg = torch.randn(img.numel(), device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    dimg[idle.repeat(3)] = 0.0
+    runs = []
+    for value in (0.0, 1e26):
+        d = torch.where(idle.repeat(3), torch.full_like(dimg, value), dimg).reshape(img.shape)
+        grads = grads_like(params)
+        rz.backward(sc, d.contiguous(), grads)
+        runs.append(grads)
+    for k in ("log_scales", "quats"):
+        assert torch.equal(runs[0][k], runs[1][k]), k
