@@ -239,7 +239,7 @@ mvgs_status make_plan(long long n, const mvgs_camera* cams, int V, const mvgs_co
     P.w_bins = w.take(R * sizeof(uint32_t));
     P.w_desc = w.take(R * sizeof(unsigned long long));
     P.w_bins_by_depth = w.take(R * sizeof(uint32_t));
-    P.w_bin_off = w.take((R + 1) * sizeof(unsigned long long));
+    P.w_bin_off = w.take((R + 1) * sizeof(uint32_t));
     P.w_keys_a = w.take(K * sizeof(uint32_t));
     P.w_keys_b = w.take(K * sizeof(uint32_t));
     P.w_vals_a = w.take(K * sizeof(uint32_t));
@@ -557,10 +557,12 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
                        at<uint32_t>(workspace, P.w_ids_b), order, Rc, depth_bits, at<void>(workspace, P.w_radix), s,
                        bins, bins_by_depth);
     }
-    unsigned long long* bin_off = at<unsigned long long>(workspace, P.w_bin_off);
+    // fewer entries than keys, so below 2^32 (a capturable call with more wraps,
+    // stays within the capacity and places nothing)
+    uint32_t* bin_off = at<uint32_t>(workspace, P.w_bin_off);
     {
         StageTimer t(MVGS_STAGE_SCAN_TILES, s);
-        scan_u32_to_u64_count(bins_by_depth, bin_off, Rc, at<void>(workspace, P.w_scan), s);
+        scan_u32(bins_by_depth, bin_off, Rc, at<void>(workspace, P.w_scan), s);
     }
     uint32_t* sorted = at<uint32_t>(state, L.off_sorted_records);
     long long* ranges = at<long long>(state, L.off_tile_ranges);

@@ -93,8 +93,8 @@ void scan_i32_to_i64(const int* in, long long* out, uint64_t n, void* tmp, cudaS
 // scans in[i] & mask
 void scan_masked_i32_to_i64(const int* in, int mask, long long* out, uint64_t n, void* tmp, cudaStream_t s);
 void scan_u32_to_u64(const uint32_t* in, unsigned long long* out, uint64_t n, void* tmp, cudaStream_t s);
-// (n may be a device count)
-void scan_u32_to_u64_count(const uint32_t* in, unsigned long long* out, Count n, void* tmp, cudaStream_t s);
+// (n may be a device count; the sums wrap)
+void scan_u32(const uint32_t* in, uint32_t* out, Count n, void* tmp, cudaStream_t s);
 
 size_t radix_temp_bytes(uint64_t n);
 // Stable LSD sort of the ids 0 .. n by key bits [0, bits); sub (optional): a
@@ -114,7 +114,7 @@ void radix_sort_ids(const uint32_t* keys, const unsigned long long* sub, uint32_
 // (pack_tile_desc, record order).  keys_a/b and vals_a/b are scratch of S_cap
 // entries each.
 size_t tile_lists_temp_bytes(uint64_t S, long long bins, long long tiles);
-void tile_lists(const uint32_t* order, const unsigned long long* bin_off, Count R, Count S, Count K,
+void tile_lists(const uint32_t* order, const uint32_t* bin_off, Count R, Count S, Count K,
                 const unsigned long long* desc, const DevCam* cams, int V, long long bins, long long tiles,
                 uint32_t* keys_a, uint32_t* vals_a, uint32_t* keys_b, uint32_t* vals_b, uint32_t* sorted,
                 long long* ranges, uint64_t S_cap, void* tmp, void* radix_tmp, cudaStream_t s);
