@@ -166,6 +166,13 @@ __device__ __forceinline__ float sig_at(const float* S, int i, int j) {
     return lo == 0 ? S[hi] : (lo == 1 ? S[2 + hi] : S[5]);
 }
 
+// v / t for a tile side, a power of two: by its exact reciprocal.  Four divisions
+// per (Gaussian, view) were a tenth of the participation pass: 3M x 8 views 201
+// -> 177 us.
+__device__ __forceinline__ float over_side(float v, int t) {
+    return v * __uint_as_float((254u << 23) - __float_as_uint((float)t));
+}
+
 // Projects one Gaussian into one view; false if culled (behind the near
 // plane, degenerate covariance, or no tile of the image within its radius).
 __device__ __forceinline__ bool project(const Gauss& G, const ProjCam& cam, int tw, int th, Proj& P) {
@@ -224,10 +231,10 @@ __device__ __forceinline__ bool project(const Gauss& G, const ProjCam& cam, int 
     const float r = (float)P.radius;
     const float hx = fminf(r, sqrtf(ext * P.a) + 1e-2f), hy = fminf(r, sqrtf(ext * P.c) + 1e-2f);
     // floor on both ends keeps at least half a pixel of slack
-    const float x0 = fminf(fmaxf(floorf((P.xy.x - hx) / tw), 0.f), (float)cam.tiles_x);
-    const float x1 = fminf(fmaxf(floorf((P.xy.x + hx) / tw) + 1.f, 0.f), (float)cam.tiles_x);
-    const float y0 = fminf(fmaxf(floorf((P.xy.y - hy) / th), 0.f), (float)cam.tiles_y);
-    const float y1 = fminf(fmaxf(floorf((P.xy.y + hy) / th) + 1.f, 0.f), (float)cam.tiles_y);
+    const float x0 = fminf(fmaxf(floorf(over_side(P.xy.x - hx, tw)), 0.f), (float)cam.tiles_x);
+    const float x1 = fminf(fmaxf(floorf(over_side(P.xy.x + hx, tw)) + 1.f, 0.f), (float)cam.tiles_x);
+    const float y0 = fminf(fmaxf(floorf(over_side(P.xy.y - hy, th)), 0.f), (float)cam.tiles_y);
+    const float y1 = fminf(fmaxf(floorf(over_side(P.xy.y + hy, th)) + 1.f, 0.f), (float)cam.tiles_y);
     P.rect = make_short4((short)x0, (short)y0, (short)x1, (short)y1);
     return x0 < x1 && y0 < y1;
 }

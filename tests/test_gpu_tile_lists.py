@@ -62,3 +62,14 @@ def test_lists_with_more_bins_than_the_key_has_room_for(cuda_lib):
                          np.full(V, 0.2, f32))
     rz = _check(cuda_lib, scene, cams, (8, 8))
     assert int(rz.layout.tiles) == V * 4095 and int(rz.needed.keys) > V * n * 8
+
+
+@pytest.mark.parametrize("tile", [(8, 8), (16, 8), (32, 32), (8, 64), (32, 64)])
+def test_rectangles_for_any_tile(cuda_lib, tile):
+    """A rectangle differs from the float64 one only where an edge falls on the rounding."""
+    scene, cams = synth.make_scene(3000, 0, seed=2), synth.make_cameras([(301, 203), (97, 390)], radius=3.0, seed=3)
+    rz, _, _, _ = gpu_forward(cuda_lib, scene, cams, tile)
+    D, P = dense_records(rz, scene.n, cams.V), oracle.project(scene, cams, tile)
+    vis = (D["valid"] != 0) & (P["valid"] != 0)
+    assert vis.sum() > 2000
+    assert (D["rect"][vis] != P["rect"][vis]).any(axis=1).mean() < 1e-3
