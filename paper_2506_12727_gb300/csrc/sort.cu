@@ -26,6 +26,13 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
+// Blocks of a launch that is sized by a capacity (capturable mode): they stride
+// over what there is.  The tile lists' entries are a tenth of the key capacity
+// that bounds them: at 3M Gaussians x 8 views the blocks without entries cost a
+// captured step 0.64 ms (15.47 -> 14.83).  Kernels that the loop makes slower are
+// variants of their own (STRIDE).
+constexpr uint64_t GRID_CAP = 152 * 32;
+
 // ---------------------------------------------------------------------------
 // exclusive scan (reduce, spine, downsweep; fewer launches for fewer blocks)
 // ---------------------------------------------------------------------------
@@ -223,9 +230,12 @@ constexpr uint64_t RS_DIRECT = 64;
 struct RadixTable {
     uint32_t* counts;
     uint32_t* totals;
-    uint32_t nblocks;
     bool direct;
 };
+
+// Blocks of n keys.  A launch sized by a capacity has at most GRID_CAP blocks,
+// which go on to further ones of the actual count.
+__device__ __forceinline__ uint32_t rs_blocks(uint64_t n) { return (uint32_t)((n + RS_TILE - 1) / RS_TILE); }
 
 struct RankSmem {
     uint32_t whist[RS_WARPS * 256];  // per-warp digit counts, then per-warp prefixes
@@ -237,43 +247,51 @@ struct RankSmem {
 };
 
 // Keys of the thread's digit in all blocks and in the blocks before.
-__device__ __forceinline__ void digit_counts(const RadixTable& tab, uint32_t& tot, uint32_t& pre) {
+__device__ __forceinline__ void digit_counts(const RadixTable& tab, uint32_t nblocks, uint32_t block, uint32_t& tot,
+                                             uint32_t& pre) {
     if (tab.direct) {
         tot = pre = 0;
 #pragma unroll 8
-        for (uint32_t b = 0; b < tab.nblocks; b++) {
+        for (uint32_t b = 0; b < nblocks; b++) {
             const uint32_t c = tab.counts[b * 256 + threadIdx.x];
-            if (b < blockIdx.x) pre += c;
+            if (b < block) pre += c;
             tot += c;
         }
     } else {
-        pre = tab.counts[(uint64_t)threadIdx.x * tab.nblocks + blockIdx.x];
+        pre = tab.counts[(uint64_t)threadIdx.x * nblocks + block];
         tot = tab.totals[threadIdx.x];
     }
 }
 
 // Per-block digit histogram.  sub (optional): subtracted from every key.
+template <bool STRIDE>
 __global__ void __launch_bounds__(RS_THREADS) rs_upsweep(const uint32_t* __restrict__ keys, Count cn, int shift,
                                                         const unsigned long long* __restrict__ sub, RadixTable tab) {
     __shared__ uint32_t hist[RS_WARPS * 256];
     const uint64_t n = cn.get();
+    const uint32_t nblocks = rs_blocks(n);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint64_t base = (uint64_t)blockIdx.x * RS_TILE + warp * RS_SEG + lane;
-    uint32_t k[RS_ITEMS];
-#pragma unroll
-    for (int j = 0; j < RS_ITEMS; j++) k[j] = base + (uint64_t)j * 32 < n ? keys[base + (uint64_t)j * 32] : 0u;
     const uint32_t k0 = sub ? (uint32_t)*sub : 0u;
-    for (int i = threadIdx.x; i < RS_WARPS * 256; i += RS_THREADS) hist[i] = 0;
-    __syncthreads();
+    uint32_t block = blockIdx.x;
+    if (block >= nblocks) return;
+    do {
+        const uint64_t base = (uint64_t)block * RS_TILE + warp * RS_SEG + lane;
+        uint32_t k[RS_ITEMS];
 #pragma unroll
-    for (int j = 0; j < RS_ITEMS; j++)
-        if (base + (uint64_t)j * 32 < n) atomicAdd(&hist[warp * 256 + (((k[j] - k0) >> shift) & 0xffu)], 1u);
-    __syncthreads();
-    uint32_t sum = 0;
+        for (int j = 0; j < RS_ITEMS; j++) k[j] = base + (uint64_t)j * 32 < n ? keys[base + (uint64_t)j * 32] : 0u;
+        for (int i = threadIdx.x; i < RS_WARPS * 256; i += RS_THREADS) hist[i] = 0;
+        __syncthreads();
 #pragma unroll
-    for (int w = 0; w < RS_WARPS; w++) sum += hist[w * 256 + threadIdx.x];
-    if (tab.direct) tab.counts[(uint64_t)blockIdx.x * 256 + threadIdx.x] = sum;
-    else tab.counts[(uint64_t)threadIdx.x * tab.nblocks + blockIdx.x] = sum;
+        for (int j = 0; j < RS_ITEMS; j++)
+            if (base + (uint64_t)j * 32 < n) atomicAdd(&hist[warp * 256 + (((k[j] - k0) >> shift) & 0xffu)], 1u);
+        __syncthreads();
+        uint32_t sum = 0;
+#pragma unroll
+        for (int w = 0; w < RS_WARPS; w++) sum += hist[w * 256 + threadIdx.x];
+        if (tab.direct) tab.counts[(uint64_t)block * 256 + threadIdx.x] = sum;
+        else tab.counts[(uint64_t)threadIdx.x * nblocks + block] = sum;
+        if (STRIDE) __syncthreads();
+    } while (STRIDE && (block += gridDim.x) < nblocks);
 }
 
 // The same table for a pass whose digits take at most 32 values (few bins, or
@@ -289,38 +307,43 @@ __global__ void __launch_bounds__(RS_THREADS) rs_upsweep_narrow(const uint32_t* 
     const uint64_t n = cn.get();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t* c = cnt[warp];
-    for (int i = lane; i < 32 * 32; i += 32) c[i] = 0;
-    __syncwarp();
-    const uint64_t base = (uint64_t)blockIdx.x * RS_TILE + warp * RS_SEG + lane;
+    const uint32_t nblocks = rs_blocks(n);
+    for (uint32_t block = blockIdx.x; block < nblocks; block += gridDim.x) {
+        for (int i = lane; i < 32 * 32; i += 32) c[i] = 0;
+        __syncwarp();
+        const uint64_t base = (uint64_t)block * RS_TILE + warp * RS_SEG + lane;
 #pragma unroll
-    for (int j = 0; j < RS_ITEMS; j++) {
-        const uint64_t idx = base + (uint64_t)j * 32;
-        if (idx < n) c[((keys[idx] >> shift) & mask) * 32 + lane] += 1u;
-    }
-    __syncwarp();
-    // lane d sums digit d's column, starting at a different lane per digit
-    uint32_t sum = 0;
+        for (int j = 0; j < RS_ITEMS; j++) {
+            const uint64_t idx = base + (uint64_t)j * 32;
+            if (idx < n) c[((keys[idx] >> shift) & mask) * 32 + lane] += 1u;
+        }
+        __syncwarp();
+        // lane d sums digit d's column, starting at a different lane per digit
+        uint32_t sum = 0;
 #pragma unroll 8
-    for (int i = 0; i < 32; i++) sum += c[lane * 32 + ((i + lane) & 31)];
-    wsum[warp][lane] = sum;
-    __syncthreads();
-    uint32_t total = 0;
-    if (threadIdx.x < 32) {
+        for (int i = 0; i < 32; i++) sum += c[lane * 32 + ((i + lane) & 31)];
+        wsum[warp][lane] = sum;
+        __syncthreads();
+        uint32_t total = 0;
+        if (threadIdx.x < 32) {
 #pragma unroll
-        for (int w = 0; w < RS_WARPS; w++) total += wsum[w][threadIdx.x];
+            for (int w = 0; w < RS_WARPS; w++) total += wsum[w][threadIdx.x];
+        }
+        if (tab.direct) tab.counts[(uint64_t)block * 256 + threadIdx.x] = total;
+        else tab.counts[(uint64_t)threadIdx.x * nblocks + block] = total;
+        __syncthreads();
     }
-    if (tab.direct) tab.counts[(uint64_t)blockIdx.x * 256 + threadIdx.x] = total;
-    else tab.counts[(uint64_t)threadIdx.x * tab.nblocks + blockIdx.x] = total;
 }
 
 // One block per digit: its counts become the number of its keys in the blocks
 // before, and their sum its total.  A warp takes a stretch of the blocks.
-__global__ void __launch_bounds__(RS_THREADS) rs_scan_kernel(RadixTable tab) {
+__global__ void __launch_bounds__(RS_THREADS) rs_scan_kernel(RadixTable tab, Count cn) {
     __shared__ uint32_t buf[33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t* row = tab.counts + (uint64_t)blockIdx.x * tab.nblocks;
-    const uint32_t per = (tab.nblocks + RS_THREADS - 1) / RS_THREADS * 32;
-    const uint32_t r0 = min(warp * per, tab.nblocks), r1 = min(r0 + per, tab.nblocks);
+    const uint32_t nblocks = rs_blocks(cn.get());
+    uint32_t* row = tab.counts + (uint64_t)blockIdx.x * nblocks;
+    const uint32_t per = (nblocks + RS_THREADS - 1) / RS_THREADS * 32;
+    const uint32_t r0 = min(warp * per, nblocks), r1 = min(r0 + per, nblocks);
     uint32_t sum = 0;
 #pragma unroll 4
     for (uint32_t r = r0 + lane; r < r1; r += 32) sum += row[r];
@@ -352,8 +375,9 @@ __global__ void __launch_bounds__(RS_THREADS) rs_scan_kernel(RadixTable tab) {
 // the keys' positions (an identity permutation, generated instead of read).
 // sub: subtracted from every key (the keys written are the differences).
 // gout != nullptr: also writes gout[pos] = gsrc[value] (a per-element array
-// carried into sorted order).
-template <bool WRITE_KEYS, int NB>
+// carried into sorted order).  STRIDE: a launch sized by a capacity; a variant of
+// its own because the loop costs registers that spill.
+template <bool WRITE_KEYS, int NB, bool STRIDE>
 __global__ void __launch_bounds__(RS_THREADS, 3) rs_downsweep(const uint32_t* __restrict__ kin,
                                                              const uint32_t* __restrict__ vin,
                                                              uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
@@ -365,77 +389,82 @@ __global__ void __launch_bounds__(RS_THREADS, 3) rs_downsweep(const uint32_t* __
     const uint64_t n = cn.get();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lt = (1u << lane) - 1u;
-    const uint64_t block0 = (uint64_t)blockIdx.x * RS_TILE;
-    if (block0 >= n) return;  // a block past the keys (capturable mode)
-    const int here = (int)(n - block0 < (uint64_t)RS_TILE ? n - block0 : (uint64_t)RS_TILE);
-    const int local0 = warp * RS_SEG + lane;
-    for (int i = threadIdx.x; i < RS_WARPS * 256; i += RS_THREADS) sm.whist[i] = 0;
-    kin += block0;
-    uint32_t k[RS_ITEMS];
+    const uint32_t nblocks = rs_blocks(n);
     const uint32_t k0 = sub ? (uint32_t)*sub : 0u;
+    uint32_t block = blockIdx.x;
+    if (block >= nblocks) return;
+    do {
+        const uint64_t block0 = (uint64_t)block * RS_TILE;
+        const int here = (int)(n - block0 < (uint64_t)RS_TILE ? n - block0 : (uint64_t)RS_TILE);
+        const int local0 = warp * RS_SEG + lane;
+        for (int i = threadIdx.x; i < RS_WARPS * 256; i += RS_THREADS) sm.whist[i] = 0;
+        const uint32_t* in = kin + block0;
+        uint32_t k[RS_ITEMS];
 #pragma unroll
-    for (int j = 0; j < RS_ITEMS; j++) k[j] = (local0 + j * 32 < here ? kin[local0 + j * 32] : 0u) - k0;
-    uint32_t tot, pre;
-    digit_counts(tab, tot, pre);
-    __syncthreads();
-    uint32_t* wh = sm.whist + warp * 256;
-    uint32_t lr[RS_ITEMS];
+        for (int j = 0; j < RS_ITEMS; j++) k[j] = (local0 + j * 32 < here ? in[local0 + j * 32] : 0u) - k0;
+        uint32_t tot, pre;
+        digit_counts(tab, nblocks, block, tot, pre);
+        __syncthreads();
+        uint32_t* wh = sm.whist + warp * 256;
+        uint32_t lr[RS_ITEMS];
 #pragma unroll
-    for (int j = 0; j < RS_ITEMS; j++) {
-        const bool ok = local0 + j * 32 < here;
-        const uint32_t d = (k[j] >> shift) & 0xffu;
-        uint32_t peers = __ballot_sync(kFull, ok);
-#pragma unroll
-        for (int b = 0; b < NB; b++) {  // digit bits above NB are zero in this pass
-            const uint32_t bit = (d >> b) & 1u;
-            const uint32_t bb = __ballot_sync(kFull, bit);
-            peers &= bit ? bb : ~bb;
-        }
-        const uint32_t rank = __popc(peers & lt);
-        const uint32_t before = wh[d];
-        __syncwarp();
-        if (ok && rank == 0) wh[d] = before + __popc(peers);
-        __syncwarp();
-        lr[j] = before + rank;
-    }
-    uint32_t vv[RS_ITEMS];
-#pragma unroll
-    for (int j = 0; j < RS_ITEMS; j++)
-        vv[j] = !vin ? (uint32_t)block0 + local0 + j * 32 : local0 + j * 32 < here ? vin[block0 + local0 + j * 32] : 0u;
-    __syncthreads();
-    uint32_t run = 0;
-#pragma unroll
-    for (int w = 0; w < RS_WARPS; w++) {
-        const uint32_t c = sm.whist[w * 256 + threadIdx.x];
-        sm.whist[w * 256 + threadIdx.x] = run;
-        run += c;
-    }
-    // both prefixes over the digits in one scan: of the totals (high words) and
-    // of the block's counts
-    unsigned long long all;
-    const unsigned long long at =
-        block_exclusive_scan<unsigned long long>((unsigned long long)tot << 32 | run, sm.scan_buf, all);
-    sm.dstart[threadIdx.x] = (uint32_t)at;
-    sm.boff[threadIdx.x] = (uint32_t)(at >> 32) + pre;
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < RS_ITEMS; j++) {
-        if (local0 + j * 32 < here) {
+        for (int j = 0; j < RS_ITEMS; j++) {
+            const bool ok = local0 + j * 32 < here;
             const uint32_t d = (k[j] >> shift) & 0xffu;
-            const uint32_t lp = sm.dstart[d] + wh[d] + lr[j];
-            sm.skeys[lp] = k[j];
-            sm.svals[lp] = vv[j];
+            uint32_t peers = __ballot_sync(kFull, ok);
+#pragma unroll
+            for (int b = 0; b < NB; b++) {  // digit bits above NB are zero in this pass
+                const uint32_t bit = (d >> b) & 1u;
+                const uint32_t bb = __ballot_sync(kFull, bit);
+                peers &= bit ? bb : ~bb;
+            }
+            const uint32_t rank = __popc(peers & lt);
+            const uint32_t before = wh[d];
+            __syncwarp();
+            if (ok && rank == 0) wh[d] = before + __popc(peers);
+            __syncwarp();
+            lr[j] = before + rank;
         }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < here; i += RS_THREADS) {
-        const uint32_t key = sm.skeys[i];
-        const uint32_t d = (key >> shift) & 0xffu;
-        const uint32_t pos = sm.boff[d] + (uint32_t)i - sm.dstart[d];
-        vout[pos] = sm.svals[i];
-        if (WRITE_KEYS) kout[pos] = key;
-        if (gout) gout[pos] = gsrc[sm.svals[i]];
-    }
+        uint32_t vv[RS_ITEMS];
+#pragma unroll
+        for (int j = 0; j < RS_ITEMS; j++)
+            vv[j] = !vin ? (uint32_t)block0 + local0 + j * 32 : local0 + j * 32 < here ? vin[block0 + local0 + j * 32] : 0u;
+        __syncthreads();
+        uint32_t run = 0;
+#pragma unroll
+        for (int w = 0; w < RS_WARPS; w++) {
+            const uint32_t c = sm.whist[w * 256 + threadIdx.x];
+            sm.whist[w * 256 + threadIdx.x] = run;
+            run += c;
+        }
+        // both prefixes over the digits in one scan: of the totals (high words) and
+        // of the block's counts
+        unsigned long long all;
+        const unsigned long long at =
+            block_exclusive_scan<unsigned long long>((unsigned long long)tot << 32 | run, sm.scan_buf, all);
+        sm.dstart[threadIdx.x] = (uint32_t)at;
+        sm.boff[threadIdx.x] = (uint32_t)(at >> 32) + pre;
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < RS_ITEMS; j++) {
+            if (local0 + j * 32 < here) {
+                const uint32_t d = (k[j] >> shift) & 0xffu;
+                const uint32_t lp = sm.dstart[d] + wh[d] + lr[j];
+                sm.skeys[lp] = k[j];
+                sm.svals[lp] = vv[j];
+            }
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < here; i += RS_THREADS) {
+            const uint32_t key = sm.skeys[i];
+            const uint32_t d = (key >> shift) & 0xffu;
+            const uint32_t pos = sm.boff[d] + (uint32_t)i - sm.dstart[d];
+            vout[pos] = sm.svals[i];
+            if (WRITE_KEYS) kout[pos] = key;
+            if (gout) gout[pos] = gsrc[sm.svals[i]];
+        }
+        if (STRIDE) __syncthreads();
+    } while (STRIDE && (block += gridDim.x) < nblocks);
 }
 
 // ---------------------------------------------------------------------------
@@ -558,22 +587,25 @@ __global__ void __launch_bounds__(256) bin_entries_kernel(const uint32_t* __rest
 
 // First and one past the last position of every bin's entries (zeroed before:
 // a bin without entries keeps an empty range).
+template <bool STRIDE>
 __global__ void __launch_bounds__(256) bin_bounds_kernel(const uint32_t* __restrict__ keys, Count Sc, int shift,
                                                          uint32_t* __restrict__ begin, uint32_t* __restrict__ end) {
     const uint64_t S = Sc.get();
-    const uint64_t i0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
+    uint64_t i0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (i0 >= S) return;
-    uint32_t b[6];
-    b[0] = i0 > 0 ? keys[i0 - 1] >> shift : 0xffffffffu;
+    do {
+        uint32_t b[6];
+        b[0] = i0 > 0 ? keys[i0 - 1] >> shift : 0xffffffffu;
 #pragma unroll
-    for (int q = 1; q < 6; q++) b[q] = i0 + q - 1 < S ? keys[i0 + q - 1] >> shift : 0xffffffffu;
+        for (int q = 1; q < 6; q++) b[q] = i0 + q - 1 < S ? keys[i0 + q - 1] >> shift : 0xffffffffu;
 #pragma unroll
-    for (int q = 1; q < 5; q++) {
-        const uint64_t i = i0 + q - 1;
-        if (i >= S) break;
-        if (i == 0 || b[q] != b[q - 1]) begin[b[q]] = (uint32_t)i;
-        if (i + 1 == S || b[q] != b[q + 1]) end[b[q]] = (uint32_t)i + 1;
-    }
+        for (int q = 1; q < 5; q++) {
+            const uint64_t i = i0 + q - 1;
+            if (i >= S) break;
+            if (i == 0 || b[q] != b[q - 1]) begin[b[q]] = (uint32_t)i;
+            if (i + 1 == S || b[q] != b[q + 1]) end[b[q]] = (uint32_t)i + 1;
+        }
+    } while (STRIDE && (i0 += (uint64_t)gridDim.x * 1024) < S);
 }
 
 // First chunk of every bin (one block; bins that no entry touches have none).
@@ -653,36 +685,38 @@ __device__ __forceinline__ uint2 entry_mask(const BinLists& L, uint64_t p, int b
 template <bool LOCAL>
 __global__ void __launch_bounds__(BC_THREADS) bin_count_kernel(BinLists L, const DevCam* __restrict__ cams, int V) {
     __shared__ uint32_t part[BC_WARPS][64];
-    const uint32_t c = blockIdx.x;
-    if (c >= L.chunk_off[L.bins]) return;
+    const uint32_t chunks = L.chunk_off[L.bins];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t b = bin_of_chunk(L.chunk_off, L.bins, c, lane);
-    const uint32_t p0 = L.begin[b] + (c - L.chunk_off[b]) * BC_CHUNK;
-    const uint32_t cnt = min(L.end[b] - p0, (uint32_t)BC_CHUNK);
-    int bx = 0, by = 0;
-    if (!LOCAL) {
-        const DevCam& cam = cams[find_bin_view(cams, V, b)];
-        const long long lb = (long long)b - cam.bin_base;
-        bx = (int)(lb % bins_across(cam.tiles_x));
-        by = (int)(lb / bins_across(cam.tiles_x));
-    }
-    uint32_t lo = 0, hi = 0;
+    for (uint32_t c = blockIdx.x; c < chunks; c += gridDim.x) {
+        const uint32_t b = bin_of_chunk(L.chunk_off, L.bins, c, lane);
+        const uint32_t p0 = L.begin[b] + (c - L.chunk_off[b]) * BC_CHUNK;
+        const uint32_t cnt = min(L.end[b] - p0, (uint32_t)BC_CHUNK);
+        int bx = 0, by = 0;
+        if (!LOCAL) {
+            const DevCam& cam = cams[find_bin_view(cams, V, b)];
+            const long long lb = (long long)b - cam.bin_base;
+            bx = (int)(lb % bins_across(cam.tiles_x));
+            by = (int)(lb / bins_across(cam.tiles_x));
+        }
+        uint32_t lo = 0, hi = 0;
 #pragma unroll
-    for (int q = 0; q < BC_GROUPS / BC_WARPS; q++) {
-        const uint32_t e = (warp * (BC_GROUPS / BC_WARPS) + q) * 32 + lane;
-        const uint2 m = e < cnt ? entry_mask<LOCAL>(L, (uint64_t)p0 + e, bx, by) : make_uint2(0u, 0u);
-        lo += __popc(warp_transpose(m.x, lane));
-        hi += __popc(warp_transpose(m.y, lane));
-    }
-    part[warp][lane] = lo;
-    part[warp][32 + lane] = hi;
-    if (threadIdx.x == 0) L.chunk_bin[c] = b;
-    __syncthreads();
-    if (threadIdx.x < 64) {
-        uint32_t sum = 0;
+        for (int q = 0; q < BC_GROUPS / BC_WARPS; q++) {
+            const uint32_t e = (warp * (BC_GROUPS / BC_WARPS) + q) * 32 + lane;
+            const uint2 m = e < cnt ? entry_mask<LOCAL>(L, (uint64_t)p0 + e, bx, by) : make_uint2(0u, 0u);
+            lo += __popc(warp_transpose(m.x, lane));
+            hi += __popc(warp_transpose(m.y, lane));
+        }
+        part[warp][lane] = lo;
+        part[warp][32 + lane] = hi;
+        if (threadIdx.x == 0) L.chunk_bin[c] = b;
+        __syncthreads();
+        if (threadIdx.x < 64) {
+            uint32_t sum = 0;
 #pragma unroll
-        for (int w = 0; w < BC_WARPS; w++) sum += part[w][threadIdx.x];
-        L.counts[(uint64_t)c * 64 + threadIdx.x] = sum;
+            for (int w = 0; w < BC_WARPS; w++) sum += part[w][threadIdx.x];
+            L.counts[(uint64_t)c * 64 + threadIdx.x] = sum;
+        }
+        __syncthreads();
     }
 }
 
@@ -725,7 +759,7 @@ __global__ void __launch_bounds__(64 * BS_PARTS) bin_scan_kernel(BinLists L, con
 // (32 entries), a warp scan of the popcounts gives each lane its part of the
 // run, the set bits are compacted in shared memory and the run is stored by
 // consecutive lanes.
-template <bool LOCAL>
+template <bool LOCAL, bool STRIDE>
 __global__ void __launch_bounds__(BC_THREADS) bin_place_kernel(BinLists L, const DevCam* __restrict__ cams, int V,
                                                                const long long* __restrict__ ranges,
                                                                const unsigned long long* __restrict__ total, Count Kc,
@@ -734,58 +768,62 @@ __global__ void __launch_bounds__(BC_THREADS) bin_place_kernel(BinLists L, const
     __shared__ uint32_t recs[BC_CHUNK];
     __shared__ uint32_t first[64];
     __shared__ uint16_t stage[BC_WARPS][BC_CHUNK];
-    const uint32_t c = blockIdx.x;
     // nothing is placed when the lists do not fit (capturable mode)
-    if (c >= L.chunk_off[L.bins] || *total > Kc.max) return;
+    const uint32_t chunks = *total > Kc.max ? 0u : L.chunk_off[L.bins];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t b = L.chunk_bin[c];
-    const uint32_t p0 = L.begin[b] + (c - L.chunk_off[b]) * BC_CHUNK;
-    const uint32_t cnt = min(L.end[b] - p0, (uint32_t)BC_CHUNK);
-    const DevCam& cam = cams[find_bin_view(cams, V, b)];
-    const int lb = (int)((long long)b - cam.bin_base), across = bins_across(cam.tiles_x);
-    const int bx = lb % across, by = lb / across;
-    if (threadIdx.x < 64) {
-        const int tx = bx * 8 + (threadIdx.x & 7), ty = by * 8 + (threadIdx.x >> 3);
-        first[threadIdx.x] = tx < cam.tiles_x && ty < cam.tiles_y
-                                 ? (uint32_t)ranges[2 * (cam.tile_base + (long long)ty * cam.tiles_x + tx)] +
-                                       L.counts[(uint64_t)c * 64 + threadIdx.x]
-                                 : 0u;
-    }
+    uint32_t c = blockIdx.x;
+    if (c >= chunks) return;
+    do {
+        const uint32_t b = L.chunk_bin[c];
+        const uint32_t p0 = L.begin[b] + (c - L.chunk_off[b]) * BC_CHUNK;
+        const uint32_t cnt = min(L.end[b] - p0, (uint32_t)BC_CHUNK);
+        const DevCam& cam = cams[find_bin_view(cams, V, b)];
+        const int lb = (int)((long long)b - cam.bin_base), across = bins_across(cam.tiles_x);
+        const int bx = lb % across, by = lb / across;
+        if (threadIdx.x < 64) {
+            const int tx = bx * 8 + (threadIdx.x & 7), ty = by * 8 + (threadIdx.x >> 3);
+            first[threadIdx.x] = tx < cam.tiles_x && ty < cam.tiles_y
+                                     ? (uint32_t)ranges[2 * (cam.tile_base + (long long)ty * cam.tiles_x + tx)] +
+                                           L.counts[(uint64_t)c * 64 + threadIdx.x]
+                                     : 0u;
+        }
 #pragma unroll
-    for (int q = 0; q < BC_GROUPS / BC_WARPS; q++) {
-        const int g = warp * (BC_GROUPS / BC_WARPS) + q;
-        const uint32_t e = g * 32 + lane;
-        uint2 m = make_uint2(0u, 0u);
-        if (e < cnt) {
-            m = entry_mask<LOCAL>(L, (uint64_t)p0 + e, bx, by);
-            recs[e] = L.vals[(uint64_t)p0 + e];
+        for (int q = 0; q < BC_GROUPS / BC_WARPS; q++) {
+            const int g = warp * (BC_GROUPS / BC_WARPS) + q;
+            const uint32_t e = g * 32 + lane;
+            uint2 m = make_uint2(0u, 0u);
+            if (e < cnt) {
+                m = entry_mask<LOCAL>(L, (uint64_t)p0 + e, bx, by);
+                recs[e] = L.vals[(uint64_t)p0 + e];
+            }
+            words[lane][g] = warp_transpose(m.x, lane);
+            words[32 + lane][g] = warp_transpose(m.y, lane);
         }
-        words[lane][g] = warp_transpose(m.x, lane);
-        words[32 + lane][g] = warp_transpose(m.y, lane);
-    }
-    __syncthreads();
-    uint16_t* st = stage[warp];
-    for (int t = warp; t < 64; t += BC_WARPS) {
-        uint32_t word = words[t][lane];
-        const uint32_t n = __popc(word);
-        uint32_t inc = n;
+        __syncthreads();
+        uint16_t* st = stage[warp];
+        for (int t = warp; t < 64; t += BC_WARPS) {
+            uint32_t word = words[t][lane];
+            const uint32_t n = __popc(word);
+            uint32_t inc = n;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(kFull, inc, o);
-            if (lane >= o) inc += y;
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFull, inc, o);
+                if (lane >= o) inc += y;
+            }
+            const uint32_t all = __shfl_sync(kFull, inc, 31);
+            if (all == 0) continue;
+            uint32_t at = inc - n;
+            while (word) {
+                st[at++] = (uint16_t)(lane * 32 + __ffs(word) - 1);
+                word &= word - 1;
+            }
+            __syncwarp();
+            uint32_t* out = sorted + first[t];
+            for (uint32_t j = lane; j < all; j += 32) out[j] = recs[st[j]];
+            __syncwarp();
         }
-        const uint32_t all = __shfl_sync(kFull, inc, 31);
-        if (all == 0) continue;
-        uint32_t at = inc - n;
-        while (word) {
-            st[at++] = (uint16_t)(lane * 32 + __ffs(word) - 1);
-            word &= word - 1;
-        }
-        __syncwarp();
-        uint32_t* out = sorted + first[t];
-        for (uint32_t j = lane; j < all; j += 32) out[j] = recs[st[j]];
-        __syncwarp();
-    }
+        if (STRIDE) __syncthreads();
+    } while (STRIDE && (c += gridDim.x) < chunks);
 }
 
 // Blend processing order: tiles by decreasing list length, in 256 length
@@ -897,21 +935,24 @@ void radix_pass(const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32
                 bool write_keys, const unsigned long long* sub, void* tmp, cudaStream_t s,
                 const uint32_t* gsrc = nullptr, uint32_t* gout = nullptr) {
     const uint64_t nb64 = radix_blocks(n.max);
-    const unsigned nb = (unsigned)nb64;
+    const unsigned nb = (unsigned)(n.dev && nb64 > GRID_CAP ? GRID_CAP : nb64);
     uint32_t* totals = static_cast<uint32_t*>(tmp);
-    const RadixTable tab{totals + 256, totals, nb, nb64 <= RS_DIRECT};
+    const RadixTable tab{totals + 256, totals, nb64 <= RS_DIRECT};
     if (bits <= 5 && !sub) rs_upsweep_narrow<<<nb, RS_THREADS, 0, s>>>(kin, n, shift, (1u << bits) - 1u, tab);
-    else rs_upsweep<<<nb, RS_THREADS, 0, s>>>(kin, n, shift, sub, tab);
+    else if (nb < nb64) rs_upsweep<true><<<nb, RS_THREADS, 0, s>>>(kin, n, shift, sub, tab);
+    else rs_upsweep<false><<<nb, RS_THREADS, 0, s>>>(kin, n, shift, sub, tab);
     if (!tab.direct) {
-        rs_scan_kernel<<<256, RS_THREADS, 0, s>>>(tab);
+        rs_scan_kernel<<<256, RS_THREADS, 0, s>>>(tab, n);
         note_launches(1);
     }
-#define MVGS_DOWN(W, B) \
-    rs_downsweep<W, B><<<nb, RS_THREADS, 0, s>>>(kin, vin, kout, vout, n, shift, sub, tab, gsrc, gout)
+#define MVGS_DOWN2(W, B, T) \
+    rs_downsweep<W, B, T><<<nb, RS_THREADS, 0, s>>>(kin, vin, kout, vout, n, shift, sub, tab, gsrc, gout)
+#define MVGS_DOWN(W, B) (nb < nb64 ? (MVGS_DOWN2(W, B, true)) : (MVGS_DOWN2(W, B, false)))
     if (bits <= 5 && !sub && write_keys) MVGS_DOWN(true, 5);
     else if (write_keys) MVGS_DOWN(true, 8);
     else MVGS_DOWN(false, 8);
 #undef MVGS_DOWN
+#undef MVGS_DOWN2
     note_launches(2);
 }
 }  // namespace
@@ -973,7 +1014,8 @@ void tile_lists(const uint32_t* order, const uint32_t* bin_off, Count R, Count S
     const bool any = S.max > 0 && R.max > 0;
     const bool local = bins <= BIN_LOCAL_MAX;
     BinLists L{};
-    const unsigned chunks = (unsigned)bin_chunks(S.max, bins);
+    const auto grid = [&](uint64_t blocks) { return (unsigned)(S.dev && blocks > GRID_CAP ? GRID_CAP : blocks); };
+    const unsigned chunks = grid(bin_chunks(S.max, bins));
     if (!any) {
         cudaMemsetAsync(tile_counts, 0, (size_t)tiles * sizeof(uint32_t), s);
     } else {
@@ -1000,7 +1042,9 @@ void tile_lists(const uint32_t* order, const uint32_t* bin_off, Count R, Count S
                      part<uint32_t>(tmp, T.counts), (uint32_t)bins};
         if (bins > 1) {
             cudaMemsetAsync(begin, 0, T.chunk_off - T.begin, s);  // begin and end
-            bin_bounds_kernel<<<(unsigned)ceil_div_u64(S.max, 1024), 256, 0, s>>>(kin, S, low, begin, end);
+            const uint64_t blocks = ceil_div_u64(S.max, 1024);
+            if (grid(blocks) < blocks) bin_bounds_kernel<true><<<grid(blocks), 256, 0, s>>>(kin, S, low, begin, end);
+            else bin_bounds_kernel<false><<<grid(blocks), 256, 0, s>>>(kin, S, low, begin, end);
             note_launches(1);
         }
         bin_chunks_kernel<<<1, SPINE_THREADS, 0, s>>>(begin, end, S, bins, chunk_off);
@@ -1017,10 +1061,12 @@ void tile_lists(const uint32_t* order, const uint32_t* bin_off, Count R, Count S
     }
     if (any) {
         StageTimer timer(MVGS_STAGE_TILE_SORT, s);
-        if (local)
-            bin_place_kernel<true><<<chunks, BC_THREADS, 0, s>>>(L, cams, V, ranges, starts + tiles, K, sorted);
-        else
-            bin_place_kernel<false><<<chunks, BC_THREADS, 0, s>>>(L, cams, V, ranges, starts + tiles, K, sorted);
+#define MVGS_PLACE(L_, T) \
+    bin_place_kernel<L_, T><<<chunks, BC_THREADS, 0, s>>>(L, cams, V, ranges, starts + tiles, K, sorted)
+        const bool stride = chunks < bin_chunks(S.max, bins);
+        if (local) stride ? (MVGS_PLACE(true, true)) : (MVGS_PLACE(true, false));
+        else stride ? (MVGS_PLACE(false, true)) : (MVGS_PLACE(false, false));
+#undef MVGS_PLACE
         note_launches(1);
     }
 }

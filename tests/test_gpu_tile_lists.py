@@ -73,3 +73,22 @@ def test_rectangles_for_any_tile(cuda_lib, tile):
     vis = (D["valid"] != 0) & (P["valid"] != 0)
     assert vis.sum() > 2000
     assert (D["rect"][vis] != P["rect"][vis]).any(axis=1).mean() < 1e-3
+
+
+def test_lists_sized_by_a_capacity_equal_the_exact_ones(cuda_lib):
+    """A capturable render with room to spare, its launches striding over more radix
+    blocks and chunks than they have blocks, against one sized by the counts."""
+    scene = synth.make_scene(1_400_000, 0, seed=6)
+    cams = synth.make_cameras([(1264, 832)] * 4, radius=4.0, seed=7)
+    rz, sc, _, img = gpu_forward(cuda_lib, scene, cams, (16, 16))
+    exact = rz.records()
+    keys, records = exact["sorted"].shape[0], exact["g"].shape[0]
+    assert keys > 4864 * 4096 * 14  # about 15 tiles per entry: more than 4864 radix blocks of 4096, and chunks by far
+    cap = cuda_lib.Rasterizer(cams, tile=(16, 16), capturable=True)
+    cap.reserve(scene.n, 6_000_000, keys + keys // 4)
+    got = cap.forward(sc)
+    assert bool((got == img).all())
+    lists = cap.records()
+    assert bool((lists["ranges"] == exact["ranges"]).all())
+    assert bool((lists["sorted"][:keys] == exact["sorted"]).all())
+    assert records <= 6_000_000
