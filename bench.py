@@ -768,11 +768,11 @@ def stage_work(rz, needed, V, pixels, blended):
 # configuration and for the blend sources it was taken on (their hash is
 # kept with it); otherwise the line reports no traffic.
 BLEND_TRAFFIC = {
-    "workload": "uneven_3m_8views", "tile": "32x64", "smem_batch": 64, "blended": 2118024889,
-    "blend_forward": 3720.0e6 + 170.8e6,
-    "blend_backward": 7450.7e6 + 419.6e6,
+    "workload": "uneven_3m_8views", "tile": "32x64", "blended": 2118024889,
+    "blend_forward": 756.6e6 + 167.7e6,
+    "blend_backward": 1996.9e6 + 228.0e6,
     "capture": "profiles/launches_uneven_3m_8views.md",
-    "sources_sha256": "a114b24ee0915ba63bfb74ce3df782c2859888aed9232cb2cd9b4c1a09a8e591",
+    "sources_sha256": "b296e217eac81e20d0af2ee0a2e0e410c3bc3682d2de220bca099379204fcbef",
 }
 
 
@@ -824,7 +824,7 @@ def roofline(stages, args, needed, rz, clk, V, pixels, blended):
     if dom in ("blend_forward", "blend_backward") and blended:
         same_launch = (args.workload == BLEND_TRAFFIC["workload"] and
                        f"{rz.cfg.tile_w}x{rz.cfg.tile_h}" == BLEND_TRAFFIC["tile"] and
-                       rz.cfg.smem_batch == BLEND_TRAFFIC["smem_batch"] and blended == BLEND_TRAFFIC["blended"])
+                       blended == BLEND_TRAFFIC["blended"])
         if not same_launch:
             d["traffic_source"] = "null: no ncu capture of this workload and launch configuration"
         elif BLEND_TRAFFIC["sources_sha256"] != blend_sources_hash():
@@ -832,7 +832,7 @@ def roofline(stages, args, needed, rz, clk, V, pixels, blended):
         else:
             d["traffic"] = int(BLEND_TRAFFIC[dom])
             d["traffic_source"] = (f"ncu dram__bytes_read.sum + dram__bytes_write.sum of this kernel's launch "
-                                   f"in {BLEND_TRAFFIC['capture']} (same workload, tile, batch and sources)")
+                                   f"in {BLEND_TRAFFIC['capture']} (same workload, tile and sources)")
     if d["bound"] == "alu":
         per = FWD_FLOP_PER_BLENDED if dom == "blend_forward" else BWD_FLOP_PER_BLENDED
         d["algorithmic"] = f"{per} FLOP x {blended} blended (pixel, Gaussian) pairs per launch"

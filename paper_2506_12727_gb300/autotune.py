@@ -2,9 +2,9 @@
 rasterizer.
 
 The tile size decides how many (Gaussian, tile) entries are sorted; the strip
-shape decides how the blend kernels spread a tile over warps; the batch is how
-many Gaussians a warp stages in shared memory at a time.  None of them
-changes the rendered image.  `autotune` times one forward + backward of each candidate
+shape decides how the blend kernels spread a tile over warps; the batch was how
+many Gaussians a warp stages in shared memory at a time (the kernels size that
+themselves now, so batches tie).  None of them changes the rendered image.  `autotune` times one forward + backward of each candidate
 on the caller's scene and cameras (CUDA events, after one warm-up) and returns
 the fastest; results are cached per (Gaussians, view resolutions) signature.
 """
