@@ -84,7 +84,8 @@ __device__ __forceinline__ BlockPos block_pos(const Views& vw) {
 // threads: a second round a third full).  The row-blurred rows lie in a ring of
 // HSY; the next tile's rows arrive during the column pass.  Bound by the issue
 // slots in the forward (79%) and by loads and address arithmetic in the
-// backward.  Eight 1264 x 832 views: 439 + 351 -> 348 + 282 us.  The sums' order
+// backward.  Eight 1264 x 832 views: 439 + 351 -> 348 + 282 us, then 258 with the
+// backward's image reads issued before its column pass.  The sums' order
 // is the tile's own, so results do not depend on the runs; packed arithmetic (I1
 // and I2 side by side) saves a fifth of the instructions but its 64-bit column
 // reads conflict, 357 us.
@@ -296,6 +297,15 @@ __global__ void __launch_bounds__(256) dssim_backward_kernel(Views vw, const flo
         const int c = threadIdx.x % TSX;
         const float inv_n = 1.f / (3.f * (float)p.H * (float)p.W);
         const int r0 = (threadIdx.x / TSX) * ROWS;
+        float i1[ROWS], i2[ROWS];  // on their way during the column pass
+#pragma unroll
+        for (int q = 0; q < ROWS; q++) {
+            const int x = p.x0 + c, y = y0 + r0 + q;
+            const bool in = x < p.W && y < p.H;
+            const long long o = p.plane + (long long)y * p.W + x;
+            i1[q] = in ? img[o] : 0.f;
+            i2[q] = in ? tgt[o] : 0.f;
+        }
         float bv[ROWS][3];
 #pragma unroll
         for (int q = 0; q < ROWS; q++) bv[q][0] = bv[q][1] = bv[q][2] = 0.f;
@@ -321,10 +331,9 @@ __global__ void __launch_bounds__(256) dssim_backward_kernel(Views vw, const flo
             if (x >= p.W || y >= p.H) continue;
             const float B1 = bv[q][0], B11 = bv[q][1], B12 = bv[q][2];
             const long long o = p.plane + (long long)y * p.W + x;
-            const float i1 = img[o], i2 = tgt[o];
-            const float diff = i1 - i2;
+            const float diff = i1[q] - i2[q];
             const float sgn = diff > 0.f ? 1.f : (diff < 0.f ? -1.f : 0.f);
-            const float dssim = B1 + 2.f * i1 * B11 + i2 * B12;
+            const float dssim = B1 + 2.f * i1[q] * B11 + i2[q] * B12;
             dimg[o] = inv_views * inv_n * ((1.f - lambda) * sgn - lambda * dssim);
         }
         base = ring(base + TSY);
