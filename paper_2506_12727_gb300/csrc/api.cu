@@ -320,7 +320,9 @@ SceneArgs scene_args(const mvgs_scene* sc) {
 // counts block of the state: records and keys in the arrays, tiles, pixels,
 // records and keys the batch needed (larger only after a capturable call ran
 // out of capacity)
-__global__ void set_counts_kernel(long long* c, long long R, long long K, long long T, long long P) {
+__global__ void set_counts_kernel(long long* c, long long R, long long K, long long T, long long P, int* queue) {
+    chained();
+    *queue = 0;
     c[0] = R;
     c[1] = K;
     c[2] = T;
@@ -335,6 +337,7 @@ __global__ void set_counts_kernel(long long* c, long long R, long long K, long l
 // and how far the largest is above it.
 __global__ void total_counts_kernel(const long long* rec_total, const unsigned long long* sums, long long rec_cap,
                                     long long key_cap, unsigned long long* dcnt) {
+    chained();
     unsigned long long k = 0, b = 0;
     uint32_t lo = 0, hi = 0;
     for (int i = threadIdx.x; i < kSumSlots; i += 32) {
@@ -363,7 +366,9 @@ __global__ void total_counts_kernel(const long long* rec_total, const unsigned l
 }
 
 __global__ void set_counts_dev_kernel(long long* c, const long long* rec_total, const unsigned long long* dcnt,
-                                      long long T, long long P) {
+                                      long long T, long long P, int* queue) {
+    chained();
+    *queue = 0;
     c[0] = (long long)dcnt[0];
     c[1] = (long long)dcnt[2];
     c[2] = T;
@@ -506,7 +511,7 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
     {
         StageTimer t(MVGS_STAGE_PREPROCESS, s);
         launch_preprocess(sc, dcams, V, tw, th, at<uint8_t>(workspace, P.w_vis), rec, bins, desc, sums, s);
-        total_counts_kernel<<<1, 32, 0, s>>>(rec.rec_off + n, sums, cap->records, cap->keys, dcnt);
+        launch_chained(total_counts_kernel, 1, 32, 0, s, rec.rec_off + n, sums, cap->records, cap->keys, dcnt);
         note_launches(1);
     }
     // Without MVGS_FLAG_CAPTURABLE the counts are read back to size the sorts
@@ -574,10 +579,12 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
         StageTimer t(MVGS_STAGE_RANGES, s);
         tile_order(ranges, P.tiles, at<uint32_t>(state, L.off_tile_order), at<void>(workspace, P.w_torder), s);
     }
+    int* queue = at<int>(workspace, P.w_counter);  // the blend's, set to 0 with the counts
     if (capt)
-        set_counts_dev_kernel<<<1, 1, 0, s>>>(counts_dev, rec.rec_off + n, dcnt, P.tiles, P.pixels);
+        launch_chained(set_counts_dev_kernel, 1, 1, 0, s, counts_dev, rec.rec_off + n, dcnt, P.tiles, P.pixels, queue);
     else
-        set_counts_kernel<<<1, 1, 0, s>>>(counts_dev, (long long)c[0], (long long)c[1], P.tiles, P.pixels);
+        launch_chained(set_counts_kernel, 1, 1, 0, s, counts_dev, (long long)c[0], (long long)c[1], P.tiles, P.pixels,
+                       queue);
     note_launches(1);
 
     BlendArgs ba;
@@ -602,7 +609,7 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
     {
         StageTimer t(MVGS_STAGE_BLEND_FORWARD, s);
         attach_samples(ba, smp, cfg, P, workspace, P.w_chunk_off, P.w_chunk_map, P.w_chunk_tmp, P.w_mask, s);
-        launch_blend_forward(ba, at<int>(workspace, P.w_counter), images, at<float>(state, L.off_final_T),
+        launch_blend_forward(ba, queue, images, at<float>(state, L.off_final_T),
                              at<uint32_t>(state, L.off_n_contrib),
                              (cfg->flags & MVGS_FLAG_PIXEL_STATS) ? at<uint2>(state, L.off_pixel_stats) : nullptr,
                              s);

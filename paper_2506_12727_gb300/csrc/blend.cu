@@ -925,7 +925,6 @@ int blend_forward_pixels_per_thread(int tw, int th, int req, long long tiles) {
 void launch_blend_forward(const BlendArgs& a, int* counter, float* img, float* final_T, uint32_t* n_contrib,
                           uint2* pixel_stats, cudaStream_t s) {
     if (a.tiles == 0) return;
-    cudaMemsetAsync(counter, 0, sizeof(int), s);
     const bool sampled = a.s_off != nullptr;
     // sampled mode: the number of runs is only known on the device; launch a
     // full persistent grid

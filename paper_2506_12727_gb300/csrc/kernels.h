@@ -159,7 +159,8 @@ int blend_strip_width(int tw);
 int blend_pixels_per_thread(int tw, int th, int req);
 // of a forward over all pixels
 int blend_forward_pixels_per_thread(int tw, int th, int req, long long tiles);
-// Persistent launches; `counter` is one device int of scratch (reset here).
+// Persistent launches; `counter` is one device int of scratch (0 for the forward,
+// reset by the backward).
 void launch_blend_forward(const BlendArgs& a, int* counter, float* img, float* final_T, uint32_t* n_contrib,
                           uint2* pixel_stats, cudaStream_t s);
 void launch_blend_backward(const BlendArgs& a, int* counter, const float* dimg, const float* final_T,

@@ -241,6 +241,7 @@ __device__ __forceinline__ bool project(const Gauss& G, const ProjCam& cam, int 
 
 // ---- kernels ---------------------------------------------------------------
 __global__ void upload_cams_kernel(CamChunk chunk, int count, DevCam* dst, unsigned long long* zero, int zero_count) {
+    chained();
     if ((int)threadIdx.x < count) dst[threadIdx.x] = chunk.c[threadIdx.x];
     for (int i = threadIdx.x; i < zero_count; i += blockDim.x) zero[i] = 0ull;
 }
@@ -251,6 +252,7 @@ __global__ void upload_cams_kernel(CamChunk chunk, int count, DevCam* dst, unsig
 __global__ void __launch_bounds__(256) count_visible_kernel(SceneArgs sc, const DevCam* __restrict__ cams, int V,
                                                             int tw, int th, int* __restrict__ counts,
                                                             uint8_t* __restrict__ vis) {
+    chained();
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= sc.n) return;
     Gauss G;
@@ -355,6 +357,7 @@ __global__ void __launch_bounds__(PRE_THREADS, SHARED_CAMS ? 10 : 8) preprocess_
                                                                  RecordArgs rec, uint32_t* __restrict__ bins,
                                                                  unsigned long long* __restrict__ tile_desc,
                                                                  unsigned long long* __restrict__ sums) {
+    chained();
     constexpr int E = (DEG + 1) * (DEG + 1) * 3, PITCH = sh_pitch(E);
     const int lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
@@ -984,7 +987,7 @@ void upload_cams(const DevCam* host, int V, DevCam* dst, cudaStream_t s, unsigne
         CamChunk chunk;
         const int cnt = V - start < kCamChunk ? V - start : kCamChunk;
         for (int i = 0; i < cnt; i++) chunk.c[i] = host[start + i];
-        upload_cams_kernel<<<1, kCamChunk, 0, s>>>(chunk, cnt, dst + start, zero, start == 0 ? zero_count : 0);
+        launch_chained(upload_cams_kernel, 1, kCamChunk, 0, s, chunk, cnt, dst + start, zero, start == 0 ? zero_count : 0);
         note_launches(1);
     }
 }
@@ -999,7 +1002,7 @@ void launch_count_keys(const SceneArgs& sc, const DevCam* cams, int V, int tw, i
 void launch_count_visible(const SceneArgs& sc, const DevCam* cams, int V, int tw, int th, int* counts,
                           uint8_t* vis, cudaStream_t s) {
     if (sc.n == 0) return;
-    count_visible_kernel<<<blocks_for(sc.n, 256), 256, 0, s>>>(sc, cams, V, tw, th, counts, vis);
+    launch_chained(count_visible_kernel, blocks_for(sc.n, 256), 256, 0, s, sc, cams, V, tw, th, counts, vis);
     note_launches(1);
 }
 
@@ -1011,8 +1014,7 @@ void launch_preprocess(const SceneArgs& sc, const DevCam* cams, int V, int tw, i
     const long long warps = (sc.n + gpw - 1) / gpw;
     const unsigned nb = (unsigned)((warps + PRE_THREADS / 32 - 1) / (PRE_THREADS / 32));
 #define MVGS_PP2(D, C)                                                                                        \
-    preprocess_kernel<D, C>                                                                                   \
-        <<<nb, PRE_THREADS, (PRE_THREADS / 32) * gpw * sh_pitch(3 * (D + 1) * (D + 1)) * sizeof(float), s>>>( \
+    launch_chained(preprocess_kernel<D, C>, nb, PRE_THREADS, (PRE_THREADS / 32) * gpw * sh_pitch(3 * (D + 1) * (D + 1)) * sizeof(float), s,  \
             sc, cams, V, tw, th, vis, rec, bins, tile_desc, sums)
 #define MVGS_PP(D)          \
     if (V >= 7) {           \

@@ -87,6 +87,7 @@ struct LoadMasked {
 
 template <class Load, class T>
 __global__ void __launch_bounds__(SC_THREADS) scan_reduce_kernel(Load ld, Count cn, T* partials) {
+    chained();
     __shared__ T buf[33];
     const uint64_t n = cn.get();
     const uint64_t base = (uint64_t)blockIdx.x * SC_TILE;
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(SC_THREADS) scan_reduce_kernel(Load ld, Count 
 template <class T>
 __global__ void __launch_bounds__(SPINE_THREADS) scan_spine_kernel(T* partials, uint64_t nb, T* total_out,
                                                                    T* end_out, Count cn) {
+    chained();
     __shared__ T buf[33];
     T carry = 0;
     for (uint64_t start = 0; start < nb; start += SPINE_THREADS) {
@@ -127,6 +129,7 @@ enum ScanBase { SPINE, PARTIALS, INPUT };
 template <class Load, class T>
 __global__ void __launch_bounds__(SC_THREADS) scan_down_kernel(Load ld, Count cn, ScanBase mode, const T* partials, T* out,
                                                                T* total_out, T* end_out) {
+    chained();
     __shared__ T tile[SC_TILE + SC_TILE / 32];
     __shared__ T buf[33];
     const uint64_t n = cn.get();
@@ -193,14 +196,14 @@ void scan_impl(Load ld, T* out, Count n, bool write_end, T* total_out, void* tmp
     // lies before them from the input, up to 1024 from the blocks' sums.
     const ScanBase mode = nb <= 5 ? INPUT : nb <= 1024 ? PARTIALS : SPINE;
     if (mode != INPUT) {
-        scan_reduce_kernel<Load, T><<<(unsigned)nb, SC_THREADS, 0, s>>>(ld, n, partials);
+        launch_chained(scan_reduce_kernel<Load, T>, (unsigned)nb, SC_THREADS, 0, s, ld, n, partials);
         note_launches(1);
     }
     if (mode == SPINE) {
-        scan_spine_kernel<T><<<1, SPINE_THREADS, 0, s>>>(partials, nb, total_out, end, n);
+        launch_chained(scan_spine_kernel<T>, 1, SPINE_THREADS, 0, s, partials, nb, total_out, end, n);
         note_launches(1);
     }
-    scan_down_kernel<Load, T><<<(unsigned)nb, SC_THREADS, 0, s>>>(ld, n, mode, partials, out, total_out, end);
+    launch_chained(scan_down_kernel<Load, T>, (unsigned)nb, SC_THREADS, 0, s, ld, n, mode, partials, out, total_out, end);
     note_launches(1);
 }
 
@@ -267,6 +270,7 @@ __device__ __forceinline__ void digit_counts(const RadixTable& tab, uint32_t nbl
 template <bool STRIDE>
 __global__ void __launch_bounds__(RS_THREADS) rs_upsweep(const uint32_t* __restrict__ keys, Count cn, int shift,
                                                         const unsigned long long* __restrict__ sub, RadixTable tab) {
+    chained();
     __shared__ uint32_t hist[RS_WARPS * 256];
     const uint64_t n = cn.get();
     const uint32_t nblocks = rs_blocks(n);
@@ -302,6 +306,7 @@ __global__ void __launch_bounds__(RS_THREADS) rs_upsweep(const uint32_t* __restr
 // Shared-memory atomics from 32 lanes on a handful of digits serialise.
 __global__ void __launch_bounds__(RS_THREADS) rs_upsweep_narrow(const uint32_t* __restrict__ keys, Count cn, int shift,
                                                                uint32_t mask, RadixTable tab) {
+    chained();
     __shared__ uint32_t cnt[RS_WARPS][32 * 32];
     __shared__ uint32_t wsum[RS_WARPS][32];
     const uint64_t n = cn.get();
@@ -338,6 +343,7 @@ __global__ void __launch_bounds__(RS_THREADS) rs_upsweep_narrow(const uint32_t* 
 // One block per digit: its counts become the number of its keys in the blocks
 // before, and their sum its total.  A warp takes a stretch of the blocks.
 __global__ void __launch_bounds__(RS_THREADS) rs_scan_kernel(RadixTable tab, Count cn) {
+    chained();
     __shared__ uint32_t buf[33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t nblocks = rs_blocks(cn.get());
@@ -385,6 +391,7 @@ __global__ void __launch_bounds__(RS_THREADS, 3) rs_downsweep(const uint32_t* __
                                                              const unsigned long long* __restrict__ sub, RadixTable tab,
                                                              const uint32_t* __restrict__ gsrc = nullptr,
                                                              uint32_t* __restrict__ gout = nullptr) {
+    chained();
     __shared__ RankSmem sm;
     const uint64_t n = cn.get();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -524,7 +531,7 @@ __device__ __forceinline__ int find_bin_view(const DevCam* cams, int V, long lon
 // the records' bin counts in that order.  A warp takes 32 records and walks
 // their entries 32 at a time (each lane finds its entry's record by a search
 // over the warp's offsets), so the stores are coalesced however uneven the
-// records' counts are. 32-bit offsets:
+// records' counts are.  The bins' bounds are zeroed on the way.  32-bit offsets:
 // 22M records (3M Gaussians x 8 views) are scanned in 80 us instead of 147 and
 // read here in 376 us with the descriptors, 394 before; the descriptors' random
 // 32-byte sectors are most of that.
@@ -533,9 +540,12 @@ __global__ void __launch_bounds__(256) bin_entries_kernel(const uint32_t* __rest
                                                           const uint32_t* __restrict__ off, Count Rc,
                                                           Count Sc, const unsigned long long* __restrict__ desc,
                                                           const DevCam* __restrict__ cams,
-                                                          uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+                                                          uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
+                                                          uint32_t* __restrict__ zero, long long zero_count) {
+    chained();
     const uint64_t R = Rc.get(), S = Sc.get();
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (long long k = (long long)i; k < zero_count; k += (long long)gridDim.x * blockDim.x) zero[k] = 0;
     const int lane = threadIdx.x & 31;
     const uint64_t w0 = i - lane;
     if (w0 >= R) return;  // the whole warp
@@ -590,6 +600,7 @@ __global__ void __launch_bounds__(256) bin_entries_kernel(const uint32_t* __rest
 template <bool STRIDE>
 __global__ void __launch_bounds__(256) bin_bounds_kernel(const uint32_t* __restrict__ keys, Count Sc, int shift,
                                                          uint32_t* __restrict__ begin, uint32_t* __restrict__ end) {
+    chained();
     const uint64_t S = Sc.get();
     uint64_t i0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (i0 >= S) return;
@@ -613,6 +624,7 @@ __global__ void __launch_bounds__(256) bin_bounds_kernel(const uint32_t* __restr
 __global__ void __launch_bounds__(SPINE_THREADS) bin_chunks_kernel(uint32_t* __restrict__ begin,
                                                                    uint32_t* __restrict__ end, Count Sc, long long bins,
                                                                    uint32_t* __restrict__ chunk_off) {
+    chained();
     __shared__ uint32_t buf[33];
     if (bins == 1) {
         if (threadIdx.x == 0) {
@@ -684,6 +696,7 @@ __device__ __forceinline__ uint2 entry_mask(const BinLists& L, uint64_t p, int b
 // Entries per tile of every chunk.
 template <bool LOCAL>
 __global__ void __launch_bounds__(BC_THREADS) bin_count_kernel(BinLists L, const DevCam* __restrict__ cams, int V) {
+    chained();
     __shared__ uint32_t part[BC_WARPS][64];
     const uint32_t chunks = L.chunk_off[L.bins];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -725,6 +738,7 @@ __global__ void __launch_bounds__(BC_THREADS) bin_count_kernel(BinLists L, const
 constexpr int BS_PARTS = 8;  // stretches of chunks scanned side by side
 __global__ void __launch_bounds__(64 * BS_PARTS) bin_scan_kernel(BinLists L, const DevCam* __restrict__ cams, int V,
                                                                  uint32_t* __restrict__ tile_counts) {
+    chained();
     __shared__ uint32_t sums[BS_PARTS][64];
     const uint32_t b = blockIdx.x;
     const int t = threadIdx.x & 63, part = threadIdx.x >> 6;
@@ -764,6 +778,7 @@ __global__ void __launch_bounds__(BC_THREADS) bin_place_kernel(BinLists L, const
                                                                const long long* __restrict__ ranges,
                                                                const unsigned long long* __restrict__ total, Count Kc,
                                                                uint32_t* __restrict__ sorted) {
+    chained();
     __shared__ uint32_t words[64][BC_GROUPS + 1];
     __shared__ uint32_t recs[BC_CHUNK];
     __shared__ uint32_t first[64];
@@ -845,6 +860,7 @@ __device__ __forceinline__ uint32_t length_class(long long len) {
 
 __global__ void __launch_bounds__(TO_THREADS) tile_order_kernel(const long long* __restrict__ ranges, long long tiles,
                                                                 uint32_t* __restrict__ order) {
+    chained();
     __shared__ uint32_t off[256];                // per class: next output position
     __shared__ uint32_t wcnt[TO_WARPS][256];     // per warp and class, within a chunk
     __shared__ uint32_t buf[33];
@@ -894,6 +910,7 @@ __global__ void __launch_bounds__(TO_THREADS) tile_order_kernel(const long long*
 // capacity: nothing is placed then, so no range may point at the array).
 __global__ void ranges_kernel(const unsigned long long* __restrict__ starts, long long tiles, Count Kc,
                               long long* __restrict__ ranges) {
+    chained();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= tiles) return;
     const bool fits = starts[tiles] <= Kc.max;
@@ -938,15 +955,15 @@ void radix_pass(const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32
     const unsigned nb = (unsigned)(n.dev && nb64 > GRID_CAP ? GRID_CAP : nb64);
     uint32_t* totals = static_cast<uint32_t*>(tmp);
     const RadixTable tab{totals + 256, totals, nb64 <= RS_DIRECT};
-    if (bits <= 5 && !sub) rs_upsweep_narrow<<<nb, RS_THREADS, 0, s>>>(kin, n, shift, (1u << bits) - 1u, tab);
-    else if (nb < nb64) rs_upsweep<true><<<nb, RS_THREADS, 0, s>>>(kin, n, shift, sub, tab);
-    else rs_upsweep<false><<<nb, RS_THREADS, 0, s>>>(kin, n, shift, sub, tab);
+    if (bits <= 5 && !sub) launch_chained(rs_upsweep_narrow, nb, RS_THREADS, 0, s, kin, n, shift, (1u << bits) - 1u, tab);
+    else if (nb < nb64) launch_chained(rs_upsweep<true>, nb, RS_THREADS, 0, s, kin, n, shift, sub, tab);
+    else launch_chained(rs_upsweep<false>, nb, RS_THREADS, 0, s, kin, n, shift, sub, tab);
     if (!tab.direct) {
-        rs_scan_kernel<<<256, RS_THREADS, 0, s>>>(tab, n);
+        launch_chained(rs_scan_kernel, 256, RS_THREADS, 0, s, tab, n);
         note_launches(1);
     }
 #define MVGS_DOWN2(W, B, T) \
-    rs_downsweep<W, B, T><<<nb, RS_THREADS, 0, s>>>(kin, vin, kout, vout, n, shift, sub, tab, gsrc, gout)
+    launch_chained(rs_downsweep<W, B, T>, nb, RS_THREADS, 0, s, kin, vin, kout, vout, n, shift, sub, tab, gsrc, gout)
 #define MVGS_DOWN(W, B) (nb < nb64 ? (MVGS_DOWN2(W, B, true)) : (MVGS_DOWN2(W, B, false)))
     if (bits <= 5 && !sub && write_keys) MVGS_DOWN(true, 5);
     else if (write_keys) MVGS_DOWN(true, 8);
@@ -1022,8 +1039,13 @@ void tile_lists(const uint32_t* order, const uint32_t* bin_off, Count R, Count S
         StageTimer timer(MVGS_STAGE_TILE_SORT, s);
         uint32_t *kin = keys_a, *vin = vals_a, *kout = keys_b, *vout = vals_b;
         const unsigned rblocks = (unsigned)ceil_div_u64(R.max, 256);
-        if (local) bin_entries_kernel<true><<<rblocks, 256, 0, s>>>(order, bin_off, R, S, desc, cams, kin, vin);
-        else bin_entries_kernel<false><<<rblocks, 256, 0, s>>>(order, bin_off, R, S, desc, cams, kin, vin);
+        uint32_t* begin = part<uint32_t>(tmp, T.begin);
+        uint32_t* end = part<uint32_t>(tmp, T.end);
+        const long long zeroed = bins > 1 ? (long long)((T.chunk_off - T.begin) / sizeof(uint32_t)) : 0;  // begin and end
+        if (local) launch_chained(bin_entries_kernel<true>, rblocks, 256, 0, s, order, bin_off, R, S, desc, cams, kin, vin,
+                                  begin, zeroed);
+        else launch_chained(bin_entries_kernel<false>, rblocks, 256, 0, s, order, bin_off, R, S, desc, cams, kin, vin,
+                                  begin, zeroed);
         const int low = local ? BIN_LOCAL_BITS : 0;
         int bits = 0;
         while ((1LL << bits) < bins) bits++;
@@ -1035,34 +1057,31 @@ void tile_lists(const uint32_t* order, const uint32_t* bin_off, Count R, Count S
             kout = nk;
             vout = nv;
         }
-        uint32_t* begin = part<uint32_t>(tmp, T.begin);
-        uint32_t* end = part<uint32_t>(tmp, T.end);
         uint32_t* chunk_off = part<uint32_t>(tmp, T.chunk_off);
         L = BinLists{kin, vin, desc, begin, end, chunk_off, part<uint32_t>(tmp, T.chunk_bin),
                      part<uint32_t>(tmp, T.counts), (uint32_t)bins};
         if (bins > 1) {
-            cudaMemsetAsync(begin, 0, T.chunk_off - T.begin, s);  // begin and end
             const uint64_t blocks = ceil_div_u64(S.max, 1024);
-            if (grid(blocks) < blocks) bin_bounds_kernel<true><<<grid(blocks), 256, 0, s>>>(kin, S, low, begin, end);
-            else bin_bounds_kernel<false><<<grid(blocks), 256, 0, s>>>(kin, S, low, begin, end);
+            if (grid(blocks) < blocks) launch_chained(bin_bounds_kernel<true>, grid(blocks), 256, 0, s, kin, S, low, begin, end);
+            else launch_chained(bin_bounds_kernel<false>, grid(blocks), 256, 0, s, kin, S, low, begin, end);
             note_launches(1);
         }
-        bin_chunks_kernel<<<1, SPINE_THREADS, 0, s>>>(begin, end, S, bins, chunk_off);
-        if (local) bin_count_kernel<true><<<chunks, BC_THREADS, 0, s>>>(L, cams, V);
-        else bin_count_kernel<false><<<chunks, BC_THREADS, 0, s>>>(L, cams, V);
-        bin_scan_kernel<<<(unsigned)bins, 64 * BS_PARTS, 0, s>>>(L, cams, V, tile_counts);
+        launch_chained(bin_chunks_kernel, 1, SPINE_THREADS, 0, s, begin, end, S, bins, chunk_off);
+        if (local) launch_chained(bin_count_kernel<true>, chunks, BC_THREADS, 0, s, L, cams, V);
+        else launch_chained(bin_count_kernel<false>, chunks, BC_THREADS, 0, s, L, cams, V);
+        launch_chained(bin_scan_kernel, (unsigned)bins, 64 * BS_PARTS, 0, s, L, cams, V, tile_counts);
         note_launches(4);
     }
     {
         StageTimer timer(MVGS_STAGE_RANGES, s);
         scan_u32_to_u64(tile_counts, starts, (uint64_t)tiles, part<void>(tmp, T.scan), s);
-        ranges_kernel<<<(unsigned)ceil_div_u64((uint64_t)tiles, 256), 256, 0, s>>>(starts, tiles, K, ranges);
+        launch_chained(ranges_kernel, (unsigned)ceil_div_u64((uint64_t)tiles, 256), 256, 0, s, starts, tiles, K, ranges);
         note_launches(1);
     }
     if (any) {
         StageTimer timer(MVGS_STAGE_TILE_SORT, s);
 #define MVGS_PLACE(L_, T) \
-    bin_place_kernel<L_, T><<<chunks, BC_THREADS, 0, s>>>(L, cams, V, ranges, starts + tiles, K, sorted)
+    launch_chained(bin_place_kernel<L_, T>, chunks, BC_THREADS, 0, s, L, cams, V, ranges, starts + tiles, K, sorted)
         const bool stride = chunks < bin_chunks(S.max, bins);
         if (local) stride ? (MVGS_PLACE(true, true)) : (MVGS_PLACE(true, false));
         else stride ? (MVGS_PLACE(false, true)) : (MVGS_PLACE(false, false));
@@ -1075,7 +1094,7 @@ size_t tile_order_temp_bytes(long long) { return 256; }
 
 void tile_order(const long long* ranges, long long tiles, uint32_t* order, void*, cudaStream_t s) {
     if (tiles <= 0) return;
-    tile_order_kernel<<<1, TO_THREADS, 0, s>>>(ranges, tiles, order);
+    launch_chained(tile_order_kernel, 1, TO_THREADS, 0, s, ranges, tiles, order);
     note_launches(1);
 }
 
