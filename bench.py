@@ -769,10 +769,10 @@ def stage_work(rz, needed, V, pixels, blended):
 # kept with it); otherwise the line reports no traffic.
 BLEND_TRAFFIC = {
     "workload": "uneven_3m_8views", "tile": "32x64", "blended": 2118024889,
-    "blend_forward": 756.6e6 + 167.7e6,
-    "blend_backward": 1996.9e6 + 228.0e6,
+    "blend_forward": 753.8e6 + 167.7e6,
+    "blend_backward": 2020.0e6 + 230.2e6,
     "capture": "profiles/launches_uneven_3m_8views.md",
-    "sources_sha256": "b296e217eac81e20d0af2ee0a2e0e410c3bc3682d2de220bca099379204fcbef",
+    "sources_sha256": "24754f6c7437fee6b42b6132d932922a58d4172e8f672fef31aea15c77a924c4",
 }
 
 
