@@ -769,10 +769,10 @@ def stage_work(rz, needed, V, pixels, blended):
 # kept with it); otherwise the line reports no traffic.
 BLEND_TRAFFIC = {
     "workload": "uneven_3m_8views", "tile": "32x64", "blended": 2118024889,
-    "blend_forward": 753.8e6 + 167.7e6,
-    "blend_backward": 2020.0e6 + 230.2e6,
+    "blend_forward": 754.3e6 + 167.7e6,
+    "blend_backward": 2002.1e6 + 229.1e6,
     "capture": "profiles/launches_uneven_3m_8views.md",
-    "sources_sha256": "24754f6c7437fee6b42b6132d932922a58d4172e8f672fef31aea15c77a924c4",
+    "sources_sha256": "cdbed7e399b5571221719cb12eeed8ec0caa1e001eb07ca3dcd158dd5586d331",
 }
 
 
