@@ -56,8 +56,15 @@ struct Count {
 // Kernels launched with launch_chained begin while the kernel before them on the
 // stream ends: chained() comes first in every thread, before any return, lets the
 // next kernel's blocks take their places and then waits until the kernel before is
-// complete and its writes are visible -- so what a chained kernel sees is what it
-// would see after a plain launch, also of the kernels before that one.  The 30
+// complete and its writes are visible.  The predecessor has waited for its own in
+// the same way, so this holds for every kernel before on the stream, whatever it
+// wrote: the chain's arrays, and the scene a caller's kernel has just updated.
+// The wait orders ordinary loads only.  A const __restrict__ pointer (or __ldg)
+// would promise that nobody writes the data while the kernel runs, which is not so
+// -- it may be resident while all of those still write -- and would allow loads
+// through the non-coherent cache or ahead of the wait.  So no pointer of a chained
+// kernel is __restrict__; where that costs something (a load behind a store that
+// might alias it), the kernel loads first.  The 30
 // launches from the participation to the blend wait about 1 us less each: a
 // 500k-Gaussian frame 531 -> 483 us, 20k in three small views 877 -> 839, 500k x 4
 // views 2900 -> 2845.  Not for the persistent blends: their waiting blocks cost

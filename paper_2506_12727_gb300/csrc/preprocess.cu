@@ -249,20 +249,24 @@ __global__ void upload_cams_kernel(CamChunk chunk, int count, DevCam* dst, unsig
 // Visibility of every (Gaussian, view) pair: one byte per pair (view-minor)
 // and the count per Gaussian.  The fill pass reads these bytes instead of
 // deciding again, so the record count is exact by construction.
-__global__ void __launch_bounds__(256) count_visible_kernel(SceneArgs sc, const DevCam* __restrict__ cams, int V,
-                                                            int tw, int th, int* __restrict__ counts,
-                                                            uint8_t* __restrict__ vis) {
+__global__ void __launch_bounds__(256) count_visible_kernel(SceneArgs sc, const DevCam* cams, int V,
+                                                            int tw, int th, int* counts,
+                                                            uint8_t* vis) {
     chained();
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= sc.n) return;
     Gauss G;
     load_gauss(sc, g, G, true);
     int cnt = 0;
-    for (int v = 0; v < V; v++) {
-        Proj P;
-        const bool ok = project(G, cams[v], tw, th, P);
-        vis[g * V + v] = ok ? 1 : 0;
-        cnt += ok ? 1 : 0;
+    for (int c = 0; c < V; c += 32) {  // 32 views at a time: no view's fields wait behind a store
+        const int views = min(V - c, 32);
+        uint32_t seen = 0;
+        for (int v = 0; v < views; v++) {
+            Proj P;
+            seen |= (project(G, cams[c + v], tw, th, P) ? 1u : 0u) << v;
+        }
+        for (int v = 0; v < views; v++) vis[g * V + c + v] = (uint8_t)(seen >> v & 1u);
+        cnt += __popc(seen);
     }
     counts[g] = cnt;
 }
@@ -278,7 +282,7 @@ static_assert(sizeof(ProjCam) % 4 == 0 && (sizeof(SharedCam) / 4) % 2 == 1, "odd
 
 // Called by every thread of the block, a copy group of its own; the caller waits
 // for it and synchronises.
-__device__ __forceinline__ void stage_cams(const DevCam* __restrict__ cams, int count, SharedCam* s_cam) {
+__device__ __forceinline__ void stage_cams(const DevCam* cams, int count, SharedCam* s_cam) {
     constexpr int W = sizeof(ProjCam) / 4;
     for (int i = threadIdx.x; i < count * W; i += blockDim.x) {
         const int v = i / W, w = i - v * W;
@@ -296,7 +300,7 @@ __host__ __device__ constexpr int sh_pitch(int E) { return E % 4 == 0 && (E / 4)
 // floats apart, without holding them in registers; cp_async_wait and
 // __syncwarp before they are read.
 template <int E, int PITCH>
-__device__ __forceinline__ void stage_sh(const float* __restrict__ rows, int count, float* dst, int lane) {
+__device__ __forceinline__ void stage_sh(const float* rows, int count, float* dst, int lane) {
     constexpr int N = E % 4 == 0 ? 4 : 1;  // floats per copy
     if (N == 4 && (reinterpret_cast<uintptr_t>(rows) & 15) == 0) {
         for (int i = lane; i < count * (E / N); i += 32) {
@@ -352,11 +356,11 @@ constexpr int PRE_THREADS = 128;
 // views that is 60% of the measured copy bandwidth on the 3.5 GB it must move;
 // the arithmetic issues in two thirds of the cycles.
 template <int DEG, bool SHARED_CAMS>
-__global__ void __launch_bounds__(PRE_THREADS, SHARED_CAMS ? 10 : 8) preprocess_kernel(SceneArgs sc, const DevCam* __restrict__ cams, int V,
-                                                                 int tw, int th, const uint8_t* __restrict__ vis,
-                                                                 RecordArgs rec, uint32_t* __restrict__ bins,
-                                                                 unsigned long long* __restrict__ tile_desc,
-                                                                 unsigned long long* __restrict__ sums) {
+__global__ void __launch_bounds__(PRE_THREADS, SHARED_CAMS ? 10 : 8) preprocess_kernel(SceneArgs sc, const DevCam* cams, int V,
+                                                                 int tw, int th, const uint8_t* vis,
+                                                                 RecordArgs rec, uint32_t* bins,
+                                                                 unsigned long long* tile_desc,
+                                                                 unsigned long long* sums) {
     chained();
     constexpr int E = (DEG + 1) * (DEG + 1) * 3, PITCH = sh_pitch(E);
     const int lane = threadIdx.x & 31;

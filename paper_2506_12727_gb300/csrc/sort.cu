@@ -268,8 +268,8 @@ __device__ __forceinline__ void digit_counts(const RadixTable& tab, uint32_t nbl
 
 // Per-block digit histogram.  sub (optional): subtracted from every key.
 template <bool STRIDE>
-__global__ void __launch_bounds__(RS_THREADS) rs_upsweep(const uint32_t* __restrict__ keys, Count cn, int shift,
-                                                        const unsigned long long* __restrict__ sub, RadixTable tab) {
+__global__ void __launch_bounds__(RS_THREADS) rs_upsweep(const uint32_t* keys, Count cn, int shift,
+                                                        const unsigned long long* sub, RadixTable tab) {
     chained();
     __shared__ uint32_t hist[RS_WARPS * 256];
     const uint64_t n = cn.get();
@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(RS_THREADS) rs_upsweep(const uint32_t* __restr
 // hit its own bank, and are plain read-modify-writes, not atomics, since no
 // other lane touches the column), then a skewed sweep sums the columns.
 // Shared-memory atomics from 32 lanes on a handful of digits serialise.
-__global__ void __launch_bounds__(RS_THREADS) rs_upsweep_narrow(const uint32_t* __restrict__ keys, Count cn, int shift,
+__global__ void __launch_bounds__(RS_THREADS) rs_upsweep_narrow(const uint32_t* keys, Count cn, int shift,
                                                                uint32_t mask, RadixTable tab) {
     chained();
     __shared__ uint32_t cnt[RS_WARPS][32 * 32];
@@ -384,13 +384,13 @@ __global__ void __launch_bounds__(RS_THREADS) rs_scan_kernel(RadixTable tab, Cou
 // carried into sorted order).  STRIDE: a launch sized by a capacity; a variant of
 // its own because the loop costs registers that spill.
 template <bool WRITE_KEYS, int NB, bool STRIDE>
-__global__ void __launch_bounds__(RS_THREADS, 3) rs_downsweep(const uint32_t* __restrict__ kin,
-                                                             const uint32_t* __restrict__ vin,
-                                                             uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
+__global__ void __launch_bounds__(RS_THREADS, 3) rs_downsweep(const uint32_t* kin,
+                                                             const uint32_t* vin,
+                                                             uint32_t* kout, uint32_t* vout,
                                                              Count cn, int shift,
-                                                             const unsigned long long* __restrict__ sub, RadixTable tab,
-                                                             const uint32_t* __restrict__ gsrc = nullptr,
-                                                             uint32_t* __restrict__ gout = nullptr) {
+                                                             const unsigned long long* sub, RadixTable tab,
+                                                             const uint32_t* gsrc = nullptr,
+                                                             uint32_t* gout = nullptr) {
     chained();
     __shared__ RankSmem sm;
     const uint64_t n = cn.get();
@@ -462,13 +462,25 @@ __global__ void __launch_bounds__(RS_THREADS, 3) rs_downsweep(const uint32_t* __
             }
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < here; i += RS_THREADS) {
-            const uint32_t key = sm.skeys[i];
-            const uint32_t d = (key >> shift) & 0xffu;
-            const uint32_t pos = sm.boff[d] + (uint32_t)i - sm.dstart[d];
-            vout[pos] = sm.svals[i];
-            if (WRITE_KEYS) kout[pos] = key;
-            if (gout) gout[pos] = gsrc[sm.svals[i]];
+        // four at a time: no carried value's fetch waits behind a store
+        for (int i0 = threadIdx.x; i0 < here; i0 += 4 * RS_THREADS) {
+            uint32_t carried[4] = {0u, 0u, 0u, 0u};
+            if (gout) {
+#pragma unroll
+                for (int q = 0; q < 4; q++)
+                    if (i0 + q * RS_THREADS < here) carried[q] = gsrc[sm.svals[i0 + q * RS_THREADS]];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const int i = i0 + q * RS_THREADS;
+                if (i >= here) break;
+                const uint32_t key = sm.skeys[i];
+                const uint32_t d = (key >> shift) & 0xffu;
+                const uint32_t pos = sm.boff[d] + (uint32_t)i - sm.dstart[d];
+                vout[pos] = sm.svals[i];
+                if (WRITE_KEYS) kout[pos] = key;
+                if (gout) gout[pos] = carried[q];
+            }
         }
         if (STRIDE) __syncthreads();
     } while (STRIDE && (block += gridDim.x) < nblocks);
@@ -536,12 +548,12 @@ __device__ __forceinline__ int find_bin_view(const DevCam* cams, int V, long lon
 // read here in 376 us with the descriptors, 394 before; the descriptors' random
 // 32-byte sectors are most of that.
 template <bool LOCAL>
-__global__ void __launch_bounds__(256) bin_entries_kernel(const uint32_t* __restrict__ order,
-                                                          const uint32_t* __restrict__ off, Count Rc,
-                                                          Count Sc, const unsigned long long* __restrict__ desc,
-                                                          const DevCam* __restrict__ cams,
-                                                          uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
-                                                          uint32_t* __restrict__ zero, long long zero_count) {
+__global__ void __launch_bounds__(256) bin_entries_kernel(const uint32_t* order,
+                                                          const uint32_t* off, Count Rc,
+                                                          Count Sc, const unsigned long long* desc,
+                                                          const DevCam* cams,
+                                                          uint32_t* keys, uint32_t* vals,
+                                                          uint32_t* zero, long long zero_count) {
     chained();
     const uint64_t R = Rc.get(), S = Sc.get();
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -598,8 +610,8 @@ __global__ void __launch_bounds__(256) bin_entries_kernel(const uint32_t* __rest
 // First and one past the last position of every bin's entries (zeroed before:
 // a bin without entries keeps an empty range).
 template <bool STRIDE>
-__global__ void __launch_bounds__(256) bin_bounds_kernel(const uint32_t* __restrict__ keys, Count Sc, int shift,
-                                                         uint32_t* __restrict__ begin, uint32_t* __restrict__ end) {
+__global__ void __launch_bounds__(256) bin_bounds_kernel(const uint32_t* keys, Count Sc, int shift,
+                                                         uint32_t* begin, uint32_t* end) {
     chained();
     const uint64_t S = Sc.get();
     uint64_t i0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
@@ -621,9 +633,9 @@ __global__ void __launch_bounds__(256) bin_bounds_kernel(const uint32_t* __restr
 
 // First chunk of every bin (one block; bins that no entry touches have none).
 // A single bin holds all S entries.
-__global__ void __launch_bounds__(SPINE_THREADS) bin_chunks_kernel(uint32_t* __restrict__ begin,
-                                                                   uint32_t* __restrict__ end, Count Sc, long long bins,
-                                                                   uint32_t* __restrict__ chunk_off) {
+__global__ void __launch_bounds__(SPINE_THREADS) bin_chunks_kernel(uint32_t* begin,
+                                                                   uint32_t* end, Count Sc, long long bins,
+                                                                   uint32_t* chunk_off) {
     chained();
     __shared__ uint32_t buf[33];
     if (bins == 1) {
@@ -695,7 +707,7 @@ __device__ __forceinline__ uint2 entry_mask(const BinLists& L, uint64_t p, int b
 
 // Entries per tile of every chunk.
 template <bool LOCAL>
-__global__ void __launch_bounds__(BC_THREADS) bin_count_kernel(BinLists L, const DevCam* __restrict__ cams, int V) {
+__global__ void __launch_bounds__(BC_THREADS) bin_count_kernel(BinLists L, const DevCam* cams, int V) {
     chained();
     __shared__ uint32_t part[BC_WARPS][64];
     const uint32_t chunks = L.chunk_off[L.bins];
@@ -736,8 +748,8 @@ __global__ void __launch_bounds__(BC_THREADS) bin_count_kernel(BinLists L, const
 // One block per bin: every chunk's counts become the number of entries in the
 // chunks before it, tile by tile, and the totals the tiles' list lengths.
 constexpr int BS_PARTS = 8;  // stretches of chunks scanned side by side
-__global__ void __launch_bounds__(64 * BS_PARTS) bin_scan_kernel(BinLists L, const DevCam* __restrict__ cams, int V,
-                                                                 uint32_t* __restrict__ tile_counts) {
+__global__ void __launch_bounds__(64 * BS_PARTS) bin_scan_kernel(BinLists L, const DevCam* cams, int V,
+                                                                 uint32_t* tile_counts) {
     chained();
     __shared__ uint32_t sums[BS_PARTS][64];
     const uint32_t b = blockIdx.x;
@@ -774,10 +786,10 @@ __global__ void __launch_bounds__(64 * BS_PARTS) bin_scan_kernel(BinLists L, con
 // run, the set bits are compacted in shared memory and the run is stored by
 // consecutive lanes.
 template <bool LOCAL, bool STRIDE>
-__global__ void __launch_bounds__(BC_THREADS) bin_place_kernel(BinLists L, const DevCam* __restrict__ cams, int V,
-                                                               const long long* __restrict__ ranges,
-                                                               const unsigned long long* __restrict__ total, Count Kc,
-                                                               uint32_t* __restrict__ sorted) {
+__global__ void __launch_bounds__(BC_THREADS) bin_place_kernel(BinLists L, const DevCam* cams, int V,
+                                                               const long long* ranges,
+                                                               const unsigned long long* total, Count Kc,
+                                                               uint32_t* sorted) {
     chained();
     __shared__ uint32_t words[64][BC_GROUPS + 1];
     __shared__ uint32_t recs[BC_CHUNK];
@@ -858,8 +870,8 @@ __device__ __forceinline__ uint32_t length_class(long long len) {
     return 255u - (b < 255u ? b : 255u);      // 0: the longest lists
 }
 
-__global__ void __launch_bounds__(TO_THREADS) tile_order_kernel(const long long* __restrict__ ranges, long long tiles,
-                                                                uint32_t* __restrict__ order) {
+__global__ void __launch_bounds__(TO_THREADS) tile_order_kernel(const long long* ranges, long long tiles,
+                                                                uint32_t* order) {
     chained();
     __shared__ uint32_t off[256];                // per class: next output position
     __shared__ uint32_t wcnt[TO_WARPS][256];     // per warp and class, within a chunk
@@ -878,10 +890,12 @@ __global__ void __launch_bounds__(TO_THREADS) tile_order_kernel(const long long*
     __syncthreads();
     // stable scatter, chunk by chunk in tile order: rank inside the warp by
     // matching classes, then add the counts of the warps before
+    uint32_t next = threadIdx.x < tiles ? cls(threadIdx.x) : 256u;
     for (long long base = 0; base < tiles; base += TO_THREADS) {
         const long long t = base + threadIdx.x;
         const bool valid = t < tiles;
-        const uint32_t c = valid ? cls(t) : 256u;
+        const uint32_t c = next;
+        next = t + TO_THREADS < tiles ? cls(t + TO_THREADS) : 256u;  // read ahead of this chunk's stores
         const uint32_t peers = __match_any_sync(kFull, c);
         for (int i = lane; i < 256; i += 32) wcnt[warp][i] = 0;
         __syncwarp();
@@ -908,8 +922,8 @@ __global__ void __launch_bounds__(TO_THREADS) tile_order_kernel(const long long*
 // [start, end) of every tile's list.  All lists are empty when they hold more
 // entries than there is room for (a capturable call that ran out of key
 // capacity: nothing is placed then, so no range may point at the array).
-__global__ void ranges_kernel(const unsigned long long* __restrict__ starts, long long tiles, Count Kc,
-                              long long* __restrict__ ranges) {
+__global__ void ranges_kernel(const unsigned long long* starts, long long tiles, Count Kc,
+                              long long* ranges) {
     chained();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= tiles) return;
