@@ -282,28 +282,48 @@ __device__ __forceinline__ Geom load_geom(const Geom* g) {
     return Geom{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 }
 
+// Whether the quadratic form of a conic stays clear of its rounding: with B^2 <=
+// 0.99 AC it is at least 1/400 of the sum of its terms' magnitudes.  The bounds
+// on A and C keep the terms of a pixel distance (0, or at least 2^-25) clear of
+// underflow and overflow.  NaN fails.
+__device__ __forceinline__ bool well_conditioned(float4 co) {
+    const float A = co.x, B = co.y, C = co.z;
+    return (A >= 1e-15f) & (A <= 1e10f) & (C >= 1e-15f) & (C <= 1e10f) & (B * B <= 0.99f * (A * C));
+}
+
 // Whether two tests of pair_eval cannot matter for a Gaussian, so that the
 // forward blend may leave them out, and blending it with alpha 0 changes
 // nothing:
-//   - e <= 0: with B^2 <= 0.99 AC the quadratic form is at least 1/400 of the
-//     sum of its terms' magnitudes, which rounding (a few 2^-24 of that sum)
-//     cannot turn negative.  The bounds on A and C keep the terms of a pixel
-//     distance (0, or at least 2^-25) clear of underflow and overflow.
+//   - e <= 0: rounding (a few 2^-24 of the sum of the terms' magnitudes) cannot
+//     turn a well-conditioned form negative.
 //   - the clamp at 0.99: o G stays below it when o does (G <= 1 up to the
 //     error of ex2.approx).
 //   - colour and depth are finite (and the colour small enough for its product
 //     with any image gradient the backward takes this way, see there).
 // NaN fails every comparison.
 __device__ __forceinline__ bool plain_gaussian(float4 co, float3 rgb, float depth) {
-    const float A = co.x, B = co.y, C = co.z;
-    return (A >= 1e-15f) & (A <= 1e10f) & (C >= 1e-15f) & (C <= 1e10f) & (B * B <= 0.99f * (A * C)) &
-           (co.w <= 0.989f) & (fabsf(rgb.x) + fabsf(rgb.y) + fabsf(rgb.z) <= 1e10f) & (fabsf(depth) <= 3e38f);
+    return well_conditioned(co) & (co.w <= 0.989f) & (fabsf(rgb.x) + fabsf(rgb.y) + fabsf(rgb.z) <= 1e10f) &
+           (fabsf(depth) <= 3e38f);
 }
 
 __device__ __forceinline__ Geom make_geom(float2 m, float4 co, float radius, bool plain) {
     const float4 q = exp2_coeffs(co);
     const float l2 = __log2f(255.f * co.w);  // o G >= 1/255 where the exponent is -l2 or more
-    return Geom{m.x, m.y, q.x, q.y, q.z, co.w, plain ? radius : -radius, l2 > 0.f ? l2 * 1.001f + 1e-3f : -1.f};
+    float reach = -1.f;
+    if (l2 > 0.f) {
+        reach = l2 * 1.001f + 1e-3f;
+        // What rounding may add to a pixel's exponent and take from rect_reaches'
+        // maximum: 3 2^-24 each of the terms' magnitudes, together below 2^-21 of
+        // their sum at the support's corner (rect_reaches may look up to a work
+        // item's 64 pixels past it).  At most 400 l2 2^-21 for a well-conditioned
+        // form, inside the margin above; of the order of 1 for needles of 500
+        // pixels, whose terms are a million times the exponent.
+        if (!well_conditioned(co)) {
+            const float far = radius + 64.f;
+            reach += 0x1p-21f * (fabsf(q.x) + fabsf(q.y) + fabsf(q.z)) * far * far;
+        }
+    }
+    return Geom{m.x, m.y, q.x, q.y, q.z, co.w, plain ? radius : -radius, reach};
 }
 
 // Whether a Gaussian can pass the support rule and alpha >= 1/255 at any
@@ -314,8 +334,10 @@ __device__ __forceinline__ Geom make_geom(float2 m, float4 co, float radius, boo
 // exponent is a 1D quadratic with its maximum in closed form.  (On an axis on
 // which the rectangle holds the mean there is no such edge; its candidate below
 // is then some point of the rectangle, and the mean itself when that is
-// inside.)  The margin in `reach` keeps the test a superset of what any pixel's
-// float32 evaluation lets through; a maximiser off by a relative 1e-7 (the
+// inside.)  The margin in `reach` (make_geom) keeps the test a superset of what
+// any pixel's float32 evaluation lets through, so what a pixel blends does not
+// depend on the work item it is in, and the forward and the backward, whose strips
+// may differ, blend the same pairs; a maximiser off by a relative 1e-7 (the
 // approximate reciprocals) lowers the exponent by a second-order amount, far
 // inside it.  NaN fails the first comparisons or the last.
 __device__ __forceinline__ bool rect_reaches(float sx0, float sx1, float sy0, float sy1, const Geom& g) {

@@ -224,7 +224,8 @@ __device__ __forceinline__ bool project(const Gauss& G, const ProjCam& cam, int 
     // The second needs d^T Sigma'^-1 d <= 2 ln(255 o), an ellipse whose
     // bounding box has half-widths sqrt(2 ln(255 o) Sigma'_xx) and
     // sqrt(2 ln(255 o) Sigma'_yy); the margins keep the box a superset of the
-    // pixels any float32 evaluation of alpha lets through.
+    // pixels a float32 evaluation of alpha lets through, but for needles hundreds
+    // of pixels long, whose rounded alpha may pass 1/255 some pixels past a tip.
     const float lo = logf(255.f * G.o);
     if (!(lo > 0.f)) return false;  // o <= 1/255: no pixel reaches 1/255
     const float ext = 2.f * lo * 1.001f + 1e-3f;
