@@ -542,7 +542,7 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
         needed->keys = -1;
     }
     const Count Rc = capt ? Count((unsigned long long)cap->records, dcnt) : Count(c[0]);
-    const Count Kc = capt ? Count((unsigned long long)cap->keys, dcnt + 2) : Count(c[1]);
+    const Count Kc = capt ? Count((unsigned long long)cap->keys, dcnt + 1) : Count(c[1]);
     const Count Sc = capt ? Count((unsigned long long)cap->keys, dcnt + 3) : Count(c[3]);
 
     // records by depth (the keys are the records' float32 depths, positive, so

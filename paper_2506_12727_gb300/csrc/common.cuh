@@ -51,6 +51,7 @@ struct Count {
         const unsigned long long v = *dev;
         return v < max ? v : max;
     }
+    __device__ __forceinline__ bool over() const { return dev && *dev > max; }
 };
 
 // Kernels launched with launch_chained begin while the kernel before them on the

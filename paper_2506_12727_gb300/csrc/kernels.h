@@ -109,8 +109,8 @@ void radix_sort_ids(const uint32_t* keys, const unsigned long long* sub, uint32_
 // The per-tile lists: record ids by (view, tile, depth), of one entry per
 // (record, covered tile), and every tile's [start, end).  `order`: records
 // sorted by depth; bin_off: exclusive scan of their bin counts in that order;
-// S: (record, bin) entries; K: room in `sorted` (nothing is placed, and every
-// range is empty, when the lists hold more); desc: tile descriptors
+// S: (record, bin) entries; K: entries of the lists, at most the room in `sorted`
+// (nothing is placed, and every range is empty, when there are more); desc: tile descriptors
 // (pack_tile_desc, record order).  keys_a/b and vals_a/b are scratch of S_cap
 // entries each.
 size_t tile_lists_temp_bytes(uint64_t S, long long bins, long long tiles);

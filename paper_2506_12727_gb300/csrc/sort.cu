@@ -787,16 +787,14 @@ __global__ void __launch_bounds__(64 * BS_PARTS) bin_scan_kernel(BinLists L, con
 // consecutive lanes.
 template <bool LOCAL, bool STRIDE>
 __global__ void __launch_bounds__(BC_THREADS) bin_place_kernel(BinLists L, const DevCam* cams, int V,
-                                                               const long long* ranges,
-                                                               const unsigned long long* total, Count Kc,
-                                                               uint32_t* sorted) {
+                                                               const long long* ranges, Count Kc, uint32_t* sorted) {
     chained();
     __shared__ uint32_t words[64][BC_GROUPS + 1];
     __shared__ uint32_t recs[BC_CHUNK];
     __shared__ uint32_t first[64];
     __shared__ uint16_t stage[BC_WARPS][BC_CHUNK];
     // nothing is placed when the lists do not fit (capturable mode)
-    const uint32_t chunks = *total > Kc.max ? 0u : L.chunk_off[L.bins];
+    const uint32_t chunks = Kc.over() ? 0u : L.chunk_off[L.bins];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t c = blockIdx.x;
     if (c >= chunks) return;
@@ -919,15 +917,17 @@ __global__ void __launch_bounds__(TO_THREADS) tile_order_kernel(const long long*
     }
 }
 
-// [start, end) of every tile's list.  All lists are empty when they hold more
+// [start, end) of every tile's list.  All lists are empty when they need more
 // entries than there is room for (a capturable call that ran out of key
-// capacity: nothing is placed then, so no range may point at the array).
+// capacity: nothing is placed then, so no range may point at the array).  The
+// needed count decides, not the starts: those are of the (record, bin) entries
+// that were kept, which may fill the room exactly.
 __global__ void ranges_kernel(const unsigned long long* starts, long long tiles, Count Kc,
                               long long* ranges) {
     chained();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= tiles) return;
-    const bool fits = starts[tiles] <= Kc.max;
+    const bool fits = !Kc.over();
     ranges[2 * t] = fits ? (long long)starts[t] : 0;
     ranges[2 * t + 1] = fits ? (long long)starts[t + 1] : 0;
 }
@@ -1095,7 +1095,7 @@ void tile_lists(const uint32_t* order, const uint32_t* bin_off, Count R, Count S
     if (any) {
         StageTimer timer(MVGS_STAGE_TILE_SORT, s);
 #define MVGS_PLACE(L_, T) \
-    launch_chained(bin_place_kernel<L_, T>, chunks, BC_THREADS, 0, s, L, cams, V, ranges, starts + tiles, K, sorted)
+    launch_chained(bin_place_kernel<L_, T>, chunks, BC_THREADS, 0, s, L, cams, V, ranges, K, sorted)
         const bool stride = chunks < bin_chunks(S.max, bins);
         if (local) stride ? (MVGS_PLACE(true, true)) : (MVGS_PLACE(true, false));
         else stride ? (MVGS_PLACE(false, true)) : (MVGS_PLACE(false, false));
