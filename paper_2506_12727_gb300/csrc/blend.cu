@@ -32,6 +32,7 @@
 // and adds the sum to the record with one atomic.
 #include <map>
 #include <mutex>
+#include <type_traits>
 
 #include "kernels.h"
 
@@ -169,10 +170,10 @@ struct alignas(16) FwdEntry {
     float4 qab;   // qa, qa, qb, qb
     float4 qco;   // qc, qc, -o, -o
     float4 rg;    // -r, -r, -g, -g
-    float4 brp;   // -b, -b, radius, list position (bit 31: every test of pair_eval is needed)
+    float4 brp;   // -b, -b, radius, list position (bit 31: pixel by pixel)
 };
 static_assert(sizeof(FwdEntry) == 80, "five 16-byte reads");
-constexpr uint32_t kTestAll = 0x80000000u;  // a list has fewer than 2^31 entries, one per record at most
+constexpr uint32_t kByPixel = 0x80000000u;  // a list has fewer than 2^31 entries, one per record at most
 
 // The forward looks at FWD_SCAN list entries at a time until more than FWD_FLUSH
 // of them reach the work item (or the list ends), then blends those: where few
@@ -196,8 +197,12 @@ constexpr int fwd_min_blocks(int ppt, bool extra) { return ppt == 4 && !extra ? 
 // pixel that the Gaussian does not reach blends it with alpha 0, which leaves T
 // and C as they are, bit for bit; a stopped pixel's threshold is raised out of
 // reach; the rare stop is found with one vote per Gaussian.  Gaussians for which
-// that could differ (plain_gaussian) take the pixels one by one with every
-// test.  Warp instructions per staged Gaussian (128 pixels) 109 -> 75, per 32
+// that could differ (not ordinary_gaussian) take the pixels one by one.  Batches
+// with a Gaussian that the clamp at 0.99 or a rounded exponent above 0 may touch
+// (not plain_gaussian) take a variant of the step with those two tests, two
+// instructions more per pixel: 500k x 4 views with 0, 10, 40, 100% of the
+// opacities above 0.993 618, 708, 652, 607 us, where taking those Gaussians pixel
+// by pixel cost 618, 740, 777, 879.  Warp instructions per staged Gaussian (128 pixels) 109 -> 75, per 32
 // list entries scanned 193 -> 110, L2 sectors per entry 3.1 -> 1.4 (Geom).
 // 3M Gaussians x 8 views at 32 x 64 tiles (2.1e9 blended pairs) 5.46 -> 3.13 ms,
 // 1M x 16 views at 16 x 64 3.59 -> 2.60, 500k x 4 views 0.94 -> 0.62, 2M x 5
@@ -252,9 +257,11 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, fwd_min_blocks(PPT, DEPT
         };
         const uint32_t len = (uint32_t)(end - start);  // one entry per record at most: below 2^31
         const uint32_t* list = a.sorted + start;
-        // one Gaussian that plain_gaussian lets through, on all pixels; true
-        // when the warp's last pixel has stopped (votes keep the warp together)
-        auto plain_step = [&](const FwdEntry& e, float dep) {
+        // one ordinary Gaussian on all pixels, with the tests of pair_eval that a
+        // plain one does without (TESTS); true when the warp's last pixel has
+        // stopped (votes keep the warp together)
+        auto packed_step = [&](auto tests, const FwdEntry& e, float dep) {
+            constexpr bool TESTS = decltype(tests)::value;
             const float4 em = e.m, eq = e.qab, eo = e.qco, ec = e.rg, eb = e.brp;
             const uint32_t pos1 = __float_as_uint(eb.w) + 1;
             const float radius = eb.z;
@@ -280,8 +287,12 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, fwd_min_blocks(PPT, DEPT
                 unpack2(dy, dy0, dy1);
                 unpack2(fma2(dy, fma2(qc, dy, x), xx), e0, e1);
                 unpack2(mul2(no, pack2(ex2_approx(e0), ex2_approx(e1))), v0, v1);
-                ok[k] = in0 & (fabsf(dy0) <= radius) & (v0 <= nmin[k]);
-                ok[l] = in1 & (fabsf(dy1) <= radius) & (v1 <= nmin[l]);
+                if (TESTS) {
+                    v0 = fmaxf(v0, -kAlphaMax);
+                    v1 = fmaxf(v1, -kAlphaMax);
+                }
+                ok[k] = in0 & (fabsf(dy0) <= radius) & (v0 <= nmin[k]) & (!TESTS || e0 <= 0.f);
+                ok[l] = in1 & (fabsf(dy1) <= radius) & (v1 <= nmin[l]) & (!TESTS || e1 <= 0.f);
                 na[p] = pack2(ok[k] ? v0 : 0.f, ok[l] ? v1 : 0.f);
                 om[p] = add2(na[p], one);
                 unpack2(mul2(T[p], om[p]), t0, t1);
@@ -333,12 +344,12 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, fwd_min_blocks(PPT, DEPT
             }
             return (bool)__all_sync(kFull, all_stopped());
         };
-        // any Gaussian, pixel by pixel with every test
+        // any Gaussian, pixel by pixel
         auto general_step = [&](const FwdEntry& e, float dep) {
             const float4 em = e.m, eq = e.qab, eo = e.qco, ec = e.rg, eb = e.brp;
             const float radius = eb.z;
             const float4 q = make_float4(eq.x, eq.z, eo.x, -eo.z);
-            const uint32_t pos1 = (__float_as_uint(eb.w) & ~kTestAll) + 1;
+            const uint32_t pos1 = (__float_as_uint(eb.w) & ~kByPixel) + 1;
             auto blend_one = [&](int k, float fx, float fy, float& Tk, float& c0, float& c1, float& c2, float& d) {
                 if (nmin[k] == -kStopped) return;
                 const float dx = fx + em.x;
@@ -405,7 +416,7 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, fwd_min_blocks(PPT, DEPT
             // stage the Gaussians that can reach a pixel of the work item
             __syncwarp();
             int n = 0;
-            bool odd = false;
+            bool odd = false, tests = false;
             do {
 #pragma unroll
                 for (int h = 0; h < 2; h++) {
@@ -413,12 +424,14 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, fwd_min_blocks(PPT, DEPT
                     const uint32_t bal = __ballot_sync(kFull, hit);
                     if (hit) {
                         const int slot = n + __popc(bal & lt);
-                        const bool plain = g[h].radius >= 0.f;
-                        odd |= !plain;
+                        const bool ordinary = g[h].radius >= 0.f;
+                        odd |= !ordinary;
+                        tests |= g[h].o < 0.f;
+                        const float no = -fabsf(g[h].o);
                         ent[slot].m = make_float4(-g[h].mx, -g[h].mx, -g[h].my, -g[h].my);
                         ent[slot].qab = make_float4(g[h].qa, g[h].qa, g[h].qb, g[h].qb);
-                        ent[slot].qco = make_float4(g[h].qc, g[h].qc, -g[h].o, -g[h].o);
-                        ent[slot].brp.w = __uint_as_float((b + 32 * h + lane) | (plain ? 0u : kTestAll));
+                        ent[slot].qco = make_float4(g[h].qc, g[h].qc, no, no);
+                        ent[slot].brp.w = __uint_as_float((b + 32 * h + lane) | (ordinary ? 0u : kByPixel));
                         wrid[slot] = rec[h];
                     }
                     n += __popc(bal);
@@ -446,14 +459,16 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, fwd_min_blocks(PPT, DEPT
                 }
             }
             __syncwarp();
-            if (!__any_sync(kFull, odd)) {
+            odd = __any_sync(kFull, odd);
+            if (!odd && !__any_sync(kFull, tests)) {
                 for (int j = 0; j < n; j++)
-                    if (plain_step(ent[j], DEPTH ? wdep[j] : 0.f)) break;
+                    if (packed_step(std::false_type(), ent[j], DEPTH ? wdep[j] : 0.f)) break;
             } else {
                 for (int j = 0; j < n; j++) {
                     const float dep = DEPTH ? wdep[j] : 0.f;
-                    if (__any_sync(kFull, __float_as_uint(ent[j].brp.w) >= kTestAll) ? general_step(ent[j], dep)
-                                                                                     : plain_step(ent[j], dep))
+                    if (odd && __any_sync(kFull, __float_as_uint(ent[j].brp.w) >= kByPixel)
+                            ? general_step(ent[j], dep)
+                            : packed_step(std::true_type(), ent[j], dep))
                         break;
                 }
             }
@@ -494,7 +509,7 @@ struct alignas(16) BwdEntry {
     float4 qab;   // qa, qa, qb, qb
     float4 qco;   // qc, qc, -o, -o
     float4 rg;    // r, r, g, g
-    float4 brp;   // b, b, radius, list position (bit 31: every test of pair_eval is needed)
+    float4 brp;   // b, b, radius, list position (bit 31: pixel by pixel)
 };
 
 // The lane sums of a group of Gaussians: ten rows of 32 lanes each, added up by
@@ -514,8 +529,12 @@ constexpr int bwd_min_blocks(int ppt) { return ppt == 4 ? 4 : 1; }
 // taken two at a time with packed arithmetic and without branches: a pixel that
 // the Gaussian does not reach takes part with alpha 0, which leaves T and the
 // sums as they are.  That needs finite factors: strips with an image gradient
-// that is not of ordinary size, and Gaussians that are not plain, take every
-// pixel with every test.  The steps of a group of three Gaussians follow each
+// that is not of ordinary size, and Gaussians that are not ordinary, take the
+// pixels one by one.  Batches with one that is not plain take the variant with
+// the two tests, four instructions more per pixel: 500k x 4 views with 0, 10, 40,
+// 100% of the opacities above 0.993 1328, 1376, 1274, 1178 us; 20k in three small
+// views 546, 592, 596, 618 us, where pixel by pixel they cost 548, 652, 843, 866.
+// The steps of a group of three Gaussians follow each
 // other without a branch, so one's latency hides behind the next.  A warp's
 // sums go through shared memory (ten stores a lane, 16 reads by one lane
 // per value: half the instructions of a shuffle reduction with its selects).  Every sum is
@@ -653,7 +672,8 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
         // One Gaussian on all pixels: the lane's sums over its pixels -- minus
         // dL/dpower times 1, dy, dy^2, dx, dx^2 and dx dy, minus the colour
         // gradients, the E_1 term -- into place u of the group.
-        auto plain_step = [&](const BwdEntry& e, int u) {
+        auto packed_step = [&](auto tests, const BwdEntry& e, int u) {
+            constexpr bool TESTS = decltype(tests)::value;
             const float4 em = e.m, eq = e.qab, eo = e.qco, ec = e.rg, eb = e.brp;
             const uint32_t tag = __float_as_uint(eb.w);
             const float radius = eb.z;
@@ -684,8 +704,12 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
                 unpack2(dy, dy0, dy1);
                 unpack2(fma2(dy, fma2(qc, dy, x), xx), e0, e1);
                 unpack2(mul2(no, pack2(ex2_approx(e0), ex2_approx(e1))), v0, v1);
-                const bool ok0 = in0 & (fabsf(dy0) <= radius) & (v0 <= -kAlphaMin) & (tag < last[k]);
-                const bool ok1 = in1 & (fabsf(dy1) <= radius) & (v1 <= -kAlphaMin) & (tag < last[l]);
+                if (TESTS) {
+                    v0 = fmaxf(v0, -kAlphaMax);
+                    v1 = fmaxf(v1, -kAlphaMax);
+                }
+                const bool ok0 = in0 & (fabsf(dy0) <= radius) & (v0 <= -kAlphaMin) & (tag < last[k]) & (!TESTS || e0 <= 0.f);
+                const bool ok1 = in1 & (fabsf(dy1) <= radius) & (v1 <= -kAlphaMin) & (tag < last[l]) & (!TESTS || e1 <= 0.f);
                 const f32x2 na = pack2(ok0 ? v0 : 0.f, ok1 ? v1 : 0.f);  // minus alpha
                 unpack2(add2(na, one), o0, o1);
                 const f32x2 inv = pack2(rcp_approx(o0), rcp_approx(o1));
@@ -694,7 +718,11 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
                 const f32x2 dc = fma2(d2[p], b2, fma2(d0[p], r2, mul2(d1[p], g2)));
                 const f32x2 da = fma2(T[p], dc, mul2(V[p], inv));  // dL/dalpha
                 V[p] = fma2(dc, nw, V[p]);
-                const f32x2 nd = mul2(da, na);  // minus dL/dpower
+                f32x2 nd = mul2(da, na);  // minus dL/dpower
+                if (TESTS) {  // 0 at the clamp
+                    nd.x = v0 > -kAlphaMax ? nd.x : 0.f;
+                    nd.y = v1 > -kAlphaMax ? nd.y : 0.f;
+                }
                 const f32x2 ed = mul2(nd, dy);
                 const f32x2 ax = fma2(qb, dy, t2), ay = fma2(qc2, dy, x);
                 float n0, n1, h0, h1, w0, w1;
@@ -733,13 +761,13 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
             }
             hand_over(u, Sx, P1, P0, sum(sr), sum(sg), sum(sb), E, Sxx, Sxy, P2);
         };
-        // the same for any Gaussian and gradient, pixel by pixel with every test
+        // the same for any Gaussian and gradient, pixel by pixel
         auto general_step = [&](const BwdEntry& e, int u) {
             const float4 em = e.m, eq = e.qab, eo = e.qco, ec = e.rg, eb = e.brp;
             const uint32_t tag = __float_as_uint(eb.w);
             const float radius = eb.z;
             const float4 q = make_float4(eq.x, eq.z, eo.x, -eo.z);
-            const uint32_t pos = tag & ~kTestAll;
+            const uint32_t pos = tag & ~kByPixel;
             float P0 = 0.f, P1 = 0.f, P2 = 0.f, Sx = 0.f, Sxx = 0.f, Sxy = 0.f, R = 0.f, Gn = 0.f, B = 0.f, E = 0.f;
             auto one_pixel = [&](int k, float fx, float fy, float e0, float e1, float e2, float& Tk, float& Vk) {
                 if (pos >= last[k]) return;
@@ -784,7 +812,7 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
                 T[p] = pack2(t[0], t[1]);
                 V[p] = pack2(u[0], u[1]);
             }
-            if (!SAMPLED) {  // one column per lane: the products of the sums, as in plain_step
+            if (!SAMPLED) {  // one column per lane: the products of the sums, as in packed_step
                 float f0, f1;
                 unpack2(FX[0], f0, f1);
                 const float dx0 = f0 + em.x;
@@ -803,6 +831,7 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
             // stage the Gaussians that can reach a pixel of the work item
             __syncwarp();
             int n = 0;
+            bool tests = false;
             do {
 #pragma unroll
                 for (int h = 0; h < 2; h++) {
@@ -811,10 +840,12 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
                     const uint32_t bal = __ballot_sync(kFull, hit);
                     if (hit) {
                         const int slot = n + __popc(bal & lt);
+                        tests |= g[h].o < 0.f;
+                        const float no = -fabsf(g[h].o);
                         ent[slot].m = make_float4(-g[h].mx, -g[h].mx, -g[h].my, -g[h].my);
                         ent[slot].qab = make_float4(g[h].qa, g[h].qa, g[h].qb, g[h].qb);
-                        ent[slot].qco = make_float4(g[h].qc, g[h].qc, -g[h].o, -g[h].o);
-                        ent[slot].brp.w = __uint_as_float((len - 1 - i) | (g[h].radius >= 0.f && !odd_pixels ? 0u : kTestAll));
+                        ent[slot].qco = make_float4(g[h].qc, g[h].qc, no, no);
+                        ent[slot].brp.w = __uint_as_float((len - 1 - i) | (g[h].radius >= 0.f && !odd_pixels ? 0u : kByPixel));
                         wrid[slot] = rec[h];
                     }
                     n += __popc(bal);
@@ -845,14 +876,20 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
                 ent[n + lane].m = ent[n + lane].qab = ent[n + lane].qco = ent[n + lane].rg = ent[n + lane].brp = zero;
             }
             __syncwarp();
+            tests = __any_sync(kFull, tests);
             // in groups, straight through: the steps of a group overlap
             for (int j = 0; j < n; j += BWD_GROUP) {
                 uint32_t tags = 0;
 #pragma unroll
                 for (int u = 0; u < BWD_GROUP; u++) tags |= __float_as_uint(ent[j + u].brp.w);
-                if (!__any_sync(kFull, tags >= kTestAll)) {
+                if (!__any_sync(kFull, tags >= kByPixel)) {
+                    if (!tests) {
 #pragma unroll
-                    for (int u = 0; u < BWD_GROUP; u++) plain_step(ent[j + u], u);
+                        for (int u = 0; u < BWD_GROUP; u++) packed_step(std::false_type(), ent[j + u], u);
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < BWD_GROUP; u++) packed_step(std::true_type(), ent[j + u], u);
+                    }
                 } else {
 #pragma unroll 1
                     for (int u = 0; u < BWD_GROUP; u++) general_step(ent[j + u], u);

@@ -272,8 +272,8 @@ __device__ __forceinline__ bool pair_eval(float dx, float dy, ColTerms ct, float
 struct alignas(32) Geom {
     float mx, my;        // projected mean
     float qa, qb, qc;    // base-2 exponent coefficients (exp2_coeffs)
-    float o;             // opacity
-    float radius;        // in pixels; negative: not plain (plain_gaussian)
+    float o;             // opacity; negative: blended with the tests that a plain one does without
+    float radius;        // in pixels; negative: blended pixel by pixel (ordinary_gaussian)
     float reach;         // alpha >= 1/255 needs an exponent of at least -reach (base 2), with a margin
 };
 static_assert(sizeof(Geom) == 32, "one sector");
@@ -293,21 +293,25 @@ __device__ __forceinline__ bool well_conditioned(float4 co) {
 }
 
 // Whether two tests of pair_eval cannot matter for a Gaussian, so that the
-// forward blend may leave them out, and blending it with alpha 0 changes
-// nothing:
+// packed blend steps may leave them out:
 //   - e <= 0: rounding (a few 2^-24 of the sum of the terms' magnitudes) cannot
 //     turn a well-conditioned form negative.
 //   - the clamp at 0.99: o G stays below it when o does (G <= 1 up to the
 //     error of ex2.approx).
-//   - colour and depth are finite (and the colour small enough for its product
-//     with any image gradient the backward takes this way, see there).
-// NaN fails every comparison.
-__device__ __forceinline__ bool plain_gaussian(float4 co, float3 rgb, float depth) {
-    return well_conditioned(co) & (co.w <= 0.989f) & (fabsf(rgb.x) + fabsf(rgb.y) + fabsf(rgb.z) <= 1e10f) &
-           (fabsf(depth) <= 3e38f);
+__device__ __forceinline__ bool plain_gaussian(float4 co) { return well_conditioned(co) & (co.w <= 0.989f); }
+
+// Whether blending a Gaussian with alpha 0 changes nothing, so that the packed
+// steps may take it without branches: everything they multiply with that 0 is
+// finite -- the exponent's terms and the squares of its derivatives over the
+// support (and a work item's 64 pixels past it), the colour (small enough for its
+// product with any image gradient the backward takes this way, see there) and the
+// depth.  NaN fails every comparison.
+__device__ __forceinline__ bool ordinary_gaussian(float4 co, float radius, float3 rgb, float depth) {
+    return ((fabsf(co.x) + fabsf(co.y) + fabsf(co.z)) * (radius + 64.f) <= 1e15f) & (co.w <= 1.f) &
+           (fabsf(rgb.x) + fabsf(rgb.y) + fabsf(rgb.z) <= 1e10f) & (fabsf(depth) <= 3e38f);
 }
 
-__device__ __forceinline__ Geom make_geom(float2 m, float4 co, float radius, bool plain) {
+__device__ __forceinline__ Geom make_geom(float2 m, float4 co, float radius, float3 rgb, float depth) {
     const float4 q = exp2_coeffs(co);
     const float l2 = __log2f(255.f * co.w);  // o G >= 1/255 where the exponent is -l2 or more
     float reach = -1.f;
@@ -324,7 +328,8 @@ __device__ __forceinline__ Geom make_geom(float2 m, float4 co, float radius, boo
             reach += 0x1p-21f * (fabsf(q.x) + fabsf(q.y) + fabsf(q.z)) * far * far;
         }
     }
-    return Geom{m.x, m.y, q.x, q.y, q.z, co.w, plain ? radius : -radius, reach};
+    return Geom{m.x, m.y, q.x, q.y, q.z, plain_gaussian(co) ? co.w : -co.w,
+                ordinary_gaussian(co, radius, rgb, depth) ? radius : -radius, reach};
 }
 
 // Whether a Gaussian can pass the support rule and alpha >= 1/255 at any
