@@ -533,7 +533,7 @@ constexpr int bwd_min_blocks(int ppt) { return ppt == 4 ? 4 : 1; }
 // pixels one by one.  Batches with one that is not plain take the variant with
 // the two tests, four instructions more per pixel: 500k x 4 views with 0, 10, 40,
 // 100% of the opacities above 0.993 1328, 1376, 1274, 1178 us; 20k in three small
-// views 546, 592, 596, 618 us, where pixel by pixel they cost 548, 652, 843, 866.
+// views 534, 580, 572, 576 us, where pixel by pixel they cost 548, 652, 843, 866.
 // The steps of a group of three Gaussians follow each
 // other without a branch, so one's latency hides behind the next.  A warp's
 // sums go through shared memory (ten stores a lane, 16 reads by one lane
@@ -585,7 +585,10 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
         const float sum = t[0].x + t[0].y;
         const float other = __shfl_xor_sync(kFull, sum, 1);
         float out = my_factor * sum;
-        if (my_group < k) {
+        // a Gaussian that no pixel of the strip blends has sums of 0: not added (the
+        // atomics of 20k Gaussians in three small views 546 -> 534 us, with all
+        // opaque 618 -> 576; the position takes both its sums, so it always is)
+        if (my_group < k && (my_val < 2 || sum != 0.f)) {
             const BwdEntry& e = ent[j + my_group];
             const uint32_t r = wrid[j + my_group];
             // dL/d mean = sum dL/dpower (A dx + B dy, B dx + C dy), in base-2 coefficients
