@@ -58,17 +58,6 @@ __device__ __forceinline__ int image_of(const Images& im, long long b) {
     return i;
 }
 
-// Kernel weight of neighbour q for centre p (p == q: 1).  Forward and
-// backward evaluate it with this one function.
-__device__ __forceinline__ float k3d(float px, float py, float pz, float sp, float qx, float qy, float qz, float sq,
-                                     bool same) {
-    if (same) return 1.f;
-    if (!(sp > 0.f) || !(sq > 0.f)) return 0.f;
-    const float dx = qx - px, dy = qy - py, dz = qz - pz;
-    const float d2 = dx * dx + dy * dy + dz * dz;
-    return __expf(-d2 / (2.f * sp * sp));
-}
-
 struct Blk {
     int i, H, W, x0, y0;
     long long pix;
@@ -114,15 +103,16 @@ __device__ __forceinline__ void add_tap(Sums& s, float w, f32x2 a, f32x2 q, f32x
 // Whether the fast loops below may take these values: images finite (a zero
 // weight then adds nothing), and where there is a surface point, coordinates and
 // widths far from the ends of the float range.
-constexpr float kMaxCoord = 0x1p20f, kMinWidth = 0x1p-20f, kMaxWidth = 0x1p20f;
+constexpr float kMaxCoord = 0x1p30f, kMinWidth = 0x1p-30f, kMaxWidth = 0x1p20f;
 __device__ __forceinline__ bool finite(float v) { return fabsf(v) <= FLT_MAX; }
 __device__ __forceinline__ bool in_domain(float x, float y, float z, float s) {
     if (!(s > 0.f)) return true;
     return fabsf(x) <= kMaxCoord && fabsf(y) <= kMaxCoord && fabsf(z) <= kMaxCoord && s >= kMinWidth && s <= kMaxWidth;
 }
 // A pixel without a surface point sits this far off as a neighbour, and as far on
-// the other side as a centre: its distance to any other gives a weight of zero.
-constexpr float kFar = 0x1p42f;
+// the other side as a centre: its distance to any other gives a weight of zero
+// (at least 2^63 over 2^41), and d2 y stays below 2^126.
+constexpr float kFar = 0x1p32f;
 
 // The weights of one neighbour for two centres (or of two neighbours for one
 // centre) whose squared distances are d2: exp(-d2 / c), c = 2 s^2, nc = -c, y
@@ -140,27 +130,42 @@ __device__ __forceinline__ f32x2 dist2(f32x2 dx, f32x2 dy, f32x2 dz) {
     return fma2(dz, dz, fma2(dx, dx, mul2(dy, dy)));
 }
 
-// The sums of any centre, straight from memory: for blocks whose values are out
-// of the fast loops' domain.
-__device__ __noinline__ Sums general_sums(const Blk& b, long long HW, const float* __restrict__ img,
-                                          const float* __restrict__ tgt, const float* __restrict__ pts,
-                                          const float* __restrict__ sig, int x, int y) {
-    const float* X = pts + 3 * b.pix;
-    const float* I1 = img + 3 * b.pix;
-    const float* I2 = tgt + 3 * b.pix;
-    const long long p = (long long)y * b.W + x;
-    const float px = X[p], py = X[HW + p], pz = X[2 * HW + p], sp = sig[b.pix + p];
-    Sums s{};
-    for (int yy = max(y - RAD, 0); yy <= min(y + RAD, b.H - 1); yy++) {
-        for (int xx = max(x - RAD, 0); xx <= min(x + RAD, b.W - 1); xx++) {
-            const long long o = (long long)yy * b.W + xx;
-            const float w = k3d(px, py, pz, sp, X[o], X[HW + o], X[2 * HW + o], sig[b.pix + o], o == p);
-            if (w == 0.f) continue;
-            add_tap(s, w, pack2(I1[o], I1[HW + o]), pack2(I2[o], I2[HW + o]), pack2(I1[2 * HW + o], I2[2 * HW + o]));
+// Blocks with values out of the fast loops' domain: a pixel without a surface
+// point is marked in the staged x coordinate by a NaN of its own (one that comes in
+// as a coordinate is made another), and the loops below test for it.
+__device__ __forceinline__ float no_point() { return __uint_as_float(0x7fffdeadu); }
+__device__ __forceinline__ bool is_point(float x) { return __float_as_uint(x) != 0x7fffdeadu; }
+
+// Called by every thread of the block.
+__device__ __forceinline__ void mark_points(const Blk& b, long long HW, const float* __restrict__ pts,
+                                            const float* __restrict__ sig, float (&sX)[HSY][HSX + 1]) {
+    for (int k = threadIdx.x; k < HSX * HSY; k += THREADS) {
+        const int r = k / HSX, c = k % HSX;
+        const int y = b.y0 + r - RAD, x = b.x0 + c - RAD;
+        const bool in = x >= 0 && y >= 0 && x < b.W && y < b.H;
+        const long long o = (long long)y * b.W + x;
+        float v = no_point();
+        if (in && sig[b.pix + o] > 0.f) {
+            v = pts[3 * b.pix + o];
+            if (!is_point(v)) v = __uint_as_float(0x7fffffffu);
         }
+        sX[r][c] = v;
     }
-    return s;
+    __syncthreads();
 }
+
+// The weights for any values: as above where nothing of that can leave the float
+// range, else by division.
+__device__ __forceinline__ float any_weight(float w, float d2, float c, float y) {
+    if (d2 * y > 200.f) w = 0.f;  // the correction may have been infinite
+    return c >= 0x1p-90f && c <= 0x1p120f ? w : __expf(-d2 / c);
+}
+__device__ __forceinline__ f32x2 any_weights(f32x2 d2, f32x2 nc, f32x2 y) {
+    const f32x2 w = weights(d2, nc, y);
+    return pack2(any_weight(w.x, d2.x, -nc.x, y.x), any_weight(w.y, d2.y, -nc.y, y.y));
+}
+// What has no weight may be anything.
+__device__ __forceinline__ f32x2 if_some(float w, f32x2 v) { return pack2(w != 0.f ? v.x : 0.f, w != 0.f ? v.y : 0.f); }
 
 // Bound by the FMA pipe (two thirds busy): for two pixels a neighbour takes 9
 // passes of the shared-memory unit, 9 packed instructions for both weights, two
@@ -207,9 +212,39 @@ __global__ void __launch_bounds__(THREADS) dssim3d_forward_kernel(Images im, lon
     const int x = b.x0 + lane, y = b.y0 + r0 - RAD;
     Sums s[2]{};
     if (odd) {
+        mark_points(b, HW, pts, sig, sX);
+        // the loops below with every test (a NaN in every block of a 1264 x 832 image:
+        // 540 us with the backward, without one 333)
+        float c2[2], npx[2];
+        bool point[2];
 #pragma unroll
-        for (int k = 0; k < 2; k++)
-            if (x < b.W && y + k < b.H) s[k] = general_sums(b, HW, img, tgt, pts, sig, x, y + k);
+        for (int k = 0; k < 2; k++) {
+            const float sp = x < b.W && y + k < b.H ? sig[b.pix + (long long)(y + k) * b.W + x] : -1.f;
+            point[k] = sp > 0.f;
+            c2[k] = point[k] ? 2.f * sp * sp : 1.f;
+            npx[k] = -sX[r0 + k][c0];
+        }
+        const f32x2 nx = pack2(npx[0], npx[1]), ny = pack2(-sY[r0][c0], -sY[r0 + 1][c0]),
+                    nz = pack2(-sZ[r0][c0], -sZ[r0 + 1][c0]);
+        const f32x2 nc = pack2(-c2[0], -c2[1]), yc = pack2(1.f / c2[0], 1.f / c2[1]);
+        for (int rr = r0 - RAD; rr <= r0 + RAD + 1; rr++) {
+            const bool upper = point[0] && rr <= r0 + RAD, lower = point[1] && rr > r0 - RAD;
+#pragma unroll
+            for (int du = -RAD; du <= RAD; du++) {
+                const int cc = c0 + du;
+                const float qx = sX[rr][cc], qy = sY[rr][cc], qz = sZ[rr][cc];
+                f32x2 w = any_weights(
+                    dist2(add2(pack2(qx, qx), nx), add2(pack2(qy, qy), ny), add2(pack2(qz, qz), nz)), nc, yc);
+                const bool neighbour = is_point(qx);
+                w.x = upper && neighbour ? w.x : 0.f;
+                w.y = lower && neighbour ? w.y : 0.f;
+                if (du == 0 && rr == r0) w.x = 1.f;
+                if (du == 0 && rr == r0 + 1) w.y = 1.f;
+                const f32x2 a = sA[rr][cc], q = sQ[rr][cc], ch2 = sC[rr][cc];
+                add_tap(s[0], w.x, if_some(w.x, a), if_some(w.x, q), if_some(w.x, ch2));
+                add_tap(s[1], w.y, if_some(w.y, a), if_some(w.y, q), if_some(w.y, ch2));
+            }
+        }
     } else {
         float sp[2], npx[2];
 #pragma unroll
@@ -294,28 +329,6 @@ __global__ void __launch_bounds__(THREADS) dssim3d_forward_kernel(Images im, lon
     }
 }
 
-// The gathered sums of any pixel, straight from memory.
-__device__ __noinline__ float3 general_gather(const Blk& b, long long HW, long long P, const float* __restrict__ pts,
-                                              const float* __restrict__ sig, const float* __restrict__ coef, float3 i1,
-                                              float3 i2, int x, int y) {
-    const float* X = pts + 3 * b.pix;
-    const float* C = coef + b.pix;
-    const long long q = (long long)y * b.W + x;
-    const float qx = X[q], qy = X[HW + q], qz = X[2 * HW + q], sq = sig[b.pix + q];
-    float3 g = make_float3(0.f, 0.f, 0.f);
-    for (int yy = min(y + RAD, b.H - 1); yy >= max(y - RAD, 0); yy--) {
-        for (int xx = min(x + RAD, b.W - 1); xx >= max(x - RAD, 0); xx--) {
-            const long long o = (long long)yy * b.W + xx;
-            const float w = k3d(X[o], X[HW + o], X[2 * HW + o], sig[b.pix + o], qx, qy, qz, sq, o == q);
-            if (w == 0.f) continue;
-            g.x = __fmaf_rn(w, __fmaf_rn(C[6 * P + o], i2.x, __fmaf_rn(2.f * C[3 * P + o], i1.x, C[o])), g.x);
-            g.y = __fmaf_rn(w, __fmaf_rn(C[7 * P + o], i2.y, __fmaf_rn(2.f * C[4 * P + o], i1.y, C[P + o])), g.y);
-            g.z = __fmaf_rn(w, __fmaf_rn(C[8 * P + o], i2.z, __fmaf_rn(2.f * C[5 * P + o], i1.z, C[2 * P + o])), g.z);
-        }
-    }
-    return g;
-}
-
 // Bound by shared memory (80% of its rate): 14 words per neighbour, for two
 // pixels.  One 1264 x 832 image: 272 -> 145 us.
 __global__ void __launch_bounds__(THREADS) dssim3d_backward_kernel(Images im, long long P, const float* __restrict__ img,
@@ -376,17 +389,40 @@ __global__ void __launch_bounds__(THREADS) dssim3d_backward_kernel(Images im, lo
         }
     }
     odd = __syncthreads_or(odd);
+    if (odd) mark_points(b, HW, pts, sig, sX);
     if (x >= b.W) return;
     float g[2][3] = {};
-    if (odd) {
+    if (odd) {  // the loops below with every test
+        const bool point[2] = {sq[0] > 0.f, sq[1] > 0.f};
+        const f32x2 nx = pack2(-sX[r0][c0], -sX[r0 + 1][c0]), ny = pack2(-sY[r0][c0], -sY[r0 + 1][c0]),
+                    nz = pack2(-sZ[r0][c0], -sZ[r0 + 1][c0]);
+        for (int rr = r0 + RAD + 1; rr >= r0 - RAD; rr--) {
+            const bool upper = point[0] && rr <= r0 + RAD, lower = point[1] && rr > r0 - RAD;
 #pragma unroll
-        for (int k = 0; k < 2; k++) {
-            if (y + k >= b.H) continue;
-            const float3 t = general_gather(b, HW, P, pts, sig, coef, make_float3(i1[k][0], i1[k][1], i1[k][2]),
-                                            make_float3(i2[k][0], i2[k][1], i2[k][2]), x, y + k);
-            g[k][0] = t.x;
-            g[k][1] = t.y;
-            g[k][2] = t.z;
+            for (int du = -RAD; du <= RAD; du++) {
+                const int cc = c0 - du;
+                const float px = sX[rr][cc], py = sY[rr][cc], pz = sZ[rr][cc], n = sN[rr][cc], rc = sR[rr][cc];
+                f32x2 w = any_weights(
+                    dist2(add2(pack2(px, px), nx), add2(pack2(py, py), ny), add2(pack2(pz, pz), nz)), pack2(n, n),
+                    pack2(rc, rc));
+                const bool centre = is_point(px);
+                w.x = upper && centre ? w.x : 0.f;
+                w.y = lower && centre ? w.y : 0.f;
+                if (du == 0 && rr == r0) w.x = 1.f;
+                if (du == 0 && rr == r0 + 1) w.y = 1.f;
+                const f32x2 A = sA[rr][cc], B = sB[rr][cc], C = sC[rr][cc], D = sD[rr][cc];
+                const float E = sE[rr][cc];
+#pragma unroll
+                for (int k = 0; k < 2; k++) {
+                    const float wk = k ? w.y : w.x;
+                    const float e0 = __fmaf_rn(C.x, i2[k][0], __fmaf_rn(B.x, i1[k][0], A.x)),
+                                e1 = __fmaf_rn(C.y, i2[k][1], __fmaf_rn(B.y, i1[k][1], A.y)),
+                                e2 = __fmaf_rn(E, i2[k][2], __fmaf_rn(D.y, i1[k][2], D.x));
+                    g[k][0] = __fmaf_rn(wk, wk != 0.f ? e0 : 0.f, g[k][0]);
+                    g[k][1] = __fmaf_rn(wk, wk != 0.f ? e1 : 0.f, g[k][1]);
+                    g[k][2] = __fmaf_rn(wk, wk != 0.f ? e2 : 0.f, g[k][2]);
+                }
+            }
         }
     } else {
         f32x2 u[2], v[2], G[2];
