@@ -270,9 +270,13 @@ __global__ void __launch_bounds__(THREADS) dssim3d_forward_kernel(Images im, lon
                 if (lower) add_tap(s[1], w.y, a, q, ch2);
             }
         };
-        row(r0 - RAD, true, false);
-        for (int rr = r0 - RAD + 1; rr <= r0 + RAD; rr++) row(rr, true, true);
-        row(r0 + RAD + 1, false, true);
+        // a warp of background, without a surface point, has nothing to add up (an
+        // image of it 335 -> 117 us with the backward)
+        if (__any_sync(0xffffffffu, sp[0] > 0.f || sp[1] > 0.f)) {
+            row(r0 - RAD, true, false);
+            for (int rr = r0 - RAD + 1; rr <= r0 + RAD; rr++) row(rr, true, true);
+            row(r0 + RAD + 1, false, true);
+        }
 #pragma unroll
         for (int k = 0; k < 2; k++) {
             if (sp[k] > 0.f) continue;
@@ -390,6 +394,7 @@ __global__ void __launch_bounds__(THREADS) dssim3d_backward_kernel(Images im, lo
     }
     odd = __syncthreads_or(odd);
     if (odd) mark_points(b, HW, pts, sig, sX);
+    const bool some = __any_sync(0xffffffffu, sq[0] > 0.f || sq[1] > 0.f);  // else background: nothing to add up
     if (x >= b.W) return;
     float g[2][3] = {};
     if (odd) {  // the loops below with every test
@@ -452,9 +457,11 @@ __global__ void __launch_bounds__(THREADS) dssim3d_backward_kernel(Images im, lo
                 if (lower) add(1, w.y, rr, cc);
             }
         };
-        row(r0 + RAD + 1, false, true);
-        for (int rr = r0 + RAD; rr > r0 - RAD; rr--) row(rr, true, true);
-        row(r0 - RAD, true, false);
+        if (some) {
+            row(r0 + RAD + 1, false, true);
+            for (int rr = r0 + RAD; rr > r0 - RAD; rr--) row(rr, true, true);
+            row(r0 - RAD, true, false);
+        }
 #pragma unroll
         for (int k = 0; k < 2; k++) {
             if (!(sq[k] > 0.f)) {  // no surface point: only the pixel's own window reaches it

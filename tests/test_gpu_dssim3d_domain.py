@@ -45,3 +45,13 @@ def test_large_coordinates_take_no_longer(cuda_lib):
     odd[0][0, 3::8, 7::32] = np.nan  # a pixel in every block
     general = _ms(cuda_lib, odd)
     assert far < 1.25 * plain and general < 3.0 * plain, (plain, far, general)
+
+
+def test_background_is_passed_over(cuda_lib):
+    """Pixels without a surface point have no window: an image of them takes less
+    than two thirds of the time (as much when every warp walked its windows)."""
+    arrays = _inputs(1264, 832, 8)
+    plain = _ms(cuda_lib, arrays)
+    arrays[3][:] = 0.0
+    background = _ms(cuda_lib, arrays)
+    assert background < 0.67 * plain, (plain, background)
