@@ -532,8 +532,8 @@ constexpr int bwd_min_blocks(int ppt) { return ppt == 4 ? 4 : 1; }
 // that is not of ordinary size, and Gaussians that are not ordinary, take the
 // pixels one by one.  Batches with one that is not plain take the variant with
 // the two tests, four instructions more per pixel: 500k x 4 views with 0, 10, 40,
-// 100% of the opacities above 0.993 1328, 1376, 1274, 1178 us; 20k in three small
-// views 534, 580, 572, 576 us, where pixel by pixel they cost 548, 652, 843, 866.
+// 100% of the opacities above 0.993 1308, 1376, 1267, 1160 us, where pixel by
+// pixel they cost 1341, 1397, 1440, 1383.
 // The steps of a group of three Gaussians follow each
 // other without a branch, so one's latency hides behind the next.  A warp's
 // sums go through shared memory (ten stores a lane, 16 reads by one lane
@@ -541,12 +541,13 @@ constexpr int bwd_min_blocks(int ppt) { return ppt == 4 ? 4 : 1; }
 // taken in a fixed order -- a lane's pixels one after the other, then lanes 16,
 // 8, 4, 2, 1 apart: the conic gradients of long thin Gaussians cancel to a small
 // rest, and their error is the order's.
+// With LOOK a group's alphas come first, and a group that no pixel blends is
+// passed over (launch_blend_backward says where that pays).
 // Warp instructions per staged Gaussian (128 pixels) 240 -> 180.  3M Gaussians x
-// 8 views at 32 x 64 tiles 8.44 -> 6.49 ms, 1M x 16 views at 16 x 64 7.70 ->
-// 5.47, 500k x 4 views 1.74 -> 1.34, the sampled pixels of 500k x 4 at 16 x 16
-// 1.21 -> 1.02, 10k at 128 x 128 0.224 -> 0.125.
-
-template <int PPT, bool SAMPLED>
+// 8 views at 32 x 64 tiles 8.44 -> 6.35 ms, 1M x 16 views at 16 x 64 7.70 ->
+// 5.36, 500k x 4 views 1.74 -> 1.31, the sampled pixels of 500k x 4 at 16 x 16
+// 1.21 -> 1.02, 10k at 128 x 128 0.224 -> 0.123.
+template <int PPT, bool SAMPLED, bool LOOK>
 __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
     blend_backward_kernel(BlendArgs a, int* __restrict__ counter, const float* __restrict__ dimg,
                           const float* __restrict__ final_T, const uint32_t* __restrict__ n_contrib,
@@ -672,30 +673,23 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
 #pragma unroll
             for (int i = 0; i < 10; i++) sums.v[(10 * u + i) * BwdSums::ROW + lane] = v[i];
         };
-        // One Gaussian on all pixels: the lane's sums over its pixels -- minus
-        // dL/dpower times 1, dy, dy^2, dx, dx^2 and dx dy, minus the colour
-        // gradients, the E_1 term -- into place u of the group.
-        auto packed_step = [&](auto tests, const BwdEntry& e, int u) {
+        // Minus one Gaussian's alpha at all pixels, 0 where it takes no part; with the
+        // tests of pair_eval that a plain one does without (TESTS).
+        auto packed_alpha = [&](auto tests, const BwdEntry& e, f32x2* na) {
             constexpr bool TESTS = decltype(tests)::value;
-            const float4 em = e.m, eq = e.qab, eo = e.qco, ec = e.rg, eb = e.brp;
+            const float4 em = e.m, eq = e.qab, eo = e.qco, eb = e.brp;
             const uint32_t tag = __float_as_uint(eb.w);
             const float radius = eb.z;
             const f32x2 nmx = pack2(em.x, em.y), nmy = pack2(em.z, em.w), qa = pack2(eq.x, eq.y),
-                        qb = pack2(eq.z, eq.w), qc = pack2(eo.x, eo.y), no = pack2(eo.z, eo.w),
-                        r2 = pack2(ec.x, ec.y), g2 = pack2(ec.z, ec.w), b2 = pack2(eb.x, eb.y);
-            const f32x2 qc2 = add2(qc, qc);
-            f32x2 dx{}, t2{}, xx{}, x{}, sr{}, sg{}, sb{};
-            float P0 = 0.f, P1 = 0.f, P2 = 0.f, Sx = 0.f, Sxx = 0.f, Sxy = 0.f;
+                        qb = pack2(eq.z, eq.w), qc = pack2(eo.x, eo.y), no = pack2(eo.z, eo.w);
+            f32x2 xx{}, x{};
             bool in0 = true, in1 = true;
-            float E = 0.f;
 #pragma unroll
             for (int p = 0; p < NP; p++) {
                 const int k = 2 * p, l = 2 * p + 1;
                 if (SAMPLED || p == 0) {
-                    dx = add2(FX[SAMPLED ? p : 0], nmx);
-                    const f32x2 t = mul2(qa, dx);
-                    t2 = add2(t, t);
-                    xx = mul2(t, dx);
+                    const f32x2 dx = add2(FX[SAMPLED ? p : 0], nmx);
+                    xx = mul2(mul2(qa, dx), dx);
                     x = mul2(qb, dx);
                     float dx0, dx1;
                     unpack2(dx, dx0, dx1);
@@ -703,7 +697,7 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
                     in1 = SAMPLED ? fabsf(dx1) <= radius : in0;
                 }
                 const f32x2 dy = add2(FY[p], nmy);
-                float dy0, dy1, e0, e1, v0, v1, o0, o1;
+                float dy0, dy1, e0, e1, v0, v1;
                 unpack2(dy, dy0, dy1);
                 unpack2(fma2(dy, fma2(qc, dy, x), xx), e0, e1);
                 unpack2(mul2(no, pack2(ex2_approx(e0), ex2_approx(e1))), v0, v1);
@@ -713,18 +707,44 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
                 }
                 const bool ok0 = in0 & (fabsf(dy0) <= radius) & (v0 <= -kAlphaMin) & (tag < last[k]) & (!TESTS || e0 <= 0.f);
                 const bool ok1 = in1 & (fabsf(dy1) <= radius) & (v1 <= -kAlphaMin) & (tag < last[l]) & (!TESTS || e1 <= 0.f);
-                const f32x2 na = pack2(ok0 ? v0 : 0.f, ok1 ? v1 : 0.f);  // minus alpha
-                unpack2(add2(na, one), o0, o1);
+                na[p] = pack2(ok0 ? v0 : 0.f, ok1 ? v1 : 0.f);
+            }
+        };
+        // One Gaussian with these on all pixels: the lane's sums over its pixels -- minus
+        // dL/dpower times 1, dy, dy^2, dx, dx^2 and dx dy, minus the colour
+        // gradients, the E_1 term -- into place u of the group.
+        auto packed_step = [&](auto tests, const BwdEntry& e, int u, const f32x2* na) {
+            constexpr bool TESTS = decltype(tests)::value;
+            const float4 em = e.m, eq = e.qab, eo = e.qco, ec = e.rg, eb = e.brp;
+            const f32x2 nmx = pack2(em.x, em.y), nmy = pack2(em.z, em.w), qa = pack2(eq.x, eq.y),
+                        qb = pack2(eq.z, eq.w), qc = pack2(eo.x, eo.y), r2 = pack2(ec.x, ec.y),
+                        g2 = pack2(ec.z, ec.w), b2 = pack2(eb.x, eb.y);
+            const f32x2 qc2 = add2(qc, qc);
+            f32x2 dx{}, t2{}, x{}, sr{}, sg{}, sb{};
+            float P0 = 0.f, P1 = 0.f, P2 = 0.f, Sx = 0.f, Sxx = 0.f, Sxy = 0.f;
+            float E = 0.f;
+#pragma unroll
+            for (int p = 0; p < NP; p++) {
+                if (SAMPLED || p == 0) {
+                    dx = add2(FX[SAMPLED ? p : 0], nmx);
+                    const f32x2 t = mul2(qa, dx);
+                    t2 = add2(t, t);
+                    x = mul2(qb, dx);
+                }
+                const f32x2 dy = add2(FY[p], nmy);
+                float dy0, dy1, o0, o1;
+                unpack2(dy, dy0, dy1);
+                unpack2(add2(na[p], one), o0, o1);
                 const f32x2 inv = pack2(rcp_approx(o0), rcp_approx(o1));
                 T[p] = mul2(T[p], inv);  // transmittance in front of this Gaussian
-                const f32x2 nw = mul2(na, T[p]);
+                const f32x2 nw = mul2(na[p], T[p]);
                 const f32x2 dc = fma2(d2[p], b2, fma2(d0[p], r2, mul2(d1[p], g2)));
                 const f32x2 da = fma2(T[p], dc, mul2(V[p], inv));  // dL/dalpha
                 V[p] = fma2(dc, nw, V[p]);
-                f32x2 nd = mul2(da, na);  // minus dL/dpower
-                if (TESTS) {  // 0 at the clamp
-                    nd.x = v0 > -kAlphaMax ? nd.x : 0.f;
-                    nd.y = v1 > -kAlphaMax ? nd.y : 0.f;
+                f32x2 nd = mul2(da, na[p]);  // minus dL/dpower
+                if (TESTS) {  // none at the clamp
+                    nd.x = na[p].x > -kAlphaMax ? nd.x : 0.f;
+                    nd.y = na[p].y > -kAlphaMax ? nd.y : 0.f;
                 }
                 const f32x2 ed = mul2(nd, dy);
                 const f32x2 ax = fma2(qb, dy, t2), ay = fma2(qc2, dy, x);
@@ -886,12 +906,34 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK, bwd_min_blocks(PPT))
 #pragma unroll
                 for (int u = 0; u < BWD_GROUP; u++) tags |= __float_as_uint(ent[j + u].brp.w);
                 if (!__any_sync(kFull, tags >= kByPixel)) {
+                    f32x2 na[BWD_GROUP][NP];
+                    if (LOOK) {  // groups that no pixel blends are passed over
+                        if (!tests) {
+#pragma unroll
+                            for (int u = 0; u < BWD_GROUP; u++) packed_alpha(std::false_type(), ent[j + u], na[u]);
+                        } else {
+#pragma unroll
+                            for (int u = 0; u < BWD_GROUP; u++) packed_alpha(std::true_type(), ent[j + u], na[u]);
+                        }
+                        float least = 0.f;
+#pragma unroll
+                        for (int u = 0; u < BWD_GROUP; u++)
+#pragma unroll
+                            for (int p = 0; p < NP; p++) least = fminf(least, fminf(na[u][p].x, na[u][p].y));
+                        if (!__any_sync(kFull, least < 0.f)) continue;
+                    }
                     if (!tests) {
 #pragma unroll
-                        for (int u = 0; u < BWD_GROUP; u++) packed_step(std::false_type(), ent[j + u], u);
+                        for (int u = 0; u < BWD_GROUP; u++) {
+                            if (!LOOK) packed_alpha(std::false_type(), ent[j + u], na[u]);
+                            packed_step(std::false_type(), ent[j + u], u, na[u]);
+                        }
                     } else {
 #pragma unroll
-                        for (int u = 0; u < BWD_GROUP; u++) packed_step(std::true_type(), ent[j + u], u);
+                        for (int u = 0; u < BWD_GROUP; u++) {
+                            if (!LOOK) packed_alpha(std::true_type(), ent[j + u], na[u]);
+                            packed_step(std::true_type(), ent[j + u], u, na[u]);
+                        }
                     }
                 } else {
 #pragma unroll 1
@@ -1004,21 +1046,35 @@ void launch_blend_forward(const BlendArgs& a, int* counter, float* img, float* f
     note_launches(1);
 }
 
+// Strips up to which the backward looks at a group's alphas before it takes the
+// group.  A strip's list is walked by one warp, and the longest walks are what is
+// waited for when there are few strips, or when they are small (up to 2 pixels per
+// lane: tiles 8 high) or thinned out (a pixel mask): most of a list's Gaussians
+// then reach the strip but no pixel of it.  375k Gaussians on 64 views of some
+// 200 x 200 65 -> 32 ms, 921k x 9 views at 8 x 8 tiles 38 -> 18, 25k x 8 small
+// views at 16 x 8 1.10 -> 0.68, 20k x 3 534 -> 493 us; where every group is blended
+// it costs 3% (10k at 128 x 128 118 -> 123 us), so not for the large renders of
+// tall tiles (sampled pixels of 500k x 4 views 1028 -> 1107).
+constexpr long long kFewStrips = 7500;
+
 void launch_blend_backward(const BlendArgs& a, int* counter, const float* dimg, const float* final_T,
                            const uint32_t* n_contrib, float* rec_grad, double* rec_conic, cudaStream_t s) {
     if (a.tiles == 0) return;
     cudaMemsetAsync(counter, 0, sizeof(int), s);
     const bool sampled = a.s_off != nullptr;
     const long long items = sampled ? (1LL << 40) : a.tiles * a.strips;
-#define MVGS_BB(P, S)                                                                                      \
-    blend_backward_kernel<P, S><<<grid_for(blend_backward_kernel<P, S>, items), 32 * WARPS_PER_BLOCK, 0, s>>>( \
+#define MVGS_BB(P, S, L)                                                                                         \
+    blend_backward_kernel<P, S, L><<<grid_for(blend_backward_kernel<P, S, L>, items), 32 * WARPS_PER_BLOCK, 0, s>>>( \
         a, counter, dimg, final_T, n_contrib, rec_grad, rec_conic)
-#define MVGS_BB2(P) if (sampled) MVGS_BB(P, true); else MVGS_BB(P, false)
+#define MVGS_BB2(P, L) if (sampled) MVGS_BB(P, true, L); else MVGS_BB(P, false, L)
     switch (a.ppt) {
-        case 1: MVGS_BB2(1); break;
-        case 2: MVGS_BB2(2); break;
-        case 8: MVGS_BB2(8); break;
-        default: MVGS_BB2(4); break;
+        case 1: MVGS_BB2(1, true); break;
+        case 2: MVGS_BB2(2, true); break;
+        case 8: MVGS_BB2(8, true); break;
+        default:
+            if (a.pixel_mask || a.tiles * a.strips <= kFewStrips) MVGS_BB2(4, true);
+            else MVGS_BB2(4, false);
+            break;
     }
 #undef MVGS_BB2
 #undef MVGS_BB
