@@ -592,7 +592,9 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
     ba.V = V;
     ba.tw = tw;
     ba.th = th;
-    ba.ppt = smp ? blend_pixels_per_thread(tw, th, cfg->pixels_per_thread)
+    // (a run of samples has the backward's pixels per lane)
+    ba.ppt = smp && !(cfg->flags & MVGS_FLAG_MASKED_PARTIAL)
+                 ? blend_pixels_per_thread(tw, th, cfg->pixels_per_thread)
                  : blend_forward_pixels_per_thread(tw, th, cfg->pixels_per_thread, P.tiles);
     ba.sw = blend_strip_width(tw);
     ba.strip_h = (32 / ba.sw) * ba.ppt;

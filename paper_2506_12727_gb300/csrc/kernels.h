@@ -157,7 +157,7 @@ struct BlendArgs {
 int blend_strip_width(int tw);
 // Pixels per lane for a tile size (req > 0: the caller's choice, checked).
 int blend_pixels_per_thread(int tw, int th, int req);
-// of a forward over all pixels
+// of a forward over whole strips
 int blend_forward_pixels_per_thread(int tw, int th, int req, long long tiles);
 // Persistent launches; `counter` is one device int of scratch (0 for the forward,
 // reset by the backward).
