@@ -1054,7 +1054,9 @@ void launch_blend_forward(const BlendArgs& a, int* counter, float* img, float* f
 // 200 x 200 65 -> 32 ms, 921k x 9 views at 8 x 8 tiles 38 -> 18, 25k x 8 small
 // views at 16 x 8 1.10 -> 0.68, 20k x 3 534 -> 493 us; where every group is blended
 // it costs 3% (10k at 128 x 128 118 -> 123 us), so not for the large renders of
-// tall tiles (sampled pixels of 500k x 4 views 1028 -> 1107).
+// tall tiles (sampled pixels of 500k x 4 views 1028 -> 1107).  Sampled pixels fill
+// a part of the strips (a quarter of them with four views to a group), so their
+// line lies four times as far (61k Gaussians on 64 small views 4.98 -> 2.93 ms).
 constexpr long long kFewStrips = 7500;
 
 void launch_blend_backward(const BlendArgs& a, int* counter, const float* dimg, const float* final_T,
@@ -1072,7 +1074,7 @@ void launch_blend_backward(const BlendArgs& a, int* counter, const float* dimg, 
         case 2: MVGS_BB2(2, true); break;
         case 8: MVGS_BB2(8, true); break;
         default:
-            if (a.pixel_mask || a.tiles * a.strips <= kFewStrips) MVGS_BB2(4, true);
+            if (a.pixel_mask || a.tiles * a.strips <= (sampled ? 4 : 1) * kFewStrips) MVGS_BB2(4, true);
             else MVGS_BB2(4, false);
             break;
     }
