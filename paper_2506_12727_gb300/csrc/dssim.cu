@@ -89,8 +89,11 @@ __device__ __forceinline__ BlockPos block_pos(const Views& vw) {
 // is the tile's own, so results do not depend on the runs; packed arithmetic (I1
 // and I2 side by side) saves a fifth of the instructions but its 64-bit column
 // reads conflict, 357 us.
+// Where runs are of one tile (RUNS false: up to 3648 tiles of 32 x 32) that
+// only cost: 16 small views (0.85 Mpixel) 99 us with a tile per block, 109 with the ring.
 constexpr int HALO = 2 * RADIUS;
-__device__ __forceinline__ int ring(int row) { return row < HSY ? row : row - HSY; }
+template <bool RUNS>
+__device__ __forceinline__ int ring(int row) { return !RUNS || row < HSY ? row : row - HSY; }
 static_assert(TSY * (TSX / 4) == 256, "one item per thread");
 
 // The rows that the tile below y0 adds, fetched asynchronously (the caller waits
@@ -134,6 +137,7 @@ __device__ __forceinline__ void stage_rows(const float* const (&src)[NP], const 
     }
 }
 
+template <bool RUNS>
 __global__ void __launch_bounds__(256) dssim_forward_kernel(Views vw, const float* __restrict__ img,
                                                            const float* __restrict__ tgt,
                                                            float* __restrict__ dm1, float* __restrict__ dm11,
@@ -155,15 +159,16 @@ __global__ void __launch_bounds__(256) dssim_forward_kernel(Views vw, const floa
     };
     stage_rows(src, p, p.ty0 * TSY, s);
     int base = 0;  // ring position of the tile's first staged row
-    for (int ty = p.ty0; ty < p.ty1; ty++) {
-        const int y0 = ty * TSY, skip = ty == p.ty0 ? 0 : HALO;
-        cp_async_wait<0>();
+    int ty = p.ty0;
+    do {
+        const int y0 = ty * TSY, skip = !RUNS || ty == p.ty0 ? 0 : HALO;
+        if (RUNS) cp_async_wait<0>();
         __syncthreads();
-        if (ty > p.ty0 && threadIdx.x == 0) put_sums(ty - 1);
+        if (RUNS && ty > p.ty0 && threadIdx.x == 0) put_sums(ty - 1);
         // row pass, four adjacent outputs per item: their 14 inputs come in four
         // 16-byte reads instead of 44 scalar ones
         for (int i = threadIdx.x; i < (HSY - skip) * (TSX / 4); i += 256) {
-            const int r = i / (TSX / 4), c0 = 4 * (i % (TSX / 4)), hr = ring(base + skip + r);
+            const int r = i / (TSX / 4), c0 = 4 * (i % (TSX / 4)), hr = ring<RUNS>(base + skip + r);
             float x1[16], x2[16];
 #pragma unroll
             for (int q = 0; q < 4; q++) {
@@ -189,7 +194,7 @@ __global__ void __launch_bounds__(256) dssim_forward_kernel(Views vw, const floa
             }
         }
         __syncthreads();
-        if (ty + 1 < p.ty1) fetch_rows(src, p, y0, s);  // the row pass is done with them
+        if (RUNS && ty + 1 < p.ty1) fetch_rows(src, p, y0, s);  // the row pass is done with them
         float ssim = 0.f, l1 = 0.f;
         const int c = threadIdx.x % TSX;
         // a thread's ROWS consecutive output rows share ROWS + TAPS - 1 staged rows:
@@ -204,7 +209,7 @@ __global__ void __launch_bounds__(256) dssim_forward_kernel(Views vw, const floa
         for (int k = 0; k < ROWS + TAPS - 1; k++) {
             float hv[5];
 #pragma unroll
-            for (int i = 0; i < 5; i++) hv[i] = h[i][ring(base + r0 + k)][c];
+            for (int i = 0; i < 5; i++) hv[i] = h[i][ring<RUNS>(base + r0 + k)][c];
 #pragma unroll
             for (int q = 0; q < ROWS; q++) {
                 const int t = k - q;
@@ -233,7 +238,7 @@ __global__ void __launch_bounds__(256) dssim_forward_kernel(Views vw, const floa
                 dm1[o] = 2.f * (m2 * (a2 - a1) * q + m1 * sv * (ib2 - ib1));
                 dm11[o] = -sv * ib2;
                 dm12[o] = 2.f * a1 * q;
-                l1 += fabsf(img[o] - tgt[o]);
+                l1 += RUNS ? fabsf(img[o] - tgt[o]) : fabsf(s[0][r + RADIUS][c + RADIUS] - s[1][r + RADIUS][c + RADIUS]);
             }
         }
         // block sums of SSIM and |I1 - I2|
@@ -246,12 +251,13 @@ __global__ void __launch_bounds__(256) dssim_forward_kernel(Views vw, const floa
             red[0][threadIdx.x >> 5] = ssim;
             red[1][threadIdx.x >> 5] = l1;
         }
-        base = ring(base + TSY);
-    }
+        if (RUNS) base = ring<RUNS>(base + TSY);
+    } while (RUNS && ++ty < p.ty1);
     __syncthreads();
-    if (threadIdx.x == 0) put_sums(p.ty1 - 1);
+    if (threadIdx.x == 0) put_sums(RUNS ? p.ty1 - 1 : p.ty0);
 }
 
+template <bool RUNS>
 __global__ void __launch_bounds__(256) dssim_backward_kernel(Views vw, const float* __restrict__ img,
                                                             const float* __restrict__ tgt,
                                                             const float* __restrict__ dm1,
@@ -264,12 +270,13 @@ __global__ void __launch_bounds__(256) dssim_backward_kernel(Views vw, const flo
     const float* const src[3] = {dm1, dm11, dm12};
     stage_rows(src, p, p.ty0 * TSY, s);
     int base = 0;
-    for (int ty = p.ty0; ty < p.ty1; ty++) {
-        const int y0 = ty * TSY, skip = ty == p.ty0 ? 0 : HALO;
-        cp_async_wait<0>();
+    int ty = p.ty0;
+    do {
+        const int y0 = ty * TSY, skip = !RUNS || ty == p.ty0 ? 0 : HALO;
+        if (RUNS) cp_async_wait<0>();
         __syncthreads();
         for (int i = threadIdx.x; i < (HSY - skip) * (TSX / 4); i += 256) {
-            const int r = i / (TSX / 4), c0 = 4 * (i % (TSX / 4)), hr = ring(base + skip + r);
+            const int r = i / (TSX / 4), c0 = 4 * (i % (TSX / 4)), hr = ring<RUNS>(base + skip + r);
             float x[3][16];
 #pragma unroll
             for (int m = 0; m < 3; m++)
@@ -293,7 +300,7 @@ __global__ void __launch_bounds__(256) dssim_backward_kernel(Views vw, const flo
             }
         }
         __syncthreads();
-        if (ty + 1 < p.ty1) fetch_rows(src, p, y0, s);
+        if (RUNS && ty + 1 < p.ty1) fetch_rows(src, p, y0, s);
         const int c = threadIdx.x % TSX;
         const float inv_n = 1.f / (3.f * (float)p.H * (float)p.W);
         const int r0 = (threadIdx.x / TSX) * ROWS;
@@ -311,7 +318,7 @@ __global__ void __launch_bounds__(256) dssim_backward_kernel(Views vw, const flo
         for (int q = 0; q < ROWS; q++) bv[q][0] = bv[q][1] = bv[q][2] = 0.f;
 #pragma unroll
         for (int k = 0; k < ROWS + TAPS - 1; k++) {
-            const int hr = ring(base + r0 + k);
+            const int hr = ring<RUNS>(base + r0 + k);
             const float h0 = h[0][hr][c], h1 = h[1][hr][c], h2 = h[2][hr][c];
 #pragma unroll
             for (int q = 0; q < ROWS; q++) {
@@ -336,8 +343,8 @@ __global__ void __launch_bounds__(256) dssim_backward_kernel(Views vw, const flo
             const float dssim = B1 + 2.f * i1[q] * B11 + i2[q] * B12;
             dimg[o] = inv_views * inv_n * ((1.f - lambda) * sgn - lambda * dssim);
         }
-        base = ring(base + TSY);
-    }
+        if (RUNS) base = ring<RUNS>(base + TSY);
+    } while (RUNS && ++ty < p.ty1);
 }
 
 __global__ void dssim_reduce_kernel(Views vw, const float2* __restrict__ bsum, long long blk_offset, float lambda,
@@ -444,11 +451,12 @@ void launch_dssim(const float* img, const float* target, const int* hw, int V, f
         const Views vw = make_views(hw, first, count);
         const long long nb = vw.blk[count], ctas = vw.cta[count];
         if (nb > 0) {
-            dssim_forward_kernel<<<(unsigned)ctas, 256, 0, s>>>(vw, img, target, dm1, dm11, dm12, bsum, blk_offset);
+            const auto forward = ctas < nb ? dssim_forward_kernel<true> : dssim_forward_kernel<false>;
+            const auto backward = ctas < nb ? dssim_backward_kernel<true> : dssim_backward_kernel<false>;
+            forward<<<(unsigned)ctas, 256, 0, s>>>(vw, img, target, dm1, dm11, dm12, bsum, blk_offset);
             note_launches(1);
             if (dimg)
-                dssim_backward_kernel<<<(unsigned)ctas, 256, 0, s>>>(vw, img, target, dm1, dm11, dm12, lambda,
-                                                                   1.f / (float)V, dimg);
+                backward<<<(unsigned)ctas, 256, 0, s>>>(vw, img, target, dm1, dm11, dm12, lambda, 1.f / (float)V, dimg);
             if (dimg) note_launches(1);
         }
         dssim_reduce_kernel<<<count, 256, 0, s>>>(vw, bsum, blk_offset, lambda, loss_per_view);
