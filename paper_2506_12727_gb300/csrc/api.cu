@@ -112,6 +112,7 @@ struct Carver {
         off = align256(off + bytes);
         return o;
     }
+    void reach(const Carver& c) { off = off > c.off ? off : c.off; }
 };
 
 struct Plan {
@@ -227,23 +228,36 @@ mvgs_status make_plan(long long n, const mvgs_camera* cams, int V, const mvgs_co
 
     Carver w;
     P.w_cams = w.take((size_t)V * sizeof(DevCam));
-    P.w_counts = w.take((size_t)(n > 0 ? n : 1) * sizeof(int));
-    P.w_vis = w.take((size_t)(n > 0 ? n : 1) * V);
     const size_t big = R > K ? R : K;
     P.w_scan = w.take(scan_temp_bytes(big > (size_t)n ? big : (size_t)n));
-    P.w_dkeys_a = w.take(R * sizeof(uint32_t));
-    P.w_dkeys_b = w.take(R * sizeof(uint32_t));
-    P.w_ids_a = w.take(R * sizeof(uint32_t));
-    P.w_ids_b = w.take(R * sizeof(uint32_t));
-    P.w_order = w.take(R * sizeof(uint32_t));
-    P.w_bins = w.take(R * sizeof(uint32_t));
-    P.w_desc = w.take(R * sizeof(unsigned long long));
-    P.w_bins_by_depth = w.take(R * sizeof(uint32_t));
-    P.w_bin_off = w.take((R + 1) * sizeof(uint32_t));
+    // Two zones that are used twice.  The first: the records' bin counts, with the
+    // participation beside them until the records are there and the depth sort's
+    // arrays after that; then the (record, bin) entries as they are generated.
+    Carver z1{w.off};
+    P.w_bins = z1.take(R * sizeof(uint32_t));
+    Carver part = z1;
+    P.w_counts = part.take((size_t)(n > 0 ? n : 1) * sizeof(int));
+    P.w_vis = part.take((size_t)(n > 0 ? n : 1) * V);
+    P.w_dkeys_a = z1.take(R * sizeof(uint32_t));
+    P.w_dkeys_b = z1.take(R * sizeof(uint32_t));
+    P.w_ids_a = z1.take(R * sizeof(uint32_t));
+    P.w_ids_b = z1.take(R * sizeof(uint32_t));
+    P.w_bins_by_depth = z1.take(R * sizeof(uint32_t));
     P.w_keys_a = w.take(K * sizeof(uint32_t));
-    P.w_keys_b = w.take(K * sizeof(uint32_t));
     P.w_vals_a = w.take(K * sizeof(uint32_t));
+    w.reach(z1);
+    w.reach(part);
+    // The second: what the entries are generated from; then their other half in the
+    // passes by bin.
+    const bool keep_desc = tile_lists_keep_desc(bins);
+    if (keep_desc) P.w_desc = w.take(R * sizeof(unsigned long long));
+    Carver z2{w.off};
+    P.w_order = z2.take(R * sizeof(uint32_t));
+    P.w_bin_off = z2.take((R + 1) * sizeof(uint32_t));
+    if (!keep_desc) P.w_desc = z2.take(R * sizeof(unsigned long long));
+    P.w_keys_b = w.take(K * sizeof(uint32_t));
     P.w_vals_b = w.take(K * sizeof(uint32_t));
+    w.reach(z2);
     P.w_radix = w.take(radix_temp_bytes(big));
     // every (record, bin) entry holds at least one tile: at most K of them
     P.w_lists = w.take(tile_lists_temp_bytes(K, bins, tiles));

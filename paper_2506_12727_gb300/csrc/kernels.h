@@ -114,6 +114,9 @@ void radix_sort_ids(const uint32_t* keys, const unsigned long long* sub, uint32_
 // (pack_tile_desc, record order).  keys_a/b and vals_a/b are scratch of S_cap
 // entries each.
 size_t tile_lists_temp_bytes(uint64_t S, long long bins, long long tiles);
+// Whether `desc` is read after the first write to keys_b / vals_b (else those,
+// and `order` and `bin_off`, may share their memory).
+bool tile_lists_keep_desc(long long bins);
 void tile_lists(const uint32_t* order, const uint32_t* bin_off, Count R, Count S, Count K,
                 const unsigned long long* desc, const DevCam* cams, int V, long long bins, long long tiles,
                 uint32_t* keys_a, uint32_t* vals_a, uint32_t* keys_b, uint32_t* vals_b, uint32_t* sorted,

@@ -1035,6 +1035,8 @@ T* part(void* tmp, size_t off) { return reinterpret_cast<T*>(static_cast<char*>(
 
 size_t tile_lists_temp_bytes(uint64_t S, long long bins, long long tiles) { return BinTemp(S, bins, tiles).bytes; }
 
+bool tile_lists_keep_desc(long long bins) { return bins > BIN_LOCAL_MAX; }
+
 void tile_lists(const uint32_t* order, const uint32_t* bin_off, Count R, Count S, Count K,
                 const unsigned long long* desc, const DevCam* cams, int V, long long bins, long long tiles,
                 uint32_t* keys_a, uint32_t* vals_a, uint32_t* keys_b, uint32_t* vals_b, uint32_t* sorted,
@@ -1043,7 +1045,7 @@ void tile_lists(const uint32_t* order, const uint32_t* bin_off, Count R, Count S
     uint32_t* tile_counts = part<uint32_t>(tmp, T.tile_counts);
     unsigned long long* starts = part<unsigned long long>(tmp, T.starts);
     const bool any = S.max > 0 && R.max > 0;
-    const bool local = bins <= BIN_LOCAL_MAX;
+    const bool local = !tile_lists_keep_desc(bins);
     BinLists L{};
     const auto grid = [&](uint64_t blocks) { return (unsigned)(S.dev && blocks > GRID_CAP ? GRID_CAP : blocks); };
     const unsigned chunks = grid(bin_chunks(S.max, bins));
