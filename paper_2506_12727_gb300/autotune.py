@@ -1,12 +1,12 @@
-"""Tile-size / pixels-per-thread / shared-memory-batch autotuner for the
-rasterizer.
+"""Tile-size / pixels-per-thread autotuner for the rasterizer.
 
 The tile size decides how many (Gaussian, tile) entries are sorted; the strip
-shape decides how the blend kernels spread a tile over warps; the batch was how
-many Gaussians a warp stages in shared memory at a time (the kernels size that
-themselves now, so batches tie).  None of them changes the rendered image.  `autotune` times one forward + backward of each candidate
+shape decides how the blend kernels spread a tile over warps.  Neither changes
+the rendered image.  `autotune` times one forward + backward of each candidate
 on the caller's scene and cameras (CUDA events, after one warm-up) and returns
 the fastest; results are cached per (Gaussians, view resolutions) signature.
+(Candidates and the result carry a third value, the shared-memory batch, which
+the library still checks but no longer uses: 0, automatic.)
 """
 from __future__ import annotations
 
@@ -14,10 +14,10 @@ import torch
 
 from . import mvgs
 
-# (tile, pixels per lane (0: automatic), Gaussians per shared-memory batch (0: automatic))
+# (tile, pixels per lane (0: automatic), shared-memory batch (0: automatic; nothing depends on it))
 CANDIDATES = (
     ((16, 16), 0, 0), ((16, 32), 0, 0), ((16, 32), 2, 0), ((32, 32), 0, 0), ((16, 64), 0, 0), ((16, 64), 2, 0),
-    ((16, 64), 0, 64), ((16, 64), 0, 192), ((32, 64), 0, 0), ((32, 64), 0, 64), ((32, 64), 0, 192), ((32, 16), 0, 0),
+    ((32, 64), 0, 0), ((32, 16), 0, 0),
 )
 
 _cache: dict = {}
