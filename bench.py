@@ -61,7 +61,7 @@ def parse():
     ap.add_argument("--workload", default=WORKLOAD)
     ap.add_argument("--tile", default="auto", help="WxH, or auto (timed choice before the measured steps)")
     ap.add_argument("--ppt", type=int, default=0, help="blend pixels per thread (0 = automatic)")
-    ap.add_argument("--smem-batch", type=int, default=0, help="Gaussians per shared-memory batch (0 = automatic)")
+    ap.add_argument("--smem-batch", type=int, default=0, help="0, 64, 128 or 192: checked by the library, without effect")
     ap.add_argument("--no-loop", action="store_true", help="skip the per-view launch loop")
     ap.add_argument("--no-cpu", action="store_true", help="skip the CPU oracle baseline")
     ap.add_argument("--no-e2e", action="store_true", help="skip the end-to-end (host buffers) measurement")
@@ -704,7 +704,7 @@ def run_serving(args, torch, mvgs):
                    "mean_views_per_batch": float(np.mean([b[1] for b in log])) if log else 0,
                    # per batch: device time of the render call (CUDA events on the
                    # worker's stream) and host time from taking the batch to its
-                   # completion (adds the two count read-backs' waits, launches and
+                   # completion (adds the count read-back's wait, launches and
                    # the Python around the call)
                    "batch_device_ms_mean": float(np.mean([b[4] for b in log])) if log else 0,
                    "batch_host_ms_mean": float(np.mean([b[5] for b in log])) if log else 0})
@@ -735,9 +735,9 @@ def stage_work(rz, needed, V, pixels, blended):
     bits = max(1, int(np.ceil(np.log2(max(tiles, 2)))))
     passes = max(1, (bits + 7) // 8)
     vb = max(1, int(R - 1).bit_length())  # record-id bits
-    # the measure of the tile sort's work: the bytes a radix sort of all (record,
-    # tile) entries moves, so that its fraction stays comparable (the lists are
-    # built through coarser bins and move fewer bytes than this)
+    # tile_sort: the bytes of a radix sort of all (record, tile) entries, a measure
+    # of the task; list_work has those of the kernels that run, which the reported
+    # rates are taken from
     if passes == 2 and (bits - 8) + vb <= 32:
         # packed two passes: a 16-bit tile id and a record id generated, read
         # and written as one word, which is read twice (histogram, scatter) and
@@ -748,7 +748,7 @@ def stage_work(rz, needed, V, pixels, blended):
     return {
         "count_visible": ("hbm", 44.0 * n + 4.0 * n + n * V, "B"),
         "scan_records": ("hbm", 12.0 * n, "B"),
-        "preprocess": ("hbm", 236.0 * n + n * V + 8.0 * n + 76.0 * R, "B"),
+        "preprocess": ("hbm", 236.0 * n + n * V + 8.0 * n + 108.0 * R, "B"),
         "depth_sort": ("hbm", 4 * 16.0 * R, "B"),
         "scan_tiles": ("hbm", 12.0 * R, "B"),
         "tile_sort": ("hbm", tile_sort_bytes, "B"),
@@ -756,10 +756,41 @@ def stage_work(rz, needed, V, pixels, blended):
         "blend_forward": ("alu", FWD_FLOP_PER_BLENDED * blended, "FLOP"),
         "zero_grads": ("hbm", 56.0 * R, "B"),  # 8 float and 3 double slots per record
         "blend_backward": ("alu", BWD_FLOP_PER_BLENDED * blended, "FLOP"),
-        "preprocess_backward": ("hbm", 472.0 * n + 76.0 * R, "B"),
+        "preprocess_backward": ("hbm", 472.0 * n + 80.0 * R, "B"),
         "dssim": ("hbm", 44.0 * 3 * pixels, "B"),
         "adc": ("hbm", 12.0 * R + 32.0 * n, "B"),
     }, blended
+
+
+def list_work(rz, needed):
+    """Bytes that the kernels building the tile lists move (see stage_work): every
+    radix pass reads its keys twice (histogram, scatter) and its values, and writes
+    both; entries are (record, bin) pairs, a bin being 8 x 8 tiles of a view."""
+    import torch
+    R, K = needed
+    rec = rz.records()
+    rc = rec["rect"].to(torch.int32)
+    some = (rc[:, 2] > rc[:, 0]) & (rc[:, 3] > rc[:, 1])
+    across = ((rc[:, 2] - 1) >> 3) - (rc[:, 0] >> 3) + 1
+    down = ((rc[:, 3] - 1) >> 3) - (rc[:, 1] >> 3) + 1
+    S = int((across * down * some).sum(dtype=torch.int64).item())
+    bits = rec["depth"].view(torch.int32)
+    spread = int(bits.max().item()) - int(bits.min().item()) if R else 0
+    passes = max(1, (spread.bit_length() + 7) // 8)
+    # the first pass makes its ids, the last writes no keys but carries the bin counts
+    depth = 20.0 * R if passes == 1 else (16.0 + 20.0 * (passes - 2) + 24.0) * R
+    tw, th = rz.cfg.tile_w, rz.cfg.tile_h
+    bins = sum((-(-int(w) // tw) + 7) // 8 * ((-(-int(h) // th) + 7) // 8)
+               for w, h in zip(rz.cams_np.width, rz.cams_np.height))
+    by_bin = ((bins - 1).bit_length() + 7) // 8
+    return {
+        "depth_sort": ("hbm", depth, "B"),
+        # order, offset and descriptor per record; entries written, sorted, read for the
+        # bins' bounds, the counts and the placement; the lists written
+        "tile_sort": ("hbm", 16.0 * R + (24.0 + 20.0 * by_bin) * S + 4.0 * K, "B"),
+        # lengths scanned, ranges, and the processing order (which reads them twice)
+        "ranges": ("hbm", 72.0 * int(rz.layout.tiles), "B"),
+    }
 
 
 # DRAM bytes (read + write) per launch of the blend kernels, from the ncu
@@ -802,6 +833,7 @@ def roofline(stages, args, needed, rz, clk, V, pixels, blended):
     mhz = (clk or {}).get("sm_mhz") or peaks.get("clocks_under_load", {}).get("sm_mhz_median", 1455.0)
     alu_peak = sms * FP32_LANES_PER_SM * 2 * mhz * 1e6 / 1e12
     work, blended = stage_work(rz, needed, V, pixels, blended)
+    work.update(list_work(rz, needed))
     table = {}
     for name, (ms_total, launches) in stages.items():
         if not launches or name not in work:
