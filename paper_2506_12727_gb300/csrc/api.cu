@@ -125,7 +125,7 @@ struct Plan {
     // workspace offsets (forward)
     size_t w_cams = 0, w_counts = 0, w_vis = 0, w_scan = 0, w_dkeys_a = 0, w_dkeys_b = 0, w_ids_a = 0, w_ids_b = 0,
            w_order = 0, w_bins = 0, w_desc = 0, w_bins_by_depth = 0, w_bin_off = 0, w_keys_a = 0, w_keys_b = 0, w_vals_a = 0, w_vals_b = 0,
-           w_radix = 0, w_lists = 0, w_torder = 0, w_counter = 0, w_dcount = 0;
+           w_radix = 0, w_lists = 0, w_counter = 0, w_dcount = 0;
     // workspace offsets of the sampled blend (forward and backward each carve their own)
     size_t w_chunk_off = 0, w_chunk_map = 0, w_chunk_tmp = 0, w_mask = 0;
     size_t b_chunk_off = 0, b_chunk_map = 0, b_chunk_tmp = 0, b_mask = 0;
@@ -228,8 +228,7 @@ mvgs_status make_plan(long long n, const mvgs_camera* cams, int V, const mvgs_co
 
     Carver w;
     P.w_cams = w.take((size_t)V * sizeof(DevCam));
-    const size_t big = R > K ? R : K;
-    P.w_scan = w.take(scan_temp_bytes(big > (size_t)n ? big : (size_t)n));
+    P.w_scan = w.take(scan_temp_bytes(R > (size_t)n ? R : (size_t)n));
     // Two zones that are used twice.  The first: the records' bin counts, with the
     // participation beside them until the records are there and the depth sort's
     // arrays after that; then the (record, bin) entries as they are generated.
@@ -258,10 +257,9 @@ mvgs_status make_plan(long long n, const mvgs_camera* cams, int V, const mvgs_co
     P.w_keys_b = w.take(K * sizeof(uint32_t));
     P.w_vals_b = w.take(K * sizeof(uint32_t));
     w.reach(z2);
-    P.w_radix = w.take(radix_temp_bytes(big));
+    P.w_radix = w.take(radix_temp_bytes(R > K ? R : K));
     // every (record, bin) entry holds at least one tile: at most K of them
     P.w_lists = w.take(tile_lists_temp_bytes(K, bins, tiles));
-    P.w_torder = w.take(tile_order_temp_bytes(tiles));
     P.w_counter = w.take(sizeof(int));
     P.w_dcount = w.take((8 + kSumWords) * sizeof(unsigned long long));
     // runs of at least 32 samples: at most one partial run per tile
@@ -591,7 +589,7 @@ static mvgs_status render_impl(const mvgs_scene* scene, const mvgs_camera* cams,
                at<void>(workspace, P.w_lists), at<void>(workspace, P.w_radix), s);
     {
         StageTimer t(MVGS_STAGE_RANGES, s);
-        tile_order(ranges, P.tiles, at<uint32_t>(state, L.off_tile_order), at<void>(workspace, P.w_torder), s);
+        tile_order(ranges, P.tiles, at<uint32_t>(state, L.off_tile_order), s);
     }
     int* queue = at<int>(workspace, P.w_counter);  // the blend's, set to 0 with the counts
     if (capt)

@@ -189,12 +189,6 @@ __device__ __forceinline__ float4 exp2_coeffs(float4 co) {
     return make_float4(__fmul_rn(-0.5f * L, co.x), __fmul_rn(-L, co.y), __fmul_rn(-0.5f * L, co.z), co.w);
 }
 
-// Conic (A, B, C) back from the base-2 coefficients (gradients need it).
-__device__ __forceinline__ float3 conic_of(float4 q) {
-    constexpr float LN2 = 0.6931471805599453f;
-    return make_float3(-2.f * LN2 * q.x, -LN2 * q.y, -2.f * LN2 * q.z);
-}
-
 // A record's tile rectangle and view for the duplication, in 8 bytes: the
 // corners x0, y0, x1, y1 (tile coordinates, end exclusive, each below 2^12)
 // in bits 0-47 and the view in bits 48-63.

@@ -123,8 +123,7 @@ void tile_lists(const uint32_t* order, const uint32_t* bin_off, Count R, Count S
                 long long* ranges, uint64_t S_cap, void* tmp, void* radix_tmp, cudaStream_t s);
 
 // Tiles ordered by decreasing list length (the blend's processing order).
-size_t tile_order_temp_bytes(long long tiles);
-void tile_order(const long long* ranges, long long tiles, uint32_t* order, void* tmp, cudaStream_t s);
+void tile_order(const long long* ranges, long long tiles, uint32_t* order, cudaStream_t s);
 
 // ---- blend.cu --------------------------------------------------------------
 struct BlendArgs {

@@ -103,8 +103,7 @@ __global__ void __launch_bounds__(SC_THREADS) scan_reduce_kernel(Load ld, Count 
 }
 
 template <class T>
-__global__ void __launch_bounds__(SPINE_THREADS) scan_spine_kernel(T* partials, uint64_t nb, T* total_out,
-                                                                   T* end_out, Count cn) {
+__global__ void __launch_bounds__(SPINE_THREADS) scan_spine_kernel(T* partials, uint64_t nb, T* end_out, Count cn) {
     chained();
     __shared__ T buf[33];
     T carry = 0;
@@ -116,8 +115,7 @@ __global__ void __launch_bounds__(SPINE_THREADS) scan_spine_kernel(T* partials, 
         if (i < nb) partials[i] = ex + carry;
         carry += tot;
     }
-    if (threadIdx.x == 0 && total_out) *total_out = carry;
-    if (threadIdx.x == 0 && end_out) end_out[cn.get()] = carry;
+    if (threadIdx.x == 0) end_out[cn.get()] = carry;
 }
 
 __device__ __forceinline__ int pad_index(int i) { return i + (i >> 5); }
@@ -127,8 +125,7 @@ __device__ __forceinline__ int pad_index(int i) { return i + (i >> 5); }
 enum ScanBase { SPINE, PARTIALS, INPUT };
 
 template <class Load, class T>
-__global__ void __launch_bounds__(SC_THREADS) scan_down_kernel(Load ld, Count cn, ScanBase mode, const T* partials, T* out,
-                                                               T* total_out, T* end_out) {
+__global__ void __launch_bounds__(SC_THREADS) scan_down_kernel(Load ld, Count cn, ScanBase mode, const T* partials, T* out) {
     chained();
     __shared__ T tile[SC_TILE + SC_TILE / 32];
     __shared__ T buf[33];
@@ -162,10 +159,7 @@ __global__ void __launch_bounds__(SC_THREADS) scan_down_kernel(Load ld, Count cn
     }
     T total;
     T run = block_exclusive_scan<T>(sum, buf, total) + first;
-    if (mode != SPINE && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
-        if (total_out) *total_out = first + total;
-        if (end_out) end_out[n] = first + total;
-    }
+    if (mode != SPINE && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = first + total;
 #pragma unroll
     for (int k = 0; k < SC_ITEMS; k++) {
         tile[pad_index(threadIdx.x * SC_ITEMS + k)] = run;
@@ -180,18 +174,15 @@ __global__ void __launch_bounds__(SC_THREADS) scan_down_kernel(Load ld, Count cn
 
 uint64_t ceil_div_u64(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
 
-// Exclusive scan of ld(0 .. n); the total goes to out[n] when write_end, and
-// to *total_out when given.
+// Exclusive scan of ld(0 .. n); the total goes to out[n].
 template <class Load, class T>
-void scan_impl(Load ld, T* out, Count n, bool write_end, T* total_out, void* tmp, cudaStream_t s) {
+void scan_impl(Load ld, T* out, Count n, void* tmp, cudaStream_t s) {
     if (n.max == 0) {
-        if (total_out) cudaMemsetAsync(total_out, 0, sizeof(T), s);
-        if (write_end) cudaMemsetAsync(out, 0, sizeof(T), s);
+        cudaMemsetAsync(out, 0, sizeof(T), s);
         return;
     }
     const uint64_t nb = ceil_div_u64(n.max, SC_TILE);
     T* partials = static_cast<T*>(tmp);
-    T* end = write_end ? out : nullptr;
     // A launch costs a dependent kernel some 3 us: up to 5 blocks sum what
     // lies before them from the input, up to 1024 from the blocks' sums.
     const ScanBase mode = nb <= 5 ? INPUT : nb <= 1024 ? PARTIALS : SPINE;
@@ -200,10 +191,10 @@ void scan_impl(Load ld, T* out, Count n, bool write_end, T* total_out, void* tmp
         note_launches(1);
     }
     if (mode == SPINE) {
-        launch_chained(scan_spine_kernel<T>, 1, SPINE_THREADS, 0, s, partials, nb, total_out, end, n);
+        launch_chained(scan_spine_kernel<T>, 1, SPINE_THREADS, 0, s, partials, nb, out, n);
         note_launches(1);
     }
-    launch_chained(scan_down_kernel<Load, T>, (unsigned)nb, SC_THREADS, 0, s, ld, n, mode, partials, out, total_out, end);
+    launch_chained(scan_down_kernel<Load, T>, (unsigned)nb, SC_THREADS, 0, s, ld, n, mode, partials, out);
     note_launches(1);
 }
 
@@ -940,19 +931,19 @@ __global__ void ranges_kernel(const unsigned long long* starts, long long tiles,
 size_t scan_temp_bytes(uint64_t n) { return (ceil_div_u64(n, SC_TILE) + 1) * sizeof(unsigned long long); }
 
 void scan_i32_to_i64(const int* in, long long* out, uint64_t n, void* tmp, cudaStream_t s) {
-    scan_impl(LoadDirect<int, long long>{in}, out, n, true, (long long*)nullptr, tmp, s);
+    scan_impl(LoadDirect<int, long long>{in}, out, n, tmp, s);
 }
 
 void scan_masked_i32_to_i64(const int* in, int mask, long long* out, uint64_t n, void* tmp, cudaStream_t s) {
-    scan_impl(LoadMasked{in, mask}, out, n, true, (long long*)nullptr, tmp, s);
+    scan_impl(LoadMasked{in, mask}, out, n, tmp, s);
 }
 
 void scan_u32_to_u64(const uint32_t* in, unsigned long long* out, uint64_t n, void* tmp, cudaStream_t s) {
-    scan_impl(LoadDirect<uint32_t, unsigned long long>{in}, out, n, true, (unsigned long long*)nullptr, tmp, s);
+    scan_impl(LoadDirect<uint32_t, unsigned long long>{in}, out, n, tmp, s);
 }
 
 void scan_u32(const uint32_t* in, uint32_t* out, Count n, void* tmp, cudaStream_t s) {
-    scan_impl(LoadDirect<uint32_t, uint32_t>{in}, out, n, true, (uint32_t*)nullptr, tmp, s);
+    scan_impl(LoadDirect<uint32_t, uint32_t>{in}, out, n, tmp, s);
 }
 
 static uint64_t radix_blocks(uint64_t n) { return ceil_div_u64(n, RS_TILE); }
@@ -1106,9 +1097,7 @@ void tile_lists(const uint32_t* order, const uint32_t* bin_off, Count R, Count S
     }
 }
 
-size_t tile_order_temp_bytes(long long) { return 256; }
-
-void tile_order(const long long* ranges, long long tiles, uint32_t* order, void*, cudaStream_t s) {
+void tile_order(const long long* ranges, long long tiles, uint32_t* order, cudaStream_t s) {
     if (tiles <= 0) return;
     launch_chained(tile_order_kernel, 1, TO_THREADS, 0, s, ranges, tiles, order);
     note_launches(1);
