@@ -199,7 +199,7 @@ constexpr int fwd_min_blocks(int ppt, bool extra) { return ppt == 4 && !extra ? 
 // reach; the rare stop is found with one vote per Gaussian.  Gaussians for which
 // that could differ (not ordinary_gaussian) take the pixels one by one.  Batches
 // with a Gaussian that the clamp at 0.99 or a rounded exponent above 0 may touch
-// (not plain_gaussian) take a variant of the step with those two tests, two
+// (not plain, make_geom) take a variant of the step with those two tests, two
 // instructions more per pixel: 500k x 4 views with 0, 10, 40, 100% of the
 // opacities above 0.993 618, 708, 652, 607 us, where taking those Gaussians pixel
 // by pixel cost 618, 740, 777, 879.  Warp instructions per staged Gaussian (128 pixels) 109 -> 75, per 32

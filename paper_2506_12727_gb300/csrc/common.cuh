@@ -277,35 +277,28 @@ __device__ __forceinline__ Geom load_geom(const Geom* g) {
     return Geom{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 }
 
-// Whether the quadratic form of a conic stays clear of its rounding: with B^2 <=
-// 0.99 AC it is at least 1/400 of the sum of its terms' magnitudes.  The bounds
-// on A and C keep the terms of a pixel distance (0, or at least 2^-25) clear of
-// underflow and overflow.  NaN fails.
-__device__ __forceinline__ bool well_conditioned(float4 co) {
-    const float A = co.x, B = co.y, C = co.z;
-    return (A >= 1e-15f) & (A <= 1e10f) & (C >= 1e-15f) & (C <= 1e10f) & (B * B <= 0.99f * (A * C));
+// Whether the quadratic form of the conic (A, B, C) of a covariance (a, b, c) stays
+// clear of its rounding: with det = ac - b^2 >= 0.01 ac, so B^2 <= 0.99 AC, it is
+// at least 1/400 of the sum of its terms' magnitudes.  With the dilation's 0.3 in a
+// and c, A and C are at most 334; the bound on a and c keeps the terms of a pixel
+// distance (0, or at least 2^-25) clear of underflow.  NaN fails.
+__device__ __forceinline__ bool well_conditioned(float a, float c, float det) {
+    return (det >= 0.01f * (a * c)) & (a + c <= 1e15f);
 }
-
-// Whether two tests of pair_eval cannot matter for a Gaussian, so that the
-// packed blend steps may leave them out:
-//   - e <= 0: rounding (a few 2^-24 of the sum of the terms' magnitudes) cannot
-//     turn a well-conditioned form negative.
-//   - the clamp at 0.99: o G stays below it when o does (G <= 1 up to the
-//     error of ex2.approx).
-__device__ __forceinline__ bool plain_gaussian(float4 co) { return well_conditioned(co) & (co.w <= 0.989f); }
 
 // Whether blending a Gaussian with alpha 0 changes nothing, so that the packed
-// steps may take it without branches: everything they multiply with that 0 is
-// finite -- the exponent's terms and the squares of its derivatives over the
-// support (and a work item's 64 pixels past it), the colour (small enough for its
-// product with any image gradient the backward takes this way, see there) and the
-// depth.  NaN fails every comparison.
-__device__ __forceinline__ bool ordinary_gaussian(float4 co, float radius, float3 rgb, float depth) {
-    return ((fabsf(co.x) + fabsf(co.y) + fabsf(co.z)) * (radius + 64.f) <= 1e15f) & (co.w <= 1.f) &
-           (fabsf(rgb.x) + fabsf(rgb.y) + fabsf(rgb.z) <= 1e10f) & (fabsf(depth) <= 3e38f);
+// blend steps may take it without branches: everything they multiply with that 0
+// is finite -- the exponent's terms and the squares of its derivatives over the
+// support (and a work item's 64 pixels past it), the colour (not negative, and small
+// enough for its product with any image gradient the backward takes this way, see
+// there) and the depth.  NaN fails every comparison.
+__device__ __forceinline__ bool ordinary_gaussian(float4 co, float radius, float3 rgb, float depth, bool well) {
+    return (well || (fabsf(co.x) + fabsf(co.y) + fabsf(co.z)) * (radius + 64.f) <= 1e15f) &&
+           (co.w <= 1.f) & (rgb.x + rgb.y + rgb.z <= 1e10f) & (fabsf(depth) <= 3e38f);
 }
 
-__device__ __forceinline__ Geom make_geom(float2 m, float4 co, float radius, float3 rgb, float depth) {
+// A record's Geom; well: well_conditioned.
+__device__ __forceinline__ Geom make_geom(float2 m, float4 co, float radius, float3 rgb, float depth, bool well) {
     const float4 q = exp2_coeffs(co);
     const float l2 = __log2f(255.f * co.w);  // o G >= 1/255 where the exponent is -l2 or more
     float reach = -1.f;
@@ -317,13 +310,19 @@ __device__ __forceinline__ Geom make_geom(float2 m, float4 co, float radius, flo
         // item's 64 pixels past it).  At most 400 l2 2^-21 for a well-conditioned
         // form, inside the margin above; of the order of 1 for needles of 500
         // pixels, whose terms are a million times the exponent.
-        if (!well_conditioned(co)) {
+        if (!well) {
             const float far = radius + 64.f;
             reach += 0x1p-21f * (fabsf(q.x) + fabsf(q.y) + fabsf(q.z)) * far * far;
         }
     }
-    return Geom{m.x, m.y, q.x, q.y, q.z, plain_gaussian(co) ? co.w : -co.w,
-                ordinary_gaussian(co, radius, rgb, depth) ? radius : -radius, reach};
+    // plain: two tests of pair_eval cannot matter, and the packed steps leave them out
+    //   - e <= 0: rounding (a few 2^-24 of the sum of the terms' magnitudes) cannot
+    //     turn a well-conditioned form negative.
+    //   - the clamp at 0.99: o G stays below it when o does (G <= 1 up to the
+    //     error of ex2.approx).
+    const bool plain = well & (co.w <= 0.989f);
+    return Geom{m.x, m.y, q.x, q.y, q.z, plain ? co.w : -co.w,
+                ordinary_gaussian(co, radius, rgb, depth, well) ? radius : -radius, reach};
 }
 
 // Whether a Gaussian can pass the support rule and alpha >= 1/255 at any

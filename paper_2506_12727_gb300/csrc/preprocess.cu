@@ -411,6 +411,7 @@ __global__ void __launch_bounds__(PRE_THREADS, SHARED_CAMS ? 10 : 8) preprocess_
         uint32_t nt = 0, nb = 0, depth = 0;  // the record's tiles, bins and depth
         if (write) {
             const float inv = 1.f / P.det;
+            const bool well = well_conditioned(P.a, P.c, P.det);
             rec.rec_g[r] = (int)g;
             rec.rec_v[r] = v;
             rec.xy[r] = P.xy;
@@ -442,7 +443,7 @@ __global__ void __launch_bounds__(PRE_THREADS, SHARED_CAMS ? 10 : 8) preprocess_
                 if (rgb[ch] < 0.f) { clamp |= 1 << ch; rgb[ch] = 0.f; }
             }
             rec.rgb_r[r] = make_float4(rgb[0], rgb[1], rgb[2], (float)P.radius);
-            const Geom ge = make_geom(P.xy, co, (float)P.radius, make_float3(rgb[0], rgb[1], rgb[2]), P.depth);
+            const Geom ge = make_geom(P.xy, co, (float)P.radius, make_float3(rgb[0], rgb[1], rgb[2]), P.depth, well);
             float4* gout = reinterpret_cast<float4*>(rec.geom + r);
             gout[0] = make_float4(ge.mx, ge.my, ge.qa, ge.qb);
             gout[1] = make_float4(ge.qc, ge.o, ge.radius, ge.reach);
