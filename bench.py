@@ -800,10 +800,10 @@ def list_work(rz, needed):
 # kept with it); otherwise the line reports no traffic.
 BLEND_TRAFFIC = {
     "workload": "uneven_3m_8views", "tile": "32x64", "blended": 2118024889,
-    "blend_forward": 754.3e6 + 167.7e6,
-    "blend_backward": 2002.1e6 + 229.1e6,
+    "blend_forward": 755.4e6 + 167.6e6,
+    "blend_backward": 1931.1e6 + 200.4e6,
     "capture": "profiles/launches_uneven_3m_8views.md",
-    "sources_sha256": "cdbed7e399b5571221719cb12eeed8ec0caa1e001eb07ca3dcd158dd5586d331",
+    "sources_sha256": "77fe1cd5c3373a5618f030d87055d1b2aa9ea3d3cd73849d18c9e24b42af30ae",
 }
 
 
