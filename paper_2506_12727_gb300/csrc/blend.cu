@@ -1049,14 +1049,17 @@ void launch_blend_forward(const BlendArgs& a, int* counter, float* img, float* f
 // Strips up to which the backward looks at a group's alphas before it takes the
 // group.  A strip's list is walked by one warp, and the longest walks are what is
 // waited for when there are few strips, or when they are small (up to 2 pixels per
-// lane: tiles 8 high) or thinned out (a pixel mask): most of a list's Gaussians
-// then reach the strip but no pixel of it.  375k Gaussians on 64 views of some
-// 200 x 200 65 -> 32 ms, 921k x 9 views at 8 x 8 tiles 38 -> 18, 25k x 8 small
-// views at 16 x 8 1.10 -> 0.68, 20k x 3 534 -> 493 us; where every group is blended
-// it costs 3% (10k at 128 x 128 118 -> 123 us), so not for the large renders of
-// tall tiles (sampled pixels of 500k x 4 views 1028 -> 1107).  Sampled pixels fill
-// a part of the strips (a quarter of them with four views to a group), so their
-// line lies four times as far (61k Gaussians on 64 small views 4.98 -> 2.93 ms).
+// lane: tiles 8 high): most of a list's Gaussians then reach the strip but no pixel
+// of it.  375k Gaussians on 64 views of some 200 x 200 65 -> 32 ms, 921k x 9 views
+// at 8 x 8 tiles 38 -> 18, 25k x 8 small views at 16 x 8 1.10 -> 0.68, 20k x 3 534
+// -> 493 us; where every group is blended it costs 3 to 10% (500k at 1000 x 800
+// 458 -> 500 us), so not for the large renders of tall tiles (sampled pixels of 500k
+// x 4 views 1028 -> 1107, masked ones of 3M x 8 6.1 -> 6.6 ms).  Over 400 random
+// calls it gives 1.08 to 1.21x (geometric mean per range of strips, 0.82 to 2.04x)
+// up to this line and 1.00x beyond it.  Sampled or masked pixels fill a part of the
+// strips (a quarter of them with four views to a group), so their line lies four
+// times as far: 1.23 and 1.34x beyond 7500 and 15000 strips (61k Gaussians on 64
+// small views 4.98 -> 2.93 ms).
 constexpr long long kFewStrips = 7500;
 
 void launch_blend_backward(const BlendArgs& a, int* counter, const float* dimg, const float* final_T,
@@ -1074,7 +1077,7 @@ void launch_blend_backward(const BlendArgs& a, int* counter, const float* dimg, 
         case 2: MVGS_BB2(2, true); break;
         case 8: MVGS_BB2(8, true); break;
         default:
-            if (a.pixel_mask || a.tiles * a.strips <= (sampled ? 4 : 1) * kFewStrips) MVGS_BB2(4, true);
+            if (a.tiles * a.strips <= (sampled || a.pixel_mask ? 4 : 1) * kFewStrips) MVGS_BB2(4, true);
             else MVGS_BB2(4, false);
             break;
     }
