@@ -800,10 +800,10 @@ def list_work(rz, needed):
 # kept with it); otherwise the line reports no traffic.
 BLEND_TRAFFIC = {
     "workload": "uneven_3m_8views", "tile": "32x64", "blended": 2118024889,
-    "blend_forward": 755.4e6 + 167.6e6,
-    "blend_backward": 1931.1e6 + 200.4e6,
+    "blend_forward": 758.3e6 + 167.8e6,
+    "blend_backward": 1924.3e6 + 199.4e6,
     "capture": "profiles/launches_uneven_3m_8views.md",
-    "sources_sha256": "77fe1cd5c3373a5618f030d87055d1b2aa9ea3d3cd73849d18c9e24b42af30ae",
+    "sources_sha256": "1c37adcd134a2abef308cbe581db7685f11701e1d2179d3be540381a883dce99",
 }
 
 
